@@ -315,6 +315,16 @@ fa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
         return ((long long)b * Sq + row_token(r)) * p.Hq + hk * g_all + hh;
     };
 
+    if (tid == 0) {
+        for (int i = 0; i < 2 * kStages; ++i) mbar_init(smem_u32(&bars[i]), 1);
+        for (int i = 0; i < kStages; ++i) mbar_init(smem_u32(&bars[2 * kStages + i]), 4);  // one arrival per consumer warp
+        abort_flag = 0;
+        fence_mbar_init();
+        tma_prefetch_desc(&tm_k);
+        tma_prefetch_desc(&tm_v);
+    }
+    grid_dep_launch();
+    grid_dep_wait();
     int len = p.seqlens[b];
     len = max(0, min(len, p.Smax));
     const int k_begin = c * p.chunk;
@@ -334,12 +344,6 @@ fa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
     }
     const int n_tiles = (k_end - k_begin + kDecTile - 1) / kDecTile;
 
-    if (tid == 0) {
-        for (int i = 0; i < 2 * kStages; ++i) mbar_init(smem_u32(&bars[i]), 1);
-        for (int i = 0; i < kStages; ++i) mbar_init(smem_u32(&bars[2 * kStages + i]), 4);  // one arrival per consumer warp
-        abort_flag = 0;
-        fence_mbar_init();
-    }
     __syncthreads();
 
     if (warp == 4) {
@@ -628,12 +632,11 @@ fa_decode_combine_kernel(const DecodeParams p, T* o, float* lse) {
     // lse is [B,Hq,Sq]
     const long long lse_at = ((long long)b * p.Hq + bh % p.Hq) * p.Sq + (bh / p.Hq) % p.Sq;
     const int tid = threadIdx.x;
+    grid_dep_launch();
+    grid_dep_wait();   // the split kernel's partial results are complete and visible from here on
     int len = p.seqlens[b];
     len = max(0, min(len, p.Smax));
     const int nc = (len + p.chunk - 1) / p.chunk;
-    // launched as a programmatic dependent of the split kernel: its partial results are
-    // complete and visible from here on (returns at once in an ordinary launch)
-    asm volatile("griddepcontrol.wait;" ::: "memory");
     const float* lp = p.lse_part + (long long)bh * p.n_chunks;
     const float* op = p.o_part + (long long)bh * p.n_chunks * D;
     float M = -INFINITY;

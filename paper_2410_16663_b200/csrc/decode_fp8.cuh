@@ -58,6 +58,16 @@ fa_decode_split_fp8_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
     const int h0 = hk * g_all + sub * 16;          // first query head of this CTA
     const int G = min(16, g_all - sub * 16);       // its number of query heads
 
+    if (tid == 0) {
+        for (int i = 0; i < 2 * kDec8Stages; ++i) mbar_init(smem_u32(&bars[i]), 1);
+        for (int i = 0; i < kDec8Stages; ++i) mbar_init(smem_u32(&bars[2 * kDec8Stages + i]), kDec8Warps);  // one arrival per consumer warp
+        abort_flag = 0;
+        fence_mbar_init();
+        tma_prefetch_desc(&tm_k);
+        tma_prefetch_desc(&tm_v);
+    }
+    grid_dep_launch();
+    grid_dep_wait();
     int len = p.seqlens[b];
     len = max(0, min(len, p.Smax));
     const int k_begin = c * p.chunk;
@@ -74,12 +84,6 @@ fa_decode_split_fp8_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
     }
     const int n_tiles = (k_end - k_begin + kDecTile - 1) / kDecTile;
 
-    if (tid == 0) {
-        for (int i = 0; i < 2 * kDec8Stages; ++i) mbar_init(smem_u32(&bars[i]), 1);
-        for (int i = 0; i < kDec8Stages; ++i) mbar_init(smem_u32(&bars[2 * kDec8Stages + i]), kDec8Warps);  // one arrival per consumer warp
-        abort_flag = 0;
-        fence_mbar_init();
-    }
     __syncthreads();
 
     if (warp == kDec8Warps) {

@@ -288,8 +288,7 @@ int forward_impl(const fa_params& in, cudaStream_t st) {
         if (int ce = fa::prepare_big_smem_kernel(reinterpret_cast<const void*>(kern), fa::kD64SlimSmem, &sm_count))
             return cuda_fail(static_cast<cudaError_t>(ce));
         dim3 grid(fp.n_qtiles, fp.Hq, fp.B);
-        kern<<<grid, 128, fa::kD64SlimSmem, st>>>(tq, tk, tv, fp);
-        cudaError_t e = cudaGetLastError();
+        const cudaError_t e = fa::launch_dependent(kern, grid, 128, fa::kD64SlimSmem, st, tq, tk, tv, fp);
         return e == cudaSuccess ? FA_OK : cuda_fail(e);
     }
 
@@ -302,8 +301,7 @@ int forward_impl(const fa_params& in, cudaStream_t st) {
         rc = encode_map(&tvh, p.v, p.B, p.Skv, p.Hkv, p.v_stride[0], p.v_stride[1], p.v_stride[2], 64, bf16, p.d);
         if (rc) return rc;
         dim3 grid(fp.n_qtiles, fp.Hq, fp.B);
-        kern<<<grid, fa::kD256Threads, fa::kD256Smem, st>>>(tq, tk, tvh, fp);
-        cudaError_t e = cudaGetLastError();
+        const cudaError_t e = fa::launch_dependent(kern, grid, fa::kD256Threads, fa::kD256Smem, st, tq, tk, tvh, fp);
         return e == cudaSuccess ? FA_OK : cuda_fail(e);
     }
 
@@ -726,17 +724,7 @@ int decode_check_args(const void* q, const void* k_cache, const void* v_cache, c
 // writes are visible.
 template <typename T, int D>
 cudaError_t launch_combine(const fa::DecodeParams& dp, int blocks, void* o, float* lse, cudaStream_t st) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(blocks);
-    cfg.blockDim = dim3(D);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, fa::fa_decode_combine_kernel<T, D>, dp, static_cast<T*>(o), lse);
+    return fa::launch_dependent(fa::fa_decode_combine_kernel<T, D>, dim3(blocks), D, 0, st, dp, static_cast<T*>(o), lse);
 }
 
 // Launch of the split kernel and of the merge for one head dimension.
@@ -760,8 +748,7 @@ int decode_launch(const CUtensorMap& tk, const CUtensorMap& tv, const fa::Decode
         if (int ce = fa::prepare_big_smem_kernel(reinterpret_cast<const void*>(kern), smem, &sm_count))
             return cuda_fail(static_cast<cudaError_t>(ce));
         dim3 grid(Hkv * ((g * Sq + 15) / 16), dp.n_chunks, B);   // 16 (token, head) rows per CTA
-        kern<<<grid, fa::kDecMmaThreads, smem, st>>>(tk, tv, dp);
-        cudaError_t e = cudaGetLastError();
+        const cudaError_t e = fa::launch_dependent(kern, grid, fa::kDecMmaThreads, smem, st, tk, tv, dp);
         if (e != cudaSuccess) return cuda_fail(e);
     }
     if (direct) return FA_OK;
@@ -894,8 +881,7 @@ static int decode_fp8_impl(const void* q, const void* k_cache, const void* v_cac
         if (int ce = fa::prepare_big_smem_kernel(reinterpret_cast<const void*>(kern), smem, &sm_count))
             return cuda_fail(static_cast<cudaError_t>(ce));
         dim3 grid(Hkv * ((g + 15) / 16), dp.n_chunks, B);
-        kern<<<grid, fa::kDec8Threads, smem, st>>>(tk, tv, dp);
-        cudaError_t e = cudaGetLastError();
+        const cudaError_t e = fa::launch_dependent(kern, grid, fa::kDec8Threads, smem, st, tk, tv, dp);
         rc = e == cudaSuccess ? FA_OK : cuda_fail(e);
         if (rc) return rc;
     }

@@ -107,6 +107,8 @@ fa_fwd_d64_stream_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
         tmem_alloc(smem_u32(&tmem_holder), 512);
         tmem_relinquish();
     }
+    if (p.early_next) grid_dep_launch();
+    grid_dep_wait();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -389,8 +391,9 @@ int launch_d64_stream(const CUtensorMap& tq, const CUtensorMap& tk, const CUtens
     const long long total = (long long)n_qpairs * fp.B * fp.Hq;
     if (total > 0x7fffffffll) return -3;
     const int grid = (int)(total < sm_count ? total : sm_count);
-    kern<<<grid, kD64StThreads, kD64StSmem, st>>>(tq, tk, tv, fp, n_qpairs, (int)total);
-    cudaError_t e = cudaGetLastError();
+    FwdParams fpc = fp;
+    fpc.early_next = grid < sm_count;
+    const cudaError_t e = launch_dependent(kern, dim3(grid), kD64StThreads, kD64StSmem, st, tq, tk, tv, fpc, n_qpairs, (int)total);
     if (e != cudaSuccess) { *cuda_err = (int)e; return -7; }
     return 0;
 }

@@ -636,6 +636,8 @@ __device__ __forceinline__ bool pp_attention(const CUtensorMap& tm_q, const CUte
         tmem_alloc(smem_u32(&ss.tmem_holder), 512);
         tmem_relinquish();
     }
+    if (p.early_next) grid_dep_launch();
+    grid_dep_wait();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -956,9 +958,9 @@ int launch_pingpong(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensor
     const long long total = (long long)fp.n_qtiles * fp.B * fp.Hq;
     if (total > 0x7fffffffll) return -3;
     const int grid = (int)(total < sm_count ? total : sm_count);
-    const FwdParams fpc = pp_plan_items(fp, grid, (kF8 || D == 64) ? 256.0 : 512.0);
-    kern<<<grid, kPipeThreads, smem, st>>>(tq, tk, tv, to, fpc, (int)total);
-    e = cudaGetLastError();
+    FwdParams fpc = pp_plan_items(fp, grid, (kF8 || D == 64) ? 256.0 : 512.0);
+    fpc.early_next = grid < sm_count;
+    e = launch_dependent(kern, dim3(grid), kPipeThreads, smem, st, tq, tk, tv, to, fpc, (int)total);
     if (e != cudaSuccess) { *cuda_err = (int)e; return -7; }
     return 0;
 }

@@ -466,6 +466,8 @@ fa_fwd_pipelined_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
         tmem_alloc(smem_u32(&tmem_holder), 512);
         tmem_relinquish();
     }
+    if (p.early_next) grid_dep_launch();
+    grid_dep_wait();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -620,8 +622,9 @@ int launch_pipelined(const CUtensorMap& tq, const CUtensorMap& tk, const CUtenso
     const long long total = (long long)n_qpairs * fp.B * fp.Hq;
     if (total > 0x7fffffffll) return -3;
     const int grid = (int)(total < sm_count ? total : sm_count);
-    kern<<<grid, kPipeThreads, smem, st>>>(tq, tk, tv, fp, (int)total, n_qpairs);
-    e = cudaGetLastError();
+    FwdParams fpc = fp;
+    fpc.early_next = grid < sm_count;
+    e = launch_dependent(kern, dim3(grid), kPipeThreads, smem, st, tq, tk, tv, fpc, (int)total, n_qpairs);
     if (e != cudaSuccess) { *cuda_err = (int)e; return -7; }
     return 0;
 }

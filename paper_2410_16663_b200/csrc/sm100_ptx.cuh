@@ -117,6 +117,16 @@ __global__ void fa_selftest_wait_kernel(unsigned long long limit_ns, unsigned in
     if (!ok) atomicAdd(gave_up, 1u);
 }
 
+// ------------------------------------------------------------------ programmatic dependent launch
+// Every attention kernel is launched as a programmatic dependent of whatever precedes it in the
+// stream (launch_dependent in prefill_simple.cuh): its CTAs may start, and set up their barriers and
+// tensor memory, while the kernel before it still runs.  grid_dep_wait() blocks until that kernel
+// has completed and its writes are visible; nothing may read or write global memory before it.
+// grid_dep_launch() lets the next kernel of the stream start in the same way as soon as every CTA of
+// this one has begun.  Both do nothing in an ordinary launch.
+__device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // ------------------------------------------------------------------ proxies / fences
 __device__ __forceinline__ void fence_proxy_async_smem() {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");

@@ -1414,3 +1414,39 @@ def test_a_wait_that_cannot_be_satisfied_gives_up_and_is_reported(fa):
     o_ref, l_ref = oracle.attention_full(q, k, v, c.causal, c.scale)
     o, lse = run_forward(fa, q.to(DEV), k.to(DEV), v.to(DEV), c.causal, c.scale)
     assert_close_to_oracle(o, lse, o_ref, l_ref, what="C1 after the self-test")
+
+
+@pytest.mark.parametrize("B,H,S,d", [(1, 2, 200, 128), (1, 3, 1100, 128), (8, 16, 1100, 128), (4, 40, 300, 128), (1, 2, 100, 64),
+                                     (2, 3, 197, 64), (1, 2, 300, 256)])
+def test_calls_that_follow_each_other_in_a_stream_see_each_others_results(fa, B, H, S, d):
+    # every kernel is launched as a programmatic dependent of the one before it and may set itself
+    # up while that one still runs; it must read nothing that is not final, and write over nothing
+    # that is still read.  Eight calls, each on the output of the one before, through two buffers in
+    # turn, against the same calls with the GPU waited for in between: bit for bit the same.
+    def chain(wait):
+        gen = torch.Generator(device=DEV)
+        gen.manual_seed(4)
+        x = torch.randn(B, S, H, d, device=DEV, generator=gen).to(torch.float16)
+        y = torch.empty_like(x)
+        lse = torch.empty(B, H, S, device=DEV)
+        cache = torch.randn(B, S, H, 128, device=DEV, generator=gen).to(torch.float16)
+        lens = torch.full((B,), S, dtype=torch.int32, device=DEV)
+        ws = torch.empty(fa.fa_decode_workspace_bytes(B, H, H, S, 128) + 16, dtype=torch.uint8, device=DEV)
+        outs = []
+        for i in range(8):
+            fa.fa_forward(x, x, x, y, lse, bool(i & 1), 0.4)
+            if wait:
+                torch.cuda.synchronize()
+            if d == 128:   # the last row of every sequence through the decode kernels, in place
+                row = y[:, -1:].contiguous()
+                fa.fa_decode(row, y, cache, row, None, lens, 0.3, ws)
+                if wait:
+                    torch.cuda.synchronize()
+                y[:, -1:] = row
+            x, y = y, x
+            outs.append(x.clone())
+        torch.cuda.synchronize()
+        return outs
+    for a, b in zip(chain(True), chain(False)):
+        assert torch.equal(a, b)
+    check_status(fa)
