@@ -82,7 +82,6 @@ fa_fwd_d256_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     const int off = p.Skv - p.Sq;
     const int n_tiles = kv_tiles_for(q0, kTile, p.Sq, p.Skv, p.causal);
 
-    grid_dep_launch();
     grid_dep_wait();
     if (tid == 128) {
         for (int i = 0; i < 13; ++i) mbar_init(smem_u32(&bars[i]), (i == 8 || i == 9) ? 128 : 1);
@@ -105,6 +104,7 @@ fa_fwd_d256_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    grid_dep_launch();
     const uint32_t tmem_base = tmem_holder;
 
     constexpr bool kBf16 = std::is_same<T, __nv_bfloat16>::value;

@@ -67,11 +67,11 @@ fa_fwd_d64_slim_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
         tmem_alloc(smem_u32(&tmem_holder), 128);
         tmem_relinquish();
     }
-    grid_dep_launch();
     grid_dep_wait();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    grid_dep_launch();
     const uint32_t tmem_base = tmem_holder;
     const uint32_t tS = tmem_base + (static_cast<uint32_t>(warp * 32) << 16);
 

@@ -636,11 +636,11 @@ __device__ __forceinline__ bool pp_attention(const CUtensorMap& tm_q, const CUte
         tmem_alloc(smem_u32(&ss.tmem_holder), 512);
         tmem_relinquish();
     }
-    if (p.early_next) grid_dep_launch();
     grid_dep_wait();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    if (p.early_next) grid_dep_launch();
     const uint32_t tmem_base = ss.tmem_holder;
     const int off = p.Skv - p.Sq;
 

@@ -466,11 +466,11 @@ fa_fwd_pipelined_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
         tmem_alloc(smem_u32(&tmem_holder), 512);
         tmem_relinquish();
     }
-    if (p.early_next) grid_dep_launch();
     grid_dep_wait();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    if (p.early_next) grid_dep_launch();
     const uint32_t tmem_base = tmem_holder;
     const int off = p.Skv - p.Sq;
 

@@ -123,7 +123,10 @@ __global__ void fa_selftest_wait_kernel(unsigned long long limit_ns, unsigned in
 // tensor memory, while the kernel before it still runs.  grid_dep_wait() blocks until that kernel
 // has completed and its writes are visible; nothing may read or write global memory before it.
 // grid_dep_launch() lets the next kernel of the stream start in the same way as soon as every CTA of
-// this one has begun.  Both do nothing in an ordinary launch.
+// this one has issued it (the first thread of a CTA counts).  A kernel with tensor memory issues it
+// after the barrier behind its allocation: an early CTA of the next kernel on the same SM could
+// otherwise get columns that a CTA of this one still needs, and each would wait for the other.
+// Both do nothing in an ordinary launch.
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
