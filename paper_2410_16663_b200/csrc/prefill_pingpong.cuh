@@ -40,6 +40,7 @@ namespace fa {
 constexpr int kPpNK = FA_PP_NK;   // K ring slots
 constexpr int kPpNV = FA_PP_NV;   // V ring slots
 constexpr int kPpQBufs = 2;
+constexpr int kPpSlots = 4;       // work items the Q/K loader may be ahead of the slowest role
 static_assert((kPpQBufs + kPpNK + kPpNV) * kTileBytes + 3072 <= 232448, "shared memory budget");
 
 // What changes with FP8 e4m3 operands (kF8; Appendix D.2 evaluates the operator with 8-bit
@@ -76,8 +77,11 @@ constexpr int v_empty = v_full + kPpNV;         // [NV]
 constexpr int s_full = v_empty + kPpNV;         // [2]  S thread (commit) -> softmax
 constexpr int pv_done = s_full + 2;             // [2]  PV thread (commit) -> softmax
 constexpr int o_final = pv_done + 2;            // [2]  PV thread (commit) -> epilogue, by item parity
+constexpr int item_full = o_final + 2;          // [kPpSlots] Q/K loader -> every other role: a work item is in the slot
+constexpr int item_empty = item_full + kPpSlots;   // [kPpSlots] back: three single-thread roles and eight softmax warps
+constexpr int claim = item_empty + kPpSlots;    // [1]  answer to a claim of work (cluster launch control) -> Q/K loader
 // barriers every thread of a softmax warpgroup arrives on (count 128)
-constexpr int p_full = o_final + 2;             // [2]  softmax -> PV thread
+constexpr int p_full = claim + 1;               // [2]  softmax -> PV thread
 constexpr int m_ready = p_full + 2;             // [2]  softmax of step g -> softmax of step g+1 (reference max
                                                 //      published) and -> S thread (scores read out of S_{g&1})
 constexpr int l_pub = m_ready + 2;              // [2]  softmax of an item's last-but-one step -> of its last step
@@ -85,23 +89,26 @@ constexpr int o_free = l_pub + 2;               // [1]  epilogue -> PV thread
 constexpr int count = o_free + 1;
 }  // namespace ppb
 
+struct __align__(16) PpItem {
+    int q0, n;      // first query row of the tile, kv tiles it visits (0: no further item)
+    int b, h, hk;
+    // packed variable-length batches only: first row of the sequence in q/o and in k/v, and
+    // the sequence's own lengths
+    int q_base, k_base, Sq, Skv;
+    int page0;   // paged K/V: the sequence's first table entry (-1 for a sequence without keys)
+};
+
 struct PpStatic {
     uint64_t bars[ppb::count];
     uint32_t tmem_holder;
     uint32_t abort_flag;
     float m_xch[2][128];   // [warpgroup][row]: reference max after that warpgroup's latest step
     float l_xch[2][128];   // [item parity][row]: row sum of the warpgroup that does not run the last step
-    uint8_t pad[3072 - ppb::count * 8 - 8 - 4 * 128 * 4];
+    PpItem items[kPpSlots];    // decoded work items, written by the Q/K loader (see PpSource)
+    uint4 claim_answer;
 };
-static_assert(sizeof(PpStatic) == 3072, "static shared state must fill exactly 3 KiB");
-
-struct PpItem {
-    int b, h, hk, q0, n;
-    // packed variable-length batches only: first row of the sequence in q/o and in k/v, and
-    // the sequence's own lengths
-    int q_base, k_base, Sq, Skv;
-    int page0;   // paged K/V: the sequence's first table entry (-1 for a sequence without keys)
-};
+constexpr int kPpStaticBytes = 3072;   // the static shared memory of the kernels: PpStatic and padding
+static_assert(sizeof(PpStatic) <= kPpStaticBytes && sizeof(PpStatic) > kPpStaticBytes - 1024, "static shared state fills 3 KiB");
 
 // Work item `idx`.  The query tiles of a head are taken in classes of C = 2^cls_log2 consecutive
 // tiles, the class of the last (longest) tiles first; inside a class the items go head by head,
@@ -110,10 +117,6 @@ struct PpItem {
 // read them, and the rounds still get shorter and shorter items, which keeps the static
 // assignment balanced (the launcher picks C from the K/V bytes of a head, see launch_pingpong).
 // C >= n_qtiles is the plain head-by-head order used for very long sequences.
-// kVarlen: the sequence's lengths come from the prefix sums; n == 0 marks an item past the end
-// of its sequence (every role skips it), and a live item visits at least one kv tile (so that
-// rows without any visible key are still written, as zeros).
-template <bool kVarlen>
 __device__ __forceinline__ void pp_class_order(const FwdParams& p, int idx, int& bh, int& qt) {
     int c, rem;  // class, index inside the class
     p.by_class.divmod(idx, c, rem);
@@ -128,11 +131,15 @@ __device__ __forceinline__ void pp_class_order(const FwdParams& p, int idx, int&
     qt = p.n_qtiles - 1 - first - j;
 }
 
-// The work item that is query tile qt of (batch, head) pair bh.
+// The work item that is query tile qt of head h of batch entry b.
+// kVarlen: the sequence's lengths come from the prefix sums; n == 0 marks an item past the end
+// of its sequence (nobody works on it), and a live item visits at least one kv tile (so that
+// rows without any visible key are still written, as zeros).
 template <bool kVarlen>
-__device__ __forceinline__ PpItem pp_decode_item(const FwdParams& p, int bh, int qt) {
+__device__ __forceinline__ PpItem pp_decode_item(const FwdParams& p, int b, int h, int qt) {
     PpItem it;
-    p.by_hq.divmod(bh, it.b, it.h);
+    it.b = b;
+    it.h = h;
     it.hk = p.by_group.div(it.h);
     it.q0 = qt * kTile;
     if (kVarlen) {
@@ -157,47 +164,143 @@ __device__ __forceinline__ PpItem pp_decode_item(const FwdParams& p, int bh, int
     return it;
 }
 
-// The items of this CTA in order.  `ord` counts the items the CTA works on (it selects the
-// double buffers); with variable-length batches the items past the end of their sequence are
-// passed over, identically in every role.
-// Very long sequences (rounds_per_head > 0; one head's K and V no longer fit in L2) go head by
-// head, and every head takes a whole number of rounds of the grid: in round r of a head CTA b
-// takes the head's (r * gridDim.x + b)-th longest tile -- b counted from the other end in every
-// second round, and the other way around for every second head -- and nothing if the head has no
-// such tile (only in a head's last round, whose items are its shortest).  The CTAs of a round
-// then all walk the same head's keys from the first on, a few dozen tiles apart at most, and
+// Where a CTA's work items come from.  One thread, the Q/K loader, decides and decodes them and
+// hands them to the other roles through a ring of slots in shared memory (PpItem, item_full,
+// item_empty): an item costs the others one barrier wait and one or two 16-byte reads instead of
+// the divisions and, in packed batches, the dependent global loads of the decoding.
+//
+// The list is dealt to the CTAs for its first p.deal_rounds rounds, in alternating direction, and
+// claimed from there on (p.claim_items): the grid has one CTA for every remaining item on top of the
+// deal_ctas that run, and a running CTA claims the items of CTAs that have not started through
+// cluster launch control when it requests the last keys of the item it is on.  The launcher says
+// how much of which list is dealt and why.
+//
+// Very long sequences (rounds_per_head > 0; one head's K and V no longer fit in L2) are all dealt,
+// head by head, and every head takes a whole number of rounds of the grid: in round r
+// of a head CTA b takes the head's (r * gridDim.x + b)-th longest tile -- b counted from the other
+// end in every second round, and the other way around for every second head -- and nothing if the
+// head has no such tile (only in a head's last round, whose items are its shortest).  The CTAs of a
+// round then all walk the same head's keys from the first on, a few dozen tiles apart at most, and
 // stay together from head to head, so a K or V tile is fetched from HBM once per round and
 // found in L2 by everyone else.  (Without the padding a round straddles two heads, the CTAs
 // that get the next head's longest tiles fall a thousand tiles behind the others, and the
-// groups, each walking the head on its own, fetch everything several times.)
+// groups, each walking the head on its own, fetch everything several times.)  A cooperative
+// launch (the fused projection) is all dealt as well.
+//
+// Packed batches: the list goes sequence by sequence and head by head, a head's tiles longest
+// first.  Sequence s takes the places from floor(cu_q[s] / 128) + s on, times Hq, which leaves
+// it at least its number of tiles and at most one more per head: the host can size the grid
+// without knowing the lengths, and a place past a sequence's end is passed over.
 template <bool kVarlen>
-struct PpItems {
-    int round = -1, ord = -1;
-    PpItem it;
-    __device__ __forceinline__ bool next(const FwdParams& p, int total_items) {
+struct PpSource {
+    const FwdParams& p;
+    int total_items;
+    uint32_t claim_bar, answer;      // shared-memory addresses
+    volatile uint32_t* abort_flag;
+    int round = -1;                  // places taken so far, less one
+    int claims = 0;                  // claims answered
+    bool pending = false;            // a claim is on its way
+    int seq = 0;                     // packed batches: sequence of the last item
+
+    __device__ __forceinline__ bool dealt(int k) const { return k < p.deal_rounds && (int)blockIdx.x < p.deal_ctas; }
+    // Asks for an item (at most once).
+    __device__ __forceinline__ void request() {
+        if (p.claim_items && !pending) {
+            fence_proxy_async_smem();   // the last answer has been read
+            mbar_expect_tx(claim_bar, 16);
+            clc_request(answer, claim_bar);
+            pending = true;
+        }
+    }
+    // The same ahead of time, if the next item is a claimed one.
+    __device__ __forceinline__ void request_next() {
+        if (!dealt(round + 1)) request();
+    }
+    __device__ __forceinline__ int place_of(int s) const { return (__ldg(p.cu_q + s) >> 7) + s; }
+    __device__ __forceinline__ void packed_place(int idx, int& b, int& h, int& qt) {
+        int v, rem;
+        p.by_hq.divmod(idx, v, rem);
+        // the last sequence that starts at or before place v: items nearly always come in rising order
+        int lo = place_of(seq) <= v ? seq : 0, hi = p.B - 1;
+        for (int k = 0; lo < hi && k < 4; ++k) {
+            if (place_of(lo + 1) > v) hi = lo;
+            else ++lo;
+        }
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (place_of(mid) <= v) lo = mid;
+            else hi = mid - 1;
+        }
+        seq = b = lo;
+        const int first = place_of(lo);
+        const int tiles = max(1, place_of(lo + 1) - first);
+        rem = idx - first * p.Hq;
+        h = rem < 0 ? -1 : rem / tiles;   // (a place before the first sequence, if cu_q[0] > 0)
+        qt = tiles - 1 - (rem - h * tiles);
+    }
+    __device__ __forceinline__ bool next(PpItem& it) {
         for (;;) {
             ++round;
+            int b, h, qt;
             if (!kVarlen && p.rounds_per_head > 0) {
                 int bh, r;
                 p.by_rph.divmod(round, bh, r);
                 if (bh >= p.B * p.Hq) return false;
-                const int g = gridDim.x, b = blockIdx.x;
-                const int j = r * g + (((r + bh) & 1) ? (g - 1 - b) : b);
+                const int g = gridDim.x, x = blockIdx.x;
+                const int j = r * g + (((r + bh) & 1) ? (g - 1 - x) : x);
                 if (j >= p.n_qtiles) continue;
-                it = pp_decode_item<kVarlen>(p, bh, p.n_qtiles - 1 - j);
-                ++ord;
-                return true;
+                p.by_hq.divmod(bh, b, h);
+                qt = p.n_qtiles - 1 - j;
+            } else {
+                int idx;
+                if (dealt(round)) {
+                    idx = round * p.deal_ctas + ((round & 1) ? (p.deal_ctas - 1 - (int)blockIdx.x) : (int)blockIdx.x);
+                    if (idx >= total_items) return false;
+                } else if (!p.claim_items) {
+                    return false;
+                } else {
+                    int x = blockIdx.x;   // (a CTA past the dealt ones that was launched after all: its own place first)
+                    if (round > 0) {
+                        request();
+                        if (!mbar_wait(claim_bar, claims & 1, abort_flag, 153)) return false;
+                        ++claims;
+                        pending = false;
+                        x = clc_answer(answer);
+                        if (x < 0) return false;
+                    }
+                    idx = p.deal_rounds * p.deal_ctas + x - p.deal_ctas;
+                }
+                if (kVarlen) {
+                    packed_place(idx, b, h, qt);
+                    if (h < 0 || h >= p.Hq || qt < 0 || qt >= p.n_qtiles) continue;
+                } else {
+                    int bh;
+                    pp_class_order(p, idx, bh, qt);
+                    p.by_hq.divmod(bh, b, h);
+                }
             }
-            const int idx = item_of_round(round, total_items);
-            if (idx >= total_items) return false;
-            int bh, qt;
-            pp_class_order<kVarlen>(p, idx, bh, qt);
-            it = pp_decode_item<kVarlen>(p, bh, qt);
-            if (!kVarlen || it.n > 0) {
-                ++ord;
-                return true;
-            }
+            it = pp_decode_item<kVarlen>(p, b, h, qt);
+            if (!kVarlen || it.n > 0) return true;
         }
+    }
+};
+
+__device__ __forceinline__ uint32_t pp_bar(uint32_t bar0, int i) { return bar0 + 8 * i; }
+
+// The other roles' end of the ring: the ord-th item, read by a single thread, which hands the slot
+// back at once.  False at the end of the list or after a wait that gave up.
+struct PpTaker {
+    const PpItem* items;
+    uint32_t bar0;
+    volatile uint32_t* abort_flag;
+    int ord = -1;
+    __device__ __forceinline__ bool next(PpItem& it, unsigned int where) {
+        ++ord;
+        const int slot = ord & (kPpSlots - 1);
+        if (!mbar_wait(pp_bar(bar0, ppb::item_full + slot), (ord / kPpSlots) & 1, abort_flag, where)) return false;
+        it = items[slot];
+        mbar_arrive(pp_bar(bar0, ppb::item_empty + slot));
+        return it.n > 0;
     }
 };
 
@@ -251,8 +354,6 @@ __device__ __forceinline__ void pp_store_p<false>(uint32_t taddr, const uint32_t
 template <>
 __device__ __forceinline__ void pp_store_p<true>(uint32_t taddr, const uint32_t (&pk)[8]) { tmem_st_x8(taddr, pk); }
 
-__device__ __forceinline__ uint32_t pp_bar(uint32_t bar0, int i) { return bar0 + 8 * i; }
-
 // Counter in global memory that one SM raises after its writes and another reads before its loads.
 __device__ __forceinline__ unsigned int ld_acquire_gpu(const unsigned int* p) {
     unsigned int v;
@@ -276,18 +377,18 @@ struct PpRing {
 };
 
 // The thread that issues S = Q K^T of every step.
-template <typename T, bool kTmaOut, bool kVarlen, bool kF8, int D>
-__device__ __forceinline__ void pp_run_s(uint32_t bar0, uint32_t sQ, uint32_t sK, uint32_t tmem, const FwdParams& p,
-                                         int total_items, volatile uint32_t* abort_flag) {
+template <typename T, bool kTmaOut, bool kF8, int D>
+__device__ __forceinline__ void pp_run_s(uint32_t bar0, uint32_t sQ, uint32_t sK, uint32_t tmem, const PpItem* slots,
+                                         volatile uint32_t* abort_flag) {
     constexpr bool kBf16 = std::is_same<T, __nv_bfloat16>::value;
     constexpr uint32_t idesc = kF8 ? instr_desc_e4m3(128, 128, false, false) : instr_desc_f16(kBf16, 128, 128, false, false);
     using Op = PpOperands<kF8, D>;
     uint32_t g = 0;
     PpRing<kPpNK> ring;
-    PpItems<kVarlen> items;
-    while (items.next(p, total_items)) {
+    PpTaker items{slots, bar0, abort_flag};
+    PpItem it;
+    while (items.next(it, 133)) {
         const int ord = items.ord;
-        const PpItem& it = items.it;
         const uint32_t qb = ord & 1;
         if (!mbar_wait(pp_bar(bar0, ppb::q_full + qb), (ord >> 1) & 1, abort_flag, 130)) return;
         const uint32_t a_lo = desc_lo(sQ + qb * kTileBytes, 16);
@@ -316,18 +417,18 @@ __device__ __forceinline__ void pp_run_s(uint32_t bar0, uint32_t sQ, uint32_t sK
 }
 
 // The thread that issues O += P V of every step.
-template <typename T, bool kVarlen, bool kF8, int D>
-__device__ __forceinline__ void pp_run_pv(uint32_t bar0, uint32_t sV, uint32_t tmem, const FwdParams& p,
-                                          int total_items, volatile uint32_t* abort_flag) {
+template <typename T, bool kF8, int D>
+__device__ __forceinline__ void pp_run_pv(uint32_t bar0, uint32_t sV, uint32_t tmem, const PpItem* slots,
+                                          volatile uint32_t* abort_flag) {
     constexpr bool kBf16 = std::is_same<T, __nv_bfloat16>::value;
     constexpr uint32_t idesc = kF8 ? instr_desc_e4m3(128, 128, false, true) : instr_desc_f16(kBf16, 128, D, false, true);
     using Op = PpOperands<kF8, D>;
     uint32_t g = 0;
     PpRing<kPpNV> ring;
-    PpItems<kVarlen> items;
-    while (items.next(p, total_items)) {
+    PpTaker items{slots, bar0, abort_flag};
+    PpItem it;
+    while (items.next(it, 143)) {
         const int ord = items.ord;
-        const PpItem& it = items.it;
         for (int j = 0; j < it.n; ++j, ++g, ring.next()) {
             const uint32_t buf = g & 1;
             if (!mbar_wait(pp_bar(bar0, ppb::v_full + ring.slot), ring.par, abort_flag, 140)) return;
@@ -380,7 +481,7 @@ __device__ __forceinline__ void pp_paged_tile(const FwdParams& p, int page, int 
     }
 }
 
-// The thread that loads Q of every item and K of every step.  (Packed batches: the tensor maps
+// The thread that picks the work items (see PpSource) and loads Q of every item and K of every step.  (Packed batches: the tensor maps
 // have one batch entry that holds every sequence back to back.)
 // One tile: two 64-element boxes of a 16-bit tensor of d = 128, or one 128-byte box (8-bit, or d = 64).
 template <bool kOneBox>
@@ -392,16 +493,21 @@ __device__ __forceinline__ void pp_load_tile(uint32_t dst, const CUtensorMap* tm
 
 template <bool kVarlen, bool kF8, int D>
 __device__ __forceinline__ void pp_run_load_qk(uint32_t bar0, uint32_t sQ, uint32_t sK, const CUtensorMap* tm_q,
-                                               const CUtensorMap* tm_k, const FwdParams& p, int total_items,
+                                               const CUtensorMap* tm_k, const FwdParams& p, int total_items, PpStatic& ss,
                                                volatile uint32_t* abort_flag) {
     tma_prefetch_desc(tm_q);
     tma_prefetch_desc(tm_k);
     const uint64_t pol_q = l2_policy_evict_first(), pol_kv = l2_policy_evict_last();
     PpRing<kPpNK> ring;
-    PpItems<kVarlen> items;
-    while (items.next(p, total_items)) {
-        const int ord = items.ord;
-        const PpItem& it = items.it;
+    PpSource<kVarlen> source{p, total_items, pp_bar(bar0, ppb::claim), smem_u32(&ss.claim_answer), abort_flag};
+    PpItem it;
+    for (int ord = 0;; ++ord) {
+        if (!source.next(it)) it.n = 0;   // no further item: the others are told so
+        const int slot = ord & (kPpSlots - 1);
+        if (!mbar_wait(pp_bar(bar0, ppb::item_empty + slot), ((ord / kPpSlots) & 1) ^ 1, abort_flag, 154)) return;
+        ss.items[slot] = it;
+        mbar_arrive(pp_bar(bar0, ppb::item_full + slot));
+        if (it.n == 0) return;
         const uint32_t qb = ord & 1;
         // passes at once the first time each buffer is used
         if (!mbar_wait(pp_bar(bar0, ppb::q_empty + qb), ((ord >> 1) & 1) ^ 1, abort_flag, 150)) return;
@@ -411,6 +517,7 @@ __device__ __forceinline__ void pp_run_load_qk(uint32_t bar0, uint32_t sQ, uint3
         int page = (kVarlen && p.block_table != nullptr) ? it.page0 : 0;
         for (int j = 0; j < it.n; ++j, ring.next()) {
             const int page_next = pp_page_of<kVarlen>(p, it.b, j + 1, it.n, it.Skv);
+            if (j == it.n - 1) source.request_next();
             if (!mbar_wait(pp_bar(bar0, ppb::k_empty + ring.slot), ring.par ^ 1, abort_flag, 151)) return;
             mbar_expect_tx(pp_bar(bar0, ppb::k_full + ring.slot), PpOperands<kF8, D>::kKvSlotBytes);
             int row = kVarlen ? it.k_base + j * kTile : j * kTile, slab = kVarlen ? 0 : it.b;
@@ -424,14 +531,13 @@ __device__ __forceinline__ void pp_run_load_qk(uint32_t bar0, uint32_t sQ, uint3
 // The thread that loads V of every step.
 template <bool kVarlen, bool kF8, int D>
 __device__ __forceinline__ void pp_run_load_v(uint32_t bar0, uint32_t sV, const CUtensorMap* tm_v, const FwdParams& p,
-                                              int total_items, volatile uint32_t* abort_flag) {
+                                              const PpItem* slots, volatile uint32_t* abort_flag) {
     tma_prefetch_desc(tm_v);
     const uint64_t pol_kv = l2_policy_evict_last();
     PpRing<kPpNV> ring;
-    PpItems<kVarlen> items;
-    while (items.next(p, total_items)) {
-        const int ord = items.ord;
-        const PpItem& it = items.it;
+    PpTaker items{slots, bar0, abort_flag};
+    PpItem it;
+    while (items.next(it, 155)) {
         int page = (kVarlen && p.block_table != nullptr) ? it.page0 : 0;
         for (int j = 0; j < it.n; ++j, ring.next()) {
             const int page_next = pp_page_of<kVarlen>(p, it.b, j + 1, it.n, it.Skv);
@@ -475,10 +581,9 @@ struct PpSoftmax {
     float m_loc;            // reference max after this warpgroup's latest step
     float m_before;         // reference max that step received from the step before it
 
-    // Step g of the CTA = step j of the item.  kMasked: the tile is crossed by the diagonal or by
+    // Step g of the CTA = step j of the item.  masked: the tile is crossed by the diagonal or by
     // the end of the keys.  Returns false when a wait gave up.
-    template <int kMasked>  // 0: no mask code; 1: masked tile; 2: decided at run time by `masked`
-    __device__ __forceinline__ bool step(uint32_t (&s)[128], uint32_t g, int j, bool masked = false) {
+    __device__ __forceinline__ bool step(uint32_t (&s)[128], uint32_t g, int j, bool masked) {
         if (!pp_warp_wait(pp_bar(bar0, ppb::s_full + w), (g >> 1) & 1, abort_flag, 110 + w)) return false;
         tc_fence_after();
         tmem_ld_x32(tS, *reinterpret_cast<uint32_t(*)[32]>(&s[0]));
@@ -489,7 +594,7 @@ struct PpSoftmax {
         tc_fence_before();  // for the arrival below that hands the S buffer back
         // probe early, look at the answer after the row max
         const bool m_there = g > 0 && mbar_test(pp_bar(bar0, ppb::m_ready + (1 - w)), ((g - 1) >> 1) & 1);
-        if (kMasked == 1 || (kMasked == 2 && masked)) {
+        if (masked) {
             // hidden scores become -inf (the scale is strictly positive, so they come out as exact zeros)
             const int kv0 = j * kTile;
             int lim = Skv - kv0;
@@ -565,7 +670,7 @@ struct PpSoftmax {
             f2_unpack(lb, b0, b1);
             l_part += (a0 + a1) + (b0 + b1);
         }
-        if (kVarlen && (kMasked == 1 || (kMasked == 2 && masked)) && Skv - j * kTile < kTile) {
+        if (kVarlen && masked && Skv - j * kTile < kTile) {
             // Packed batches, the tile that holds a sequence's last key: the rows of V after it
             // belong to the next sequence, or to the unused rest of a page, and may hold anything.
             // Their probabilities are exact zeros, but 0 * NaN would still poison O, so those
@@ -594,11 +699,6 @@ struct PpSoftmax {
 // and each warp sends its 32 rows to global memory with two TMA stores (tm_o: boxes of 32 rows x
 // 64 columns).  Rows past the end of the queries are clipped by the tensor map.  Otherwise
 // (fp32 output) every thread stores its own row.
-// kSingle: the step exists once, and a branch skips its mask code on tiles every row sees in
-// full; otherwise those tiles take a loop of their own without mask code.  The single copy is a
-// little slower per step and much smaller: with it, what an item executes from its first step
-// to its epilogue stays within the 32 KB the instruction cache serves at full rate, which is
-// what counts when an item has few steps.
 // kVarlen (needs kTmaOut): a packed batch of sequences of different lengths (see FwdParams).
 // kF8: q, k, v hold FP8 e4m3 bytes (see PpOperands); T is then the type of the output only.
 // kProj (needs kTmaOut): a projection phase follows in the same launch (proj_gemm.cuh): a warp
@@ -606,7 +706,7 @@ struct PpSoftmax {
 // and counts them in done[batch * n_qtiles + query tile]; four warps and Hq heads make a row
 // block of O complete.
 // The whole kernel but for the release of tensor memory; returns false if nothing was set up.
-template <typename T, bool kTmaOut, bool kSingle, bool kVarlen, bool kF8, bool kProj, int D = 128>
+template <typename T, bool kTmaOut, bool kVarlen, bool kF8, bool kProj, int D = 128>
 __device__ __forceinline__ bool pp_attention(const CUtensorMap& tm_q, const CUtensorMap& tm_k, const CUtensorMap& tm_v,
                                              const CUtensorMap& tm_o, const FwdParams& p, const int total_items,
                                              PpStatic& ss, const uint32_t smem_base, unsigned int* done) {
@@ -627,7 +727,8 @@ __device__ __forceinline__ bool pp_attention(const CUtensorMap& tm_q, const CUte
     if (tid == 0) {
         for (int i = 0; i < ppb::count; ++i) {
             const bool q_back = kTmaOut && (i == ppb::q_empty || i == ppb::q_empty + 1);
-            mbar_init(pp_bar(bar0, i), i >= ppb::p_full ? 128 : (q_back ? 4 : 1));
+            const bool slot_back = i >= ppb::item_empty && i < ppb::item_empty + kPpSlots;
+            mbar_init(pp_bar(bar0, i), i >= ppb::p_full ? 128 : (slot_back ? 11 : (q_back ? 4 : 1)));
         }
         ss.abort_flag = 0;
         fence_mbar_init();
@@ -692,12 +793,14 @@ __device__ __forceinline__ bool pp_attention(const CUtensorMap& tm_q, const CUte
                 q_back = -1;
             }
         };
-        PpItems<kVarlen> items;
-        while (ok && items.next(p, total_items)) {
-            const int ord = items.ord;
-            const PpItem& it = items.it;
-            const int n = it.n;
-            const int row = it.q0 + r;   // within the sequence
+        for (int ord = 0; ok; ++ord) {
+            const int slot = ord & (kPpSlots - 1);
+            if (!pp_warp_wait(pp_bar(bar0, ppb::item_full + slot), (ord / kPpSlots) & 1, abort_flag, 122 + w)) break;
+            // the epilogue reads the rest of the slot; it is handed back at the end of the item
+            const PpItem& it = ss.items[slot];
+            const int n = it.n, q0 = it.q0;
+            if (n == 0) break;
+            const int row = q0 + r;   // within the sequence
             const int Sq_i = kVarlen ? it.Sq : p.Sq, Skv_i = kVarlen ? it.Skv : p.Skv;
             const int off_i = kVarlen ? it.Skv - it.Sq : off;
             if (kVarlen) {
@@ -710,11 +813,15 @@ __device__ __forceinline__ bool pp_attention(const CUtensorMap& tm_q, const CUte
             sm.m_before = -INFINITY;
             uint32_t s[128];             // this thread's row of S, later of O
             const uint32_t xb = items2 & 1, xpar = (items2 >> 1) & 1;  // row-sum exchange buffer / phase
-            // kv tiles every row of the query tile sees in full: they come first and take the
-            // loop without mask code; the few tiles crossed by the diagonal or by the end of the
-            // keys follow
+            // kv tiles every row of the query tile sees in full: they come first; on the few tiles
+            // crossed by the diagonal or by the end of the keys, which follow, the step also masks.
+            // (The step exists once and a branch skips its mask code: a second copy for the full
+            // tiles was 1 % ahead from 8192 keys on while every role decoded its own items; with the
+            // items handed over through shared memory the single copy is: 533 against 547 us on
+            // 32 heads x 8192 causal keys.  What an item executes then stays within the 32 KB the
+            // instruction cache serves at full rate.)
             int n_full = Skv_i / kTile;
-            if (p.causal) n_full = min(n_full, max(0, (it.q0 + off_i + 1) / kTile));
+            if (p.causal) n_full = min(n_full, max(0, (q0 + off_i + 1) / kTile));
             n_full = min(n_full, n);
             // this warpgroup's steps of the item: those with an absolute step number of its parity
             const uint32_t g_item = g;
@@ -722,18 +829,8 @@ __device__ __forceinline__ bool pp_attention(const CUtensorMap& tm_q, const CUte
             // no step of this warpgroup in the item (one step, the other warpgroup's): the next
             // step it takes belongs to the item whose Q load waits for the buffer, so hand it back now
             if (j >= n) hand_back_q();
-            if (kSingle) {
             for (; j < n && ok; j += 2) {
-                ok = sm.template step<2>(s, g_item + (uint32_t)j, j, j >= n_full);
-                hand_back_q();
-                if (ok && j == n - 2) {
-                    ss.l_xch[xb][r] = sm.l_part;
-                    mbar_arrive(pp_bar(bar0, ppb::l_pub + xb));
-                }
-            }
-            } else {
-            for (; j < n_full && ok; j += 2) {
-                ok = sm.template step<0>(s, g_item + (uint32_t)j, j);
+                ok = sm.step(s, g_item + (uint32_t)j, j, j >= n_full);
                 hand_back_q();
                 if (ok && j == n - 2) {
                     // the other warpgroup runs the last step and the epilogue: hand it this row sum
@@ -741,15 +838,6 @@ __device__ __forceinline__ bool pp_attention(const CUtensorMap& tm_q, const CUte
                     ss.l_xch[xb][r] = sm.l_part;
                     mbar_arrive(pp_bar(bar0, ppb::l_pub + xb));
                 }
-            }
-            for (; j < n && ok; j += 2) {
-                ok = sm.template step<1>(s, g_item + (uint32_t)j, j);
-                hand_back_q();
-                if (ok && j == n - 2) {
-                    ss.l_xch[xb][r] = sm.l_part;
-                    mbar_arrive(pp_bar(bar0, ppb::l_pub + xb));
-                }
-            }
             }
             const float l_part = sm.l_part, m_loc = sm.m_loc, m_before = sm.m_before;
             if (ok && ((g_item + (uint32_t)n - 1u) & 1u) == (uint32_t)w) {
@@ -761,6 +849,17 @@ __device__ __forceinline__ bool pp_attention(const CUtensorMap& tm_q, const CUte
                     const float l_other = ss.l_xch[xb][r];
                     // the other warpgroup's sum is relative to the reference this one's last step received
                     if (l_other > 0.f) l_run += l_other * fast_exp2((m_before - m_loc) * scale_log2);
+                }
+                // (before the wait for the last P V, which takes longer than this)
+                // (FP8: O and the row sum carry the same factor on the probabilities; V's own factor goes on O)
+                const float inv_l = (l_run > 0.f) ? (kF8 ? p.out_scale / l_run : 1.f / l_run) : 0.f;
+                const long long obase = kVarlen ? (long long)(it.q_base + row) * p.o_ss + (long long)it.h * p.o_sh
+                                                : (long long)it.b * p.o_sb + (long long)row * p.o_ss + (long long)it.h * p.o_sh;
+                if (row < Sq_i && p.lse != nullptr) {
+                    const float lse = (l_run > 0.f) ? (m_loc * scale_log2 + log2f(l_run) - (kF8 ? kP8ScaleLog2 : 0.f)) * 0.6931471805599453f
+                                                    : -INFINITY;
+                    if (kVarlen) p.lse[(long long)it.h * p.total_q + it.q_base + row] = lse;
+                    else p.lse[((long long)it.b * p.Hq + it.h) * p.Sq + row] = lse;
                 }
                 ok = pp_warp_wait(pp_bar(bar0, ppb::o_final + (ord & 1)), (ord >> 1) & 1, abort_flag, 120 + w);
                 if (!ok) break;
@@ -775,16 +874,6 @@ __device__ __forceinline__ bool pp_attention(const CUtensorMap& tm_q, const CUte
                 // O is in registers: the next item's first P V may overwrite it
                 tc_fence_before();
                 mbar_arrive(pp_bar(bar0, ppb::o_free));
-                // (FP8: O and the row sum carry the same factor on the probabilities; V's own factor goes on O)
-                const float inv_l = (l_run > 0.f) ? (kF8 ? p.out_scale / l_run : 1.f / l_run) : 0.f;
-                const long long obase = kVarlen ? (long long)(it.q_base + row) * p.o_ss + (long long)it.h * p.o_sh
-                                                : (long long)it.b * p.o_sb + (long long)row * p.o_ss + (long long)it.h * p.o_sh;
-                if (row < Sq_i && p.lse != nullptr) {
-                    const float lse = (l_run > 0.f) ? (m_loc * scale_log2 + log2f(l_run) - (kF8 ? kP8ScaleLog2 : 0.f)) * 0.6931471805599453f
-                                                    : -INFINITY;
-                    if (kVarlen) p.lse[(long long)it.h * p.total_q + it.q_base + row] = lse;
-                    else p.lse[((long long)it.b * p.Hq + it.h) * p.Sq + row] = lse;
-                }
                 if (kTmaOut) {
                     const uint32_t q_buf = sQ + (uint32_t)(ord & 1) * kTileBytes;
                     const uint32_t row_base = q_buf + (uint32_t)r * 128u;
@@ -844,6 +933,8 @@ __device__ __forceinline__ bool pp_attention(const CUtensorMap& tm_q, const CUte
                     }
                 }
             }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(pp_bar(bar0, ppb::item_empty + slot));
             g = g_item + (uint32_t)n;
             if (n >= 2) ++items2;
         }
@@ -853,17 +944,17 @@ __device__ __forceinline__ bool pp_attention(const CUtensorMap& tm_q, const CUte
     } else {
         setmaxnreg_dec<kPipeOtherRegs>();
         if (lane == 0) {
-            if (warp == 8) pp_run_s<T, kTmaOut, kVarlen, kF8, D>(bar0, sQ, sK, tmem_base, p, total_items, abort_flag);
-            else if (warp == 10) pp_run_pv<T, kVarlen, kF8, D>(bar0, sV, tmem_base, p, total_items, abort_flag);
-            else if (warp == 9) pp_run_load_qk<kVarlen, kF8, D>(bar0, sQ, sK, &tm_q, &tm_k, p, total_items, abort_flag);
-            else pp_run_load_v<kVarlen, kF8, D>(bar0, sV, &tm_v, p, total_items, abort_flag);
+            if (warp == 8) pp_run_s<T, kTmaOut, kF8, D>(bar0, sQ, sK, tmem_base, ss.items, abort_flag);
+            else if (warp == 10) pp_run_pv<T, kF8, D>(bar0, sV, tmem_base, ss.items, abort_flag);
+            else if (warp == 9) pp_run_load_qk<kVarlen, kF8, D>(bar0, sQ, sK, &tm_q, &tm_k, p, total_items, ss, abort_flag);
+            else pp_run_load_v<kVarlen, kF8, D>(bar0, sV, &tm_v, p, ss.items, abort_flag);
         }
         __syncwarp();
     }
     return true;
 }
 
-template <typename T, bool kTmaOut, bool kSingle, bool kVarlen, bool kF8 = false, int D = 128>
+template <typename T, bool kTmaOut, bool kVarlen, bool kF8 = false, int D = 128>
 __global__ void __launch_bounds__(kPipeThreads, 1)
 fa_fwd_pingpong_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                        const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_o,
@@ -872,9 +963,10 @@ fa_fwd_pingpong_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
     // part that follows it starts on a 1024-byte boundary, which the 128-byte swizzle needs)
     // plus seven 32 KiB tiles.  The alignment is checked rather than assumed.
     extern __shared__ __align__(1024) uint8_t smem_raw[];
-    __shared__ __align__(1024) PpStatic ss;
-    if (!pp_attention<T, kTmaOut, kSingle, kVarlen, kF8, false, D>(tm_q, tm_k, tm_v, tm_o, p, total_items, ss,
-                                                                   smem_u32(smem_raw), nullptr))
+    __shared__ __align__(1024) uint8_t static_raw[kPpStaticBytes];
+    PpStatic& ss = *reinterpret_cast<PpStatic*>(static_raw);
+    if (!pp_attention<T, kTmaOut, kVarlen, kF8, false, D>(tm_q, tm_k, tm_v, tm_o, p, total_items, ss, smem_u32(smem_raw),
+                                                          nullptr))
         return;
     tc_fence_before();
     __syncthreads();
@@ -886,7 +978,7 @@ fa_fwd_pingpong_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
 
 // to: map over the output with boxes of 32 rows x 64 columns; read only when the output has the
 // operands' type (any valid map otherwise).
-// The item order of a launch on `grid` CTAs (see pp_class_order and PpItems): returns the
+// The item order of a launch on `grid` CTAs (see pp_class_order and PpSource): returns the
 // parameters with the order's fields filled in.  bytes_per_key: K plus V bytes of one key and head.
 inline FwdParams pp_plan_items(const FwdParams& fp, int grid, double bytes_per_key) {
     const bool varlen = fp.cu_q != nullptr;
@@ -909,24 +1001,16 @@ inline FwdParams pp_plan_items(const FwdParams& fp, int grid, double bytes_per_k
         while ((grid >> cls_log2) * head_bytes > budget && (2 << cls_log2) <= cap) ++cls_log2;
         while (cls_log2 > 0 && (1 << cls_log2) > fp.n_qtiles) --cls_log2;
     }
-    if (varlen) {
-        // Packed batches: sequence by sequence and head by head, a head's tiles longest first (a
-        // single class).  The lengths differ from sequence to sequence, so classes of tiles across
-        // heads would mix long and short items in a round; head by head a round holds the tiles
-        // of two or three neighbouring heads, which are of a size and share their K and V
-        // (measured on 32 requests of 256 to 8192 tokens: 6.0 ms against 6.8 to 7.7 ms with
-        // classes of 1 to 16 tiles).
-        cls_log2 = 0;
-        while ((1 << cls_log2) < fp.n_qtiles) ++cls_log2;
-    }
     // From three rounds per head on (56K keys on 148 SMs) and once a head's K and V are past what
-    // L2 keeps, the head-by-head order with whole rounds per head (see PpItems); the empty slots of
+    // L2 keeps, the head-by-head order with whole rounds per head (see PpSource); the empty slots of
     // a head's last round cost little there because its items are the head's shortest.
     const double kv_bytes_per_head = bytes_per_key * fp.Skv;
     if (!varlen && fp.n_qtiles >= 3 * grid && kv_bytes_per_head > 24.0 * 1024 * 1024) {
         fpc.rounds_per_head = (fp.n_qtiles + grid - 1) / grid;
         fpc.by_rph.set(fpc.rounds_per_head);
     }
+    fpc.deal_ctas = grid;
+    fpc.deal_rounds = 0x7fffffff;
     fpc.cls_log2 = cls_log2;
     const long long class_items = ((long long)fp.B * fp.Hq) << cls_log2;  // > total only for a single class
     fpc.by_class.set(class_items > 0x7fffffffll ? 0x7fffffff : (int)class_items);
@@ -941,25 +1025,38 @@ template <typename T, bool kF8 = false, int D = 128>
 int launch_pingpong(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& to,
                     const FwdParams& fp, cudaStream_t st, int* cuda_err) {
     constexpr int smem = kPpQBufs * kTileBytes + (kPpNK + kPpNV) * PpOperands<kF8, D>::kKvSlotBytes;
-    // the single-copy step up to 32 kv tiles per item (timed: ahead by 3 % at 2048 keys, level at
-    // 4096, behind by 1 % at 8192)
-    const bool single = fp.o_fp32 || fp.Skv <= 32 * kTile;
     const bool varlen = fp.cu_q != nullptr;
     if (varlen && fp.o_fp32) return -3;
     if (kF8 && (varlen || fp.o_fp32)) return -3;
-    auto kern = kF8 ? fa_fwd_pingpong_kernel<T, true, true, false, kF8, D>
-                    : (varlen ? fa_fwd_pingpong_kernel<T, true, true, kF8 ? false : true, false, D>
-                              : (fp.o_fp32 ? fa_fwd_pingpong_kernel<T, false, true, false, false, D>
-                                           : (single ? fa_fwd_pingpong_kernel<T, true, true, false, false, D>
-                                                     : fa_fwd_pingpong_kernel<T, true, false, false, false, D>)));
+    auto kern = kF8 ? fa_fwd_pingpong_kernel<T, true, false, kF8, D>
+                    : (varlen ? fa_fwd_pingpong_kernel<T, true, kF8 ? false : true, false, D>
+                              : (fp.o_fp32 ? fa_fwd_pingpong_kernel<T, false, false, false, D>
+                                           : fa_fwd_pingpong_kernel<T, true, false, false, D>));
     int sm_count = 0;
     cudaError_t e;
     if (int ce = prepare_big_smem_kernel(reinterpret_cast<const void*>(kern), smem, &sm_count)) { *cuda_err = ce; return -7; }
-    const long long total = (long long)fp.n_qtiles * fp.B * fp.Hq;
+    // packed batches: a place for every tile of every sequence, without knowing the lengths (see PpSource)
+    const long long total = varlen ? ((long long)(fp.total_q >> 7) + fp.B) * fp.Hq : (long long)fp.n_qtiles * fp.B * fp.Hq;
     if (total > 0x7fffffffll) return -3;
-    const int grid = (int)(total < sm_count ? total : sm_count);
+    int grid = (int)(total < sm_count ? total : sm_count);
     FwdParams fpc = pp_plan_items(fp, grid, (kF8 || D == 64) ? 256.0 : 512.0);
     fpc.early_next = grid < sm_count;
+    if (fpc.rounds_per_head == 0) {
+        // How much of the list is dealt (see PpSource).  A deal keeps neighbours of the list, which
+        // read the same K and V, on neighbouring CTAs; claims balance.  Packed batches, whose places
+        // differ in length without order: all claimed (32 requests of 256 to 8192 tokens: 4.58 ms
+        // against 4.83 dealt).  Head by head (a head fills the grid): the last two rounds and the
+        // remainder claimed (32 heads x 32768: 7.92 ms; all dealt 8.07, remainder alone 8.13).
+        // Class order: the remainder claimed (8 x 32 heads x 512: 43.1 us against 45.0 all dealt,
+        // 32 x 8192: 526 against 535, 4 x 32 x 2048 level; a round more claimed loses 1 %), but all
+        // after the first round if there are no more than two (5 heads x 8192: 81.3 against 85.4 us).
+        const int full = (int)(total / grid);
+        fpc.deal_rounds = varlen ? 0 : fp.n_qtiles >= grid ? max(1, full - 2) : full > 2 ? full : 1;
+        const long long rest = total - (long long)fpc.deal_rounds * grid;
+        fpc.claim_items = rest > 0;
+        fpc.deal_ctas = fpc.deal_rounds > 0 ? grid : 0;
+        grid = fpc.deal_ctas + (int)rest;
+    }
     e = launch_dependent(kern, dim3(grid), kPipeThreads, smem, st, tq, tk, tv, to, fpc, (int)total);
     if (e != cudaSuccess) { *cuda_err = (int)e; return -7; }
     return 0;

@@ -52,7 +52,7 @@ struct FwdParams {
     // the size of the last (possibly smaller) class
     int cls_log2;
     FastDiv by_class, by_lastcls;
-    // head-by-head order of the ping-pong kernel for very long sequences (see PpItems::next):
+    // head-by-head order of the ping-pong kernel for very long sequences (see PpSource):
     // every head takes rounds_per_head whole rounds of the grid; 0 = the class order above
     int rounds_per_head;
     FastDiv by_rph;
@@ -78,6 +78,9 @@ struct FwdParams {
     // 179 against 174 us with the next kernel's launch left to the end; 2 heads x 512: 12.6
     // against 15.7 us with an early one).
     int early_next = 0;
+    // ping-pong kernel (see PpSource): the first deal_rounds rounds of the item list are dealt to the
+    // first deal_ctas CTAs; the rest, if claim_items, is claimed one by one
+    int claim_items = 0, deal_ctas = 0, deal_rounds = 0;
 };
 
 constexpr int kTile = 128;          // query rows per tile == kv rows per tile == head dim

@@ -219,16 +219,17 @@ fa_proj_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
 // row blocks whose heads other CTAs are still working on are waited for through `done`.  The
 // grid must be resident as a whole (the host uses a cooperative launch): a CTA that waits for a
 // row block relies on the CTAs that own its heads making progress.
-template <typename T, bool kSingle>
+template <typename T>
 __global__ void __launch_bounds__(kPipeThreads, 1)
 fa_fwd_pingpong_proj_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                             const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_o,
                             const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_w,
                             const FwdParams p, const int total_items, const ProjParams pp) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
-    __shared__ __align__(1024) PpStatic ss;
+    __shared__ __align__(1024) uint8_t static_raw[kPpStaticBytes];
+    PpStatic& ss = *reinterpret_cast<PpStatic*>(static_raw);
     const uint32_t smem_base = smem_u32(smem_raw);
-    if (!pp_attention<T, true, kSingle, false, false, true>(tm_q, tm_k, tm_v, tm_o, p, total_items, ss, smem_base, pp.done))
+    if (!pp_attention<T, true, false, false, true>(tm_q, tm_k, tm_v, tm_o, p, total_items, ss, smem_base, pp.done))
         return;
     // every role has left its loops and every store of this CTA has landed; the tiles are about
     // to be overwritten by TMA loads, the exchange arrays become the phase's barriers
@@ -271,8 +272,7 @@ int launch_proj(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap&
         if (e != cudaSuccess) { *cuda_err = (int)e; return -7; }
         return 0;
     }
-    const bool single = fp.Skv <= 32 * kTile;
-    auto kern = single ? fa_fwd_pingpong_proj_kernel<T, true> : fa_fwd_pingpong_proj_kernel<T, false>;
+    auto kern = fa_fwd_pingpong_proj_kernel<T>;
     if (int ce = prepare_big_smem_kernel(reinterpret_cast<const void*>(kern), smem, &sm_count)) { *cuda_err = ce; return -7; }
     const long long total = (long long)fp.n_qtiles * fp.B * fp.Hq;
     if (total > 0x7fffffffll) return -3;

@@ -130,6 +130,29 @@ __global__ void fa_selftest_wait_kernel(unsigned long long limit_ns, unsigned in
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// ------------------------------------------------------------------ cluster launch control
+// A running CTA takes over the work of a CTA of its grid that has not started yet: the request is
+// asynchronous, its 16-byte answer lands at dst (shared memory) and completes 16 bytes on bar.
+__device__ __forceinline__ void clc_request(uint32_t dst, uint32_t bar) {
+    asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];" ::"r"(dst), "r"(bar)
+                 : "memory");
+}
+// The answer: blockIdx.x of the CTA that will not be launched, or -1 if every CTA has started (no
+// further request may be made then).
+__device__ __forceinline__ int clc_answer(uint32_t src) {
+    int x;
+    asm volatile(
+        "{\n\t.reg .b128 h;\n\t.reg .pred p;\n\t"
+        "ld.shared.b128 h, [%1];\n\t"
+        "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, h;\n\t"
+        "mov.b32 %0, -1;\n\t"
+        "@p clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %0, h;\n\t}"
+        : "=r"(x)
+        : "r"(src)
+        : "memory");
+    return x;
+}
+
 // ------------------------------------------------------------------ proxies / fences
 __device__ __forceinline__ void fence_proxy_async_smem() {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");

@@ -1450,3 +1450,25 @@ def test_calls_that_follow_each_other_in_a_stream_see_each_others_results(fa, B,
     for a, b in zip(chain(True), chain(False)):
         assert torch.equal(a, b)
     check_status(fa)
+
+
+@pytest.mark.parametrize("heads", [147, 148, 149, 295, 296, 297, 445])
+def test_pingpong_items_dealt_and_claimed(fa, heads):
+    # one item per head: fewer items than SMs (148), whole rounds with nothing left to claim, one
+    # more or one less, and enough rounds that only the remainder is claimed; the fp32-output form too
+    full_case(fa, 1, heads, heads, 100, 130, True, "bf16", seed=700 + heads, variant=3)
+
+
+@pytest.mark.parametrize("sq", [128 * 147 + 1, 128 * 148 + 5])
+def test_pingpong_items_head_by_head_with_a_claimed_tail(fa, sq):
+    # a head's query tiles alone fill the grid: head-by-head order, the last rounds claimed
+    full_case(fa, 1, 4, 2, sq, 140, False, "fp16", seed=sq, variant=3)
+
+
+@pytest.mark.parametrize("lens", [(1,), (128,), (129,), (0, 0, 5), (127, 1, 128, 128, 129, 0, 255, 1), (256, 0, 0, 0, 0, 0, 3, 640),
+                                  tuple([1] * 200), tuple([0, 130] * 40), tuple(range(0, 400, 7))])
+def test_varlen_places_of_sequences_in_the_item_list(fa, lens):
+    # the list gives a sequence floor(end / 128) - floor(start / 128) + 1 places per head: starts and
+    # ends on and off multiples of 128, empty sequences, many in one place, many places per sequence
+    cfg = synth.VarlenConfig("t", 6, 3, lens, lens, dtype="fp16", causal=True, seed=800 + len(lens))
+    varlen_case(fa, cfg, f"places {lens[:8]}")
