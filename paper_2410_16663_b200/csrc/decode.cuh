@@ -15,7 +15,6 @@ namespace fa {
 constexpr int kDecTile = 128;                 // keys per shared-memory tile
 constexpr int kDecStages = 3;                 // ring depth (K and V tiles each)
 constexpr int kDecTileBytes = 32768;          // a tile of d = 128
-constexpr int kDecHalfBytes = 16384;          // one 128-key x 64-element box
 // Head dimension D (128 or 64): a tile is 128 keys x D 16-bit elements, one or two swizzled
 // boxes, in a ring of three slots per operand.  With D = 64 a CTA's rings are 96 KiB and two
 // CTAs share an SM: the bytes in flight per SM are those of D = 128, and twice the consumer
@@ -94,6 +93,27 @@ __device__ __forceinline__ void mma_16816(float (&c)[4], const uint32_t (&a)[4],
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
+// Where a tile's bytes lie in shared memory.  A tile is loaded in boxes of `rows` keys (128, or one
+// page of 16, 32 or 64), and a box holds all of d: its 64-element blocks one after the other, `rows`
+// rows of 128 swizzled bytes each.  (A 16-key page of d = 128 as one box of 4 KiB instead of two of
+// 2 KiB: the TMA unit's cost per box, about 100 clocks, is what bounds small pages: 48 sequences
+// of 100 to 8000 keys, 8 kv heads, 164 -> 143 us; 16-key pages reach 92 to 96 % of a contiguous cache's rate.)
+template <int D>
+struct DecTileLayout {
+    int rows_log2;
+    uint32_t block;   // bytes from one 64-element block of a box to the next
+    __device__ __forceinline__ explicit DecTileLayout(const DecodeParams& p) {
+        const int rows = (p.block_table != nullptr && p.page_size < kDecTile) ? p.page_size : kDecTile;
+        rows_log2 = 31 - __clz(rows);
+        block = (uint32_t)rows * 128u;
+    }
+    // first byte of key `key` of the tile in its box's first block
+    __device__ __forceinline__ uint32_t key(int key) const {
+        const uint32_t box = (uint32_t)key >> rows_log2;
+        return (D / 64 - 1) * box * block + (uint32_t)key * 128u;
+    }
+};
+
 // The consumer warps' work in the keys-as-rows form (at most 8 rows, i.e. (token, head) pairs,
 // per kv head).  A warp-level MMA has 16 rows and 8 columns: with the query heads as rows, as in the
 // general form below, a kv head with 1 to 8 query heads leaves half or more of every MMA to
@@ -130,6 +150,10 @@ __device__ __forceinline__ bool dec_consume_key_rows(const DecodeParams& p, uint
     float m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f};  // heads 2 t4 and 2 t4 + 1
     const int key_w = warp * 32;  // this warp's keys inside a tile
     bool ok = true;
+    // this lane's key of each block of 16, for the K and for the V matrices
+    const DecTileLayout<D> lay(p);
+    const uint32_t k_at[2] = {lay.key(key_w + ((lane >> 3) & 1) * 8 + (lane & 7)), lay.key(key_w + 16 + ((lane >> 3) & 1) * 8 + (lane & 7))};
+    const uint32_t v_at[2] = {lay.key(key_w + (lane >> 4) * 8 + (lane & 7)), lay.key(key_w + 16 + (lane >> 4) * 8 + (lane & 7))};
 
     for (int t = 0; t < n_tiles; ++t) {
         const int st = t % kStages;
@@ -146,12 +170,11 @@ __device__ __forceinline__ bool dec_consume_key_rows(const DecodeParams& p, uint
 #pragma unroll
             for (int mb = 0; mb < 2; ++mb) {
                 sc[mb][0] = sc[mb][1] = sc[mb][2] = sc[mb][3] = 0.f;
-                const int key = key_w + mb * 16 + ((lane >> 3) & 1) * 8 + (lane & 7);
 #pragma unroll
                 for (int ks = 0; ks < D / 16; ++ks) {
                     // matrices: (keys 0-7, chunk 2 ks), (keys 8-15, chunk 2 ks), (keys 0-7, chunk 2 ks + 1), (keys 8-15, ...)
                     const int chunk = 2 * ks + (lane >> 4);
-                    const uint32_t addr = kt + (chunk >> 3) * kDecHalfBytes + key * 128 + (((chunk & 7) ^ (key & 7)) << 4);
+                    const uint32_t addr = kt + k_at[mb] + (chunk >> 3) * lay.block + (((chunk & 7) ^ (lane & 7)) << 4);
                     uint32_t a[4];
                     ldsm_x4(addr, a[0], a[1], a[2], a[3]);
                     if (kBf16) mma_16816_bf16(sc[mb], a, qb[ks][0], qb[ks][1]);
@@ -223,7 +246,7 @@ __device__ __forceinline__ bool dec_consume_key_rows(const DecodeParams& p, uint
                 // rows past the sequence may hold NaN bits: zero them (0 * NaN would poison O)
                 for (int i = lane; i < (32 - valid) * (D / 8); i += 32) {
                     const int key = key_w + valid + i / (D / 8), ch = i % (D / 8);
-                    const uint32_t addr = vt + (ch >> 3) * kDecHalfBytes + key * 128 + (((ch & 7) ^ (key & 7)) << 4);
+                    const uint32_t addr = vt + lay.key(key) + (ch >> 3) * lay.block + (((ch & 7) ^ (key & 7)) << 4);
                     asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(addr), "r"(0u) : "memory");
                 }
                 __syncwarp();
@@ -232,11 +255,10 @@ __device__ __forceinline__ bool dec_consume_key_rows(const DecodeParams& p, uint
 #pragma unroll
             for (int mb = 0; mb < 2; ++mb) {
                 // matrices: (keys 0-7, chunk 2 i), (keys 0-7, chunk 2 i + 1), (keys 8-15, chunk 2 i), (keys 8-15, chunk 2 i + 1)
-                const int key = key_w + mb * 16 + (lane >> 4) * 8 + (lane & 7);
 #pragma unroll
                 for (int i = 0; i < D / 16; ++i) {
                     const int ch = 2 * i + ((lane >> 3) & 1);
-                    const uint32_t addr = vt + (ch >> 3) * kDecHalfBytes + key * 128 + (((ch & 7) ^ (key & 7)) << 4);
+                    const uint32_t addr = vt + v_at[mb] + (ch >> 3) * lay.block + (((ch & 7) ^ (lane & 7)) << 4);
                     uint32_t a[4];
                     ldsm_x4_trans(addr, a[0], a[1], a[2], a[3]);
                     if (kBf16) mma_16816_bf16(o[i], a, pt[mb][0], pt[mb][1]);
@@ -379,11 +401,9 @@ fa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
                 }
                 __syncwarp();
                 if (lane < live) {
-                    const uint32_t offs = (uint32_t)(lane * ps) * 128u;
-                    tma_load_4d_hint(sK + st * kTileB + offs, &tm_k, bk, 0, hk, 0, cur, stream_policy);
-                    if (D == 128) tma_load_4d_hint(sK + st * kTileB + kDecHalfBytes + offs, &tm_k, bk, 64, hk, 0, cur, stream_policy);
-                    tma_load_4d_hint(sV + st * kTileB + offs, &tm_v, bv, 0, hk, 0, cur, stream_policy);
-                    if (D == 128) tma_load_4d_hint(sV + st * kTileB + kDecHalfBytes + offs, &tm_v, bv, 64, hk, 0, cur, stream_policy);
+                    const uint32_t offs = (uint32_t)(lane * ps) * (2u * D);
+                    tma_load_5d_hint(sK + st * kTileB + offs, &tm_k, bk, 0, 0, 0, hk, cur, stream_policy);
+                    tma_load_5d_hint(sV + st * kTileB + offs, &tm_v, bv, 0, 0, 0, hk, cur, stream_policy);
                 }
             }
         } else if (lane == 0) {
@@ -400,11 +420,9 @@ fa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
                 }
                 if (!mbar_wait(smem_u32(&bars[2 * kStages + st]), ((t / kStages) & 1) ^ 1, &abort_flag, 22)) break;
                 mbar_expect_tx(bk, kTileB);
-                tma_load_4d_hint(sK + st * kTileB, &tm_k, bk, 0, hk, row0, slab, stream_policy);
-                if (D == 128) tma_load_4d_hint(sK + st * kTileB + kDecHalfBytes, &tm_k, bk, 64, hk, row0, slab, stream_policy);
+                tma_load_5d_hint(sK + st * kTileB, &tm_k, bk, 0, row0, 0, hk, slab, stream_policy);
                 mbar_expect_tx(bv, kTileB);
-                tma_load_4d_hint(sV + st * kTileB, &tm_v, bv, 0, hk, row0, slab, stream_policy);
-                if (D == 128) tma_load_4d_hint(sV + st * kTileB + kDecHalfBytes, &tm_v, bv, 64, hk, row0, slab, stream_policy);
+                tma_load_5d_hint(sV + st * kTileB, &tm_v, bv, 0, row0, 0, hk, slab, stream_policy);
             }
         }
         __syncwarp();
@@ -444,6 +462,7 @@ fa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
         for (int i = 0; i < D / 8; ++i) o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f;
         float m_lo = -INFINITY, m_hi = -INFINITY, l_lo = 0.f, l_hi = 0.f;  // rows g and g + 8
         const int key_w = warp * 32;  // this warp's keys inside a tile
+        const DecTileLayout<D> lay(p);
 
         for (int t = 0; t < n_tiles; ++t) {
             const int st = t % kStages;
@@ -463,7 +482,7 @@ fa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
 #pragma unroll
                     for (int c4 = 0; c4 < D / 32; ++c4) {  // 4 d-chunks of 8 per ldmatrix.x4 = two k-steps
                         const int chunk = c4 * 4 + (lane >> 3);
-                        const uint32_t addr = kt + (chunk >> 3) * kDecHalfBytes + key * 128 + (((chunk & 7) ^ (key & 7)) << 4);
+                        const uint32_t addr = kt + lay.key(key) + (chunk >> 3) * lay.block + (((chunk & 7) ^ (key & 7)) << 4);
                         uint32_t b0, b1, b2, b3;
                         ldsm_x4(addr, b0, b1, b2, b3);
                         if (std::is_same<T, __nv_bfloat16>::value) {
@@ -534,7 +553,7 @@ fa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
                     // rows past the sequence may hold NaN bits: zero them (0 * NaN would poison O)
                     for (int i = lane; i < (32 - valid) * (D / 8); i += 32) {
                         const int key = key_w + valid + i / (D / 8), ch = i % (D / 8);
-                        const uint32_t addr = vt + (ch >> 3) * kDecHalfBytes + key * 128 + (((ch & 7) ^ (key & 7)) << 4);
+                        const uint32_t addr = vt + lay.key(key) + (ch >> 3) * lay.block + (((ch & 7) ^ (key & 7)) << 4);
                         asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(addr), "r"(0u) : "memory");
                     }
                     __syncwarp();
@@ -551,7 +570,7 @@ fa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
 #pragma unroll
                     for (int n2 = 0; n2 < D / 16; ++n2) {  // two output blocks per ldmatrix.x4.trans
                         const int ch = n2 * 2 + (lane >> 4);
-                        const uint32_t addr = vt + (ch >> 3) * kDecHalfBytes + key * 128 + (((ch & 7) ^ (key & 7)) << 4);
+                        const uint32_t addr = vt + lay.key(key) + (ch >> 3) * lay.block + (((ch & 7) ^ (key & 7)) << 4);
                         uint32_t b0, b1, b2, b3;
                         ldsm_x4_trans(addr, b0, b1, b2, b3);
                         if (std::is_same<T, __nv_bfloat16>::value) {

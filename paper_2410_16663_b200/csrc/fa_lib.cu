@@ -74,6 +74,28 @@ int encode_map(CUtensorMap* tm, const void* base, int B, int S, int H, int64_t s
     return FA_OK;
 }
 
+// Tensor map over a contiguous 16-bit cache [slabs, S, H, d] (d = 128 or 64) whose box is box_rows keys
+// x all of d for one (slab, head): the dimensions are (64 elements of d, S, 64-element blocks of d, H,
+// slab), so a box lands block by block, box_rows rows of 128 swizzled bytes each.
+int encode_map_cache(CUtensorMap* tm, const void* base, int slabs, int S, int H, int box_rows, bool bf16, int d) {
+    EncodeTiledFn fn = get_encode_fn();
+    if (!fn) return FA_ERR_DEVICE;
+    const cuuint64_t row = (cuuint64_t)H * d * 2;
+    cuuint64_t dims[5] = {64, (cuuint64_t)S, (cuuint64_t)(d / 64), (cuuint64_t)H, (cuuint64_t)slabs};
+    cuuint64_t strides[4] = {row, 128, (cuuint64_t)d * 2, row * S};
+    cuuint32_t box[5] = {64, (cuuint32_t)box_rows, (cuuint32_t)(d / 64), 1, 1};
+    cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+    CUresult r = fn(tm, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 5,
+                    const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                    CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) {
+        t_last_cuda_error = static_cast<int>(r);
+        return FA_ERR_CUDA;
+    }
+    return FA_OK;
+}
+
 // Tensor map over a [B, S, H, 128] one-byte tensor, contiguous: a box is box_rows sequence
 // positions x 128 bytes for one (batch, head), 128-byte swizzled.
 int encode_map_u8(CUtensorMap* tm, const void* base, int B, int S, int H, int box_rows) {
@@ -801,11 +823,9 @@ int decode_impl(const void* q, const void* k_cache, const void* v_cache, void* o
         const int slabs = block_table ? num_pages : B;
         const int slab_rows = block_table ? page_size : Skv_max;
         const int box_rows = (block_table && page_size < fa::kDecTile) ? page_size : fa::kDecTile;
-        rc = encode_map(&tk, k_cache, slabs, slab_rows, Hkv, (int64_t)slab_rows * Hkv * d, (int64_t)Hkv * d, d,
-                        box_rows, bf16, d);
+        rc = encode_map_cache(&tk, k_cache, slabs, slab_rows, Hkv, box_rows, bf16, d);
         if (rc) return rc;
-        rc = encode_map(&tv, v_cache, slabs, slab_rows, Hkv, (int64_t)slab_rows * Hkv * d, (int64_t)Hkv * d, d,
-                        box_rows, bf16, d);
+        rc = encode_map_cache(&tv, v_cache, slabs, slab_rows, Hkv, box_rows, bf16, d);
         if (rc) return rc;
     }
     return d == 64 ? decode_launch<64>(tk, tv, dp, o, lse, g, bf16, direct, Skv_max > 0, st)
