@@ -51,6 +51,9 @@ struct DecodeParams {
     // the result itself and no merge kernel runs (nullptr otherwise)
     void* o_final;
     float* lse_final;
+    // the chunks of a sequence are a cluster's CTAs and are merged through distributed shared
+    // memory (see decode_plan); o_final and lse_final are then the result's
+    int clustered = 0;
     int bf16_io = 0;      // 8-bit cache kernel only: q and o are bf16 (fp16 otherwise)
 };
 
@@ -113,6 +116,47 @@ struct DecTileLayout {
         return (D / 64 - 1) * box * block + (uint32_t)key * 128u;
     }
 };
+
+// Merge of the chunks of one sequence whose CTAs form a cluster (rank = chunk): part holds this
+// CTA's normalised rows and their log-sum-exps.  Row r is finished by CTA r mod (chunks with
+// keys); store(r, col, value, lse) writes a column of it.  Every thread of the CTA calls this.
+constexpr int kDecPartOffset = 40960;   // bytes from the ring's start, past the warps' merge buffer
+constexpr int kDecMaxCluster = 16;
+template <int D, typename Store>
+__device__ __forceinline__ void dec_cluster_merge(const float* part, const float* part_lse, int G, int chunk_rank, int n_live,
+                                                  int tid, Store store) {
+    __syncwarp();
+    cluster_sync_all();   // (CTAs without keys have left; their chunks are not read)
+    if (tid < D) {
+        const uint32_t po = smem_u32(part) + 4 * tid, pl = smem_u32(part_lse);
+        for (int r = chunk_rank; r < G; r += n_live) {
+            float l[kDecMaxCluster], o[kDecMaxCluster];
+            float M = -INFINITY;
+#pragma unroll
+            for (int i = 0; i < kDecMaxCluster; ++i) {
+                l[i] = -INFINITY;
+                o[i] = 0.f;
+                if (i < n_live) {
+                    l[i] = cluster_ld(cluster_map(pl + 4 * r, i));
+                    o[i] = cluster_ld(cluster_map(po + 4 * D * r, i));
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < kDecMaxCluster; ++i) M = fmaxf(M, l[i]);
+            float wsum = 0.f, acc = 0.f;
+#pragma unroll
+            for (int i = 0; i < kDecMaxCluster; ++i) {
+                const float w = (l[i] == -INFINITY) ? 0.f : __expf(l[i] - M);
+                wsum += w;
+                acc = fmaf(w, o[i], acc);
+            }
+            const bool any = M != -INFINITY;   // (several query tokens: one that sees no key at all)
+            store(r, tid, any ? acc / wsum : 0.f, any ? M + logf(wsum) : -INFINITY);
+        }
+    }
+    __syncwarp();
+    cluster_sync_all();   // nobody's shared memory goes away while others read it
+}
 
 // The consumer warps' work in the keys-as-rows form (at most 8 rows, i.e. (token, head) pairs,
 // per kv head).  A warp-level MMA has 16 rows and 8 columns: with the query heads as rows, as in the
@@ -356,7 +400,7 @@ fa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
         return ((long long)b * p.Hq + hk * g_all + (kMulti ? R % g_all : R)) * Sq + row_token(r);
     };
     if (k_begin >= k_end) {  // uniform for the CTA
-        if (p.o_final != nullptr && tid < D) {   // a sequence without keys, and nobody else writes its rows
+        if (p.o_final != nullptr && c == 0 && tid < D) {   // a sequence without keys, and nobody else writes its rows
             for (int r = 0; r < G; ++r) {
                 static_cast<T*>(p.o_final)[row_index(r) * D + tid] = T(0.f);
                 if (tid == 0 && p.lse_final) p.lse_final[lse_index(r)] = -INFINITY;
@@ -365,6 +409,8 @@ fa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
         return;
     }
     const int n_tiles = (k_end - k_begin + kDecTile - 1) / kDecTile;
+    float* part = reinterpret_cast<float*>(smem_raw + (smem_base - smem_u32(smem_raw)) + kDecPartOffset);   // [16][D]
+    float* part_lse = part + 16 * D;                                                                         // [16]
 
     __syncthreads();
 
@@ -627,7 +673,10 @@ fa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
                 // (l == 0: a query token that sees none of this chunk's keys)
                 const float out = (l > 0.f) ? acc / l : 0.f;
                 const float lse = (l > 0.f) ? (M * p.scale_log2 + log2f(l)) * 0.6931471805599453f : -INFINITY;
-                if (p.o_final != nullptr) {   // the only chunk: this is the result
+                if (p.clustered) {
+                    part[r * D + tid] = out;
+                    if (tid == 0) part_lse[r] = lse;
+                } else if (p.o_final != nullptr) {   // the only chunk: this is the result
                     static_cast<T*>(p.o_final)[row_index(r) * D + tid] = T(out);
                     if (tid == 0 && p.lse_final) p.lse_final[lse_index(r)] = lse;
                 } else {
@@ -637,6 +686,13 @@ fa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
                 }
             }
         }
+    }
+    if (p.clustered) {
+        const int n_live = (len + p.chunk - 1) / p.chunk;
+        dec_cluster_merge<D>(part, part_lse, G, c, n_live, tid, [&](int r, int col, float out, float lse) {
+            static_cast<T*>(p.o_final)[row_index(r) * D + col] = T(out);
+            if (col == 0 && p.lse_final) p.lse_final[lse_index(r)] = lse;
+        });
     }
 }
 

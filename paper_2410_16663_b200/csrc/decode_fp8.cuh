@@ -16,6 +16,8 @@ constexpr int kDec8Stages = 3;            // ring slots of one K and one V tile:
 constexpr int kDec8TileBytes = 16384;   // 128 keys x 128 one-byte elements
 constexpr int kDec8Warps = 4;            // consumer warps, 32 keys of every tile each (as in the fp16 kernel)
 constexpr int kDec8Threads = (kDec8Warps + 1) * 32;
+constexpr int kDec8Smem = 1024 + 2 * kDec8Stages * kDec8TileBytes;
+static_assert(kDec8Threads == kDecMmaThreads, "the launcher asks for both kernels' cluster slots with one block size");
 
 // Four e4m3 bytes -> two fp16 pairs: (byte 0, byte 1) and (byte 2, byte 3).  (Widening on the
 // integer pipe instead -- the byte moved into the upper half of a halfword with its low seven
@@ -73,7 +75,7 @@ fa_decode_split_fp8_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
     const int k_begin = c * p.chunk;
     const int k_end = min(len, k_begin + p.chunk);
     if (k_begin >= k_end) {  // uniform for the CTA
-        if (p.o_final != nullptr && tid < 128) {   // a sequence without keys, and nobody else writes its rows
+        if (p.o_final != nullptr && c == 0 && tid < 128) {   // a sequence without keys, and nobody else writes its rows
             for (int r = 0; r < G; ++r) {
                 // (sixteen zero bits are 0.0 in fp16 and in bf16)
                 static_cast<__half*>(p.o_final)[((long long)b * p.Hq + h0 + r) * 128 + tid] = __half(0.f);
@@ -83,6 +85,8 @@ fa_decode_split_fp8_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
         return;
     }
     const int n_tiles = (k_end - k_begin + kDecTile - 1) / kDecTile;
+    float* part = reinterpret_cast<float*>(smem_raw + (smem_base - smem_u32(smem_raw)) + kDecPartOffset);   // [16][128]
+    float* part_lse = part + 16 * 128;                                                                       // [16]
 
     __syncthreads();
 
@@ -371,7 +375,10 @@ fa_decode_split_fp8_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
                 }
                 const float out = acc / l * p.v_scale;
                 const float lse = (M * p.scale_log2 + log2f(l)) * 0.6931471805599453f;
-                if (p.o_final != nullptr) {   // the only chunk: this is the result
+                if (p.clustered) {
+                    part[r * 128 + col] = out;
+                    if (col == 0) part_lse[r] = lse;
+                } else if (p.o_final != nullptr) {   // the only chunk: this is the result
                     const long long row = (long long)b * p.Hq + h0 + r;
                     if (p.bf16_io) static_cast<__nv_bfloat16*>(p.o_final)[row * 128 + col] = __nv_bfloat16(out);
                     else static_cast<__half*>(p.o_final)[row * 128 + col] = __half(out);
@@ -383,6 +390,15 @@ fa_decode_split_fp8_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
                 }
             }
         }
+    }
+    if (p.clustered) {
+        const int n_live = (len + p.chunk - 1) / p.chunk;
+        dec_cluster_merge<128>(part, part_lse, G, c, n_live, tid, [&](int r, int col, float out, float lse) {
+            const long long row = (long long)b * p.Hq + h0 + r;
+            if (p.bf16_io) static_cast<__nv_bfloat16*>(p.o_final)[row * 128 + col] = __nv_bfloat16(out);
+            else static_cast<__half*>(p.o_final)[row * 128 + col] = __half(out);
+            if (col == 0 && p.lse_final) p.lse_final[row] = lse;
+        });
     }
 }
 

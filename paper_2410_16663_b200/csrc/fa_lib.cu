@@ -9,6 +9,7 @@
 #include <stdint.h>
 #include <string.h>
 
+#include <atomic>
 #include <mutex>
 
 #include "decode.cuh"
@@ -423,6 +424,100 @@ int decode_chunk(int B, int Hkv, int Smax, bool long_ok = false) {
     return 256;
 }
 
+// How many clusters of c = 2 .. 16 CTAs of a decode kernel the device runs at a time (it depends on
+// how the SMs are grouped; on B200 with one CTA per SM: 74 of 2, 33 of 4, 15 of 8, 7 of 16).
+// Asked once per device and kind of kernel: 0 = 16-bit, d = 128; 1 = 16-bit, d = 64; 2 = 8-bit.
+struct ClusterSlots {
+    int n[fa::kDecMaxCluster + 1] = {};
+};
+int decode_cluster_slots(int kind, ClusterSlots* out) {
+    constexpr int kMaxDev = 64;
+    static ClusterSlots table[kMaxDev][3];
+    static std::atomic<bool> ready[kMaxDev][3];
+    static std::mutex mu;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return cuda_fail(e);
+    if (dev < 0 || dev >= kMaxDev) return FA_OK;   // no clusters
+    if (!ready[dev][kind].load(std::memory_order_acquire)) {
+        const void* kern = kind == 2   ? reinterpret_cast<const void*>(fa::fa_decode_split_fp8_kernel<1>)
+                           : kind == 1 ? reinterpret_cast<const void*>(fa::fa_decode_split_mma_kernel<false, __half, 64, true>)
+                                       : reinterpret_cast<const void*>(fa::fa_decode_split_mma_kernel<false, __half, 128, true>);
+        const int smem = kind == 2 ? fa::kDec8Smem : kind == 1 ? fa::DecShape<64>::kSmem : fa::DecShape<128>::kSmem;
+        int sm_count = 0;
+        if (int ce = fa::prepare_big_smem_kernel(kern, smem, &sm_count)) return cuda_fail(static_cast<cudaError_t>(ce));
+        ClusterSlots t;
+        for (int c = 2; c <= fa::kDecMaxCluster; ++c) {
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(1, c, 1);
+            cfg.blockDim = dim3(fa::kDecMmaThreads);
+            cfg.dynamicSmemBytes = smem;
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeClusterDimension;
+            attr[0].val.clusterDim.x = 1;
+            attr[0].val.clusterDim.y = c;
+            attr[0].val.clusterDim.z = 1;
+            cfg.attrs = attr;
+            cfg.numAttrs = 1;
+            if (cudaOccupancyMaxActiveClusters(&t.n[c], kern, &cfg) != cudaSuccess) {
+                t.n[c] = 0;   // this size is never used then
+                cudaGetLastError();
+            }
+        }
+        std::lock_guard<std::mutex> lock(mu);
+        if (!ready[dev][kind].load(std::memory_order_relaxed)) {
+            table[dev][kind] = t;
+            ready[dev][kind].store(true, std::memory_order_release);
+        }
+    }
+    *out = table[dev][kind];
+    return FA_OK;
+}
+
+// How a decode call is cut: keys per chunk, chunks per sequence, and whether the chunks of a
+// sequence are one cluster's CTAs, merged in the split kernel itself.
+struct DecodePlan {
+    int chunk = 256, n_chunks = 1;
+    bool clustered = false;
+};
+// ctas: CTAs per chunk over all sequences (B * Hkv, and a multiple above 16 rows per kv head).
+//
+// Few CTAs: the chunks of a sequence as one cluster, as large as the device runs for all of them at
+// once, merged through distributed shared memory.  A second launch for the merge costs 3 us and more
+// with many chunks: the partials have to reach L2, the grid has to end, and the merge starts with
+// two dependent loads.  Measured (us, cluster against split + merge): 1 sequence, 5 kv heads, 512
+// keys 6.4 / 8.6, 8192 8.3 / 12.0, 32768 17.7 / 23.9; 8 kv heads, 8192 10.9 / 11.7, 131072 81 / 83;
+// 5 x 8, 1000 keys 8.8 / 11.9.  But a cluster's chunks are fixed parts of the longest sequence, so
+// sequences of different lengths balance badly once the chunks are long (2 x 5 kv heads of up to
+// 32768 keys: 23.3 / 20.1; of up to 4096 level or ahead up to 12 tiles per chunk), and one sequence
+// with very few kv heads leaves most SMs idle (1 kv head, 65536 keys: 27.9 / 21.6; 8-bit, 5 kv heads,
+// 32768 keys: 17.7 / 16.2).
+int decode_plan(int kind, long long ctas, int B, int Hkv, int Smax, bool long_ok, DecodePlan* plan) {
+    DecodePlan pl;
+    if (Smax > 0) {
+        pl.chunk = decode_chunk(B, Hkv, Smax, long_ok);
+        pl.n_chunks = (Smax + pl.chunk - 1) / pl.chunk;
+    }
+    const int tiles = (Smax + fa::kDecTile - 1) / fa::kDecTile;
+    if (tiles > 1 && ctas <= 1024) {
+        ClusterSlots slots;
+        if (int rc = decode_cluster_slots(kind, &slots)) return rc;
+        int c = tiles < fa::kDecMaxCluster ? tiles : fa::kDecMaxCluster;
+        while (c > 1 && slots.n[c] < ctas) --c;
+        if (c > 1) {
+            const int per = (tiles + c - 1) / c;
+            // (d = 64 and 8-bit run two CTAs per SM)
+            if (per <= 12 || (B == 1 && (kind == 0 ? per <= 16 || ctas * c >= 74 : ctas * c >= 148))) {
+                pl.chunk = per * fa::kDecTile;
+                pl.n_chunks = (tiles + per - 1) / per;
+                pl.clustered = pl.n_chunks > 1;
+            }
+        }
+    }
+    *plan = pl;
+    return FA_OK;
+}
+
 }  // namespace
 
 extern "C" {
@@ -770,7 +865,7 @@ int decode_launch(const CUtensorMap& tk, const CUtensorMap& tv, const fa::Decode
         if (int ce = fa::prepare_big_smem_kernel(reinterpret_cast<const void*>(kern), smem, &sm_count))
             return cuda_fail(static_cast<cudaError_t>(ce));
         dim3 grid(Hkv * ((g * Sq + 15) / 16), dp.n_chunks, B);   // 16 (token, head) rows per CTA
-        const cudaError_t e = fa::launch_dependent(kern, grid, fa::kDecMmaThreads, smem, st, tk, tv, dp);
+        const cudaError_t e = fa::launch_dependent_clusters(kern, grid, dp.clustered ? dp.n_chunks : 1, fa::kDecMmaThreads, smem, st, tk, tv, dp);
         if (e != cudaSuccess) return cuda_fail(e);
     }
     if (direct) return FA_OK;
@@ -801,8 +896,13 @@ int decode_impl(const void* q, const void* k_cache, const void* v_cache, void* o
     dp.seqlens = seqlens_k;
     dp.B = B; dp.Hq = Hq; dp.Hkv = Hkv; dp.Smax = Skv_max;
     dp.Sq = Sq;
-    dp.chunk = Skv_max > 0 ? decode_chunk(B, Hkv, Skv_max, true) : 256;
-    dp.n_chunks = Skv_max > 0 ? (Skv_max + dp.chunk - 1) / dp.chunk : 1;
+    const int g = Hq / Hkv;
+    DecodePlan plan;
+    rc = decode_plan(d == 64 ? 1 : 0, (long long)B * Hkv * ((g * Sq + 15) / 16), B, Hkv, Skv_max, true, &plan);
+    if (rc) return rc;
+    dp.chunk = plan.chunk;
+    dp.n_chunks = plan.n_chunks;
+    dp.clustered = plan.clustered;
     if (dp.n_chunks > 65535) return FA_ERR_UNSUPPORTED;   // the chunks are the grid's second dimension
     dp.o_part = static_cast<float*>(workspace);
     dp.lse_part = dp.o_part + (size_t)B * Sq * Hq * dp.n_chunks * d;
@@ -811,11 +911,10 @@ int decode_impl(const void* q, const void* k_cache, const void* v_cache, void* o
     dp.page_size = block_table ? page_size : 1;
     dp.table_stride = table_stride;
     dp.v_scale = 1.f;
-    // one chunk per sequence: the split kernel writes the result itself, no merge kernel
-    const bool direct = Skv_max > 0 && dp.n_chunks == 1;
+    // one chunk per sequence, or one cluster: the split kernel writes the result itself, no merge kernel
+    const bool direct = Skv_max > 0 && (dp.n_chunks == 1 || dp.clustered);
     dp.o_final = direct ? o : nullptr;
     dp.lse_final = direct ? lse : nullptr;
-    const int g = Hq / Hkv;
 
     CUtensorMap tk, tv;
     if (Skv_max > 0) {
@@ -868,8 +967,13 @@ static int decode_fp8_impl(const void* q, const void* k_cache, const void* v_cac
     dp.q = q;
     dp.seqlens = seqlens_k;
     dp.B = B; dp.Hq = Hq; dp.Hkv = Hkv; dp.Smax = Skv_max;
-    dp.chunk = Skv_max > 0 ? decode_chunk(B, Hkv, Skv_max) : 256;
-    dp.n_chunks = Skv_max > 0 ? (Skv_max + dp.chunk - 1) / dp.chunk : 1;
+    const int g = Hq / Hkv;
+    DecodePlan plan;
+    rc = decode_plan(2, (long long)B * Hkv * ((g + 15) / 16), B, Hkv, Skv_max, false, &plan);
+    if (rc) return rc;
+    dp.chunk = plan.chunk;
+    dp.n_chunks = plan.n_chunks;
+    dp.clustered = plan.clustered;
     if (dp.n_chunks > 65535) return FA_ERR_UNSUPPORTED;   // the chunks are the grid's second dimension
     dp.o_part = static_cast<float*>(workspace);
     dp.lse_part = dp.o_part + (size_t)B * Hq * dp.n_chunks * 128;
@@ -880,11 +984,10 @@ static int decode_fp8_impl(const void* q, const void* k_cache, const void* v_cac
     dp.v_scale = v_scale;
     dp.Sq = 1;
     dp.bf16_io = bf16 ? 1 : 0;
-    // one chunk per sequence: the split kernel writes O and LSE itself and no merge is launched
-    const bool direct = Skv_max > 0 && dp.n_chunks == 1;
+    // one chunk per sequence, or one cluster: the split kernel writes O and LSE itself and no merge is launched
+    const bool direct = Skv_max > 0 && (dp.n_chunks == 1 || dp.clustered);
     dp.o_final = direct ? o : nullptr;
     dp.lse_final = direct ? lse : nullptr;
-    const int g = Hq / Hkv;
     if (Skv_max > 0) {
         CUtensorMap tk, tv;
         const int slabs = block_table ? num_pages : B;          // outermost dimension: the sequence, or the page
@@ -894,14 +997,14 @@ static int decode_fp8_impl(const void* q, const void* k_cache, const void* v_cac
         if (rc) return rc;
         rc = encode_map_u8(&tv, v_cache, slabs, slab_rows, Hkv, box_rows);
         if (rc) return rc;
-        constexpr int smem = 1024 + 2 * fa::kDec8Stages * fa::kDec8TileBytes;
+        constexpr int smem = fa::kDec8Smem;
         int sm_count = 0;
         // keys as the MMA's rows and up to 8 query heads as its columns (two column blocks for 9..16 heads)
         auto kern = (g > 8) ? fa::fa_decode_split_fp8_kernel<2> : fa::fa_decode_split_fp8_kernel<1>;
         if (int ce = fa::prepare_big_smem_kernel(reinterpret_cast<const void*>(kern), smem, &sm_count))
             return cuda_fail(static_cast<cudaError_t>(ce));
         dim3 grid(Hkv * ((g + 15) / 16), dp.n_chunks, B);
-        const cudaError_t e = fa::launch_dependent(kern, grid, fa::kDec8Threads, smem, st, tk, tv, dp);
+        const cudaError_t e = fa::launch_dependent_clusters(kern, grid, dp.clustered ? dp.n_chunks : 1, fa::kDec8Threads, smem, st, tk, tv, dp);
         rc = e == cudaSuccess ? FA_OK : cuda_fail(e);
         if (rc) return rc;
     }

@@ -147,25 +147,37 @@ inline int prepare_big_smem_kernel(const void* kern, int smem_bytes, int* sm_cou
     if ((e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return (int)e;
     if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes)) != cudaSuccess)
         return (int)e;
+    // (decode kernels with their chunks in one cluster: up to 16 CTAs)
+    if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess) return (int)e;
     if (cached) __atomic_store_n(&ent->sms[dev], n, __ATOMIC_RELEASE);
     *sm_count = n;
     return 0;
 }
 
-// Launch as a programmatic dependent of the kernel before it in the stream (see grid_dep_wait).
+// Launch as a programmatic dependent of the kernel before it in the stream (see grid_dep_wait), in
+// clusters of cluster_y CTAs along the grid's second dimension if that is more than one.
 template <typename... P, typename... A>
-inline cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, int threads, int smem_bytes, cudaStream_t st, A... args) {
+inline cudaError_t launch_dependent_clusters(void (*kern)(P...), dim3 grid, int cluster_y, int threads, int smem_bytes,
+                                             cudaStream_t st, A... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = smem_bytes;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = 1;
+    attr[1].val.clusterDim.y = cluster_y;
+    attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = cluster_y > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+template <typename... P, typename... A>
+inline cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, int threads, int smem_bytes, cudaStream_t st, A... args) {
+    return launch_dependent_clusters(kern, grid, 1, threads, smem_bytes, st, args...);
 }
 
 // Stores 32 consecutive rows of a 16-bit output tile, one row of 128 elements (64 packed words

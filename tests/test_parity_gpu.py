@@ -1472,3 +1472,36 @@ def test_varlen_places_of_sequences_in_the_item_list(fa, lens):
     # ends on and off multiples of 128, empty sequences, many in one place, many places per sequence
     cfg = synth.VarlenConfig("t", 6, 3, lens, lens, dtype="fp16", causal=True, seed=800 + len(lens))
     varlen_case(fa, cfg, f"places {lens[:8]}")
+
+
+@pytest.mark.parametrize("B,hq,hkv,smax,d", [(1, 5, 5, 2100, 128), (1, 2, 2, 2048, 128), (1, 4, 1, 129, 128), (2, 10, 5, 1300, 128),
+                                             (3, 5, 5, 1200, 128), (4, 5, 5, 900, 64), (5, 40, 5, 640, 128), (8, 4, 4, 512, 128),
+                                             (9, 5, 5, 390, 128), (37, 2, 2, 300, 128), (37, 2, 2, 300, 64), (75, 2, 2, 300, 128),
+                                             (2, 4, 1, 27000, 128)])
+def test_decode_chunks_in_one_cluster(fa, B, hq, hkv, smax, d):
+    # the chunks of a sequence as a cluster of 2 to 16 CTAs: whole and ragged last chunks, sequences
+    # that fill none, one, some or all of their chunks; sizes on both sides of the rule (75 x 2 kv heads
+    # and the long pair take split and merge).  One and three query rows, fp16 and (d = 128) the FP8 cache.
+    cfg = synth.DecodeConfig("t", B, hq, hkv, smax, 1, smax, d=d, seed=1500 + B + smax)
+    q, k, v, sl = synth.decode_inputs(cfg, "cpu", poison=False)
+    for b, n in enumerate([smax, 0, 1, 128, 129]):
+        if b < B:
+            sl[b] = n
+    kn, vn = k.clone(), v.clone()
+    for b in range(B):
+        kn[b, int(sl[b]):] = float("nan")
+        vn[b, int(sl[b]):] = float("nan")
+    o_ref, l_ref = oracle.decode(q, k, v, sl, cfg.scale)
+    o, lse = run_decode(fa, q.to(DEV), kn.to(DEV), vn.to(DEV), sl.to(DEV), cfg.scale)
+    assert_close_to_oracle(o[:, 0], lse, o_ref, l_ref, what=f"cluster decode B{B} {hkv} {smax}")
+    if smax < 5000:
+        q3 = torch.cat([q, q.flip(2), -q], dim=1)
+        o_ref, l_ref = oracle.decode_append(q3, k, v, sl, cfg.scale)
+        o, lse = run_decode_append(fa, q3.to(DEV), kn.to(DEV), vn.to(DEV), sl.to(DEV), cfg.scale)
+        assert_close_to_oracle(o, lse, o_ref, l_ref, what=f"cluster append B{B} {hkv} {smax}")
+    if d == 128:
+        k8, v8 = synth.fp8_cache(k, v, sl, 0.25, 0.125)
+        kc, vc = synth.fp8_cache(k, v, sl, 0.25, 0.125, poison=False)
+        o_ref, l_ref = oracle.decode_fp8(q, kc, vc, sl, cfg.scale, 0.25, 0.125)
+        o, lse = run_decode_fp8(fa, q.to(DEV), k8.to(DEV), v8.to(DEV), sl.to(DEV), cfg.scale, 0.25, 0.125)
+        assert_close_to_oracle(o[:, 0], lse, o_ref, l_ref, what=f"cluster fp8 B{B} {hkv} {smax}")
