@@ -328,11 +328,18 @@ int forward_impl(const fa_params& in, cudaStream_t st) {
         return e == cudaSuccess ? FA_OK : cuda_fail(e);
     }
 
-    // Default choice, from timings of both kernels on B200: the ping-pong kernel (one query tile
-    // per CTA, Q K^T running ahead of the softmax) wins from 1024 keys on; the paired-tile kernel
-    // keeps an edge on shorter sequences, where items change every few steps.
+    // Default choice, from timings of both kernels: the ping-pong kernel (one query tile per CTA,
+    // Q K^T running ahead of the softmax), also on short sequences: paired tiles make half as many
+    // items of twice the length, which loses when there are few (1 x 2 heads x 512: 8.0 against 12.3
+    // us; 1 x 5 x 1000: 11.7 / 20.1; 1 x 32 x 512: 9.9 / 13.3), and an item boundary costs the
+    // ping-pong kernel less than it did (8 x 32 x 512: 42.0 / 48.9; 16 x 32 x 128: 18.5 / 25.3).  What
+    // is left to the paired kernel: without a mask, items of exactly two query and two kv tiles, at least three
+    // rounds of them (16 x 64/8 x 200: 56.1 against 61.8 us; 16 x 32 x 256: 38.1 / 39.8; causal level).
     int variant = p.variant;
-    if (variant == 0) variant = (p.Skv >= 1024) ? 3 : 4;
+    if (variant == 0) {
+        const bool two_by_two = fp.n_qtiles == 2 && p.Skv > fa::kTile && p.Skv <= 2 * fa::kTile;
+        variant = (!p.causal && two_by_two && 2ll * p.B * p.Hq >= 3 * 148) ? 4 : 3;
+    }
     switch (variant) {
         case 4:  // pipelined kernel, two query tiles per CTA
             return bf16 ? fa::launch_pipelined<__nv_bfloat16>(tq, tk, tv, fp, st, &t_last_cuda_error)

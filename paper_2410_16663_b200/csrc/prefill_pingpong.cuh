@@ -987,8 +987,12 @@ inline FwdParams pp_plan_items(const FwdParams& fp, int grid, double bytes_per_k
     // L2, but at most half of a head's tiles and 16 (a class that is the whole head makes all
     // its tiles read the same K/V lines at the same moment, which measured slower).  Under the
     // causal mask the items of a class differ in length, which costs balance when a head has few
-    // tiles: heads with fewer than 16 keep the plain longest-first order.  When one head alone
-    // fills every CTA, a single class: the plain head-by-head order.
+    // tiles: heads with fewer than 16 keep the plain longest-first order as long as all keys and
+    // values together about fit in L2 (2 x 32 heads x 1900: 75 us against 81 in classes of 8; 8 x 32 x
+    // 1024, 134 MB, level); past that a longest-first round finds none of its K/V there, and heads of
+    // 6 tiles and more take classes of 8 (5 x 32 x 1800: 194 us against 214; 16 x 32 x 768: 146
+    // against 154; 8 x 32 x 1500: 220 against 232).  When one head alone fills every CTA, a single
+    // class: the plain head-by-head order.
     FwdParams fpc = fp;
     int cls_log2 = 0;
     if (fp.n_qtiles >= grid) {
@@ -997,9 +1001,12 @@ inline FwdParams pp_plan_items(const FwdParams& fp, int grid, double bytes_per_k
         const double head_bytes = bytes_per_key * fp.Skv / (fp.Hq / fp.Hkv);
         const double budget = 32.0 * 1024 * 1024;
         const int half = fp.n_qtiles / 2 < 16 ? fp.n_qtiles / 2 : 16;
-        const int cap = (fp.causal && fp.n_qtiles < 16) ? 1 : half;
-        while ((grid >> cls_log2) * head_bytes > budget && (2 << cls_log2) <= cap) ++cls_log2;
-        while (cls_log2 > 0 && (1 << cls_log2) > fp.n_qtiles) --cls_log2;
+        if (fp.causal && fp.n_qtiles < 16) {
+            if (fp.n_qtiles >= 6 && bytes_per_key * fp.Skv * fp.B * fp.Hkv > 140e6) cls_log2 = 3;
+        } else {
+            while ((grid >> cls_log2) * head_bytes > budget && (2 << cls_log2) <= half) ++cls_log2;
+            while (cls_log2 > 0 && (1 << cls_log2) > fp.n_qtiles) --cls_log2;
+        }
     }
     // From three rounds per head on (56K keys on 148 SMs) and once a head's K and V are past what
     // L2 keeps, the head-by-head order with whole rounds per head (see PpSource); the empty slots of
