@@ -127,35 +127,83 @@ __device__ __forceinline__ void dec_cluster_merge(const float* part, const float
                                                   int tid, Store store) {
     __syncwarp();
     cluster_sync_all();   // (CTAs without keys have left; their chunks are not read)
-    if (tid < D) {
-        const uint32_t po = smem_u32(part) + 4 * tid, pl = smem_u32(part_lse);
-        for (int r = chunk_rank; r < G; r += n_live) {
-            float l[kDecMaxCluster], o[kDecMaxCluster];
-            float M = -INFINITY;
+    if (tid < 128) {
+        // D / 4 lanes (16 or 32) work on a row, four columns each; lane i of them also looks after chunk i's weight
+        constexpr int kLanes = D / 4;
+        const int sl = tid % kLanes, col = 4 * sl;
+        const uint32_t po = smem_u32(part) + 4 * col, pl = smem_u32(part_lse);
+        for (int r0 = chunk_rank; r0 < G; r0 += n_live * (128 / kLanes)) {
+            const int r = r0 + n_live * (tid / kLanes);
+            const bool live = r < G;
+            float l = -INFINITY, v[8][4];
+            auto load = [&](int i0) {   // rows of eight chunks
 #pragma unroll
-            for (int i = 0; i < kDecMaxCluster; ++i) {
-                l[i] = -INFINITY;
-                o[i] = 0.f;
-                if (i < n_live) {
-                    l[i] = cluster_ld(cluster_map(pl + 4 * r, i));
-                    o[i] = cluster_ld(cluster_map(po + 4 * D * r, i));
+                for (int i = 0; i < 8; ++i) {
+                    v[i][0] = v[i][1] = v[i][2] = v[i][3] = 0.f;
+                    if (live && i0 + i < n_live) cluster_ld4(cluster_map(po + 4 * D * r, i0 + i), v[i]);
+                }
+            };
+            if (live && sl < n_live) l = cluster_ld(cluster_map(pl + 4 * r, sl));
+            load(0);   // (on their way while the weights are worked out)
+            float M = l;
+#pragma unroll
+            for (int sh = 8; sh > 0; sh >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, sh, 16));
+            M = __shfl_sync(0xffffffffu, M, 0, kLanes);
+            const float w = (l == -INFINITY) ? 0.f : __expf(l - M);
+            float wsum = w;
+#pragma unroll
+            for (int sh = 8; sh > 0; sh >>= 1) wsum += __shfl_xor_sync(0xffffffffu, wsum, sh, 16);
+            wsum = __shfl_sync(0xffffffffu, wsum, 0, kLanes);
+            float acc[4] = {0.f, 0.f, 0.f, 0.f};
+            for (int i0 = 0; i0 < n_live; i0 += 8) {
+                if (i0 > 0) load(i0);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const float wi = __shfl_sync(0xffffffffu, w, i0 + i, kLanes);   // (zero past the live chunks)
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) acc[k] = fmaf(wi, v[i][k], acc[k]);
                 }
             }
-#pragma unroll
-            for (int i = 0; i < kDecMaxCluster; ++i) M = fmaxf(M, l[i]);
-            float wsum = 0.f, acc = 0.f;
-#pragma unroll
-            for (int i = 0; i < kDecMaxCluster; ++i) {
-                const float w = (l[i] == -INFINITY) ? 0.f : __expf(l[i] - M);
-                wsum += w;
-                acc = fmaf(w, o[i], acc);
+            if (live) {
+                const bool any = M != -INFINITY;   // (several query tokens: one that sees no key at all)
+                const float inv = any ? 1.f / wsum : 0.f;
+                store(r, col, make_float4(acc[0] * inv, acc[1] * inv, acc[2] * inv, acc[3] * inv), any ? M + logf(wsum) : -INFINITY);
             }
-            const bool any = M != -INFINITY;   // (several query tokens: one that sees no key at all)
-            store(r, tid, any ? acc / wsum : 0.f, any ? M + logf(wsum) : -INFINITY);
         }
     }
     __syncwarp();
     cluster_sync_all();   // nobody's shared memory goes away while others read it
+}
+
+// Merge of the four consumer warps' states of row r (mo: [4][16][D] unnormalised rows, ml: [4][16] pairs of
+// max and sum): columns col .. col + 3, and the row's log-sum-exp.
+template <int D>
+__device__ __forceinline__ float4 dec_warp_merge(const float* mo, const float* ml, int r, int col, float scale_log2, float factor,
+                                                 float& lse) {
+    float M = -INFINITY;
+#pragma unroll
+    for (int w = 0; w < 4; ++w) M = fmaxf(M, ml[(w * 16 + r) * 2]);
+    float l = 0.f, acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int w = 0; w < 4; ++w) {
+        const float mw = ml[(w * 16 + r) * 2];
+        const float sw = (mw == -INFINITY) ? 0.f : fast_exp2((mw - M) * scale_log2);
+        const float4 v = *reinterpret_cast<const float4*>(&mo[(w * 16 + r) * D + col]);
+        l += sw * ml[(w * 16 + r) * 2 + 1];
+        acc[0] += sw * v.x;
+        acc[1] += sw * v.y;
+        acc[2] += sw * v.z;
+        acc[3] += sw * v.w;
+    }
+    // (l == 0: a query token that sees none of this chunk's keys)
+    lse = (l > 0.f) ? (M * scale_log2 + log2f(l)) * 0.6931471805599453f : -INFINITY;
+    const float inv = (l > 0.f) ? 1.f / l : 0.f;
+    return make_float4(acc[0] * inv * factor, acc[1] * inv * factor, acc[2] * inv * factor, acc[3] * inv * factor);
+}
+// Four consecutive elements of an output row.
+template <typename T>
+__device__ __forceinline__ void dec_store4(void* o, long long at, const float4& v) {
+    *reinterpret_cast<uint2*>(static_cast<T*>(o) + at) = make_uint2(pack2<T>(v.x, v.y), pack2<T>(v.z, v.w));
 }
 
 // The consumer warps' work in the keys-as-rows form (at most 8 rows, i.e. (token, head) pairs,
@@ -657,40 +705,30 @@ fa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
         }
         }
         asm volatile("bar.sync 1, 128;" ::: "memory");
-        if (ok && tid < D) {
-            for (int r = 0; r < G; ++r) {  // thread `tid` owns output column `tid` of every row
-                float M = -INFINITY;
-#pragma unroll
-                for (int w = 0; w < 4; ++w) M = fmaxf(M, ml[(w * 16 + r) * 2]);
-                float l = 0.f, acc = 0.f;
-#pragma unroll
-                for (int w = 0; w < 4; ++w) {
-                    const float mw = ml[(w * 16 + r) * 2];
-                    const float sw = (mw == -INFINITY) ? 0.f : fast_exp2((mw - M) * p.scale_log2);
-                    l += sw * ml[(w * 16 + r) * 2 + 1];
-                    acc += sw * mo[(w * 16 + r) * D + tid];
-                }
-                // (l == 0: a query token that sees none of this chunk's keys)
-                const float out = (l > 0.f) ? acc / l : 0.f;
-                const float lse = (l > 0.f) ? (M * p.scale_log2 + log2f(l)) * 0.6931471805599453f : -INFINITY;
+        if (ok) {
+            // a thread owns four output columns, so 512 / D rows go at a time
+            const int col = 4 * (tid % (D / 4));
+            for (int r = tid / (D / 4); r < G; r += 512 / D) {
+                float lse;
+                const float4 out = dec_warp_merge<D>(mo, ml, r, col, p.scale_log2, 1.f, lse);
                 if (p.clustered) {
-                    part[r * D + tid] = out;
-                    if (tid == 0) part_lse[r] = lse;
+                    *reinterpret_cast<float4*>(&part[r * D + col]) = out;
+                    if (col == 0) part_lse[r] = lse;
                 } else if (p.o_final != nullptr) {   // the only chunk: this is the result
-                    static_cast<T*>(p.o_final)[row_index(r) * D + tid] = T(out);
-                    if (tid == 0 && p.lse_final) p.lse_final[lse_index(r)] = lse;
+                    dec_store4<T>(p.o_final, row_index(r) * D + col, out);
+                    if (col == 0 && p.lse_final) p.lse_final[lse_index(r)] = lse;
                 } else {
                     const long long slot = row_index(r) * p.n_chunks + c;
-                    p.o_part[slot * D + tid] = out;
-                    if (tid == 0) p.lse_part[slot] = lse;
+                    *reinterpret_cast<float4*>(&p.o_part[slot * D + col]) = out;
+                    if (col == 0) p.lse_part[slot] = lse;
                 }
             }
         }
     }
     if (p.clustered) {
         const int n_live = (len + p.chunk - 1) / p.chunk;
-        dec_cluster_merge<D>(part, part_lse, G, c, n_live, tid, [&](int r, int col, float out, float lse) {
-            static_cast<T*>(p.o_final)[row_index(r) * D + col] = T(out);
+        dec_cluster_merge<D>(part, part_lse, G, c, n_live, tid, [&](int r, int col, const float4& out, float lse) {
+            dec_store4<T>(p.o_final, row_index(r) * D + col, out);
             if (col == 0 && p.lse_final) p.lse_final[lse_index(r)] = lse;
         });
     }

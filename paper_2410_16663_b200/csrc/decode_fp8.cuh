@@ -360,32 +360,21 @@ fa_decode_split_fp8_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
         }
         asm volatile("bar.sync 1, %0;" ::"n"(kDec8Warps * 32) : "memory");
         if (ok) {
-            const int col = tid & 127;   // a thread owns one output column
-            for (int r = tid >> 7; r < G; r += kDec8Warps / 4) {
-                float M = -INFINITY;
-#pragma unroll
-                for (int w = 0; w < kDec8Warps; ++w) M = fmaxf(M, ml[(w * 16 + r) * 2]);
-                float l = 0.f, acc = 0.f;
-#pragma unroll
-                for (int w = 0; w < kDec8Warps; ++w) {
-                    const float mw = ml[(w * 16 + r) * 2];
-                    const float sw = (mw == -INFINITY) ? 0.f : fast_exp2((mw - M) * p.scale_log2);
-                    l += sw * ml[(w * 16 + r) * 2 + 1];
-                    acc += sw * mo[(w * 16 + r) * 128 + col];
-                }
-                const float out = acc / l * p.v_scale;
-                const float lse = (M * p.scale_log2 + log2f(l)) * 0.6931471805599453f;
+            const int col = 4 * (tid & 31);   // a thread owns four output columns, so four rows go at a time
+            for (int r = tid >> 5; r < G; r += 4) {
+                float lse;
+                const float4 out = dec_warp_merge<128>(mo, ml, r, col, p.scale_log2, p.v_scale, lse);
+                const long long row = (long long)b * p.Hq + h0 + r;
                 if (p.clustered) {
-                    part[r * 128 + col] = out;
+                    *reinterpret_cast<float4*>(&part[r * 128 + col]) = out;
                     if (col == 0) part_lse[r] = lse;
                 } else if (p.o_final != nullptr) {   // the only chunk: this is the result
-                    const long long row = (long long)b * p.Hq + h0 + r;
-                    if (p.bf16_io) static_cast<__nv_bfloat16*>(p.o_final)[row * 128 + col] = __nv_bfloat16(out);
-                    else static_cast<__half*>(p.o_final)[row * 128 + col] = __half(out);
+                    if (p.bf16_io) dec_store4<__nv_bfloat16>(p.o_final, row * 128 + col, out);
+                    else dec_store4<__half>(p.o_final, row * 128 + col, out);
                     if (col == 0 && p.lse_final) p.lse_final[row] = lse;
                 } else {
-                    const long long slot = ((long long)b * p.Hq + h0 + r) * p.n_chunks + c;
-                    p.o_part[slot * 128 + col] = out;
+                    const long long slot = row * p.n_chunks + c;
+                    *reinterpret_cast<float4*>(&p.o_part[slot * 128 + col]) = out;
                     if (col == 0) p.lse_part[slot] = lse;
                 }
             }
@@ -393,10 +382,10 @@ fa_decode_split_fp8_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
     }
     if (p.clustered) {
         const int n_live = (len + p.chunk - 1) / p.chunk;
-        dec_cluster_merge<128>(part, part_lse, G, c, n_live, tid, [&](int r, int col, float out, float lse) {
+        dec_cluster_merge<128>(part, part_lse, G, c, n_live, tid, [&](int r, int col, const float4& out, float lse) {
             const long long row = (long long)b * p.Hq + h0 + r;
-            if (p.bf16_io) static_cast<__nv_bfloat16*>(p.o_final)[row * 128 + col] = __nv_bfloat16(out);
-            else static_cast<__half*>(p.o_final)[row * 128 + col] = __half(out);
+            if (p.bf16_io) dec_store4<__nv_bfloat16>(p.o_final, row * 128 + col, out);
+            else dec_store4<__half>(p.o_final, row * 128 + col, out);
             if (col == 0 && p.lse_final) p.lse_final[row] = lse;
         });
     }
