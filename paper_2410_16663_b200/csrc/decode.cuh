@@ -8,6 +8,7 @@
 
 #include <type_traits>
 
+#include "prefill_simple.cuh"
 #include "sm100_ptx.cuh"
 
 namespace fa {
@@ -121,7 +122,6 @@ struct DecTileLayout {
 // CTA's normalised rows and their log-sum-exps.  Row r is finished by CTA r mod (chunks with
 // keys); store(r, col, value, lse) writes a column of it.  Every thread of the CTA calls this.
 constexpr int kDecPartOffset = 40960;   // bytes from the ring's start, past the warps' merge buffer
-constexpr int kDecMaxCluster = 16;
 template <int D, typename Store>
 __device__ __forceinline__ void dec_cluster_merge(const float* part, const float* part_lse, int G, int chunk_rank, int n_live,
                                                   int tid, Store store) {

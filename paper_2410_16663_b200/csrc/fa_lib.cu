@@ -9,7 +9,6 @@
 #include <stdint.h>
 #include <string.h>
 
-#include <atomic>
 #include <mutex>
 
 #include "decode.cuh"
@@ -271,6 +270,7 @@ int forward_impl(const fa_params& in, cudaStream_t st) {
     if (rc) return rc;
 
     fa::FwdParams fp = dense_fwd_params(p);
+    if (p.variant == 0) fp.split = 0;   // the ping-pong launcher decides whether CTAs share a query tile
     const bool bf16 = p.dtype == FA_DTYPE_BF16;
 
     if (p.Skv == 0) {
@@ -431,54 +431,14 @@ int decode_chunk(int B, int Hkv, int Smax, bool long_ok = false) {
     return 256;
 }
 
-// How many clusters of c = 2 .. 16 CTAs of a decode kernel the device runs at a time (it depends on
-// how the SMs are grouped; on B200 with one CTA per SM: 74 of 2, 33 of 4, 15 of 8, 7 of 16).
-// Asked once per device and kind of kernel: 0 = 16-bit, d = 128; 1 = 16-bit, d = 64; 2 = 8-bit.
-struct ClusterSlots {
-    int n[fa::kDecMaxCluster + 1] = {};
-};
-int decode_cluster_slots(int kind, ClusterSlots* out) {
-    constexpr int kMaxDev = 64;
-    static ClusterSlots table[kMaxDev][3];
-    static std::atomic<bool> ready[kMaxDev][3];
-    static std::mutex mu;
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return cuda_fail(e);
-    if (dev < 0 || dev >= kMaxDev) return FA_OK;   // no clusters
-    if (!ready[dev][kind].load(std::memory_order_acquire)) {
-        const void* kern = kind == 2   ? reinterpret_cast<const void*>(fa::fa_decode_split_fp8_kernel<1>)
-                           : kind == 1 ? reinterpret_cast<const void*>(fa::fa_decode_split_mma_kernel<false, __half, 64, true>)
-                                       : reinterpret_cast<const void*>(fa::fa_decode_split_mma_kernel<false, __half, 128, true>);
-        const int smem = kind == 2 ? fa::kDec8Smem : kind == 1 ? fa::DecShape<64>::kSmem : fa::DecShape<128>::kSmem;
-        int sm_count = 0;
-        if (int ce = fa::prepare_big_smem_kernel(kern, smem, &sm_count)) return cuda_fail(static_cast<cudaError_t>(ce));
-        ClusterSlots t;
-        for (int c = 2; c <= fa::kDecMaxCluster; ++c) {
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3(1, c, 1);
-            cfg.blockDim = dim3(fa::kDecMmaThreads);
-            cfg.dynamicSmemBytes = smem;
-            cudaLaunchAttribute attr[1];
-            attr[0].id = cudaLaunchAttributeClusterDimension;
-            attr[0].val.clusterDim.x = 1;
-            attr[0].val.clusterDim.y = c;
-            attr[0].val.clusterDim.z = 1;
-            cfg.attrs = attr;
-            cfg.numAttrs = 1;
-            if (cudaOccupancyMaxActiveClusters(&t.n[c], kern, &cfg) != cudaSuccess) {
-                t.n[c] = 0;   // this size is never used then
-                cudaGetLastError();
-            }
-        }
-        std::lock_guard<std::mutex> lock(mu);
-        if (!ready[dev][kind].load(std::memory_order_relaxed)) {
-            table[dev][kind] = t;
-            ready[dev][kind].store(true, std::memory_order_release);
-        }
-    }
-    *out = table[dev][kind];
-    return FA_OK;
+// The clusters of a decode kernel that run at a time; kind: 0 = 16-bit, d = 128; 1 = 16-bit, d = 64; 2 = 8-bit.
+int decode_cluster_slots(int kind, fa::ClusterSlots* out) {
+    const void* kern = kind == 2   ? reinterpret_cast<const void*>(fa::fa_decode_split_fp8_kernel<1>)
+                       : kind == 1 ? reinterpret_cast<const void*>(fa::fa_decode_split_mma_kernel<false, __half, 64, true>)
+                                   : reinterpret_cast<const void*>(fa::fa_decode_split_mma_kernel<false, __half, 128, true>);
+    const int smem = kind == 2 ? fa::kDec8Smem : kind == 1 ? fa::DecShape<64>::kSmem : fa::DecShape<128>::kSmem;
+    const int ce = fa::cluster_slots(kern, smem, fa::kDecMmaThreads, out);
+    return ce ? cuda_fail(static_cast<cudaError_t>(ce)) : FA_OK;
 }
 
 // How a decode call is cut: keys per chunk, chunks per sequence, and whether the chunks of a
@@ -507,9 +467,9 @@ int decode_plan(int kind, long long ctas, int B, int Hkv, int Smax, bool long_ok
     }
     const int tiles = (Smax + fa::kDecTile - 1) / fa::kDecTile;
     if (tiles > 1 && ctas <= 1024) {
-        ClusterSlots slots;
+        fa::ClusterSlots slots;
         if (int rc = decode_cluster_slots(kind, &slots)) return rc;
-        int c = tiles < fa::kDecMaxCluster ? tiles : fa::kDecMaxCluster;
+        int c = tiles < fa::kMaxCluster ? tiles : fa::kMaxCluster;
         while (c > 1 && slots.n[c] < ctas) --c;
         if (c > 1) {
             const int per = (tiles + c - 1) / c;
@@ -872,7 +832,7 @@ int decode_launch(const CUtensorMap& tk, const CUtensorMap& tv, const fa::Decode
         if (int ce = fa::prepare_big_smem_kernel(reinterpret_cast<const void*>(kern), smem, &sm_count))
             return cuda_fail(static_cast<cudaError_t>(ce));
         dim3 grid(Hkv * ((g * Sq + 15) / 16), dp.n_chunks, B);   // 16 (token, head) rows per CTA
-        const cudaError_t e = fa::launch_dependent_clusters(kern, grid, dp.clustered ? dp.n_chunks : 1, fa::kDecMmaThreads, smem, st, tk, tv, dp);
+        const cudaError_t e = fa::launch_dependent_clusters(kern, grid, 1, dp.clustered ? dp.n_chunks : 1, fa::kDecMmaThreads, smem, st, tk, tv, dp);
         if (e != cudaSuccess) return cuda_fail(e);
     }
     if (direct) return FA_OK;
@@ -1011,7 +971,7 @@ static int decode_fp8_impl(const void* q, const void* k_cache, const void* v_cac
         if (int ce = fa::prepare_big_smem_kernel(reinterpret_cast<const void*>(kern), smem, &sm_count))
             return cuda_fail(static_cast<cudaError_t>(ce));
         dim3 grid(Hkv * ((g + 15) / 16), dp.n_chunks, B);
-        const cudaError_t e = fa::launch_dependent_clusters(kern, grid, dp.clustered ? dp.n_chunks : 1, fa::kDec8Threads, smem, st, tk, tv, dp);
+        const cudaError_t e = fa::launch_dependent_clusters(kern, grid, 1, dp.clustered ? dp.n_chunks : 1, fa::kDec8Threads, smem, st, tk, tv, dp);
         rc = e == cudaSuccess ? FA_OK : cuda_fail(e);
         if (rc) return rc;
     }

@@ -92,6 +92,7 @@ constexpr int count = o_free + 1;
 struct __align__(16) PpItem {
     int q0, n;      // first query row of the tile, kv tiles it visits (0: no further item)
     int b, h, hk;
+    int j0;         // the first of those kv tiles (not 0 only where CTAs share a query tile)
     // packed variable-length batches only: first row of the sequence in q/o and in k/v, and
     // the sequence's own lengths
     int q_base, k_base, Sq, Skv;
@@ -141,6 +142,7 @@ __device__ __forceinline__ PpItem pp_decode_item(const FwdParams& p, int b, int 
     it.b = b;
     it.h = h;
     it.hk = p.by_group.div(it.h);
+    it.j0 = 0;
     it.q0 = qt * kTile;
     if (kVarlen) {
         it.q_base = p.cu_q[it.b];
@@ -162,6 +164,20 @@ __device__ __forceinline__ PpItem pp_decode_item(const FwdParams& p, int b, int 
         it.n = kv_tiles_for(it.q0, kTile, p.Sq, p.Skv, p.causal);
     }
     return it;
+}
+
+// The share of this CTA where the CTAs of a cluster divide the kv tiles of one query tile: item
+// blockIdx.x / p.split of the class order, kv tiles [j0, j0 + n).  Returns n (0: nothing to do).
+__device__ __forceinline__ int pp_split_first(int n, int split, int rank) { return n * rank / split; }
+__device__ __forceinline__ int pp_split_item(const FwdParams& p, PpItem& it) {
+    const int idx = (int)blockIdx.x / p.split, rank = (int)blockIdx.x - idx * p.split;
+    int bh, qt, b, h;
+    pp_class_order(p, idx, bh, qt);
+    p.by_hq.divmod(bh, b, h);
+    it = pp_decode_item<false>(p, b, h, qt);
+    it.j0 = pp_split_first(it.n, p.split, rank);
+    it.n = pp_split_first(it.n, p.split, rank + 1) - it.j0;
+    return it.n;
 }
 
 // Where a CTA's work items come from.  One thread, the Q/K loader, decides and decodes them and
@@ -239,6 +255,10 @@ struct PpSource {
         qt = tiles - 1 - (rem - h * tiles);
     }
     __device__ __forceinline__ bool next(PpItem& it) {
+        if (!kVarlen && p.split > 1) {   // one item per cluster
+            ++round;
+            return round == 0 && pp_split_item(p, it) > 0;
+        }
         for (;;) {
             ++round;
             int b, h, qt;
@@ -520,7 +540,7 @@ __device__ __forceinline__ void pp_run_load_qk(uint32_t bar0, uint32_t sQ, uint3
             if (j == it.n - 1) source.request_next();
             if (!mbar_wait(pp_bar(bar0, ppb::k_empty + ring.slot), ring.par ^ 1, abort_flag, 151)) return;
             mbar_expect_tx(pp_bar(bar0, ppb::k_full + ring.slot), PpOperands<kF8, D>::kKvSlotBytes);
-            int row = kVarlen ? it.k_base + j * kTile : j * kTile, slab = kVarlen ? 0 : it.b;
+            int row = kVarlen ? it.k_base + j * kTile : (it.j0 + j) * kTile, slab = kVarlen ? 0 : it.b;
             pp_paged_tile<kVarlen>(p, page, j, row, slab);
             page = page_next;
             pp_load_tile<PpOperands<kF8, D>::kOneBox>(sK + ring.slot * PpOperands<kF8, D>::kKvSlotBytes, tm_k, pp_bar(bar0, ppb::k_full + ring.slot), it.hk, row, slab, pol_kv);
@@ -543,7 +563,7 @@ __device__ __forceinline__ void pp_run_load_v(uint32_t bar0, uint32_t sV, const 
             const int page_next = pp_page_of<kVarlen>(p, it.b, j + 1, it.n, it.Skv);
             if (!mbar_wait(pp_bar(bar0, ppb::v_empty + ring.slot), ring.par ^ 1, abort_flag, 152)) return;
             mbar_expect_tx(pp_bar(bar0, ppb::v_full + ring.slot), PpOperands<kF8, D>::kKvSlotBytes);
-            int row = kVarlen ? it.k_base + j * kTile : j * kTile, slab = kVarlen ? 0 : it.b;
+            int row = kVarlen ? it.k_base + j * kTile : (it.j0 + j) * kTile, slab = kVarlen ? 0 : it.b;
             pp_paged_tile<kVarlen>(p, page, j, row, slab);
             page = page_next;
             pp_load_tile<PpOperands<kF8, D>::kOneBox>(sV + ring.slot * PpOperands<kF8, D>::kKvSlotBytes, tm_v, pp_bar(bar0, ppb::v_full + ring.slot), it.hk, row, slab, pol_kv);
@@ -573,6 +593,7 @@ struct PpSoftmax {
     uint32_t tO, tS, tP;    // this warp's lane quarter of O, S_w, P_w in tensor memory
     float scale_log2;
     int causal, Skv, off;
+    int kv_first;           // first key of the item's first kv tile (0 unless CTAs share a query tile)
     uint32_t sV;            // V ring in shared memory (packed batches: see the end of step())
     int r;                  // this thread's row of the tile
     // per item
@@ -596,7 +617,7 @@ struct PpSoftmax {
         const bool m_there = g > 0 && mbar_test(pp_bar(bar0, ppb::m_ready + (1 - w)), ((g - 1) >> 1) & 1);
         if (masked) {
             // hidden scores become -inf (the scale is strictly positive, so they come out as exact zeros)
-            const int kv0 = j * kTile;
+            const int kv0 = kv_first + j * kTile;
             int lim = Skv - kv0;
             if (causal) lim = min(lim, row + off - kv0 + 1);
 #pragma unroll
@@ -694,6 +715,78 @@ struct PpSoftmax {
     }
 };
 
+// Merge of the parts that a cluster's CTAs computed of one query tile: CTA `rank` of `split` finishes
+// rows rank, rank + split, ..., one warp per row and four columns per lane, reading the parts through
+// distributed shared memory.
+constexpr uint32_t kPpPartStats = 65536;   // bytes from a part's O to its (max, sum) pairs
+template <typename T>
+__device__ __forceinline__ void pp_split_merge(const FwdParams& p, uint32_t part, int tid) {
+    const int warp = tid >> 5, lane = tid & 31;
+    const int split = p.split, idx = (int)blockIdx.x / split, rank = (int)blockIdx.x - idx * split;
+    int bh, qt, b, h;
+    pp_class_order(p, idx, bh, qt);
+    p.by_hq.divmod(bh, b, h);
+    const int q0 = qt * kTile;
+    const int n = kv_tiles_for(q0, kTile, p.Sq, p.Skv, p.causal);
+    // Weights first, one thread per row and part (a part without kv tiles holds nothing): exp2 of the
+    // part's max over the largest, divided by the row's sum.  They go where this CTA's own pairs
+    // are not.
+    const uint32_t w_at = part + kPpPartStats + 2048u;   // [row][kMaxCluster]
+    const int rows = min(kTile, p.Sq - q0);
+    for (int k = tid / kMaxCluster; ; k += 256 / kMaxCluster) {
+        const int row = rank + split * k, i = tid % kMaxCluster;
+        if (rank + split * (k - (tid & 31) / kMaxCluster) >= rows) break;   // uniform for the warp
+        float m = -INFINITY, l = 0.f;
+        if (row < rows && i < split && pp_split_first(n, split, i + 1) > pp_split_first(n, split, i))
+            cluster_ld2(cluster_map(part + kPpPartStats + (uint32_t)row * 8u, i), m, l);
+        if (!(l > 0.f)) m = -INFINITY;   // (a row that sees none of the part's keys)
+        float M = m;
+#pragma unroll
+        for (int sh = kMaxCluster / 2; sh > 0; sh >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, sh));
+        const float w = (l > 0.f) ? fast_exp2((m - M) * p.scale_log2) : 0.f;
+        float sum = w * l;
+#pragma unroll
+        for (int sh = kMaxCluster / 2; sh > 0; sh >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, sh);
+        if (row < rows) {
+            asm volatile("st.shared.f32 [%0], %1;" ::"r"(w_at + (uint32_t)(row * kMaxCluster + i) * 4u), "f"(sum > 0.f ? w / sum : 0.f) : "memory");
+            if (i == 0 && p.lse != nullptr)
+                p.lse[((long long)b * p.Hq + h) * p.Sq + q0 + row] = sum > 0.f ? (M * p.scale_log2 + log2f(sum)) * 0.6931471805599453f : -INFINITY;
+        }
+    }
+    asm volatile("bar.sync 1, 256;" ::: "memory");
+    // Then the rows, one warp and four columns per lane, four rows at a time: the loads' latency is what this takes
+    for (int k0 = warp; rank + split * k0 < rows; k0 += 32) {
+        float acc[4][4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) acc[k][0] = acc[k][1] = acc[k][2] = acc[k][3] = 0.f;
+#pragma unroll 2
+        for (int i = 0; i < split; ++i) {
+            float v[4][4], w[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int row = min(rank + split * (k0 + 8 * k), rows - 1);
+                asm volatile("ld.shared.f32 %0, [%1];" : "=f"(w[k]) : "r"(w_at + (uint32_t)(row * kMaxCluster + i) * 4u));
+                cluster_ld4(cluster_map(part + (uint32_t)row * 512u + (uint32_t)((lane ^ (row & 31)) << 4), i), v[k]);
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) acc[k][c] = w[k] > 0.f ? fmaf(w[k], v[k][c], acc[k][c]) : acc[k][c];
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int row = rank + split * (k0 + 8 * k);
+            if (row < rows) {
+                const long long at_o = (long long)b * p.o_sb + (long long)(q0 + row) * p.o_ss + (long long)h * p.o_sh + 4 * lane;
+                if (p.o_fp32)
+                    *reinterpret_cast<float4*>(static_cast<float*>(p.o) + at_o) = make_float4(acc[k][0], acc[k][1], acc[k][2], acc[k][3]);
+                else
+                    *reinterpret_cast<uint2*>(static_cast<T*>(p.o) + at_o) = make_uint2(pack2<T>(acc[k][0], acc[k][1]), pack2<T>(acc[k][2], acc[k][3]));
+            }
+        }
+    }
+}
+
 // kTmaOut: the output has the operands' 16-bit type; an item's O goes, scaled and rounded, into
 // the item's Q buffer (which Q K^T has finished with by then) in the swizzled layout of a tile,
 // and each warp sends its 32 rows to global memory with two TMA stores (tm_o: boxes of 32 rows x
@@ -706,10 +799,11 @@ struct PpSoftmax {
 // and counts them in done[batch * n_qtiles + query tile]; four warps and Hq heads make a row
 // block of O complete.
 // The whole kernel but for the release of tensor memory; returns false if nothing was set up.
-template <typename T, bool kTmaOut, bool kVarlen, bool kF8, bool kProj, int D = 128>
+template <typename T, bool kTmaOut, bool kVarlen, bool kF8, bool kProj, int D = 128, bool kSplit = false>
 __device__ __forceinline__ bool pp_attention(const CUtensorMap& tm_q, const CUtensorMap& tm_k, const CUtensorMap& tm_v,
                                              const CUtensorMap& tm_o, const FwdParams& p, const int total_items,
                                              PpStatic& ss, const uint32_t smem_base, unsigned int* done) {
+    static_assert(!kSplit || (!kTmaOut && !kVarlen && !kF8 && !kProj && D == 128), "one form shares query tiles");
     static_assert(!kProj || (kTmaOut && !kVarlen && D == 128), "the projection phase reads a contiguous 16-bit O of d = 128");
     const uint32_t sQ = smem_base;
     const uint32_t sK = sQ + kPpQBufs * kTileBytes;
@@ -770,6 +864,7 @@ __device__ __forceinline__ bool pp_attention(const CUtensorMap& tm_q, const CUte
         sm.causal = p.causal;
         sm.Skv = p.Skv;
         sm.off = off;
+        sm.kv_first = 0;
         uint32_t g = 0;        // step counter of the CTA
         uint32_t items2 = 0;   // items with at least two steps seen so far
         bool ok = true;
@@ -822,6 +917,10 @@ __device__ __forceinline__ bool pp_attention(const CUtensorMap& tm_q, const CUte
             // instruction cache serves at full rate.)
             int n_full = Skv_i / kTile;
             if (p.causal) n_full = min(n_full, max(0, (q0 + off_i + 1) / kTile));
+            if (kSplit) {
+                n_full = max(0, n_full - it.j0);
+                sm.kv_first = it.j0 * kTile;
+            }
             n_full = min(n_full, n);
             // this warpgroup's steps of the item: those with an absolute step number of its parity
             const uint32_t g_item = g;
@@ -855,7 +954,7 @@ __device__ __forceinline__ bool pp_attention(const CUtensorMap& tm_q, const CUte
                 const float inv_l = (l_run > 0.f) ? (kF8 ? p.out_scale / l_run : 1.f / l_run) : 0.f;
                 const long long obase = kVarlen ? (long long)(it.q_base + row) * p.o_ss + (long long)it.h * p.o_sh
                                                 : (long long)it.b * p.o_sb + (long long)row * p.o_ss + (long long)it.h * p.o_sh;
-                if (row < Sq_i && p.lse != nullptr) {
+                if (!kSplit && row < Sq_i && p.lse != nullptr) {
                     const float lse = (l_run > 0.f) ? (m_loc * scale_log2 + log2f(l_run) - (kF8 ? kP8ScaleLog2 : 0.f)) * 0.6931471805599453f
                                                     : -INFINITY;
                     if (kVarlen) p.lse[(long long)it.h * p.total_q + it.q_base + row] = lse;
@@ -874,7 +973,17 @@ __device__ __forceinline__ bool pp_attention(const CUtensorMap& tm_q, const CUte
                 // O is in registers: the next item's first P V may overwrite it
                 tc_fence_before();
                 mbar_arrive(pp_bar(bar0, ppb::o_free));
-                if (kTmaOut) {
+                if (kSplit) {
+                    // this CTA's part, for the merge below: the row of O as it is and its max and sum,
+                    // in the K ring (read to the end by now); 16-byte chunks are swizzled by the row
+                    const uint32_t part = sK + (uint32_t)r * 512u;
+#pragma unroll
+                    for (int c = 0; c < D / 4; ++c)
+                        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(part + (uint32_t)((c ^ (r & 31)) << 4)), "r"(s[4 * c]),
+                                     "r"(s[4 * c + 1]), "r"(s[4 * c + 2]), "r"(s[4 * c + 3])
+                                     : "memory");
+                    asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(sK + kPpPartStats + (uint32_t)r * 8u), "f"(m_loc), "f"(l_run) : "memory");
+                } else if (kTmaOut) {
                     const uint32_t q_buf = sQ + (uint32_t)(ord & 1) * kTileBytes;
                     const uint32_t row_base = q_buf + (uint32_t)r * 128u;
 #pragma unroll
@@ -951,7 +1060,32 @@ __device__ __forceinline__ bool pp_attention(const CUtensorMap& tm_q, const CUte
         }
         __syncwarp();
     }
+    if constexpr (kSplit) {
+        __syncwarp();
+        cluster_sync_all();
+        if (warp < 8) pp_split_merge<T>(p, sK, tid);
+        __syncwarp();
+        cluster_sync_all();   // nobody's shared memory goes away while others read it
+    }
     return true;
+}
+
+// Few query tiles: the CTAs of a cluster share one (see pp_split_item and the launcher).
+template <typename T>
+__global__ void __launch_bounds__(kPipeThreads, 1)
+fa_fwd_pingpong_split_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
+                             const __grid_constant__ CUtensorMap tm_v, const FwdParams p) {
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    __shared__ __align__(1024) uint8_t static_raw[kPpStaticBytes];
+    PpStatic& ss = *reinterpret_cast<PpStatic*>(static_raw);
+    if (!pp_attention<T, false, false, false, false, 128, true>(tm_q, tm_k, tm_v, tm_q, p, 0, ss, smem_u32(smem_raw), nullptr))
+        return;
+    tc_fence_before();
+    __syncthreads();
+    if ((threadIdx.x >> 5) == 8) {
+        __syncwarp();
+        tmem_dealloc(ss.tmem_holder, 512);
+    }
 }
 
 template <typename T, bool kTmaOut, bool kVarlen, bool kF8 = false, int D = 128>
@@ -1045,8 +1179,37 @@ int launch_pingpong(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensor
     // packed batches: a place for every tile of every sequence, without knowing the lengths (see PpSource)
     const long long total = varlen ? ((long long)(fp.total_q >> 7) + fp.B) * fp.Hq : (long long)fp.n_qtiles * fp.B * fp.Hq;
     if (total > 0x7fffffffll) return -3;
+    // Few query tiles over many keys: the CTAs of a cluster divide the kv tiles of a query tile and
+    // merge their parts through distributed shared memory, as many CTAs to a tile as the device runs
+    // for all tiles at once.  A step takes 0.8 to 1 us, and the exchange of the parts (64 KiB a CTA,
+    // two cluster barriers, the launch of clusters) about five more than an ordinary epilogue, so it
+    // pays from eight steps saved on the longest tile: 15 tiles over 157 kv tiles 128 -> 33 us, 32
+    // over 63 55 -> 25, 64 over 32 31.2 -> 23.3, 64 over 16 19.1 -> 17.9; 60 over 12 15.2 / 15.5.
+    if constexpr (!kF8 && D == 128) {
+        if (fp.split == 0 && !varlen) {
+            const int kv_tiles = (fp.Skv + kTile - 1) / kTile;   // of the longest item
+            int c = kv_tiles < kMaxCluster ? kv_tiles : kMaxCluster;
+            if (c > 1 && 2 * total <= sm_count) {
+                auto split_kern = fa_fwd_pingpong_split_kernel<T>;
+                ClusterSlots slots;
+                if (int ce = cluster_slots(reinterpret_cast<const void*>(split_kern), smem, kPipeThreads, &slots)) { *cuda_err = ce; return -7; }
+                while (c > 1 && slots.n[c] < total) --c;
+                if (c > 1 && kv_tiles - (kv_tiles + c - 1) / c >= 8) {
+                    FwdParams fps = fp;   // the plain longest-first order
+                    fps.by_class.set(fp.B * fp.Hq);
+                    fps.cls_log2 = 0;
+                    fps.split = c;
+                    fps.early_next = total * c < sm_count;
+                    e = launch_dependent_clusters(split_kern, dim3((unsigned)total * c), c, 1, kPipeThreads, smem, st, tq, tk, tv, fps);
+                    if (e != cudaSuccess) { *cuda_err = (int)e; return -7; }
+                    return 0;
+                }
+            }
+        }
+    }
     int grid = (int)(total < sm_count ? total : sm_count);
     FwdParams fpc = pp_plan_items(fp, grid, (kF8 || D == 64) ? 256.0 : 512.0);
+    fpc.split = 1;
     fpc.early_next = grid < sm_count;
     if (fpc.rounds_per_head == 0) {
         // How much of the list is dealt (see PpSource).  A deal keeps neighbours of the list, which

@@ -10,6 +10,8 @@
 
 #include <type_traits>
 
+#include <mutex>
+
 #include "sm100_ptx.cuh"
 
 namespace fa {
@@ -81,6 +83,7 @@ struct FwdParams {
     // ping-pong kernel (see PpSource): the first deal_rounds rounds of the item list are dealt to the
     // first deal_ctas CTAs; the rest, if claim_items, is claimed one by one
     int claim_items = 0, deal_ctas = 0, deal_rounds = 0;
+    int split = 1;   // ping-pong kernel: CTAs (a cluster) that share the kv tiles of a query tile
 };
 
 constexpr int kTile = 128;          // query rows per tile == kv rows per tile == head dim
@@ -147,18 +150,73 @@ inline int prepare_big_smem_kernel(const void* kern, int smem_bytes, int* sm_cou
     if ((e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return (int)e;
     if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes)) != cudaSuccess)
         return (int)e;
-    // (decode kernels with their chunks in one cluster: up to 16 CTAs)
+    // (kernels whose CTAs share a sequence or a query tile in one cluster: up to 16 CTAs)
     if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess) return (int)e;
     if (cached) __atomic_store_n(&ent->sms[dev], n, __ATOMIC_RELEASE);
     *sm_count = n;
     return 0;
 }
 
+// How many clusters of c = 2 .. 16 CTAs of a kernel the current device runs at a time (it depends on
+// how the SMs are grouped; on B200 with one CTA per SM: 74 of 2, 33 of 4, 15 of 8, 7 of 16).  Asked
+// once per kernel and device; returns 0 or the CUDA error code.
+constexpr int kMaxCluster = 16;
+struct ClusterSlots {
+    int n[kMaxCluster + 1] = {};
+};
+inline int cluster_slots(const void* kern, int smem_bytes, int threads, ClusterSlots* out) {
+    struct Entry {
+        const void* kern = nullptr;
+        int dev = 0;
+        ClusterSlots slots;
+    };
+    constexpr int kMaxEntries = 256;
+    static Entry table[kMaxEntries];
+    static int used = 0;
+    static std::mutex mu;
+    int dev = 0, sm_count = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return (int)e;
+    std::lock_guard<std::mutex> lock(mu);
+    for (int i = 0; i < used; ++i)
+        if (table[i].kern == kern && table[i].dev == dev) {
+            *out = table[i].slots;
+            return 0;
+        }
+    if (int ce = prepare_big_smem_kernel(kern, smem_bytes, &sm_count)) return ce;
+    ClusterSlots t;
+    for (int c = 2; c <= kMaxCluster; ++c) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(c);
+        cfg.blockDim = dim3(threads);
+        cfg.dynamicSmemBytes = smem_bytes;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = c;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        if (cudaOccupancyMaxActiveClusters(&t.n[c], kern, &cfg) != cudaSuccess) {
+            t.n[c] = 0;   // this size is never used then
+            cudaGetLastError();
+        }
+    }
+    if (used < kMaxEntries) {
+        table[used].kern = kern;
+        table[used].dev = dev;
+        table[used].slots = t;
+        ++used;
+    }
+    *out = t;
+    return 0;
+}
+
 // Launch as a programmatic dependent of the kernel before it in the stream (see grid_dep_wait), in
-// clusters of cluster_y CTAs along the grid's second dimension if that is more than one.
+// clusters of cluster_x * cluster_y CTAs if that is more than one.
 template <typename... P, typename... A>
-inline cudaError_t launch_dependent_clusters(void (*kern)(P...), dim3 grid, int cluster_y, int threads, int smem_bytes,
-                                             cudaStream_t st, A... args) {
+inline cudaError_t launch_dependent_clusters(void (*kern)(P...), dim3 grid, int cluster_x, int cluster_y, int threads,
+                                             int smem_bytes, cudaStream_t st, A... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3(threads);
@@ -168,16 +226,16 @@ inline cudaError_t launch_dependent_clusters(void (*kern)(P...), dim3 grid, int 
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = 1;
+    attr[1].val.clusterDim.x = cluster_x;
     attr[1].val.clusterDim.y = cluster_y;
     attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = cluster_y > 1 ? 2 : 1;
+    cfg.numAttrs = cluster_x * cluster_y > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
 }
 template <typename... P, typename... A>
 inline cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, int threads, int smem_bytes, cudaStream_t st, A... args) {
-    return launch_dependent_clusters(kern, grid, 1, threads, smem_bytes, st, args...);
+    return launch_dependent_clusters(kern, grid, 1, 1, threads, smem_bytes, st, args...);
 }
 
 // Stores 32 consecutive rows of a 16-bit output tile, one row of 128 elements (64 packed words

@@ -1505,3 +1505,14 @@ def test_decode_chunks_in_one_cluster(fa, B, hq, hkv, smax, d):
         o_ref, l_ref = oracle.decode_fp8(q, kc, vc, sl, cfg.scale, 0.25, 0.125)
         o, lse = run_decode_fp8(fa, q.to(DEV), k8.to(DEV), v8.to(DEV), sl.to(DEV), cfg.scale, 0.25, 0.125)
         assert_close_to_oracle(o[:, 0], lse, o_ref, l_ref, what=f"cluster fp8 B{B} {hkv} {smax}")
+
+
+@pytest.mark.parametrize("causal", [False, True])
+@pytest.mark.parametrize("B,hq,hkv,sq,skv,dtype", [(1, 2, 2, 1500, 1500, "fp16"), (1, 3, 3, 1279, 1281, "fp16"), (1, 8, 1, 128, 4000, "bf16"),
+                                                   (1, 1, 1, 1, 2100, "fp16"), (1, 1, 1, 100, 1300, "bf16"), (2, 4, 2, 300, 1500, "fp16"),
+                                                   (1, 37, 37, 129, 2100, "fp16"), (1, 25, 5, 257, 2100, "fp16"), (3, 3, 1, 130, 2000, "bf16")])
+def test_query_tiles_shared_by_a_cluster(fa, B, hq, hkv, sq, skv, dtype, causal):
+    # few query tiles over many keys (up to 74 tiles on 148 SMs): 2 to 16 CTAs divide the kv tiles of each, with fewer tiles than
+    # CTAs in the first causal rows, ragged last tiles and rows that see nothing of a part; 75 items do not.
+    # (bf16 also with the fp32 output)
+    full_case(fa, B, hq, hkv, sq, skv, causal, dtype, seed=1700 + sq + skv)
