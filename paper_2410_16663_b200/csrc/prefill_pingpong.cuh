@@ -206,7 +206,10 @@ __device__ __forceinline__ int pp_split_item(const FwdParams& p, PpItem& it) {
 // Packed batches: the list goes sequence by sequence and head by head, a head's tiles longest
 // first.  Sequence s takes the places from floor(cu_q[s] / 128) + s on, times Hq, which leaves
 // it at least its number of tiles and at most one more per head: the host can size the grid
-// without knowing the lengths, and a place past a sequence's end is passed over.
+// without knowing the lengths, and a place past a sequence's end is passed over.  Where it is not more,
+// every sequence has the longest one's number of places instead (p.fixed_places): chunks of 512 new
+// tokens have four tiles, for which the other count keeps five places, and a claim that finds an empty
+// place is a round trip for nothing (10 chunks over up to 5300 keys, 32 heads: 365 -> 362 us; 20 of up to 666, 85.6 -> 83.7).
 template <bool kVarlen>
 struct PpSource {
     const FwdParams& p;
@@ -235,6 +238,12 @@ struct PpSource {
     __device__ __forceinline__ int place_of(int s) const { return (__ldg(p.cu_q + s) >> 7) + s; }
     __device__ __forceinline__ void packed_place(int idx, int& b, int& h, int& qt) {
         int v, rem;
+        if (p.fixed_places) {
+            p.by_qtiles.divmod(idx, v, rem);
+            p.by_hq.divmod(v, b, h);
+            qt = p.n_qtiles - 1 - rem;
+            return;
+        }
         p.by_hq.divmod(idx, v, rem);
         // the last sequence that starts at or before place v: items nearly always come in rising order
         int lo = place_of(seq) <= v ? seq : 0, hi = p.B - 1;
@@ -1177,7 +1186,9 @@ int launch_pingpong(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensor
     cudaError_t e;
     if (int ce = prepare_big_smem_kernel(reinterpret_cast<const void*>(kern), smem, &sm_count)) { *cuda_err = ce; return -7; }
     // packed batches: a place for every tile of every sequence, without knowing the lengths (see PpSource)
-    const long long total = varlen ? ((long long)(fp.total_q >> 7) + fp.B) * fp.Hq : (long long)fp.n_qtiles * fp.B * fp.Hq;
+    const long long all_tiles = (long long)fp.n_qtiles * fp.B, packed_tiles = (long long)(fp.total_q >> 7) + fp.B;
+    const bool fixed_places = !varlen || all_tiles <= packed_tiles;
+    const long long total = (fixed_places ? all_tiles : packed_tiles) * fp.Hq;
     if (total > 0x7fffffffll) return -3;
     // Few query tiles over many keys: the CTAs of a cluster divide the kv tiles of a query tile and
     // merge their parts through distributed shared memory, as many CTAs to a tile as the device runs
@@ -1210,6 +1221,7 @@ int launch_pingpong(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensor
     int grid = (int)(total < sm_count ? total : sm_count);
     FwdParams fpc = pp_plan_items(fp, grid, (kF8 || D == 64) ? 256.0 : 512.0);
     fpc.split = 1;
+    fpc.fixed_places = fixed_places;
     fpc.early_next = grid < sm_count;
     if (fpc.rounds_per_head == 0) {
         // How much of the list is dealt (see PpSource).  A deal keeps neighbours of the list, which

@@ -64,6 +64,7 @@ struct FwdParams {
     const int* cu_q;
     const int* cu_k;
     int total_q;
+    int fixed_places;  // the item list has n_qtiles places for every sequence and head (see PpSource)
     // packed batch over a paged K/V cache (block_table != nullptr; cu_k unused): sequence b has
     // seqlens_k[b] keys, key j in row j % page_size of page block_table[b * table_stride + j / page_size];
     // page_size is a multiple of the 128-key tile and the K/V tensor maps run over the pages

@@ -1466,10 +1466,12 @@ def test_pingpong_items_head_by_head_with_a_claimed_tail(fa, sq):
 
 
 @pytest.mark.parametrize("lens", [(1,), (128,), (129,), (0, 0, 5), (127, 1, 128, 128, 129, 0, 255, 1), (256, 0, 0, 0, 0, 0, 3, 640),
-                                  tuple([1] * 200), tuple([0, 130] * 40), tuple(range(0, 400, 7))])
+                                  tuple([1] * 200), tuple([0, 130] * 40), tuple(range(0, 400, 7)),
+                                  (512, 384, 512, 257), (512, 0, 512, 512, 500)])
 def test_varlen_places_of_sequences_in_the_item_list(fa, lens):
     # the list gives a sequence floor(end / 128) - floor(start / 128) + 1 places per head: starts and
     # ends on and off multiples of 128, empty sequences, many in one place, many places per sequence
+    # (or, where that is not more, the longest one's number of tiles: nearly equal lengths)
     cfg = synth.VarlenConfig("t", 6, 3, lens, lens, dtype="fp16", causal=True, seed=800 + len(lens))
     varlen_case(fa, cfg, f"places {lens[:8]}")
 
