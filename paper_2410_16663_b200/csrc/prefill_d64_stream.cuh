@@ -29,8 +29,9 @@
 // loop takes its masks from warp-uniform counts (cfull, cend) and not by a vote per chunk, whole
 // chunks are read two at a time, an item is decoded by precomputed reciprocals, one lane arrives for
 // its warp, and a row's maxima cross between the two warps that share the row, not between the
-// warpgroups.  Vision batch (1024 x 12 x 197, fp16) 0.409 -> 0.376 ms; 512 x 12 sequences of 144, 176,
-// 256 tokens 0.169, 0.184, 0.241 -> 0.134, 0.163, 0.230 ms.
+// warpgroups.  Vision batch (1024 x 12 x 197, fp16) 0.411 -> 0.373 ms (0.377 with the last chunk's
+// upper half always computed); 512 x 12 sequences of 144, 176, 256 tokens 0.169, 0.184, 0.241 ->
+// 0.134, 0.163, 0.230 ms.
 #pragma once
 
 #include "prefill_d64.cuh"
@@ -205,8 +206,13 @@ fa_fwd_d64_stream_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
                     tmem_wait_ld();
                     const int live = lim - 16 * c;
 #pragma unroll
-                    for (int i = 0; i < 16; ++i)
+                    for (int i = 0; i < 8; ++i)
                         if (i < live) m = fmaxf(m, __uint_as_float(s[i]));
+                    if (warp_lim - 16 * c > 8) {
+#pragma unroll
+                        for (int i = 8; i < 16; ++i)
+                            if (i < live) m = fmaxf(m, __uint_as_float(s[i]));
+                    }
                 }
                 *hm_mine = m;
                 const uint32_t xch = d64_bar(bar0, d64b::row_max + 4 * pr + (warp & 3));   // with the warp that has the rows' other half
@@ -255,12 +261,18 @@ fa_fwd_d64_stream_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
                         tmem_ld_x16(tS + 16 * c, s);
                         tmem_wait_ld();
                         const int live = lim - 16 * c;
-#pragma unroll
-                        for (int i = 0; i < 16; i += 2) {
+                        auto masked_pair = [&](int i) {
                             const float e0 = (i < live) ? fast_exp2(fmaf(__uint_as_float(s[i]), scale_log2, neg_ms)) : 0.f;
                             const float e1 = (i + 1 < live) ? fast_exp2(fmaf(__uint_as_float(s[i + 1]), scale_log2, neg_ms)) : 0.f;
                             l += e0 + e1;
                             pk[i >> 1] = pack2<T>(e0, e1);
+                        };
+#pragma unroll
+                        for (int i = 0; i < 8; i += 2) masked_pair(i);
+                        pk[4] = pk[5] = pk[6] = pk[7] = 0u;
+                        if (warp_lim - 16 * c > 8) {   // (197 tokens: five keys in the last chunk)
+#pragma unroll
+                            for (int i = 8; i < 16; i += 2) masked_pair(i);
                         }
                         tmem_st_x8(tP + 8 * (c - cs), pk);
                     }

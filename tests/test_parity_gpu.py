@@ -407,6 +407,14 @@ def test_d64_short_sequence_every_split_of_the_keys(fa, skv):
     full_case_d64(fa, 2, 3, 3, skv, skv, True, "bf16", seed=700 + skv)
 
 
+@pytest.mark.parametrize("skv", [135, 136, 137, 200, 201, 248, 249])
+def test_d64_short_sequence_half_a_last_chunk(fa, skv):
+    # the last 16 keys are computed in halves of eight: up to eight live keys and one more, in both
+    # halves of the keys, and under the mask with every count of live keys in a warp's last chunk
+    full_case_d64(fa, 3, 4, 2, 197, skv, False, "fp16", seed=500 + skv)
+    full_case_d64(fa, 2, 3, 3, 130, skv, True, "bf16", seed=550 + skv)
+
+
 @pytest.mark.parametrize("dtype", ["fp16", "bf16"])
 def test_d64_gqa_and_both_types(fa, dtype):
     full_case_d64(fa, 2, 8, 2, 333, 333, True, dtype, seed=71)
