@@ -180,15 +180,38 @@ __device__ __forceinline__ int pp_split_item(const FwdParams& p, PpItem& it) {
     return it.n;
 }
 
+// The places of the item list that a CTA takes: its share.  The first deal_ctas CTAs of the grid have
+// deal_rounds places each, dealt in alternating direction; every CTA after them has one place.
+// A CTA walks its own share and then the share of every CTA whose launch it has cancelled.  That can be
+// any CTA that has not started, one of the dealing ones included: while a kernel of another stream
+// holds some SMs, CTAs that found one may be through with their deal before the others get theirs.
+struct PpWalk {
+    int deal_ctas, deal_rounds;
+    int share;       // CTA whose share this is
+    int round = 0;   // places of it taken so far
+
+    __host__ __device__ __forceinline__ bool used_up() const { return round >= (share < deal_ctas ? deal_rounds : 1); }
+    // The next place of the share (only if it is not used up).
+    __host__ __device__ __forceinline__ int next() {
+        const int r = round++;
+        if (share >= deal_ctas) return deal_rounds * deal_ctas + share - deal_ctas;
+        return r * deal_ctas + ((r & 1) ? deal_ctas - 1 - share : share);
+    }
+    __host__ __device__ __forceinline__ void take_over(int cta) {
+        share = cta;
+        round = 0;
+    }
+};
+
 // Where a CTA's work items come from.  One thread, the Q/K loader, decides and decodes them and
 // hands them to the other roles through a ring of slots in shared memory (PpItem, item_full,
 // item_empty): an item costs the others one barrier wait and one or two 16-byte reads instead of
 // the divisions and, in packed batches, the dependent global loads of the decoding.
 //
-// The list is dealt to the CTAs for its first p.deal_rounds rounds, in alternating direction, and
-// claimed from there on (p.claim_items): the grid has one CTA for every remaining item on top of the
-// deal_ctas that run, and a running CTA claims the items of CTAs that have not started through
-// cluster launch control when it requests the last keys of the item it is on.  The launcher says
+// The list is dealt to the first p.deal_ctas CTAs for its first p.deal_rounds rounds and claimed from
+// there on (p.claim_items): the grid has one CTA for every remaining item on top of the dealing ones,
+// and a running CTA takes over the share (see PpWalk) of a CTA that has not started through
+// cluster launch control when it requests the last keys of the last item it has.  The launcher says
 // how much of which list is dealt and why.
 //
 // Very long sequences (rounds_per_head > 0; one head's K and V no longer fit in L2) are all dealt,
@@ -216,12 +239,12 @@ struct PpSource {
     int total_items;
     uint32_t claim_bar, answer;      // shared-memory addresses
     volatile uint32_t* abort_flag;
-    int round = -1;                  // places taken so far, less one
+    PpWalk walk;
+    int round = -1;                  // (rounds_per_head) rounds taken so far, less one
     int claims = 0;                  // claims answered
     bool pending = false;            // a claim is on its way
     int seq = 0;                     // packed batches: sequence of the last item
 
-    __device__ __forceinline__ bool dealt(int k) const { return k < p.deal_rounds && (int)blockIdx.x < p.deal_ctas; }
     // Asks for an item (at most once).
     __device__ __forceinline__ void request() {
         if (p.claim_items && !pending) {
@@ -233,7 +256,7 @@ struct PpSource {
     }
     // The same ahead of time, if the next item is a claimed one.
     __device__ __forceinline__ void request_next() {
-        if (!dealt(round + 1)) request();
+        if (walk.used_up()) request();
     }
     __device__ __forceinline__ int place_of(int s) const { return (__ldg(p.cu_q + s) >> 7) + s; }
     __device__ __forceinline__ void packed_place(int idx, int& b, int& h, int& qt) {
@@ -281,24 +304,18 @@ struct PpSource {
                 p.by_hq.divmod(bh, b, h);
                 qt = p.n_qtiles - 1 - j;
             } else {
-                int idx;
-                if (dealt(round)) {
-                    idx = round * p.deal_ctas + ((round & 1) ? (p.deal_ctas - 1 - (int)blockIdx.x) : (int)blockIdx.x);
-                    if (idx >= total_items) return false;
-                } else if (!p.claim_items) {
-                    return false;
-                } else {
-                    int x = blockIdx.x;   // (a CTA past the dealt ones that was launched after all: its own place first)
-                    if (round > 0) {
-                        request();
-                        if (!mbar_wait(claim_bar, claims & 1, abort_flag, 153)) return false;
-                        ++claims;
-                        pending = false;
-                        x = clc_answer(answer);
-                        if (x < 0) return false;
-                    }
-                    idx = p.deal_rounds * p.deal_ctas + x - p.deal_ctas;
+                if (walk.used_up()) {
+                    if (!p.claim_items) return false;
+                    request();
+                    if (!mbar_wait(claim_bar, claims & 1, abort_flag, 153)) return false;
+                    ++claims;
+                    pending = false;
+                    const int cta = clc_answer(answer);
+                    if (cta < 0) return false;
+                    walk.take_over(cta);
                 }
+                const int idx = walk.next();
+                if (idx >= total_items) return false;   // (a list that is all dealt)
                 if (kVarlen) {
                     packed_place(idx, b, h, qt);
                     if (h < 0 || h >= p.Hq || qt < 0 || qt >= p.n_qtiles) continue;
@@ -528,7 +545,8 @@ __device__ __forceinline__ void pp_run_load_qk(uint32_t bar0, uint32_t sQ, uint3
     tma_prefetch_desc(tm_k);
     const uint64_t pol_q = l2_policy_evict_first(), pol_kv = l2_policy_evict_last();
     PpRing<kPpNK> ring;
-    PpSource<kVarlen> source{p, total_items, pp_bar(bar0, ppb::claim), smem_u32(&ss.claim_answer), abort_flag};
+    PpSource<kVarlen> source{p, total_items, pp_bar(bar0, ppb::claim), smem_u32(&ss.claim_answer), abort_flag,
+                             {p.deal_ctas, p.deal_rounds, (int)blockIdx.x}};
     PpItem it;
     for (int ord = 0;; ++ord) {
         if (!source.next(it)) it.n = 0;   // no further item: the others are told so

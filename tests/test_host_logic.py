@@ -11,17 +11,29 @@ ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 
 
-@pytest.mark.skipif(not os.path.exists(NVCC) and shutil.which("nvcc") is None, reason="nvcc not found")
-def test_fastdiv_matches_integer_division(tmp_path):
+def run_host_check(name, tmp_path):
     nvcc = NVCC if os.path.exists(NVCC) else shutil.which("nvcc")
-    exe = str(tmp_path / "fastdiv_check")
-    src = os.path.join(ROOT, "tests", "host_checks", "fastdiv_check.cu")
+    exe = str(tmp_path / name)
+    src = os.path.join(ROOT, "tests", "host_checks", name + ".cu")
     subprocess.run([nvcc, "-std=c++17", "-O2", "-gencode", "arch=compute_100a,code=sm_100a", src, "-o", exe],
                    check=True, timeout=600)
     out = subprocess.run([exe], capture_output=True, text=True, timeout=600)
     sys.stdout.write(out.stdout)
     assert out.returncode == 0, out.stdout[-2000:]
     assert out.stdout.strip().startswith("OK")
+
+
+needs_nvcc = pytest.mark.skipif(not os.path.exists(NVCC) and shutil.which("nvcc") is None, reason="nvcc not found")
+
+
+@needs_nvcc
+def test_fastdiv_matches_integer_division(tmp_path):
+    run_host_check("fastdiv_check", tmp_path)
+
+
+@needs_nvcc
+def test_every_place_of_the_item_list_is_taken_once_whatever_cta_starts_when(tmp_path):
+    run_host_check("item_walk_check", tmp_path)
 
 
 def test_paged_from_packed_keeps_every_row_where_the_table_says():

@@ -1,0 +1,116 @@
+"""Calls beside another kernel: what else is resident on the GPU must not change a result.
+
+The persistent prefill kernel hands part of its work to whichever CTA is free, decode and small
+prefills run as clusters, and every kernel starts while the one before it in its stream still runs;
+all of this goes another way when a kernel of another stream keeps some of the SMs."""
+import pytest
+import torch
+
+from paper_2410_16663_b200 import inputs as synth
+from tests.test_parity_gpu import check_status, fa  # noqa: F401  (fa: the fixture)
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+
+
+def _rand(shape, dtype, seed):
+    gen = torch.Generator(device=DEV)
+    gen.manual_seed(seed)
+    return torch.randn(shape, device=DEV, generator=gen).to(dtype)
+
+
+class Neighbour:
+    """A finite call that holds one SM per head: one query tile over `keys` keys, about 0.6 us per 128 keys."""
+
+    def __init__(self, fa, sms, keys):
+        self.fa, self.sms = fa, sms
+        self.q = _rand((1, 128, sms, 128), torch.float16, 1)
+        self.k, self.v = (_rand((1, keys, 1, 128), torch.float16, s) for s in (2, 3))
+        self.o = torch.empty_like(self.q)
+
+    def run(self):
+        self.fa.fa_forward_ex(self.q, self.k, self.v, self.o, None, False, 0.1, variant=3)
+
+
+def beside_neighbour(fa, call, outs, sms, keys=131072, overlaps=True):
+    """Runs call() alone and again beside a Neighbour that outlasts it; the outputs, filled with NaN
+    before each run, must be the same bit for bit."""
+    near = Neighbour(fa, sms, keys)
+
+    def clear():
+        for t in outs:
+            t.fill_(float("nan"))
+
+    near.run()
+    clear()
+    call()
+    torch.cuda.synchronize()
+    alone = [t.clone() for t in outs]
+    s1, s2 = torch.cuda.Stream(), torch.cuda.Stream()
+    end1, end2 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    clear()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(s1):
+        near.run()
+        end1.record()
+    with torch.cuda.stream(s2):
+        call()
+        end2.record()
+    torch.cuda.synchronize()
+    check_status(fa)
+    if overlaps:   # else the neighbour was gone too early and nothing has been tested
+        assert end2.elapsed_time(end1) > 0
+    for a, b in zip(alone, outs):
+        assert not torch.isnan(a).any()
+        assert torch.equal(a, b), f"{int((a != b).sum())} of {a.numel()} values differ"
+
+
+def _dense(B, H, Hkv, Sq, Skv, d, dtype, o_dtype=None, seed=5):
+    q = _rand((B, Sq, H, d), dtype, seed)
+    k, v = (_rand((B, Skv, Hkv, d), dtype, seed + i) for i in (1, 2))
+    o = torch.empty(q.shape, dtype=o_dtype or dtype, device=DEV)
+    return q, k, v, o, torch.empty(B, H, Sq, device=DEV)
+
+
+# (16, 32, 128): three rounds of items on 148 SMs and a remainder; then six and thirteen; the head-by-head
+# order with its last two rounds claimed; d = 64 and the fp32 output
+@pytest.mark.parametrize("sms", [1, 16, 32])
+@pytest.mark.parametrize("B,H,Hkv,Sq,Skv,d,dtype,o_dtype", [
+    (16, 32, 32, 128, 128, 128, torch.float16, None),
+    (8, 32, 32, 512, 512, 128, torch.float16, None),
+    (4, 32, 32, 2048, 2048, 128, torch.bfloat16, None),
+    (1, 4, 2, 148 * 128 + 1, 300, 128, torch.float16, None),
+    (8, 32, 8, 512, 512, 64, torch.float16, None),
+    (8, 32, 32, 512, 512, 128, torch.bfloat16, torch.float32),
+])
+def test_prefill_beside_a_kernel_that_holds_sms(fa, B, H, Hkv, Sq, Skv, d, dtype, o_dtype, sms):  # noqa: F811
+    q, k, v, o, lse = _dense(B, H, Hkv, Sq, Skv, d, dtype, o_dtype)
+    beside_neighbour(fa, lambda: fa.fa_forward_ex(q, k, v, o, lse, Sq == Skv, 0.1), [o, lse], sms)
+
+
+@pytest.mark.parametrize("sms", [16, 32])
+def test_prefill_fp8_beside_a_kernel_that_holds_sms(fa, sms):  # noqa: F811
+    q, k, v, o, lse = _dense(8, 32, 32, 512, 512, 128, torch.float16)
+    q8, k8, v8 = synth.fp8_operands(q, k, v, 0.125, 0.25, 0.0625)
+    beside_neighbour(fa, lambda: fa.fa_forward_fp8(q8, k8, v8, o, lse, True, 0.1, 0.125, 0.25, 0.0625), [o, lse], sms)
+
+
+@pytest.mark.parametrize("sms", [16, 32])
+def test_other_forms_beside_a_kernel_that_holds_sms(fa, sms):  # noqa: F811
+    # a packed batch (all of its list claimed)
+    lens = [700, 33, 1290, 128, 512, 1] * 3
+    cu = torch.tensor([0] + lens).cumsum(0).to(torch.int32).to(DEV)
+    q, k, v = (_rand((sum(lens), 16, 128), torch.bfloat16, s) for s in (7, 8, 9))
+    o, lse = torch.empty_like(q), torch.empty(16, sum(lens), device=DEV)
+    beside_neighbour(fa, lambda: fa.fa_forward_varlen(q, k, v, o, lse, cu, cu, max(lens), max(lens), True, 0.1), [o, lse], sms)
+    # a query tile shared by a cluster's CTAs, d = 256, the short d = 64 kernels
+    for B, H, Hkv, Sq, Skv, d in ((1, 8, 2, 200, 4000, 128), (1, 8, 8, 700, 700, 256), (40, 12, 12, 197, 197, 64), (64, 12, 12, 100, 100, 64)):
+        q, k, v, o, lse = _dense(B, H, Hkv, Sq, Skv, d, torch.float16)
+        beside_neighbour(fa, lambda: fa.fa_forward(q, k, v, o, lse, True, 0.1), [o, lse], sms, overlaps=False)
+    # decode: chunks merged in one cluster, and split with a merge kernel
+    for B, Hkv, smax in ((1, 5, 8192), (16, 8, 9000)):
+        q, o, lse = _rand((B, 1, 2 * Hkv, 128), torch.float16, 11), torch.empty(B, 1, 2 * Hkv, 128, dtype=torch.float16, device=DEV), torch.empty(B, 2 * Hkv, device=DEV)
+        k, v = (_rand((B, smax, Hkv, 128), torch.float16, s) for s in (12, 13))
+        sl = torch.tensor([smax - 77 * b for b in range(B)], dtype=torch.int32, device=DEV)
+        ws = torch.empty(fa.fa_decode_workspace_bytes(B, 2 * Hkv, Hkv, smax, 128) + 16, dtype=torch.uint8, device=DEV)
+        beside_neighbour(fa, lambda: fa.fa_decode(q, k, v, o, lse, sl, 0.1, ws), [o, lse], sms, overlaps=False)
