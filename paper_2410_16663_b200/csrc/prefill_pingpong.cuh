@@ -755,9 +755,10 @@ __device__ __forceinline__ void pp_split_merge(const FwdParams& p, uint32_t part
     p.by_hq.divmod(bh, b, h);
     const int q0 = qt * kTile;
     const int n = kv_tiles_for(q0, kTile, p.Sq, p.Skv, p.causal);
-    // Weights first, one thread per row and part (a part without kv tiles holds nothing): exp2 of the
-    // part's max over the largest, divided by the row's sum.  They go where this CTA's own pairs
-    // are not.
+    // Weights first, one thread per row and part: exp2 of the part's max over the largest, divided by the
+    // row's sum; -1 for a part without kv tiles, which holds nothing, and one whose keys the row does
+    // not see.  A sum that is NaN (a NaN or infinite score) makes every weight of the row NaN.  They go
+    // where this CTA's own pairs are not.
     const uint32_t w_at = part + kPpPartStats + 2048u;   // [row][kMaxCluster]
     const int rows = min(kTile, p.Sq - q0);
     for (int k = tid / kMaxCluster; ; k += 256 / kMaxCluster) {
@@ -766,16 +767,16 @@ __device__ __forceinline__ void pp_split_merge(const FwdParams& p, uint32_t part
         float m = -INFINITY, l = 0.f;
         if (row < rows && i < split && pp_split_first(n, split, i + 1) > pp_split_first(n, split, i))
             cluster_ld2(cluster_map(part + kPpPartStats + (uint32_t)row * 8u, i), m, l);
-        if (!(l > 0.f)) m = -INFINITY;   // (a row that sees none of the part's keys)
-        float M = m;
+        const bool nothing = l == 0.f;
+        float M = nothing ? -INFINITY : m;
 #pragma unroll
         for (int sh = kMaxCluster / 2; sh > 0; sh >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, sh));
-        const float w = (l > 0.f) ? fast_exp2((m - M) * p.scale_log2) : 0.f;
+        const float w = nothing ? 0.f : fast_exp2((m - M) * p.scale_log2);
         float sum = w * l;
 #pragma unroll
         for (int sh = kMaxCluster / 2; sh > 0; sh >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, sh);
         if (row < rows) {
-            asm volatile("st.shared.f32 [%0], %1;" ::"r"(w_at + (uint32_t)(row * kMaxCluster + i) * 4u), "f"(sum > 0.f ? w / sum : 0.f) : "memory");
+            asm volatile("st.shared.f32 [%0], %1;" ::"r"(w_at + (uint32_t)(row * kMaxCluster + i) * 4u), "f"(nothing ? -1.f : w / sum) : "memory");
             if (i == 0 && p.lse != nullptr)
                 p.lse[((long long)b * p.Hq + h) * p.Sq + q0 + row] = sum > 0.f ? (M * p.scale_log2 + log2f(sum)) * 0.6931471805599453f : -INFINITY;
         }
@@ -798,7 +799,7 @@ __device__ __forceinline__ void pp_split_merge(const FwdParams& p, uint32_t part
 #pragma unroll
             for (int k = 0; k < 4; ++k)
 #pragma unroll
-                for (int c = 0; c < 4; ++c) acc[k][c] = w[k] > 0.f ? fmaf(w[k], v[k][c], acc[k][c]) : acc[k][c];
+                for (int c = 0; c < 4; ++c) acc[k][c] = w[k] < 0.f ? acc[k][c] : fmaf(w[k], v[k][c], acc[k][c]);
         }
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
@@ -974,7 +975,8 @@ __device__ __forceinline__ bool pp_attention(const CUtensorMap& tm_q, const CUte
                     if (!ok) break;
                     const float l_other = ss.l_xch[xb][r];
                     // the other warpgroup's sum is relative to the reference this one's last step received
-                    if (l_other > 0.f) l_run += l_other * fast_exp2((m_before - m_loc) * scale_log2);
+                    // (a NaN, from a NaN or infinite score, must stay one: where CTAs share a tile the sum is all the merge looks at)
+                    if (l_other != 0.f) l_run += l_other * fast_exp2((m_before - m_loc) * scale_log2);
                 }
                 // (before the wait for the last P V, which takes longer than this)
                 // (FP8: O and the row sum carry the same factor on the probabilities; V's own factor goes on O)

@@ -1526,3 +1526,51 @@ def test_query_tiles_shared_by_a_cluster(fa, B, hq, hkv, sq, skv, dtype, causal)
     # CTAs in the first causal rows, ragged last tiles and rows that see nothing of a part; 75 items do not.
     # (bf16 also with the fp32 output)
     full_case(fa, B, hq, hkv, sq, skv, causal, dtype, seed=1700 + sq + skv)
+
+
+def expect_nonfinite(o, lse, q, k, v, causal, scale):
+    """Rows whose visible scores hold a NaN or an infinity have a NaN output and no finite LSE; every
+    other row is the oracle's (its inputs with the bad keys and queries, which it does not see, as zeros)."""
+    g = q.shape[2] // k.shape[2]
+    s = torch.einsum("bqhd,bkhd->bhqk", q.float().double(), k.float().double().repeat_interleave(g, 2))
+    hide = torch.ones(s.shape[-2:], dtype=torch.bool).triu(s.shape[-1] - s.shape[-2] + 1) if causal else torch.zeros(1, 1, dtype=torch.bool)
+    # (a score of -inf beside finite ones only has weight zero)
+    bad = ((torch.isnan(s) | torch.isposinf(s)) & ~hide).any(-1)   # [B,H,Sq]
+    assert bad.any()
+    o, lse = o.float().cpu(), lse.float().cpu()
+    assert torch.isnan(o.transpose(1, 2)[bad]).all(), "a row that sees a non-finite score has a finite output"
+    assert not torch.isfinite(lse[bad]).any()
+    o_ref, l_ref = oracle.attention_full(q.nan_to_num(0, 0, 0), k.nan_to_num(0, 0, 0), v, causal, scale)
+    good = ~bad & ~(torch.isneginf(s) & ~hide).any(-1)
+    keep = good[:, :, :, None].transpose(1, 2).expand(o.shape)
+    assert_close_to_oracle(torch.where(keep, o.double(), o_ref), torch.where(good, lse.double(), l_ref), o_ref, l_ref, what="rows that see only finite scores")
+
+
+@pytest.mark.parametrize("value", [float("nan"), float("inf"), float("-inf")])
+@pytest.mark.parametrize("where", ["k_early", "k_late", "q"])
+@pytest.mark.parametrize("B,hq,hkv,sq,skv,causal", [(1, 2, 2, 1500, 1500, True), (1, 2, 1, 200, 2100, False), (1, 8, 2, 128, 4000, True),
+                                                    (8, 32, 32, 200, 300, True)])
+def test_nonfinite_scores_are_not_hidden(fa, B, hq, hkv, sq, skv, causal, where, value):
+    # the first three share query tiles among a cluster's CTAs: one part's non-finite row sum must reach the row
+    cfg = synth.PrefillConfig("t", B, hq, hkv, sq, skv, dtype="fp16", causal=causal, seed=1900 + skv)
+    q, k, v = synth.prefill_inputs(cfg, "cpu")
+    if where == "q":
+        q[0, sq // 2, 0, 3] = value
+    else:
+        k[0, skv // 3 if where == "k_early" else skv - 2, 0, 5] = value
+    o, lse = run_forward(fa, q.to(DEV), k.to(DEV), v.to(DEV), causal, cfg.scale)
+    expect_nonfinite(o, lse, q, k, v, causal, cfg.scale)
+
+
+@pytest.mark.parametrize("key", [100, 1700])
+def test_shared_query_tiles_with_an_infinite_value(fa, key):
+    # an infinite entry of V reaches its column of every row that sees the key, whatever the key's weight
+    cfg = synth.PrefillConfig("t", 1, 2, 2, 300, 2000, dtype="fp16", causal=False, seed=1950)
+    q, k, v = synth.prefill_inputs(cfg, "cpu")
+    v[0, key, 1, 7] = float("inf")
+    k[0, key] *= 20   # weights from nearly 1 down to 0
+    o, _ = run_forward(fa, q.to(DEV), k.to(DEV), v.to(DEV), False, cfg.scale)
+    fin = torch.isfinite(o.cpu())
+    assert not fin[0, :, 1, 7].any()
+    fin[0, :, 1, 7] = True
+    assert fin.all()
