@@ -165,7 +165,7 @@ __device__ __forceinline__ void dec_cluster_merge(const float* part, const float
                 }
             }
             if (live) {
-                const bool any = M != -INFINITY;   // (several query tokens: one that sees no key at all)
+                const bool any = wsum != 0.f;   // (several query tokens: one that sees no key at all)
                 const float inv = any ? 1.f / wsum : 0.f;
                 store(r, col, make_float4(acc[0] * inv, acc[1] * inv, acc[2] * inv, acc[3] * inv), any ? M + logf(wsum) : -INFINITY);
             }
@@ -195,9 +195,13 @@ __device__ __forceinline__ float4 dec_warp_merge(const float* mo, const float* m
         acc[2] += sw * v.z;
         acc[3] += sw * v.w;
     }
-    // (l == 0: a query token that sees none of this chunk's keys)
-    lse = (l > 0.f) ? (M * scale_log2 + log2f(l)) * 0.6931471805599453f : -INFINITY;
-    const float inv = (l > 0.f) ? 1.f / l : 0.f;
+    if (l == 0.f) {   // a query token that sees none of this chunk's keys, whatever their values are
+        lse = -INFINITY;
+        return make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    // (a NaN sum, from a NaN or infinite score, makes the row and its log-sum-exp NaN here and in the merges)
+    lse = (M * scale_log2 + log2f(l)) * 0.6931471805599453f;
+    const float inv = 1.f / l;
     return make_float4(acc[0] * inv * factor, acc[1] * inv * factor, acc[2] * inv * factor, acc[3] * inv * factor);
 }
 // Four consecutive elements of an output row.
@@ -753,8 +757,12 @@ fa_decode_combine_kernel(const DecodeParams p, T* o, float* lse) {
     const float* lp = p.lse_part + (long long)bh * p.n_chunks;
     const float* op = p.o_part + (long long)bh * p.n_chunks * D;
     float M = -INFINITY;
-    for (int c = 0; c < nc; ++c) M = fmaxf(M, lp[c]);
-    if (nc == 0 || M == -INFINITY) {   // no keys, or (several query rows) a token that sees none
+    bool none = true;   // no keys, or (several query rows) a token that sees none
+    for (int c = 0; c < nc; ++c) {
+        M = fmaxf(M, lp[c]);
+        none = none && lp[c] == -INFINITY;   // (a NaN is skipped by the max)
+    }
+    if (none) {
         o[(long long)bh * D + tid] = T(0.f);
         if (lse && tid == 0) lse[lse_at] = -INFINITY;
         return;

@@ -1574,3 +1574,64 @@ def test_shared_query_tiles_with_an_infinite_value(fa, key):
     assert not fin[0, :, 1, 7].any()
     fin[0, :, 1, 7] = True
     assert fin.all()
+
+
+def expect_nonfinite_decode(o, lse, q, k, v, sl, scale, o_ref, l_ref):
+    """As expect_nonfinite for [B,Sq,Hq,d] rows that are the last of every sequence; the LSE is NaN as well."""
+    B, Sq, Hq, _ = q.shape
+    g = Hq // k.shape[2]
+    s = torch.einsum("bqhd,bkhd->bqhk", q.float().double(), k.float().double().repeat_interleave(g, 2))
+    at = torch.arange(k.shape[1])[None, None, :]
+    seen = at <= sl[:, None, None].long() - Sq + torch.arange(Sq)[None, :, None]   # [B,Sq,keys]
+    seen = seen & (at < sl[:, None, None])
+    bad = ((torch.isnan(s) | torch.isposinf(s)) & seen[:, :, None, :]).any(-1)     # [B,Sq,Hq]
+    unsure = (torch.isneginf(s) & seen[:, :, None, :]).any(-1) & ~bad              # (a weight of zero: not in the reference's inputs)
+    o, lse = o.float().cpu(), lse.float().cpu().transpose(1, 2)
+    assert bad.any()
+    assert torch.isnan(o[bad]).all() and torch.isnan(lse[bad]).all()
+    good = ~bad & ~unsure
+    o = torch.where(good[..., None], o.double(), o_ref)
+    lse = torch.where(good, lse.double(), l_ref.transpose(1, 2))
+    assert_close_to_oracle(o, lse, o_ref, l_ref.transpose(1, 2), what="rows that see only finite scores")
+
+
+# one query row and four, keys as rows and heads as rows, the chunks in one cluster and split with a merge kernel
+@pytest.mark.parametrize("where", ["k_nan", "k_inf", "q_nan", "q_inf"])
+@pytest.mark.parametrize("B,hq,hkv,Sq,smax,d", [(1, 5, 5, 1, 4000, 128), (2, 24, 2, 1, 700, 128), (1, 8, 2, 4, 900, 64), (2, 32, 2, 3, 600, 128),
+                                                (40, 8, 8, 1, 2600, 128), (40, 8, 8, 2, 2600, 64), (1, 4, 4, 1, 90, 128)])
+def test_decode_nonfinite_scores_are_not_hidden(fa, B, hq, hkv, Sq, smax, d, where):
+    cfg = synth.DecodeConfig("t", B, hq, hkv, smax, smax // 2, smax, d=d, seed=1970 + B + smax)
+    q, k, v, sl = synth.decode_inputs(cfg, "cpu", poison=False)
+    if Sq > 1:
+        q = torch.cat([q, q.flip(2), -q, q.flip(3)][:Sq], dim=1)
+    o_ref, l_ref = oracle.decode_append(q, k, v, sl, cfg.scale)
+    bad = float(where[2:])
+    qb, kb = q.clone(), k.clone()
+    if where[0] == "q":
+        qb[0, Sq - 1, 0, 3] = bad
+    else:
+        # (the first of several query rows sees it as its last key; the infinity's sign makes one head's score +inf at least)
+        kb[0, int(sl[0]) - Sq, hkv - 1, 5] = math.copysign(bad, float(q[0, 0, hq - 1, 5]))
+    o, lse = run_decode_append(fa, qb.to(DEV), kb.to(DEV), v.to(DEV), sl.to(DEV), cfg.scale)
+    expect_nonfinite_decode(o, lse, qb, kb, v, sl, cfg.scale, o_ref, l_ref)
+    if d == 128 and Sq == 1 and not where == "k_inf":   # the FP8 cache has no infinity
+        k8, v8 = synth.fp8_cache(k, v, sl, 0.25, 0.125, poison=False)
+        o_ref, l_ref = oracle.decode_fp8(q, k8, v8, sl, cfg.scale, 0.25, 0.125)
+        if where == "k_nan":
+            k8[0, int(sl[0]) - Sq, hkv - 1, 5] = 0x7f
+        o, lse = run_decode_fp8(fa, qb.to(DEV), k8.to(DEV), v8.to(DEV), sl.to(DEV), cfg.scale, 0.25, 0.125)
+        expect_nonfinite_decode(o, lse[:, :, None], qb, kb, v, sl, cfg.scale, o_ref[:, None], l_ref[:, :, None])
+
+
+@pytest.mark.parametrize("B,hkv,smax,length", [(1, 5, 1025, 1025), (40, 8, 2600, 2049)])
+def test_append_a_token_does_not_see_the_values_of_a_later_chunk(fa, B, hkv, smax, length):
+    # the last key is alone in its chunk (128-key chunks in a cluster; 2048-key chunks and a merge kernel), and the
+    # first of two query rows does not see it: a NaN there must not reach that row
+    cfg = synth.DecodeConfig("t", B, hkv, hkv, smax, length, length, seed=1990 + B)
+    q, k, v, sl = synth.decode_inputs(cfg, "cpu", poison=False)
+    q = torch.cat([q, -q], dim=1)
+    o_ref, l_ref = oracle.decode_append(q, k, v, sl, cfg.scale)
+    v[:, length - 1] = float("nan")
+    o, lse = run_decode_append(fa, q.to(DEV), k.to(DEV), v.to(DEV), sl.to(DEV), cfg.scale)
+    assert torch.isnan(o[:, 1]).all()
+    assert_close_to_oracle(o[:, :1], lse[:, :, :1], o_ref[:, :1], l_ref[:, :, :1], what="row before the NaN")
