@@ -195,14 +195,14 @@ __device__ __forceinline__ float4 dec_warp_merge(const float* mo, const float* m
         acc[2] += sw * v.z;
         acc[3] += sw * v.w;
     }
-    if (l == 0.f) {   // a query token that sees none of this chunk's keys, whatever their values are
-        lse = -INFINITY;
-        return make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    // (a NaN sum, from a NaN or infinite score, makes the row and its log-sum-exp NaN here and in the merges)
-    lse = (M * scale_log2 + log2f(l)) * 0.6931471805599453f;
-    const float inv = 1.f / l;
-    return make_float4(acc[0] * inv * factor, acc[1] * inv * factor, acc[2] * inv * factor, acc[3] * inv * factor);
+    // l == 0: a query token that sees none of this chunk's keys, whatever their values are.  (A NaN sum, from a
+    // NaN or infinite score, makes the row and its log-sum-exp NaN here and in the merges.)
+    const bool none = l == 0.f;
+    lse = none ? -INFINITY : (M * scale_log2 + log2f(l)) * 0.6931471805599453f;
+    const float inv = none ? 0.f : 1.f / l;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) acc[k] = none ? 0.f : acc[k] * inv * factor;
+    return make_float4(acc[0], acc[1], acc[2], acc[3]);
 }
 // Four consecutive elements of an output row.
 template <typename T>
@@ -757,11 +757,10 @@ fa_decode_combine_kernel(const DecodeParams p, T* o, float* lse) {
     const float* lp = p.lse_part + (long long)bh * p.n_chunks;
     const float* op = p.o_part + (long long)bh * p.n_chunks * D;
     float M = -INFINITY;
-    bool none = true;   // no keys, or (several query rows) a token that sees none
-    for (int c = 0; c < nc; ++c) {
-        M = fmaxf(M, lp[c]);
-        none = none && lp[c] == -INFINITY;   // (a NaN is skipped by the max)
-    }
+    for (int c = 0; c < nc; ++c) M = fmaxf(M, lp[c]);
+    bool none = M == -INFINITY;   // no keys, or (several query rows) a token that sees none ...
+    if (none)                     // ... unless there is a NaN, which the max skips
+        for (int c = 0; c < nc; ++c) none = none && lp[c] == -INFINITY;
     if (none) {
         o[(long long)bh * D + tid] = T(0.f);
         if (lse && tid == 0) lse[lse_at] = -INFINITY;
