@@ -15,6 +15,7 @@ namespace fa {
 
 constexpr int kDecTile = 128;                 // keys per shared-memory tile
 constexpr int kDecStages = 3;                 // ring depth (K and V tiles each)
+constexpr float kDecRefDropLog2 = 6.f;        // see DecodeParams::ref_tiles
 constexpr int kDecTileBytes = 32768;          // a tile of d = 128
 // Head dimension D (128 or 64): a tile is 128 keys x D 16-bit elements, one or two swizzled
 // boxes, in a ring of three slots per operand.  With D = 64 a CTA's rings are 96 KiB and two
@@ -55,6 +56,16 @@ struct DecodeParams {
     // the chunks of a sequence are a cluster's CTAs and are merged through distributed shared
     // memory (see decode_plan); o_final and lse_final are then the result's
     int clustered = 0;
+    // Tiles (a power of two) after which the reference of the probabilities, the running max, is lowered
+    // by ref_drop.  The probabilities are rounded to 16 bits for the second product, all but that of the
+    // key that sets the reference, which is exactly 1: the fewer keys share a reference, the smaller is
+    // the rounding error.  Chunks that are longer only because a sequence is one cluster's (see
+    // decode_plan) lower it where they would end without the cluster, so that the next keys set their
+    // own (1 sequence, 5 heads, 8192 keys: 2.54e-4 from the result in 64 bits, 2.61e-4 without this).
+    // What has been summed grows by up to 2^6 each time; a cluster's chunks are at most eight times as
+    // long as without it, so it stays far inside fp32.
+    int ref_tiles = 1 << 30;
+    float ref_drop = 0.f;   // kDecRefDropLog2 / scale_log2
     int bf16_io = 0;      // 8-bit cache kernel only: q and o are bf16 (fp16 otherwise)
 };
 
@@ -223,7 +234,7 @@ __device__ __forceinline__ void dec_store4(void* o, long long at, const float4& 
 // 2 t4, 2 t4 + 1 must not see (they came after the row's token).
 // Leaves each warp's (max, sum, O) in mo / ml in the layout the merge expects; returns false
 // after a wait that gave up.
-template <bool kMulti, typename T, int D>
+template <bool kMulti, typename T, int D, bool kCluster>
 __device__ __forceinline__ bool dec_consume_key_rows(const DecodeParams& p, uint64_t* bars, volatile uint32_t* abort_flag,
                                                      uint32_t sK, uint32_t sV, float* mo, float* ml, int warp, int lane,
                                                      const T* q_col, int hide0, int hide1, int len, int k_begin, int k_end,
@@ -255,6 +266,7 @@ __device__ __forceinline__ bool dec_consume_key_rows(const DecodeParams& p, uint
         const int st = t % kStages;
         const uint32_t parity = (t / kStages) & 1;
         const int valid = min(kDecTile, k_end - (k_begin + t * kDecTile)) - key_w;  // valid keys of this warp's 32
+        const float drop = kCluster && (t & (p.ref_tiles - 1)) == 0 ? p.ref_drop : 0.f;   // see DecodeParams
         ok = mbar_wait(smem_u32(&bars[st]), parity, abort_flag, 20);
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
@@ -300,7 +312,7 @@ __device__ __forceinline__ bool dec_consume_key_rows(const DecodeParams& p, uint
             }
             // finite when key 0 of the warp is visible (always with one query token; an earlier
             // token of several may see none of the warp's keys: its state then stays empty)
-            const float mn0 = fmaxf(m_run[0], mx0), mn1 = fmaxf(m_run[1], mx1);
+            const float mn0 = fmaxf(m_run[0] - drop, mx0), mn1 = fmaxf(m_run[1] - drop, mx1);
             const float a0 = (m_run[0] == -INFINITY) ? 0.f : fast_exp2((m_run[0] - mn0) * p.scale_log2);
             const float a1 = (m_run[1] == -INFINITY) ? 0.f : fast_exp2((m_run[1] - mn1) * p.scale_log2);
             m_run[0] = mn0;
@@ -402,7 +414,10 @@ __device__ __forceinline__ bool dec_consume_key_rows(const DecodeParams& p, uint
 // D: the head dimension, 128 or 64.
 // kKeyRows (at most 8 (token, head) rows per kv head): the consumers work in the keys-as-rows
 // form (dec_consume_key_rows).
-template <bool kMulti, typename T = __half, int D = 128, bool kKeyRows = false>
+// kCluster: the chunks of a sequence are a cluster's CTAs (p.clustered).  (An instantiation of its own, as lowering
+// the reference costs every tile two instructions and the merge below registers: 200 sequences of up to 600 keys,
+// not clustered, 10.14 us in one instantiation for both, 10.33 with the reference, 9.98 apart.)
+template <bool kMulti, typename T, int D, bool kKeyRows, bool kCluster>
 __global__ void __launch_bounds__(kDecMmaThreads, DecShape<D>::kCtasPerSm)
 fa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                            const DecodeParams p) {
@@ -535,7 +550,7 @@ fa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
             const T* q_col = (g < G) ? static_cast<const T*>(p.q) + row_index(g) * D : nullptr;
             const int hide0 = kMulti ? Sq - 1 - row_token(min(2 * t4, G - 1)) : 0;
             const int hide1 = kMulti ? Sq - 1 - row_token(min(2 * t4 + 1, G - 1)) : 0;
-            ok = dec_consume_key_rows<kMulti, T, D>(p, bars, &abort_flag, sK, sV, mo, ml, warp, lane, q_col, hide0, hide1,
+            ok = dec_consume_key_rows<kMulti, T, D, kCluster>(p, bars, &abort_flag, sK, sV, mo, ml, warp, lane, q_col, hide0, hide1,
                                                     len, k_begin, k_end, n_tiles);
         } else {
         // Q as A fragments for the D / 16 k-steps (rows >= G are zero)
@@ -566,6 +581,7 @@ fa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
             const int st = t % kStages;
             const uint32_t parity = (t / kStages) & 1;
             const int valid = min(kDecTile, k_end - (k_begin + t * kDecTile)) - key_w;  // valid keys of this warp's 32
+            const float drop = kCluster && (t & (p.ref_tiles - 1)) == 0 ? p.ref_drop : 0.f;   // see DecodeParams
             ok = mbar_wait(smem_u32(&bars[st]), parity, &abort_flag, 20);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
@@ -614,7 +630,7 @@ fa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
                 mx_hi = fmaxf(mx_hi, __shfl_xor_sync(0xffffffffu, mx_hi, 2));
                 // finite when key 0 of the warp is visible (always with one query row; an earlier
                 // token of several may see none of the warp's keys: its state then stays empty)
-                const float mn_lo = fmaxf(m_lo, mx_lo), mn_hi = fmaxf(m_hi, mx_hi);
+                const float mn_lo = fmaxf(m_lo - drop, mx_lo), mn_hi = fmaxf(m_hi - drop, mx_hi);
                 const float a_lo = (m_lo == -INFINITY) ? 0.f : fast_exp2((m_lo - mn_lo) * p.scale_log2);
                 const float a_hi = (m_hi == -INFINITY) ? 0.f : fast_exp2((m_hi - mn_hi) * p.scale_log2);
                 m_lo = mn_lo;
@@ -715,7 +731,7 @@ fa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
             for (int r = tid / (D / 4); r < G; r += 512 / D) {
                 float lse;
                 const float4 out = dec_warp_merge<D>(mo, ml, r, col, p.scale_log2, 1.f, lse);
-                if (p.clustered) {
+                if (kCluster) {
                     *reinterpret_cast<float4*>(&part[r * D + col]) = out;
                     if (col == 0) part_lse[r] = lse;
                 } else if (p.o_final != nullptr) {   // the only chunk: this is the result
@@ -729,7 +745,7 @@ fa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
             }
         }
     }
-    if (p.clustered) {
+    if constexpr (kCluster) {
         const int n_live = (len + p.chunk - 1) / p.chunk;
         dec_cluster_merge<D>(part, part_lse, G, c, n_live, tid, [&](int r, int col, const float4& out, float lse) {
             dec_store4<T>(p.o_final, row_index(r) * D + col, out);

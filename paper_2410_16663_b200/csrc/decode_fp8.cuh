@@ -38,7 +38,7 @@ __device__ __forceinline__ uint32_t bf16x2_to_f16x2(uint32_t v) {
 }
 
 // grid: (Hkv * ceil(g / 16), n_chunks, B) with g = Hq / Hkv (the kv head fastest, see decode.cuh)
-template <int NB>
+template <int NB, bool kCluster>
 __global__ void __launch_bounds__(kDec8Threads, 2)
 fa_decode_split_fp8_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                            const DecodeParams p) {
@@ -196,6 +196,7 @@ fa_decode_split_fp8_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
             const int st = t % kDec8Stages;
             const uint32_t parity = (t / kDec8Stages) & 1;
             const int valid = min(kDecTile, k_end - (k_begin + t * kDecTile)) - key_w;  // valid keys of this warp's 32
+            const float drop = kCluster && (t & (p.ref_tiles - 1)) == 0 ? p.ref_drop : 0.f;   // see DecodeParams
             ok = mbar_wait(smem_u32(&bars[st]), parity, &abort_flag, 20);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
@@ -244,7 +245,7 @@ fa_decode_split_fp8_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
                         mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, sh));
                         mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, sh));
                     }
-                    const float mn0 = fmaxf(m_run[nbk][0], mx0), mn1 = fmaxf(m_run[nbk][1], mx1);  // finite: key 0 of the warp is valid
+                    const float mn0 = fmaxf(m_run[nbk][0] - drop, mx0), mn1 = fmaxf(m_run[nbk][1] - drop, mx1);  // finite: key 0 of the warp is valid
                     const float a0 = (m_run[nbk][0] == -INFINITY) ? 0.f : fast_exp2((m_run[nbk][0] - mn0) * p.scale_log2);
                     const float a1 = (m_run[nbk][1] == -INFINITY) ? 0.f : fast_exp2((m_run[nbk][1] - mn1) * p.scale_log2);
                     m_run[nbk][0] = mn0;
@@ -365,7 +366,7 @@ fa_decode_split_fp8_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
                 float lse;
                 const float4 out = dec_warp_merge<128>(mo, ml, r, col, p.scale_log2, p.v_scale, lse);
                 const long long row = (long long)b * p.Hq + h0 + r;
-                if (p.clustered) {
+                if (kCluster) {
                     *reinterpret_cast<float4*>(&part[r * 128 + col]) = out;
                     if (col == 0) part_lse[r] = lse;
                 } else if (p.o_final != nullptr) {   // the only chunk: this is the result
@@ -380,7 +381,7 @@ fa_decode_split_fp8_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
             }
         }
     }
-    if (p.clustered) {
+    if constexpr (kCluster) {
         const int n_live = (len + p.chunk - 1) / p.chunk;
         dec_cluster_merge<128>(part, part_lse, G, c, n_live, tid, [&](int r, int col, const float4& out, float lse) {
             const long long row = (long long)b * p.Hq + h0 + r;

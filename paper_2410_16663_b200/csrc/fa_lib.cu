@@ -433,9 +433,9 @@ int decode_chunk(int B, int Hkv, int Smax, bool long_ok = false) {
 
 // The clusters of a decode kernel that run at a time; kind: 0 = 16-bit, d = 128; 1 = 16-bit, d = 64; 2 = 8-bit.
 int decode_cluster_slots(int kind, fa::ClusterSlots* out) {
-    const void* kern = kind == 2   ? reinterpret_cast<const void*>(fa::fa_decode_split_fp8_kernel<1>)
-                       : kind == 1 ? reinterpret_cast<const void*>(fa::fa_decode_split_mma_kernel<false, __half, 64, true>)
-                                   : reinterpret_cast<const void*>(fa::fa_decode_split_mma_kernel<false, __half, 128, true>);
+    const void* kern = kind == 2   ? reinterpret_cast<const void*>(fa::fa_decode_split_fp8_kernel<1, true>)
+                       : kind == 1 ? reinterpret_cast<const void*>(fa::fa_decode_split_mma_kernel<false, __half, 64, true, true>)
+                                   : reinterpret_cast<const void*>(fa::fa_decode_split_mma_kernel<false, __half, 128, true, true>);
     const int smem = kind == 2 ? fa::kDec8Smem : kind == 1 ? fa::DecShape<64>::kSmem : fa::DecShape<128>::kSmem;
     const int ce = fa::cluster_slots(kern, smem, fa::kDecMmaThreads, out);
     return ce ? cuda_fail(static_cast<cudaError_t>(ce)) : FA_OK;
@@ -446,6 +446,17 @@ int decode_cluster_slots(int kind, fa::ClusterSlots* out) {
 struct DecodePlan {
     int chunk = 256, n_chunks = 1;
     bool clustered = false;
+    int plain_chunk = 256;   // keys per chunk without the cluster
+    void fill(fa::DecodeParams* dp) const {   // (after scale_log2)
+        dp->chunk = chunk;
+        dp->n_chunks = n_chunks;
+        dp->clustered = clustered;
+        // (with next to no scale all scores count alike and no probability is rounded)
+        if (clustered && dp->scale_log2 > 1e-20f) {
+            dp->ref_tiles = plain_chunk / fa::kDecTile;
+            dp->ref_drop = fa::kDecRefDropLog2 / dp->scale_log2;
+        }
+    }
 };
 // ctas: CTAs per chunk over all sequences (B * Hkv, and a multiple above 16 rows per kv head).
 //
@@ -475,6 +486,7 @@ int decode_plan(int kind, long long ctas, int B, int Hkv, int Smax, bool long_ok
             const int per = (tiles + c - 1) / c;
             // (d = 64 and 8-bit run two CTAs per SM)
             if (per <= 12 || (B == 1 && (kind == 0 ? per <= 16 || ctas * c >= 74 : ctas * c >= 148))) {
+                pl.plain_chunk = pl.chunk;
                 pl.chunk = per * fa::kDecTile;
                 pl.n_chunks = (tiles + per - 1) / per;
                 pl.clustered = pl.n_chunks > 1;
@@ -821,14 +833,15 @@ int decode_launch(const CUtensorMap& tk, const CUtensorMap& tv, const fa::Decode
         int sm_count = 0;
         // at most 8 (token, head) rows per kv head: the keys-as-rows form of the consumers
         const bool key_rows = g * Sq <= 8;
-        auto kern = bf16 ? ((Sq > 1) ? (key_rows ? fa::fa_decode_split_mma_kernel<true, __nv_bfloat16, D, true>
-                                                 : fa::fa_decode_split_mma_kernel<true, __nv_bfloat16, D>)
-                                     : (key_rows ? fa::fa_decode_split_mma_kernel<false, __nv_bfloat16, D, true>
-                                                 : fa::fa_decode_split_mma_kernel<false, __nv_bfloat16, D>))
-                         : ((Sq > 1) ? (key_rows ? fa::fa_decode_split_mma_kernel<true, __half, D, true>
-                                                 : fa::fa_decode_split_mma_kernel<true, __half, D>)
-                                     : (key_rows ? fa::fa_decode_split_mma_kernel<false, __half, D, true>
-                                                 : fa::fa_decode_split_mma_kernel<false, __half, D>));
+        using Kernel = void (*)(CUtensorMap, CUtensorMap, fa::DecodeParams);
+        // by type, several query rows, consumer form, and whether the chunks of a sequence are one cluster
+        static const Kernel kernels[2][2][2][2] = {
+#define FA_DEC(T, M, R) {fa::fa_decode_split_mma_kernel<M, T, D, R, false>, fa::fa_decode_split_mma_kernel<M, T, D, R, true>}
+            {{FA_DEC(__half, false, false), FA_DEC(__half, false, true)}, {FA_DEC(__half, true, false), FA_DEC(__half, true, true)}},
+            {{FA_DEC(__nv_bfloat16, false, false), FA_DEC(__nv_bfloat16, false, true)},
+             {FA_DEC(__nv_bfloat16, true, false), FA_DEC(__nv_bfloat16, true, true)}}};
+#undef FA_DEC
+        const Kernel kern = kernels[bf16][Sq > 1][key_rows][dp.clustered != 0];
         if (int ce = fa::prepare_big_smem_kernel(reinterpret_cast<const void*>(kern), smem, &sm_count))
             return cuda_fail(static_cast<cudaError_t>(ce));
         dim3 grid(Hkv * ((g * Sq + 15) / 16), dp.n_chunks, B);   // 16 (token, head) rows per CTA
@@ -867,13 +880,11 @@ int decode_impl(const void* q, const void* k_cache, const void* v_cache, void* o
     DecodePlan plan;
     rc = decode_plan(d == 64 ? 1 : 0, (long long)B * Hkv * ((g * Sq + 15) / 16), B, Hkv, Skv_max, true, &plan);
     if (rc) return rc;
-    dp.chunk = plan.chunk;
-    dp.n_chunks = plan.n_chunks;
-    dp.clustered = plan.clustered;
+    dp.scale_log2 = scale * 1.4426950408889634f;
+    plan.fill(&dp);
     if (dp.n_chunks > 65535) return FA_ERR_UNSUPPORTED;   // the chunks are the grid's second dimension
     dp.o_part = static_cast<float*>(workspace);
     dp.lse_part = dp.o_part + (size_t)B * Sq * Hq * dp.n_chunks * d;
-    dp.scale_log2 = scale * 1.4426950408889634f;
     dp.block_table = block_table;
     dp.page_size = block_table ? page_size : 1;
     dp.table_stride = table_stride;
@@ -938,13 +949,11 @@ static int decode_fp8_impl(const void* q, const void* k_cache, const void* v_cac
     DecodePlan plan;
     rc = decode_plan(2, (long long)B * Hkv * ((g + 15) / 16), B, Hkv, Skv_max, false, &plan);
     if (rc) return rc;
-    dp.chunk = plan.chunk;
-    dp.n_chunks = plan.n_chunks;
-    dp.clustered = plan.clustered;
+    dp.scale_log2 = scale * k_scale * 1.4426950408889634f;   // the scores are q . (k_scale * k8)
+    plan.fill(&dp);
     if (dp.n_chunks > 65535) return FA_ERR_UNSUPPORTED;   // the chunks are the grid's second dimension
     dp.o_part = static_cast<float*>(workspace);
     dp.lse_part = dp.o_part + (size_t)B * Hq * dp.n_chunks * 128;
-    dp.scale_log2 = scale * k_scale * 1.4426950408889634f;   // the scores are q . (k_scale * k8)
     dp.block_table = block_table;
     dp.page_size = block_table ? page_size : 1;
     dp.table_stride = table_stride;
@@ -967,7 +976,8 @@ static int decode_fp8_impl(const void* q, const void* k_cache, const void* v_cac
         constexpr int smem = fa::kDec8Smem;
         int sm_count = 0;
         // keys as the MMA's rows and up to 8 query heads as its columns (two column blocks for 9..16 heads)
-        auto kern = (g > 8) ? fa::fa_decode_split_fp8_kernel<2> : fa::fa_decode_split_fp8_kernel<1>;
+        auto kern = dp.clustered ? ((g > 8) ? fa::fa_decode_split_fp8_kernel<2, true> : fa::fa_decode_split_fp8_kernel<1, true>)
+                                 : ((g > 8) ? fa::fa_decode_split_fp8_kernel<2, false> : fa::fa_decode_split_fp8_kernel<1, false>);
         if (int ce = fa::prepare_big_smem_kernel(reinterpret_cast<const void*>(kern), smem, &sm_count))
             return cuda_fail(static_cast<cudaError_t>(ce));
         dim3 grid(Hkv * ((g + 15) / 16), dp.n_chunks, B);

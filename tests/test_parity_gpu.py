@@ -1635,3 +1635,32 @@ def test_append_a_token_does_not_see_the_values_of_a_later_chunk(fa, B, hkv, sma
     o, lse = run_decode_append(fa, q.to(DEV), k.to(DEV), v.to(DEV), sl.to(DEV), cfg.scale)
     assert torch.isnan(o[:, 1]).all()
     assert_close_to_oracle(o[:, :1], lse[:, :, :1], o_ref[:, :1], l_ref[:, :, :1], what="row before the NaN")
+
+
+@pytest.mark.parametrize("hq,hkv,Sq,d,fp8", [(5, 5, 1, 128, False), (45, 5, 1, 128, False), (5, 5, 4, 64, False), (5, 5, 1, 128, True),
+                                             (45, 5, 1, 128, True)])
+def test_decode_in_a_cluster_rounds_no_more_than_in_short_chunks(fa, hq, hkv, Sq, d, fp8):
+    # One key of every 256 counts (score 6, the others -40), and neighbours among them differ by 3/64 in the score and
+    # in the sign of their value: O is (sum over pairs of 1 - e^(-3/64)) / (sum of 1 + e^(-3/64)).  With a reference of its
+    # own for every 256 keys each of these probabilities is exactly 1 when it is rounded, and what is left is fp32 and the
+    # rounding of the stored output: 2^-11 of it, plus 2^-19.  A common reference would round e^(-3/64) to
+    # fp16, which is 1.05e-4 off, and half of that in O.
+    S, delta = 8192, 3 / 64
+    k = torch.zeros(1, S, hkv, d, dtype=torch.float64)
+    v = torch.zeros(1, S, hkv, d, dtype=torch.float64)
+    k[..., 0] = -40
+    at = torch.arange(5, S, 256)
+    k[:, at, :, 0] = 6
+    k[:, at[1::2], :, 1] = -3   # times 1/64 from the query: exact in e4m3 as well
+    v[:, at] = 1
+    v[:, at[1::2]] = -1
+    q = torch.zeros(1, Sq, hq, d, dtype=torch.float16, device=DEV)
+    q[..., 0], q[..., 1] = 1, 1 / 64
+    sl = torch.tensor([S], dtype=torch.int32, device=DEV)
+    if fp8:
+        k8, v8 = (t.float().to(torch.float8_e4m3fn).view(torch.uint8).to(DEV) for t in (k, v))
+        o, _ = run_decode_fp8(fa, q, k8, v8, sl, 1.0, 1.0, 1.0)
+    else:
+        o, _ = run_decode_append(fa, q, k.to(torch.float16).to(DEV), v.to(torch.float16).to(DEV), sl, 1.0)
+    want = (1 - math.exp(-delta)) / (1 + math.exp(-delta))
+    assert float((o.double() - want).abs().max()) <= 2 ** -11 * want + 2 ** -19
