@@ -152,7 +152,7 @@ __device__ __forceinline__ PpItem pp_decode_item(const FwdParams& p, int b, int 
             // the first table entry is fetched together with the lengths, so that a loader does
             // not start an item with two dependent global loads (the entry exists for every
             // sequence; its value is ignored when the sequence has no keys)
-            const int first_page = __ldg(p.block_table + (long long)it.b * p.table_stride);
+            const int first_page = p.block_table[(long long)it.b * p.table_stride];
             it.Skv = p.seqlens_k[it.b];
             it.page0 = it.Skv > 0 ? first_page : -1;
         } else {
@@ -258,7 +258,7 @@ struct PpSource {
     __device__ __forceinline__ void request_next() {
         if (walk.used_up()) request();
     }
-    __device__ __forceinline__ int place_of(int s) const { return (__ldg(p.cu_q + s) >> 7) + s; }
+    __device__ __forceinline__ int place_of(int s) const { return (p.cu_q[s] >> 7) + s; }
     __device__ __forceinline__ void packed_place(int idx, int& b, int& h, int& qt) {
         int v, rem;
         if (p.fixed_places) {
@@ -512,9 +512,10 @@ __device__ __forceinline__ int pp_page_of(const FwdParams& p, int b, int j, int 
     if (kVarlen && p.block_table != nullptr && j < n) {
         // (volatile: issued here, ahead of the wait that follows, not where the value is used)
         int page;
-        asm volatile("ld.global.nc.s32 %0, [%1];"
+        asm volatile("ld.global.s32 %0, [%1];"
                      : "=r"(page)
-                     : "l"(p.block_table + (long long)b * p.table_stride + p.by_tiles_per_page.div(j)));
+                     : "l"(p.block_table + (long long)b * p.table_stride + p.by_tiles_per_page.div(j))
+                     : "memory");
         return page;
     }
     return 0;

@@ -121,7 +121,9 @@ __global__ void fa_selftest_wait_kernel(unsigned long long limit_ns, unsigned in
 // Every attention kernel is launched as a programmatic dependent of whatever precedes it in the
 // stream (launch_dependent in prefill_simple.cuh): its CTAs may start, and set up their barriers and
 // tensor memory, while the kernel before it still runs.  grid_dep_wait() blocks until that kernel
-// has completed and its writes are visible; nothing may read or write global memory before it.
+// has completed and its writes are visible; nothing may read or write global memory before it, and
+// nothing at all is read through the non-coherent path (__ldg, ld.global.nc), which wants data that
+// nobody writes while the kernel lives: its life begins while the kernel before it still writes.
 // grid_dep_launch() lets the next kernel of the stream start in the same way as soon as every CTA of
 // this one has issued it (the first thread of a CTA counts).  A kernel with tensor memory issues it
 // after the barrier behind its allocation: an early CTA of the next kernel on the same SM could

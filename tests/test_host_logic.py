@@ -36,6 +36,16 @@ def test_every_place_of_the_item_list_is_taken_once_whatever_cta_starts_when(tmp
     run_host_check("item_walk_check", tmp_path)
 
 
+def test_kernels_read_nothing_through_the_non_coherent_path():
+    """A kernel launched as a programmatic dependent lives while the one before it still writes, so its
+    inputs are not read-only for its lifetime, which __ldg and ld.global.nc require."""
+    csrc = os.path.join(ROOT, "paper_2410_16663_b200", "csrc")
+    for name in sorted(os.listdir(csrc)):
+        for n, line in enumerate(open(os.path.join(csrc, name)), 1):
+            code = line.split("//")[0]
+            assert "__ldg" not in code and "global.nc" not in code, f"{name}:{n}: {line.strip()}"
+
+
 def test_paged_from_packed_keeps_every_row_where_the_table_says():
     """The page pool built from a packed batch holds, behind its block table, exactly the packed
     rows of every sequence; rows of a last page past the end of its sequence, and the spare
