@@ -121,11 +121,14 @@ def fa_last_cuda_error() -> int:
 
 
 # The current stream's handle without building a torch.cuda.Stream object around it: a call on a few
-# hundred keys is bound by what the host does for it, and the object took 3.4 us of its 10.5.
-_raw_stream, _device = torch._C._cuda_getCurrentRawStream, torch.cuda.current_device
+# hundred keys is bound by what the host does for it, and the object took 3.4 us of its 10.5.  The
+# function is torch's own and not promised: a torch without it (one without CUDA among them) takes the object.
+_raw_stream, _device = getattr(torch._C, "_cuda_getCurrentRawStream", None), torch.cuda.current_device
 
 
 def _stream() -> int:
+    if _raw_stream is None:
+        return int(torch.cuda.current_stream().cuda_stream)
     return _raw_stream(_device())
 
 

@@ -338,3 +338,21 @@ def test_forward_proj_validation(fa):
     assert call(outp=P(out) + 16) == fa.FA_ERR_ALIGN and call(wp=P(w) + 2) == fa.FA_ERR_ALIGN
     assert call(wsp=None) == fa.FA_ERR_WORKSPACE and call(wsn=2) == fa.FA_ERR_WORKSPACE
     assert call(wsp=P(ws) + 1) == fa.FA_ERR_ALIGN
+
+
+def test_binding_loads_with_a_torch_that_lacks_the_raw_stream_lookup(fa, monkeypatch):
+    # the lookup is private to torch: a build without it takes the stream object's handle instead
+    import importlib.util
+
+    if hasattr(torch._C, "_cuda_getCurrentRawStream"):
+        monkeypatch.delattr(torch._C, "_cuda_getCurrentRawStream")
+    spec = importlib.util.spec_from_file_location("binding_without_lookup", fa.__file__)
+    mod = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(mod)
+    assert mod.fa_version() == fa.fa_version()
+
+    class Stream:
+        cuda_stream = 1234
+
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: Stream())
+    assert mod._stream() == 1234
