@@ -138,17 +138,22 @@ int encode_map_matrix(CUtensorMap* tm, const void* base, int rows, int cols, boo
 // a page holds a multiple of the 128-key tile, or 16, 32 or 64 keys (several pages per tile)
 bool page_size_ok(int ps) { return ps > 0 && (ps % fa::kDecTile == 0 || ps == 16 || ps == 32 || ps == 64); }
 
-int check_device() {
-    static thread_local int cached_dev = -1, cached_rc = FA_OK;
+// sms: receives the device's SM count
+int check_device(int* sms = nullptr) {
+    static thread_local int cached_dev = -1, cached_rc = FA_OK, cached_sms = 0;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return cuda_fail(e);
-    if (dev == cached_dev) return cached_rc;
-    int major = 0;
-    e = cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev);
-    if (e != cudaSuccess) return cuda_fail(e);
-    cached_dev = dev;
-    cached_rc = (major == 10) ? FA_OK : FA_ERR_DEVICE;
+    if (dev != cached_dev) {
+        int major = 0, n = 0;
+        e = cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+        if (e != cudaSuccess) return cuda_fail(e);
+        cached_dev = dev;
+        cached_rc = (major == 10) ? FA_OK : FA_ERR_DEVICE;
+        cached_sms = n;
+    }
+    if (sms) *sms = cached_sms;
     return cached_rc;
 }
 
@@ -266,7 +271,8 @@ int forward_impl(const fa_params& in, cudaStream_t st) {
     if (!aligned16(p.q) || !aligned16(p.k) || !aligned16(p.v) || !aligned16(p.o)) return FA_ERR_ALIGN;
     if (p.lse && (reinterpret_cast<uintptr_t>(p.lse) & 3u)) return FA_ERR_ALIGN;
 
-    int rc = check_device();
+    int sms = 0;
+    int rc = check_device(&sms);
     if (rc) return rc;
 
     fa::FwdParams fp = dense_fwd_params(p);
@@ -338,7 +344,7 @@ int forward_impl(const fa_params& in, cudaStream_t st) {
     int variant = p.variant;
     if (variant == 0) {
         const bool two_by_two = fp.n_qtiles == 2 && p.Skv > fa::kTile && p.Skv <= 2 * fa::kTile;
-        variant = (!p.causal && two_by_two && 2ll * p.B * p.Hq >= 3 * 148) ? 4 : 3;
+        variant = (!p.causal && two_by_two && 2ll * p.B * p.Hq >= 3ll * sms) ? 4 : 3;
     }
     switch (variant) {
         case 4:  // pipelined kernel, two query tiles per CTA
@@ -470,22 +476,22 @@ struct DecodePlan {
 // 32768 keys: 23.3 / 20.1; of up to 4096 level or ahead up to 12 tiles per chunk), and one sequence
 // with very few kv heads leaves most SMs idle (1 kv head, 65536 keys: 27.9 / 21.6; 8-bit, 5 kv heads,
 // 32768 keys: 17.7 / 16.2).
-int decode_plan(int kind, long long ctas, int B, int Hkv, int Smax, bool long_ok, DecodePlan* plan) {
+int decode_plan(int kind, int sms, long long ctas, int B, int Hkv, int Smax, bool long_ok, DecodePlan* plan) {
     DecodePlan pl;
     if (Smax > 0) {
         pl.chunk = decode_chunk(B, Hkv, Smax, long_ok);
         pl.n_chunks = (Smax + pl.chunk - 1) / pl.chunk;
     }
     const int tiles = (Smax + fa::kDecTile - 1) / fa::kDecTile;
-    if (tiles > 1 && ctas <= 1024) {
+    if (tiles > 1 && ctas <= sms) {   // (no more clusters of two run at a time, with two CTAs per SM)
         fa::ClusterSlots slots;
         if (int rc = decode_cluster_slots(kind, &slots)) return rc;
         int c = tiles < fa::kMaxCluster ? tiles : fa::kMaxCluster;
         while (c > 1 && slots.n[c] < ctas) --c;
         if (c > 1) {
             const int per = (tiles + c - 1) / c;
-            // (d = 64 and 8-bit run two CTAs per SM)
-            if (per <= 12 || (B == 1 && (kind == 0 ? per <= 16 || ctas * c >= 74 : ctas * c >= 148))) {
+            // (a CTA for half of the SMs, or one of two for each: d = 64 and 8-bit run two per SM)
+            if (per <= 12 || (B == 1 && (kind == 0 ? per <= 16 || 2 * ctas * c >= sms : ctas * c >= sms))) {
                 pl.plain_chunk = pl.chunk;
                 pl.chunk = per * fa::kDecTile;
                 pl.n_chunks = (tiles + per - 1) / per;
@@ -867,7 +873,8 @@ int decode_impl(const void* q, const void* k_cache, const void* v_cache, void* o
     if (!aligned16(workspace)) return FA_ERR_ALIGN;
     const size_t need = fa_decode_append_workspace_bytes(B, Sq, Hq, Hkv, Skv_max, d);
     if (need > 0 && (!workspace || workspace_bytes < need)) return FA_ERR_WORKSPACE;
-    rc = check_device();
+    int sms = 0;
+    rc = check_device(&sms);
     if (rc) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
 
@@ -878,7 +885,7 @@ int decode_impl(const void* q, const void* k_cache, const void* v_cache, void* o
     dp.Sq = Sq;
     const int g = Hq / Hkv;
     DecodePlan plan;
-    rc = decode_plan(d == 64 ? 1 : 0, (long long)B * Hkv * ((g * Sq + 15) / 16), B, Hkv, Skv_max, true, &plan);
+    rc = decode_plan(d == 64 ? 1 : 0, sms, (long long)B * Hkv * ((g * Sq + 15) / 16), B, Hkv, Skv_max, true, &plan);
     if (rc) return rc;
     dp.scale_log2 = scale * 1.4426950408889634f;
     plan.fill(&dp);
@@ -937,7 +944,8 @@ static int decode_fp8_impl(const void* q, const void* k_cache, const void* v_cac
         return FA_ERR_ALIGN;
     const size_t need = fa_decode_workspace_bytes(B, Hq, Hkv, Skv_max, d);
     if (need > 0 && (!workspace || workspace_bytes < need)) return FA_ERR_WORKSPACE;
-    int rc = check_device();
+    int sms = 0;
+    int rc = check_device(&sms);
     if (rc) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
 
@@ -947,7 +955,7 @@ static int decode_fp8_impl(const void* q, const void* k_cache, const void* v_cac
     dp.B = B; dp.Hq = Hq; dp.Hkv = Hkv; dp.Smax = Skv_max;
     const int g = Hq / Hkv;
     DecodePlan plan;
-    rc = decode_plan(2, (long long)B * Hkv * ((g + 15) / 16), B, Hkv, Skv_max, false, &plan);
+    rc = decode_plan(2, sms, (long long)B * Hkv * ((g + 15) / 16), B, Hkv, Skv_max, false, &plan);
     if (rc) return rc;
     dp.scale_log2 = scale * k_scale * 1.4426950408889634f;   // the scores are q . (k_scale * k8)
     plan.fill(&dp);
