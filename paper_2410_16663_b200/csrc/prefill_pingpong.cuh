@@ -187,19 +187,24 @@ __device__ __forceinline__ int pp_split_item(const FwdParams& p, PpItem& it) {
 // holds some SMs, CTAs that found one may be through with their deal before the others get theirs.
 struct PpWalk {
     int deal_ctas, deal_rounds;
-    int share;       // CTA whose share this is
-    int round = 0;   // places of it taken so far
+    int place = 0, step = 0;   // the next place, and how far the one after it is
+    int left = 0;              // places left
 
-    __host__ __device__ __forceinline__ bool used_up() const { return round >= (share < deal_ctas ? deal_rounds : 1); }
-    // The next place of the share (only if it is not used up).
+    __host__ __device__ __forceinline__ bool used_up() const { return left == 0; }
+    // The next place (only if the share is not used up).
     __host__ __device__ __forceinline__ int next() {
-        const int r = round++;
-        if (share >= deal_ctas) return deal_rounds * deal_ctas + share - deal_ctas;
-        return r * deal_ctas + ((r & 1) ? deal_ctas - 1 - share : share);
+        const int at = place;
+        place += step;
+        step = 2 * deal_ctas - step;   // (a round that goes up is followed by one that goes down)
+        --left;
+        return at;
     }
-    __host__ __device__ __forceinline__ void take_over(int cta) {
-        share = cta;
-        round = 0;
+    // Starts on the share of a CTA.
+    __host__ __device__ __forceinline__ void take(int cta) {
+        const bool dealing = cta < deal_ctas;
+        place = dealing ? cta : deal_rounds * deal_ctas + cta - deal_ctas;
+        step = 2 * (deal_ctas - cta) - 1;
+        left = dealing ? deal_rounds : 1;
     }
 };
 
@@ -312,7 +317,7 @@ struct PpSource {
                     pending = false;
                     const int cta = clc_answer(answer);
                     if (cta < 0) return false;
-                    walk.take_over(cta);
+                    walk.take(cta);
                 }
                 const int idx = walk.next();
                 if (idx >= total_items) return false;   // (a list that is all dealt)
@@ -547,7 +552,8 @@ __device__ __forceinline__ void pp_run_load_qk(uint32_t bar0, uint32_t sQ, uint3
     const uint64_t pol_q = l2_policy_evict_first(), pol_kv = l2_policy_evict_last();
     PpRing<kPpNK> ring;
     PpSource<kVarlen> source{p, total_items, pp_bar(bar0, ppb::claim), smem_u32(&ss.claim_answer), abort_flag,
-                             {p.deal_ctas, p.deal_rounds, (int)blockIdx.x}};
+                             {p.deal_ctas, p.deal_rounds}};
+    source.walk.take(blockIdx.x);
     PpItem it;
     for (int ord = 0;; ++ord) {
         if (!source.next(it)) it.n = 0;   // no further item: the others are told so

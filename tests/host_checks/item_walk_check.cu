@@ -29,7 +29,10 @@ static bool run(int deal_ctas, int rounds, int rest, int resident, int order, un
     while (!waiting.empty() || !running.empty()) {
         // the hardware starts CTAs while there is room, and there always is when nothing runs
         while (!waiting.empty() && (int)running.size() < resident && (late_starts || running.empty() || (int)running.size() + (int)waiting.size() == grid))
-            running.push_back({dealing, rounds, next_waiting()});
+        {
+            running.push_back({dealing, rounds});
+            running.back().take(next_waiting());
+        }
         const int i = (int)(rng() % running.size());
         fa::PpWalk& w = running[i];
         if (w.used_up()) {
@@ -39,7 +42,7 @@ static bool run(int deal_ctas, int rounds, int rest, int resident, int order, un
                 running.pop_back();
                 continue;
             }
-            w.take_over(next_waiting());
+            w.take(next_waiting());
         }
         const int at = w.next();
         if (at < 0 || at >= total) {
