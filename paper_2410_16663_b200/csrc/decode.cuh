@@ -417,6 +417,10 @@ __device__ __forceinline__ bool dec_consume_key_rows(const DecodeParams& p, uint
 // kCluster: the chunks of a sequence are a cluster's CTAs (p.clustered).  (An instantiation of its own, as lowering
 // the reference costs every tile two instructions and the merge below registers: 200 sequences of up to 600 keys,
 // not clustered, 10.14 us in one instantiation for both, 10.33 with the reference, 9.98 apart.)
+// (The kernels here do not release the next one early: its CTAs would take the places of this one's, or those
+// next to it, and wait there.  16 sequences of up to 4096 keys, d = 64, 22.3 us with an early release, 20.5
+// without; one of 32768 keys, 24.9 / 23.2; 8 of up to 8000, 30.5 / 29.6; 5 heads x 8192, 7.03 / 6.85; calls
+// of 6 us level.)
 template <bool kMulti, typename T, int D, bool kKeyRows, bool kCluster>
 __global__ void __launch_bounds__(kDecMmaThreads, DecShape<D>::kCtasPerSm)
 fa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
@@ -456,7 +460,6 @@ fa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
         tma_prefetch_desc(&tm_k);
         tma_prefetch_desc(&tm_v);
     }
-    grid_dep_launch();
     grid_dep_wait();
     int len = p.seqlens[b];
     len = max(0, min(len, p.Smax));
@@ -765,7 +768,6 @@ fa_decode_combine_kernel(const DecodeParams p, T* o, float* lse) {
     // lse is [B,Hq,Sq]
     const long long lse_at = ((long long)b * p.Hq + bh % p.Hq) * p.Sq + (bh / p.Hq) % p.Sq;
     const int tid = threadIdx.x;
-    grid_dep_launch();
     grid_dep_wait();   // the split kernel's partial results are complete and visible from here on
     int len = p.seqlens[b];
     len = max(0, min(len, p.Smax));

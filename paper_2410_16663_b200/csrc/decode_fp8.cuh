@@ -68,7 +68,6 @@ fa_decode_split_fp8_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
         tma_prefetch_desc(&tm_k);
         tma_prefetch_desc(&tm_v);
     }
-    grid_dep_launch();
     grid_dep_wait();
     int len = p.seqlens[b];
     len = max(0, min(len, p.Smax));

@@ -317,6 +317,7 @@ int forward_impl(const fa_params& in, cudaStream_t st) {
         if (int ce = fa::prepare_big_smem_kernel(reinterpret_cast<const void*>(kern), fa::kD64SlimSmem, &sm_count))
             return cuda_fail(static_cast<cudaError_t>(ce));
         dim3 grid(fp.n_qtiles, fp.Hq, fp.B);
+        fp.early_next = (long long)fp.n_qtiles * fp.Hq * fp.B < 4ll * sm_count;
         const cudaError_t e = fa::launch_dependent(kern, grid, 128, fa::kD64SlimSmem, st, tq, tk, tv, fp);
         return e == cudaSuccess ? FA_OK : cuda_fail(e);
     }
@@ -330,6 +331,7 @@ int forward_impl(const fa_params& in, cudaStream_t st) {
         rc = encode_map(&tvh, p.v, p.B, p.Skv, p.Hkv, p.v_stride[0], p.v_stride[1], p.v_stride[2], 64, bf16, p.d);
         if (rc) return rc;
         dim3 grid(fp.n_qtiles, fp.Hq, fp.B);
+        fp.early_next = (long long)fp.n_qtiles * fp.Hq * fp.B < sm_count;
         const cudaError_t e = fa::launch_dependent(kern, grid, fa::kD256Threads, fa::kD256Smem, st, tq, tk, tvh, fp);
         return e == cudaSuccess ? FA_OK : cuda_fail(e);
     }

@@ -104,7 +104,7 @@ fa_fwd_d256_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    grid_dep_launch();
+    if (p.early_next) grid_dep_launch();
     const uint32_t tmem_base = tmem_holder;
 
     constexpr bool kBf16 = std::is_same<T, __nv_bfloat16>::value;

@@ -71,7 +71,7 @@ fa_fwd_d64_slim_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    grid_dep_launch();
+    if (p.early_next) grid_dep_launch();
     const uint32_t tmem_base = tmem_holder;
     const uint32_t tS = tmem_base + (static_cast<uint32_t>(warp * 32) << 16);
 

@@ -74,12 +74,12 @@ struct FwdParams {
     FastDiv by_tiles_per_page;  // page_size / 128: kv tile j lies in table entry j / that, at tile j % that of the page
     int d;  // head dimension: 128, or 64 (its own kernel)
     float out_scale;  // factor on O (FP8 operands: the factor of V; 1 otherwise)
-    // Persistent kernels: whether the next kernel of the stream may begin its set-up at once
-    // (grid_dep_launch).  Only when the grid leaves SMs free: when it fills them, the early CTAs of
-    // the next launch land on whichever SM is done first, neighbours in the item order end up on
+    // Whether the next kernel of the stream may begin its set-up at once (grid_dep_launch).  Only
+    // when the grid leaves room for CTAs: when it fills the device, the early CTAs of the next launch
+    // land on whichever SM is done first, neighbours in the item order end up on
     // different dies and their K and V are no longer shared in one L2 (4 x 32 heads x 2048 keys:
-    // 179 against 174 us with the next kernel's launch left to the end; 2 heads x 512: 12.6
-    // against 15.7 us with an early one).
+    // 179 against 174 us with the next kernel's launch left to the end; d = 64, 256 x 16 x 128: 73.4
+    // against 70.6; d = 256 level; 2 heads x 512: 12.6 against 15.7 us with an early one).
     int early_next = 0;
     // ping-pong kernel (see PpSource): the first deal_rounds rounds of the item list are dealt to the
     // first deal_ctas CTAs; the rest, if claim_items, is claimed one by one

@@ -118,9 +118,9 @@ __global__ void fa_selftest_wait_kernel(unsigned long long limit_ns, unsigned in
 }
 
 // ------------------------------------------------------------------ programmatic dependent launch
-// Every attention kernel is launched as a programmatic dependent of whatever precedes it in the
-// stream (launch_dependent in prefill_simple.cuh): its CTAs may start, and set up their barriers and
-// tensor memory, while the kernel before it still runs.  grid_dep_wait() blocks until that kernel
+// The attention kernels are launched as programmatic dependents of whatever precedes them in the
+// stream (launch_dependent in prefill_simple.cuh; not the simple kernels and not the fused projection):
+// the CTAs may start, and set up their barriers and tensor memory, while the kernel before still runs.  grid_dep_wait() blocks until that kernel
 // has completed and its writes are visible; nothing may read or write global memory before it, and
 // nothing at all is read through the non-coherent path (__ldg, ld.global.nc), which wants data that
 // nobody writes while the kernel lives: its life begins while the kernel before it still writes.
@@ -128,7 +128,8 @@ __global__ void fa_selftest_wait_kernel(unsigned long long limit_ns, unsigned in
 // this one has issued it (the first thread of a CTA counts).  A kernel with tensor memory issues it
 // after the barrier behind its allocation: an early CTA of the next kernel on the same SM could
 // otherwise get columns that a CTA of this one still needs, and each would wait for the other.
-// Both do nothing in an ordinary launch.
+// Who issues it early is a matter of measurement (FwdParams::early_next; the decode kernels never do,
+// see decode.cuh).  Both do nothing in an ordinary launch.
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
