@@ -1,7 +1,7 @@
 // Decode-stage attention (one query row per sequence over the cached K and V), split along
 // the cache: each CTA streams one chunk of one (sequence, kv head) through a TMA-fed
 // shared-memory ring and keeps running (rowmax, rowsum, O) for the query heads that share
-// the kv head; a second kernel merges the per-chunk partial results.  The work is a single
+// the kv head; the CTAs of a cluster, or a second kernel, merge the per-chunk partial results.  The work is a single
 // pass over the cache, so the kernel is written for HBM bandwidth: every cache byte is read
 // exactly once and nothing but the partials is written.
 #pragma once

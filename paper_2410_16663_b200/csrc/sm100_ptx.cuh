@@ -140,8 +140,9 @@ __device__ __forceinline__ void clc_request(uint32_t dst, uint32_t bar) {
     asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];" ::"r"(dst), "r"(bar)
                  : "memory");
 }
-// The answer: blockIdx.x of the CTA that will not be launched, or -1 if every CTA has started (no
-// further request may be made then).
+// The answer: blockIdx.x of the CTA that will not be launched -- any that has not started -- or -1 if
+// there was none to cancel: every CTA has started, or the request was declined and the others will be
+// launched.  No further request may be made then.
 __device__ __forceinline__ int clc_answer(uint32_t src) {
     int x;
     asm volatile(
