@@ -119,7 +119,7 @@ __device__ __forceinline__ void load_tile_hint(uint32_t dst, const CUtensorMap* 
 // code.  The table of what has been done is keyed by kernel address and device; concurrent first
 // calls at worst repeat the same idempotent set-up.
 inline int prepare_big_smem_kernel(const void* kern, int smem_bytes, int* sm_count) {
-    constexpr int kMaxDev = 64, kMaxKernels = 64;
+    constexpr int kMaxDev = 64, kMaxKernels = 128;   // (some sixty kernels ask; one past the end would be set up on every call)
     struct Entry {
         const void* kern;
         int sms[kMaxDev];
