@@ -37,11 +37,8 @@ namespace fa {
 #ifndef FA_PP_NK
 #define FA_PP_NK 3
 #endif
-#ifndef FA_PP_NV
-#define FA_PP_NV 2
-#endif
 constexpr int kPpNK = FA_PP_NK;   // K ring slots
-constexpr int kPpNV = FA_PP_NV;   // V ring slots
+constexpr int kPpNV = 2;          // V ring slots: those of the steps' parities
 constexpr int kPpQBufs = 2;
 constexpr int kPpSlots = 4;       // work items the Q/K loader may be ahead of the slowest role
 static_assert((kPpQBufs + kPpNK + kPpNV) * kTileBytes + 3072 <= 232448, "shared memory budget");
@@ -76,9 +73,8 @@ constexpr int q_empty = 2;                      // [2]  S thread (commit) -> loa
 constexpr int k_full = 4;                       // [NK]
 constexpr int k_empty = k_full + kPpNK;         // [NK]
 constexpr int v_full = k_empty + kPpNK;         // [NV]
-constexpr int v_empty = v_full + kPpNV;         // [NV]
-constexpr int s_full = v_empty + kPpNV;         // [2]  S thread (commit) -> softmax
-constexpr int pv_done = s_full + 2;             // [2]  PV thread (commit) -> softmax
+constexpr int s_full = v_full + kPpNV;          // [2]  S thread (commit) -> softmax
+constexpr int pv_done = s_full + 2;             // [2]  PV thread (commit) -> softmax, and -> V loader: V of step g is in slot g & 1
 constexpr int o_final = pv_done + 2;            // [2]  PV thread (commit) -> epilogue, by item parity
 constexpr int item_full = o_final + 2;          // [kPpSlots] Q/K loader -> every other role: a work item is in the slot
 constexpr int item_empty = item_full + kPpSlots;   // [kPpSlots] back: three single-thread roles and eight softmax warps
@@ -503,7 +499,6 @@ __device__ __forceinline__ void pp_run_pv(uint32_t bar0, uint32_t sV, uint32_t t
                                (ks > 0) ? 1u : (j > 0 ? 1u : 0u));
             }
             mma_commit(pp_bar(bar0, ppb::pv_done + buf));
-            mma_commit(pp_bar(bar0, ppb::v_empty + ring.slot));
             if (j == it.n - 1) mma_commit(pp_bar(bar0, ppb::o_final + (ord & 1)));
         }
     }
@@ -598,7 +593,7 @@ __device__ __forceinline__ void pp_run_load_v(uint32_t bar0, uint32_t sV, const 
         int page = (kVarlen && p.block_table != nullptr) ? it.page0 : 0;
         for (int j = 0; j < it.n; ++j, ring.next()) {
             const int page_next = pp_page_of<kVarlen>(p, it.b, j + 1, it.n, it.Skv);
-            if (!mbar_wait(pp_bar(bar0, ppb::v_empty + ring.slot), ring.par ^ 1, abort_flag, 152)) return;
+            if (!mbar_wait(pp_bar(bar0, ppb::pv_done + ring.slot), ring.par ^ 1, abort_flag, 152)) return;
             mbar_expect_tx(pp_bar(bar0, ppb::v_full + ring.slot), PpOperands<kF8, D>::kKvSlotBytes);
             int row = kVarlen ? it.k_base + j * kTile : (it.j0 + j) * kTile, slab = kVarlen ? 0 : it.b;
             pp_paged_tile<kVarlen>(p, page, j, row, slab);
@@ -686,42 +681,42 @@ struct PpSoftmax {
         const float neg_ms = -((m_new == -INFINITY) ? 0.f : m_new) * scale_log2 + (kF8 ? kP8ScaleLog2 : 0.f);
         const uint64_t sc2 = f2_pack(scale_log2, scale_log2), nm2 = f2_pack(neg_ms, neg_ms);
         uint64_t la = f2_pack(0.f, 0.f), lb = la;
-        {
-            uint32_t pk[Op::kPCols];
-            const bool p_free = g < 2 || mbar_test(pp_bar(bar0, ppb::pv_done + w), ((g >> 1) - 1) & 1);
-            pp_exp_chunk<T, kF8>(s, 0, sc2, nm2, la, lb, pk);
-            if (g >= 2) {
-                // O += P V of step g-2 has read this P buffer
-                if (!__all_sync(0xffffffffu, p_free) &&
-                    !pp_warp_wait(pp_bar(bar0, ppb::pv_done + w), ((g >> 1) - 1) & 1, abort_flag, 116 + w))
-                    return false;
-                tc_fence_after();
-            }
-            if (__builtin_expect(j > 0 && __any_sync(0xffffffffu, grow), 0)) {
-                // rare: the reference moved.  O holds the P V sums up to step g-1 once that step's
-                // MMAs have completed (those of step g-2 have, see above, so the parity wait on the
-                // other buffer's barrier is one phase at most behind).
-                if (!pp_warp_wait(pp_bar(bar0, ppb::pv_done + (1 - w)), ((g - 1) >> 1) & 1, abort_flag, 114 + w)) return false;
-                tc_fence_after();
-                const float alpha = grow ? ((m_prev == -INFINITY) ? 0.f : fast_exp2((m_prev - mx) * scale_log2)) : 1.f;
+        // All of P is formed in registers (a packed pair takes the place of two scores) and goes to tensor
+        // memory in one piece at the end.  Stored chunk by chunk, the first store had to wait for P V of
+        // step g-2, which ends about 1400 clocks after that step's P was handed over, and a warpgroup's step
+        // was that long plus the other three chunks: 32 heads x 32768 7828 -> 7615 us, 8192 keys 541 -> 527,
+        // 5 heads x 4096 32.3 -> 31.3, 1001 queries over 7951 keys 472 -> 460, short sequences level.
+        uint32_t pk[4][Op::kPCols];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) pp_exp_chunk<T, kF8>(s, c, sc2, nm2, la, lb, pk[c]);
+        const bool p_free = g < 2 || mbar_test(pp_bar(bar0, ppb::pv_done + w), ((g >> 1) - 1) & 1);
+        pp_exp_chunk<T, kF8>(s, 3, sc2, nm2, la, lb, pk[3]);
+        if (g >= 2) {
+            // O += P V of step g-2 has read this P buffer
+            if (!__all_sync(0xffffffffu, p_free) &&
+                !pp_warp_wait(pp_bar(bar0, ppb::pv_done + w), ((g >> 1) - 1) & 1, abort_flag, 116 + w))
+                return false;
+            tc_fence_after();
+        }
+        if (__builtin_expect(j > 0 && __any_sync(0xffffffffu, grow), 0)) {
+            // rare: the reference moved.  O holds the P V sums up to step g-1 once that step's
+            // MMAs have completed (those of step g-2 have, see above, so the parity wait on the
+            // other buffer's barrier is one phase at most behind).
+            if (!pp_warp_wait(pp_bar(bar0, ppb::pv_done + (1 - w)), ((g - 1) >> 1) & 1, abort_flag, 114 + w)) return false;
+            tc_fence_after();
+            const float alpha = grow ? ((m_prev == -INFINITY) ? 0.f : fast_exp2((m_prev - mx) * scale_log2)) : 1.f;
 #pragma unroll 1
-                for (int c = 0; c < D / 16; ++c) {
-                    uint32_t o[16];
-                    tmem_ld_x16(tO + c * 16, o);
-                    tmem_wait_ld();
+            for (int c = 0; c < D / 16; ++c) {
+                uint32_t o[16];
+                tmem_ld_x16(tO + c * 16, o);
+                tmem_wait_ld();
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
-                    tmem_st_x16(tO + c * 16, o);
-                }
+                for (int i = 0; i < 16; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
+                tmem_st_x16(tO + c * 16, o);
             }
-            pp_store_p<kF8>(tP, pk);
         }
 #pragma unroll
-        for (int c = 1; c < 4; ++c) {
-            uint32_t pk[Op::kPCols];
-            pp_exp_chunk<T, kF8>(s, c, sc2, nm2, la, lb, pk);
-            pp_store_p<kF8>(tP + c * Op::kPCols, pk);
-        }
+        for (int c = 0; c < 4; ++c) pp_store_p<kF8>(tP + c * Op::kPCols, pk[c]);
         {
             float a0, a1, b0, b1;
             f2_unpack(la, a0, a1);
