@@ -607,6 +607,7 @@ __device__ __forceinline__ void pp_run_load_v(uint32_t bar0, uint32_t sV, const 
 // tensor-memory instructions that follow need the whole warp).
 __device__ __forceinline__ bool pp_warp_wait(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag,
                                              unsigned int where) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;   // the usual case, in one branch
     const bool ok = mbar_wait(bar, parity, abort_flag, where);
     return __all_sync(0xffffffffu, ok);
 }
@@ -645,8 +646,9 @@ struct PpSoftmax {
         tmem_ld_x32(tS + 96, *reinterpret_cast<uint32_t(*)[32]>(&s[96]));
         tmem_wait_ld();
         tc_fence_before();  // for the arrival below that hands the S buffer back
-        // probe early, look at the answer after the row max
-        const bool m_there = g > 0 && mbar_test(pp_bar(bar0, ppb::m_ready + (1 - w)), ((g - 1) >> 1) & 1);
+        // probe and read early, look at the answer after the row max
+        const bool m_there = g == 0 || mbar_test(pp_bar(bar0, ppb::m_ready + (1 - w)), ((g - 1) >> 1) & 1);
+        float m_prev = *m_other;
         if (masked) {
             // hidden scores become -inf (the scale is strictly positive, so they come out as exact zeros)
             const int kv0 = kv_first + j * kTile;
@@ -657,14 +659,12 @@ struct PpSoftmax {
                 if (i >= lim) s[i] = 0xff800000u;
         }
         const float mx = pp_row_max(s);
-        // reference max left by step g-1 (of the other warpgroup); an item starts afresh
-        float m_prev = -INFINITY;
-        if (g > 0) {
-            if (!__all_sync(0xffffffffu, m_there) &&
-                !pp_warp_wait(pp_bar(bar0, ppb::m_ready + (1 - w)), ((g - 1) >> 1) & 1, abort_flag, 112 + w))
-                return false;
-            if (j > 0) m_prev = *m_other;
+        // reference max left by step g-1 (of the other warpgroup, read above); an item starts afresh
+        if (!__all_sync(0xffffffffu, m_there)) {
+            if (!pp_warp_wait(pp_bar(bar0, ppb::m_ready + (1 - w)), ((g - 1) >> 1) & 1, abort_flag, 112 + w)) return false;
+            m_prev = *m_other;
         }
+        if (j == 0) m_prev = -INFINITY;
         m_before = m_prev;
         // lazy reference update: the reference moves only when the row max outgrew it by more than
         // the threshold (always on the first visible score; never on -inf)
@@ -674,10 +674,9 @@ struct PpSoftmax {
         // one arrival per thread: publishes its reference max and, the scores being in registers,
         // lets Q K^T of step g+2 overwrite the S buffer
         mbar_arrive(pp_bar(bar0, ppb::m_ready + w));
-        if (m_loc != m_new) {  // this warpgroup's row sum follows the reference
-            if (l_part > 0.f) l_part *= fast_exp2((m_loc - m_new) * scale_log2);
-            m_loc = m_new;
-        }
+        // this warpgroup's row sum follows the reference (a factor of 1 rather than a branch)
+        l_part *= m_loc == m_new ? 1.f : fast_exp2((m_loc - m_new) * scale_log2);
+        m_loc = m_new;
         const float neg_ms = -((m_new == -INFINITY) ? 0.f : m_new) * scale_log2 + (kF8 ? kP8ScaleLog2 : 0.f);
         const uint64_t sc2 = f2_pack(scale_log2, scale_log2), nm2 = f2_pack(neg_ms, neg_ms);
         uint64_t la = f2_pack(0.f, 0.f), lb = la;
@@ -686,35 +685,38 @@ struct PpSoftmax {
         // step g-2, which ends about 1400 clocks after that step's P was handed over, and a warpgroup's step
         // was that long plus the other three chunks: 32 heads x 32768 7828 -> 7615 us, 8192 keys 541 -> 527,
         // 5 heads x 4096 32.3 -> 31.3, 1001 queries over 7951 keys 472 -> 460, short sequences level.
+        // From there on the steps were bound by the warpgroups' own chains, and what those lost most on were
+        // branches (about 30 clocks each until they are resolved, and a scheduler has two of these warps).
+        // So a step's fast path has five: one for each of three waits -- a vote on a first probe, and
+        // everything rare behind it --, one for the mask and one at its end.  The same four cases: 7603 -> 7368,
+        // 526 -> 509, 31.4 -> 30.1, 460 -> 442; 4 x 32 x 2048 178 -> 172, 8 x 32 x 512 44.0 -> 42.6.
         uint32_t pk[4][Op::kPCols];
 #pragma unroll
         for (int c = 0; c < 3; ++c) pp_exp_chunk<T, kF8>(s, c, sc2, nm2, la, lb, pk[c]);
         const bool p_free = g < 2 || mbar_test(pp_bar(bar0, ppb::pv_done + w), ((g >> 1) - 1) & 1);
         pp_exp_chunk<T, kF8>(s, 3, sc2, nm2, la, lb, pk[3]);
-        if (g >= 2) {
+        if (__builtin_expect(!__all_sync(0xffffffffu, p_free && !(j > 0 && grow)), 0)) {
             // O += P V of step g-2 has read this P buffer
-            if (!__all_sync(0xffffffffu, p_free) &&
-                !pp_warp_wait(pp_bar(bar0, ppb::pv_done + w), ((g >> 1) - 1) & 1, abort_flag, 116 + w))
-                return false;
-            tc_fence_after();
-        }
-        if (__builtin_expect(j > 0 && __any_sync(0xffffffffu, grow), 0)) {
-            // rare: the reference moved.  O holds the P V sums up to step g-1 once that step's
-            // MMAs have completed (those of step g-2 have, see above, so the parity wait on the
-            // other buffer's barrier is one phase at most behind).
-            if (!pp_warp_wait(pp_bar(bar0, ppb::pv_done + (1 - w)), ((g - 1) >> 1) & 1, abort_flag, 114 + w)) return false;
-            tc_fence_after();
-            const float alpha = grow ? ((m_prev == -INFINITY) ? 0.f : fast_exp2((m_prev - mx) * scale_log2)) : 1.f;
+            if (g >= 2 && !pp_warp_wait(pp_bar(bar0, ppb::pv_done + w), ((g >> 1) - 1) & 1, abort_flag, 116 + w)) return false;
+            if (j > 0 && __any_sync(0xffffffffu, grow)) {
+                // rare: the reference moved.  O holds the P V sums up to step g-1 once that step's
+                // MMAs have completed (those of step g-2 have, see above, so the parity wait on the
+                // other buffer's barrier is one phase at most behind).
+                if (!pp_warp_wait(pp_bar(bar0, ppb::pv_done + (1 - w)), ((g - 1) >> 1) & 1, abort_flag, 114 + w)) return false;
+                tc_fence_after();
+                const float alpha = grow ? ((m_prev == -INFINITY) ? 0.f : fast_exp2((m_prev - mx) * scale_log2)) : 1.f;
 #pragma unroll 1
-            for (int c = 0; c < D / 16; ++c) {
-                uint32_t o[16];
-                tmem_ld_x16(tO + c * 16, o);
-                tmem_wait_ld();
+                for (int c = 0; c < D / 16; ++c) {
+                    uint32_t o[16];
+                    tmem_ld_x16(tO + c * 16, o);
+                    tmem_wait_ld();
 #pragma unroll
-                for (int i = 0; i < 16; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
-                tmem_st_x16(tO + c * 16, o);
+                    for (int i = 0; i < 16; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
+                    tmem_st_x16(tO + c * 16, o);
+                }
             }
         }
+        tc_fence_after();
 #pragma unroll
         for (int c = 0; c < 4; ++c) pp_store_p<kF8>(tP + c * Op::kPCols, pk[c]);
         {
@@ -963,14 +965,17 @@ __device__ __forceinline__ bool pp_attention(const CUtensorMap& tm_q, const CUte
             // no step of this warpgroup in the item (one step, the other warpgroup's): the next
             // step it takes belongs to the item whose Q load waits for the buffer, so hand it back now
             if (j >= n) hand_back_q();
-            for (; j < n && ok; j += 2) {
+            for (; j < n; j += 2) {
                 ok = sm.step(s, g_item + (uint32_t)j, j, j >= n_full);
-                hand_back_q();
-                if (ok && j == n - 2) {
-                    // the other warpgroup runs the last step and the epilogue: hand it this row sum
-                    // (it is relative to the reference this step left, which that step receives)
-                    ss.l_xch[xb][r] = sm.l_part;
-                    mbar_arrive(pp_bar(bar0, ppb::l_pub + xb));
+                if (!ok) break;
+                if (q_back >= 0 || j == n - 2) {   // (one branch where there is nothing to do)
+                    hand_back_q();
+                    if (j == n - 2) {
+                        // the other warpgroup runs the last step and the epilogue: hand it this row sum
+                        // (it is relative to the reference this step left, which that step receives)
+                        ss.l_xch[xb][r] = sm.l_part;
+                        mbar_arrive(pp_bar(bar0, ppb::l_pub + xb));
+                    }
                 }
             }
             const float l_part = sm.l_part, m_loc = sm.m_loc, m_before = sm.m_before;
