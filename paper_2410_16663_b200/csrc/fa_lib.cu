@@ -74,6 +74,33 @@ int encode_map(CUtensorMap* tm, const void* base, int B, int S, int H, int64_t s
     return FA_OK;
 }
 
+// Tensor map of the ping-pong kernel over a [B, S, H, d] 16-bit tensor: for d = 128 a box is box_rows positions x
+// all of d for one (batch, head) -- the dimensions are (64 elements of d, S, 64-element blocks of d, H, B), so
+// it lands block by block, box_rows rows of 128 swizzled bytes each --, for d = 64 that of encode_map.
+int encode_map_tile(CUtensorMap* tm, const void* base, int B, int S, int H, int64_t sb, int64_t ss, int64_t sh,
+                    int box_rows, bool bf16, int d = 128) {
+    if (d == 64) return encode_map(tm, base, B, S, H, sb, ss, sh, box_rows, bf16, d);
+    EncodeTiledFn fn = get_encode_fn();
+    if (!fn) return FA_ERR_DEVICE;
+    cuuint64_t dims[5] = {64, (cuuint64_t)S, (cuuint64_t)(d / 64), (cuuint64_t)H, (cuuint64_t)B};
+    cuuint64_t strides[4] = {(cuuint64_t)ss * 2, 128, (cuuint64_t)sh * 2, (cuuint64_t)sb * 2};
+    // a dimension of extent 1 never advances; give it a harmless legal stride
+    if (H == 1) strides[2] = (cuuint64_t)d * 2;
+    if (S == 1) strides[0] = strides[2] * (cuuint64_t)H;
+    if (B == 1) strides[3] = strides[0] * (cuuint64_t)S;
+    cuuint32_t box[5] = {64, (cuuint32_t)box_rows, (cuuint32_t)(d / 64), 1, 1};
+    cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+    CUresult r = fn(tm, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 5,
+                    const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                    CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) {
+        t_last_cuda_error = static_cast<int>(r);
+        return FA_ERR_CUDA;
+    }
+    return FA_OK;
+}
+
 // Tensor map over a contiguous 16-bit cache [slabs, S, H, d] (d = 128 or 64) whose box is box_rows keys
 // x all of d for one (slab, head): the dimensions are (64 elements of d, S, 64-element blocks of d, H,
 // slab), so a box lands block by block, box_rows rows of 128 swizzled bytes each.
@@ -288,15 +315,29 @@ int forward_impl(const fa_params& in, cudaStream_t st) {
         return e == cudaSuccess ? FA_OK : cuda_fail(e);
     }
 
+    // Default choice, from timings of both kernels: the ping-pong kernel (one query tile per CTA,
+    // Q K^T running ahead of the softmax), also on short sequences: paired tiles make half as many
+    // items of twice the length, which loses when there are few (1 x 2 heads x 512: 8.0 against 12.3
+    // us; 1 x 5 x 1000: 11.7 / 20.1; 1 x 32 x 512: 9.9 / 13.3), and an item boundary costs the
+    // ping-pong kernel less than it did (8 x 32 x 512: 42.0 / 48.9; 16 x 32 x 128: 18.5 / 25.3).  What
+    // is left to the paired kernel: without a mask, items of exactly two query and two kv tiles, at least three
+    // rounds of them (16 x 64/8 x 200: 56.1 against 61.8 us; 16 x 32 x 256: 38.1 / 39.8; causal level).
+    int variant = p.variant;
+    if (variant == 0 && p.d == 64) variant = p.Skv >= kD64PingPongFrom ? 3 : 0;
+    else if (variant == 0 && p.d == 128) {
+        const bool two_by_two = fp.n_qtiles == 2 && p.Skv > fa::kTile && p.Skv <= 2 * fa::kTile;
+        variant = (!p.causal && two_by_two && 2ll * p.B * p.Hq >= 3ll * sms) ? 4 : 3;
+    }
+    const auto encode = variant == 3 ? encode_map_tile : encode_map;
     CUtensorMap tq, tk, tv;
-    rc = encode_map(&tq, p.q, p.B, p.Sq, p.Hq, p.q_stride[0], p.q_stride[1], p.q_stride[2], 128, bf16, p.d);
+    rc = encode(&tq, p.q, p.B, p.Sq, p.Hq, p.q_stride[0], p.q_stride[1], p.q_stride[2], 128, bf16, p.d);
     if (rc) return rc;
-    rc = encode_map(&tk, p.k, p.B, p.Skv, p.Hkv, p.k_stride[0], p.k_stride[1], p.k_stride[2], 128, bf16, p.d);
+    rc = encode(&tk, p.k, p.B, p.Skv, p.Hkv, p.k_stride[0], p.k_stride[1], p.k_stride[2], 128, bf16, p.d);
     if (rc) return rc;
-    rc = encode_map(&tv, p.v, p.B, p.Skv, p.Hkv, p.v_stride[0], p.v_stride[1], p.v_stride[2], 128, bf16, p.d);
+    rc = encode(&tv, p.v, p.B, p.Skv, p.Hkv, p.v_stride[0], p.v_stride[1], p.v_stride[2], 128, bf16, p.d);
     if (rc) return rc;
 
-    if (p.d == 64 && (p.variant == 3 || (p.variant == 0 && p.Skv >= kD64PingPongFrom))) {
+    if (p.d == 64 && variant == 3) {
         // long sequences: the ping-pong kernel with tiles of one 64-element box (see PpOperands)
         CUtensorMap to = tq;
         if (!fp.o_fp32) {  // the output leaves through TMA stores of 32 rows x 64 columns
@@ -336,18 +377,6 @@ int forward_impl(const fa_params& in, cudaStream_t st) {
         return e == cudaSuccess ? FA_OK : cuda_fail(e);
     }
 
-    // Default choice, from timings of both kernels: the ping-pong kernel (one query tile per CTA,
-    // Q K^T running ahead of the softmax), also on short sequences: paired tiles make half as many
-    // items of twice the length, which loses when there are few (1 x 2 heads x 512: 8.0 against 12.3
-    // us; 1 x 5 x 1000: 11.7 / 20.1; 1 x 32 x 512: 9.9 / 13.3), and an item boundary costs the
-    // ping-pong kernel less than it did (8 x 32 x 512: 42.0 / 48.9; 16 x 32 x 128: 18.5 / 25.3).  What
-    // is left to the paired kernel: without a mask, items of exactly two query and two kv tiles, at least three
-    // rounds of them (16 x 64/8 x 200: 56.1 against 61.8 us; 16 x 32 x 256: 38.1 / 39.8; causal level).
-    int variant = p.variant;
-    if (variant == 0) {
-        const bool two_by_two = fp.n_qtiles == 2 && p.Skv > fa::kTile && p.Skv <= 2 * fa::kTile;
-        variant = (!p.causal && two_by_two && 2ll * p.B * p.Hq >= 3ll * sms) ? 4 : 3;
-    }
     switch (variant) {
         case 4:  // pipelined kernel, two query tiles per CTA
             return bf16 ? fa::launch_pipelined<__nv_bfloat16>(tq, tk, tv, fp, st, &t_last_cuda_error)
@@ -360,8 +389,8 @@ int forward_impl(const fa_params& in, cudaStream_t st) {
                         : launch_simple<__half, false>(tq, tk, tv, fp, st);
         case 3: {  // ping-pong kernel: one query tile per CTA, two softmax warpgroups alternate over kv steps
             CUtensorMap to = tq;
-            if (!fp.o_fp32) {  // the output leaves through TMA stores of 32 rows x 64 columns
-                rc = encode_map(&to, p.o, p.B, p.Sq, p.Hq, p.o_stride[0], p.o_stride[1], p.o_stride[2], 32, bf16);
+            if (!fp.o_fp32) {  // the output leaves through TMA stores of 32 rows
+                rc = encode_map_tile(&to, p.o, p.B, p.Sq, p.Hq, p.o_stride[0], p.o_stride[1], p.o_stride[2], 32, bf16);
                 if (rc) return rc;
             }
             return bf16 ? fa::launch_pingpong<__nv_bfloat16>(tq, tk, tv, to, fp, st, &t_last_cuda_error)
@@ -587,7 +616,7 @@ int fa_forward_fp8(const void* q, const void* k, const void* v, void* o, float* 
     if (rc) return rc;
     rc = encode_map_u8(&tv, v, B, Skv, Hkv, 128);
     if (rc) return rc;
-    rc = encode_map(&to, o, B, Sq, Hq, (int64_t)Sq * Hq * 128, (int64_t)Hq * 128, 128, 32, bf16);
+    rc = encode_map_tile(&to, o, B, Sq, Hq, (int64_t)Sq * Hq * 128, (int64_t)Hq * 128, 128, 32, bf16);
     if (rc) return rc;
     return bf16 ? fa::launch_pingpong<__nv_bfloat16, true>(tq, tk, tv, to, fp, st, &t_last_cuda_error)
                 : fa::launch_pingpong<__half, true>(tq, tk, tv, to, fp, st, &t_last_cuda_error);
@@ -662,13 +691,13 @@ int fa_forward_proj(const void* q, const void* k, const void* v, const void* w_o
     e = cudaMemsetAsync(workspace, 0, fa_forward_proj_workspace_bytes(B, Sq), st);
     if (e != cudaSuccess) return cuda_fail(e);
     pp.done = static_cast<unsigned int*>(workspace);
-    rc = encode_map(&tq, q, B, Sq, Hq, ap.q_stride[0], ap.q_stride[1], ap.q_stride[2], 128, bf16);
+    rc = encode_map_tile(&tq, q, B, Sq, Hq, ap.q_stride[0], ap.q_stride[1], ap.q_stride[2], 128, bf16);
     if (rc) return rc;
-    rc = encode_map(&tk, k, B, Skv, Hkv, ap.k_stride[0], ap.k_stride[1], ap.k_stride[2], 128, bf16);
+    rc = encode_map_tile(&tk, k, B, Skv, Hkv, ap.k_stride[0], ap.k_stride[1], ap.k_stride[2], 128, bf16);
     if (rc) return rc;
-    rc = encode_map(&tv, v, B, Skv, Hkv, ap.v_stride[0], ap.v_stride[1], ap.v_stride[2], 128, bf16);
+    rc = encode_map_tile(&tv, v, B, Skv, Hkv, ap.v_stride[0], ap.v_stride[1], ap.v_stride[2], 128, bf16);
     if (rc) return rc;
-    rc = encode_map(&to, o, B, Sq, Hq, ap.o_stride[0], ap.o_stride[1], ap.o_stride[2], 32, bf16);
+    rc = encode_map_tile(&to, o, B, Sq, Hq, ap.o_stride[0], ap.o_stride[1], ap.o_stride[2], 32, bf16);
     if (rc) return rc;
     const fa::FwdParams fp = dense_fwd_params(ap);
     return bf16 ? fa::launch_proj<__nv_bfloat16>(tq, tk, tv, to, ta, tw, fp, pp, 1, st, &t_last_cuda_error)
@@ -750,15 +779,15 @@ static int varlen_impl(const void* q, const void* k, const void* v, void* o, flo
     }
     // the packed tensors as one batch entry; a sequence's rows are reached through the prefix sums
     CUtensorMap tq, tk, tv, to;
-    rc = encode_map(&tq, q, 1, total_q, Hq, (int64_t)total_q * Hq * d, (int64_t)Hq * d, d, 128, bf16, d);
+    rc = encode_map_tile(&tq, q, 1, total_q, Hq, (int64_t)total_q * Hq * d, (int64_t)Hq * d, d, 128, bf16, d);
     if (rc) return rc;
     // K and V: one batch entry with every sequence back to back, or one entry per page
     const int slabs = block_table ? num_pages : 1, slab_rows = block_table ? page_size : total_k;
-    rc = encode_map(&tk, k, slabs, slab_rows, Hkv, (int64_t)slab_rows * Hkv * d, (int64_t)Hkv * d, d, 128, bf16, d);
+    rc = encode_map_tile(&tk, k, slabs, slab_rows, Hkv, (int64_t)slab_rows * Hkv * d, (int64_t)Hkv * d, d, 128, bf16, d);
     if (rc) return rc;
-    rc = encode_map(&tv, v, slabs, slab_rows, Hkv, (int64_t)slab_rows * Hkv * d, (int64_t)Hkv * d, d, 128, bf16, d);
+    rc = encode_map_tile(&tv, v, slabs, slab_rows, Hkv, (int64_t)slab_rows * Hkv * d, (int64_t)Hkv * d, d, 128, bf16, d);
     if (rc) return rc;
-    rc = encode_map(&to, o, 1, total_q, Hq, (int64_t)total_q * Hq * d, (int64_t)Hq * d, d, 32, bf16, d);
+    rc = encode_map_tile(&to, o, 1, total_q, Hq, (int64_t)total_q * Hq * d, (int64_t)Hq * d, d, 32, bf16, d);
     if (rc) return rc;
     if (d == 64)
         return bf16 ? fa::launch_pingpong<__nv_bfloat16, false, 64>(tq, tk, tv, to, fp, st, &t_last_cuda_error)

@@ -533,12 +533,13 @@ __device__ __forceinline__ void pp_paged_tile(const FwdParams& p, int page, int 
 
 // The thread that picks the work items (see PpSource) and loads Q of every item and K of every step.  (Packed batches: the tensor maps
 // have one batch entry that holds every sequence back to back.)
-// One tile: two 64-element boxes of a 16-bit tensor of d = 128, or one 128-byte box (8-bit, or d = 64).
+// One tile is one box: of d = 128 and 16 bits, both 64-element blocks of the rows (see encode_map_tile), otherwise
+// rows of 128 bytes.  (Two boxes of 64 columns cost the loading thread and the TMA unit twice: 8 x 32 x 512 40.6 -> 40.1 us, 32 packed prompts of 256 to 8192 tokens 4262 -> 4164, long sequences level.)
 template <bool kOneBox>
 __device__ __forceinline__ void pp_load_tile(uint32_t dst, const CUtensorMap* tm, uint32_t bar, int h, int s0, int b,
                                              uint64_t policy) {
     if (kOneBox) tma_load_4d_hint(dst, tm, bar, 0, h, s0, b, policy);
-    else load_tile_hint(dst, tm, bar, h, s0, b, policy);
+    else tma_load_5d_hint(dst, tm, bar, 0, s0, 0, h, b, policy);
 }
 
 template <bool kVarlen, bool kF8, int D>
@@ -1034,11 +1035,13 @@ __device__ __forceinline__ bool pp_attention(const CUtensorMap& tm_q, const CUte
                     asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(sK + kPpPartStats + (uint32_t)r * 8u), "f"(m_loc), "f"(l_run) : "memory");
                 } else if (kTmaOut) {
                     const uint32_t q_buf = sQ + (uint32_t)(ord & 1) * kTileBytes;
-                    const uint32_t row_base = q_buf + (uint32_t)r * 128u;
+                    // a warp's rows: its 64-column blocks one after the other, as its store takes them
+                    const uint32_t slab = q_buf + (uint32_t)(warp & 3) * (D == 128 ? 8192u : 4096u);
+                    const uint32_t row_base = slab + (uint32_t)lane * 128u;
 #pragma unroll
                     for (int c = 0; c < D / 8; ++c) {
                         // 16-byte chunk c & 7 of the row's half c >> 3, at its swizzled place
-                        const uint32_t addr = row_base + (uint32_t)(c >> 3) * kHalfBytes + (((uint32_t)(c & 7) ^ ((uint32_t)r & 7u)) << 4);
+                        const uint32_t addr = row_base + (uint32_t)(c >> 3) * 4096u + (((uint32_t)(c & 7) ^ ((uint32_t)lane & 7u)) << 4);
                         const uint32_t w0 = pack2<T>(__uint_as_float(s[8 * c]) * inv_l, __uint_as_float(s[8 * c + 1]) * inv_l);
                         const uint32_t w1 = pack2<T>(__uint_as_float(s[8 * c + 2]) * inv_l, __uint_as_float(s[8 * c + 3]) * inv_l);
                         const uint32_t w2 = pack2<T>(__uint_as_float(s[8 * c + 4]) * inv_l, __uint_as_float(s[8 * c + 5]) * inv_l);
@@ -1052,9 +1055,8 @@ __device__ __forceinline__ bool pp_attention(const CUtensorMap& tm_q, const CUte
                     // sequence, so only a warp whose 32 rows all exist may use the box store
                     const bool box = kVarlen ? (row0 + 32 <= Sq_i) : (row0 < Sq_i);
                     if (lane == 0 && box) {
-                        const uint32_t src = q_buf + (uint32_t)(warp & 3) * 4096u;
-                        tma_store_4d(&tm_o, src, 0, it.h, kVarlen ? it.q_base + row0 : row0, kVarlen ? 0 : it.b);
-                        if (D == 128) tma_store_4d(&tm_o, src + kHalfBytes, 64, it.h, kVarlen ? it.q_base + row0 : row0, kVarlen ? 0 : it.b);
+                        if (D == 128) tma_store_5d(&tm_o, slab, 0, kVarlen ? it.q_base + row0 : row0, 0, it.h, kVarlen ? 0 : it.b);
+                        else tma_store_4d(&tm_o, slab, 0, it.h, kVarlen ? it.q_base + row0 : row0, kVarlen ? 0 : it.b);
                         tma_store_commit();
                     }
                     q_back = ord & 1;  // handed back to the loader after this warp's next step
