@@ -783,64 +783,80 @@ __device__ __forceinline__ void pp_split_merge(const FwdParams& p, uint32_t part
     p.by_hq.divmod(bh, b, h);
     const int q0 = qt * kTile;
     const int n = kv_tiles_for(q0, kTile, p.Sq, p.Skv, p.causal);
-    // Weights first, one thread per row and part: exp2 of the part's max over the largest, divided by the
+    // Rows `rank + split * k`, k < mine, are this CTA's.  Weights first, one thread per row and part, all at once (a
+    // group of 2, 4, 8 or 16 lanes has a row): exp2 of the part's max over the largest, divided by the
     // row's sum; -1 for a part without kv tiles, which holds nothing, and one whose keys the row does
     // not see.  A sum that is NaN (a NaN or infinite score) makes every weight of the row NaN.  They go
     // where this CTA's own pairs are not.
-    const uint32_t w_at = part + kPpPartStats + 2048u;   // [row][kMaxCluster]
-    const int rows = min(kTile, p.Sq - q0);
-    for (int k = tid / kMaxCluster; ; k += 256 / kMaxCluster) {
-        const int row = rank + split * k, i = tid % kMaxCluster;
-        if (rank + split * (k - (tid & 31) / kMaxCluster) >= rows) break;   // uniform for the warp
+    const uint32_t w_at = part + kPpPartStats + 2048u;   // [k][kMaxCluster]
+    const int rows = min(kTile, p.Sq - q0), mine = rank < rows ? (rows - rank + split - 1) / split : 0;
+    const int width_log2 = 32 - __clz(split - 1);
+    {
+        const int k = tid >> width_log2, i = tid & ((1 << width_log2) - 1);
+        const int row = rank + split * k;
         float m = -INFINITY, l = 0.f;
-        if (row < rows && i < split && pp_split_first(n, split, i + 1) > pp_split_first(n, split, i))
+        if (k < mine && i < split && pp_split_first(n, split, i + 1) > pp_split_first(n, split, i))
             cluster_ld2(cluster_map(part + kPpPartStats + (uint32_t)row * 8u, i), m, l);
         const bool nothing = l == 0.f;
         float M = nothing ? -INFINITY : m;
-#pragma unroll
-        for (int sh = kMaxCluster / 2; sh > 0; sh >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, sh));
+        for (int sh = 1 << width_log2 >> 1; sh > 0; sh >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, sh));
         const float w = nothing ? 0.f : fast_exp2((m - M) * p.scale_log2);
         float sum = w * l;
-#pragma unroll
-        for (int sh = kMaxCluster / 2; sh > 0; sh >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, sh);
-        if (row < rows) {
-            asm volatile("st.shared.f32 [%0], %1;" ::"r"(w_at + (uint32_t)(row * kMaxCluster + i) * 4u), "f"(nothing ? -1.f : w / sum) : "memory");
+        for (int sh = 1 << width_log2 >> 1; sh > 0; sh >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, sh);
+        if (k < mine) {
+            asm volatile("st.shared.f32 [%0], %1;" ::"r"(w_at + (uint32_t)(k * kMaxCluster + i) * 4u), "f"(nothing ? -1.f : w / sum) : "memory");
             if (i == 0 && p.lse != nullptr)
                 p.lse[((long long)b * p.Hq + h) * p.Sq + q0 + row] = sum > 0.f ? (M * p.scale_log2 + log2f(sum)) * 0.6931471805599453f : -INFINITY;
         }
     }
     asm volatile("bar.sync 1, 256;" ::: "memory");
-    // Then the rows, one warp and four columns per lane, four rows at a time: the loads' latency is what this takes
-    for (int k0 = warp; rank + split * k0 < rows; k0 += 32) {
-        float acc[4][4];
+    // Then the rows, one warp and four columns per lane, up to four rows at a time: the loads' latency is what this takes.
+    // A CTA begins with the part of the CTA after it and ends with its own: from the same part on, all
+    // would read one CTA's shared memory at a time.
+    auto merge_rows = [&](auto rows_at_a_time) {
+        constexpr int kRows = decltype(rows_at_a_time)::value;
+        for (int k0 = warp; k0 < mine; k0 += 8 * kRows) {
+            float acc[kRows][4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) acc[k][0] = acc[k][1] = acc[k][2] = acc[k][3] = 0.f;
-#pragma unroll 2
-        for (int i = 0; i < split; ++i) {
-            float v[4][4], w[4];
+            for (int q = 0; q < kRows; ++q) acc[q][0] = acc[q][1] = acc[q][2] = acc[q][3] = 0.f;
+            int i = rank;
+            auto add_part = [&](auto own) {
+                i = i + 1 == split ? 0 : i + 1;
+                const uint32_t from = decltype(own)::value ? part : cluster_map(part, i);
+                float v[kRows][4], w[kRows];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int row = min(rank + split * (k0 + 8 * k), rows - 1);
-                asm volatile("ld.shared.f32 %0, [%1];" : "=f"(w[k]) : "r"(w_at + (uint32_t)(row * kMaxCluster + i) * 4u));
-                cluster_ld4(cluster_map(part + (uint32_t)row * 512u + (uint32_t)((lane ^ (row & 31)) << 4), i), v[k]);
+                for (int q = 0; q < kRows; ++q) {
+                    const int k = min(k0 + 8 * q, mine - 1), row = rank + split * k;
+                    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(w[q]) : "r"(w_at + (uint32_t)(k * kMaxCluster + i) * 4u));
+                    const uint32_t at = from + (uint32_t)row * 512u + (uint32_t)((lane ^ (row & 31)) << 4);
+                    if (decltype(own)::value)
+                        asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v[q][0]), "=f"(v[q][1]), "=f"(v[q][2]), "=f"(v[q][3]) : "r"(at));
+                    else cluster_ld4(at, v[q]);
+                }
+#pragma unroll
+                for (int q = 0; q < kRows; ++q)
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) acc[q][c] = w[q] < 0.f ? acc[q][c] : fmaf(w[q], v[q][c], acc[q][c]);
+            };
+#pragma unroll(kRows == 4 ? 1 : 4)
+            for (int t = 0; t < split - 1; ++t) add_part(std::false_type());
+            add_part(std::true_type());
+#pragma unroll
+            for (int q = 0; q < kRows; ++q) {
+                const int k = k0 + 8 * q;
+                if (k < mine) {
+                    const long long at_o = (long long)b * p.o_sb + (long long)(q0 + rank + split * k) * p.o_ss + (long long)h * p.o_sh + 4 * lane;
+                    if (p.o_fp32)
+                        *reinterpret_cast<float4*>(static_cast<float*>(p.o) + at_o) = make_float4(acc[q][0], acc[q][1], acc[q][2], acc[q][3]);
+                    else
+                        *reinterpret_cast<uint2*>(static_cast<T*>(p.o) + at_o) = make_uint2(pack2<T>(acc[q][0], acc[q][1]), pack2<T>(acc[q][2], acc[q][3]));
+                }
             }
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-#pragma unroll
-                for (int c = 0; c < 4; ++c) acc[k][c] = w[k] < 0.f ? acc[k][c] : fmaf(w[k], v[k][c], acc[k][c]);
         }
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const int row = rank + split * (k0 + 8 * k);
-            if (row < rows) {
-                const long long at_o = (long long)b * p.o_sb + (long long)(q0 + row) * p.o_ss + (long long)h * p.o_sh + 4 * lane;
-                if (p.o_fp32)
-                    *reinterpret_cast<float4*>(static_cast<float*>(p.o) + at_o) = make_float4(acc[k][0], acc[k][1], acc[k][2], acc[k][3]);
-                else
-                    *reinterpret_cast<uint2*>(static_cast<T*>(p.o) + at_o) = make_uint2(pack2<T>(acc[k][0], acc[k][1]), pack2<T>(acc[k][2], acc[k][3]));
-            }
-        }
-    }
+    };
+    if (mine <= 8) merge_rows(std::integral_constant<int, 1>());
+    else if (mine <= 16) merge_rows(std::integral_constant<int, 2>());
+    else merge_rows(std::integral_constant<int, 4>());
 }
 
 // kTmaOut: the output has the operands' 16-bit type; an item's O goes, scaled and rounded, into
