@@ -20,7 +20,8 @@
 // memory: the warpgroup of step g takes the reference max left by step g-1, decides whether its
 // own row max moves it (only when it outgrew it by more than 2^8, see kRescaleThreshold),
 // publishes the result for step g+1 right away, and, in the rare case that it moved, rescales O
-// once O += P V of step g-1 has completed.  Each warpgroup keeps the row sum of its own steps;
+// once O += P V of step g-1 has completed.  (Waiting for that hand-over costs nothing by itself: a form that
+// took the reference to be the one its own last step left, and looked only at the step's end, was 6 % slower.)  Each warpgroup keeps the row sum of its own steps;
 // the one that runs an item's last step adds the other's and writes O and LSE.
 // Synchronisation is by mbarriers, and every wait on one is bounded (see mbar_wait).  The form whose
 // CTAs share a query tile merges behind cluster barriers and a named barrier, which are not: every
@@ -534,7 +535,8 @@ __device__ __forceinline__ void pp_paged_tile(const FwdParams& p, int page, int 
 // The thread that picks the work items (see PpSource) and loads Q of every item and K of every step.  (Packed batches: the tensor maps
 // have one batch entry that holds every sequence back to back.)
 // One tile is one box: of d = 128 and 16 bits, both 64-element blocks of the rows (see encode_map_tile), otherwise
-// rows of 128 bytes.  (Two boxes of 64 columns cost the loading thread and the TMA unit twice: 8 x 32 x 512 40.6 -> 40.1 us, 32 packed prompts of 256 to 8192 tokens 4262 -> 4164, long sequences level.)
+// rows of 128 bytes.  (Two boxes of 64 columns cost the loading thread and the TMA unit twice: 8 x 32 x 512 40.6 -> 40.1
+// us, 32 packed prompts of 256 to 8192 tokens 4262 -> 4164, long sequences level.)
 template <bool kOneBox>
 __device__ __forceinline__ void pp_load_tile(uint32_t dst, const CUtensorMap* tm, uint32_t bar, int h, int s0, int b,
                                              uint64_t policy) {
@@ -861,8 +863,8 @@ __device__ __forceinline__ void pp_split_merge(const FwdParams& p, uint32_t part
 
 // kTmaOut: the output has the operands' 16-bit type; an item's O goes, scaled and rounded, into
 // the item's Q buffer (which Q K^T has finished with by then) in the swizzled layout of a tile,
-// and each warp sends its 32 rows to global memory with two TMA stores (tm_o: boxes of 32 rows x
-// 64 columns).  Rows past the end of the queries are clipped by the tensor map.  Otherwise
+// and each warp sends its 32 rows to global memory with one TMA store (tm_o: boxes of 32
+// rows).  Rows past the end of the queries are clipped by the tensor map.  Otherwise
 // (fp32 output) every thread stores its own row.
 // kVarlen (needs kTmaOut): a packed batch of sequences of different lengths (see FwdParams).
 // kF8: q, k, v hold FP8 e4m3 bytes (see PpOperands); T is then the type of the output only.
@@ -1069,11 +1071,21 @@ __device__ __forceinline__ bool pp_attention(const CUtensorMap& tm_q, const CUte
                     for (int c = 0; c < D / 8; ++c) {
                         // 16-byte chunk c & 7 of the row's half c >> 3, at its swizzled place
                         const uint32_t addr = row_base + (uint32_t)(c >> 3) * 4096u + (((uint32_t)(c & 7) ^ ((uint32_t)lane & 7u)) << 4);
-                        const uint32_t w0 = pack2<T>(__uint_as_float(s[8 * c]) * inv_l, __uint_as_float(s[8 * c + 1]) * inv_l);
-                        const uint32_t w1 = pack2<T>(__uint_as_float(s[8 * c + 2]) * inv_l, __uint_as_float(s[8 * c + 3]) * inv_l);
-                        const uint32_t w2 = pack2<T>(__uint_as_float(s[8 * c + 4]) * inv_l, __uint_as_float(s[8 * c + 5]) * inv_l);
-                        const uint32_t w3 = pack2<T>(__uint_as_float(s[8 * c + 6]) * inv_l, __uint_as_float(s[8 * c + 7]) * inv_l);
-                        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(w0), "r"(w1), "r"(w2), "r"(w3) : "memory");
+                        // (packed multiplications: 8 x 32 x 512 42.6 -> 42.0 us, 16 x 32 x 256 34.6 -> 34.3, others level; but
+                        // the packed batches' instantiation came out 1 to 2 % slower with them)
+                        uint32_t wd[4];
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            float x0 = __uint_as_float(s[8 * c + 2 * q]), x1 = __uint_as_float(s[8 * c + 2 * q + 1]);
+                            if (kVarlen) {
+                                x0 *= inv_l;
+                                x1 *= inv_l;
+                            } else {
+                                f2_unpack(f2_mul(f2_pack(x0, x1), f2_pack(inv_l, inv_l)), x0, x1);
+                            }
+                            wd[q] = pack2<T>(x0, x1);
+                        }
+                        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(wd[0]), "r"(wd[1]), "r"(wd[2]), "r"(wd[3]) : "memory");
                     }
                     fence_proxy_async_smem();
                     __syncwarp();
@@ -1086,7 +1098,7 @@ __device__ __forceinline__ bool pp_attention(const CUtensorMap& tm_q, const CUte
                         else tma_store_4d(&tm_o, slab, 0, it.h, kVarlen ? it.q_base + row0 : row0, kVarlen ? 0 : it.b);
                         tma_store_commit();
                     }
-                    q_back = ord & 1;  // handed back to the loader after this warp's next step
+                    q_back = ord & 1;  // handed back to the loader at the start of the next item
                     if (kProj) done_slot = it.b * p.n_qtiles + it.q0 / kTile;
                     __syncwarp();
                     if (kVarlen && !box && row < Sq_i) {
@@ -1236,7 +1248,7 @@ inline FwdParams pp_plan_items(const FwdParams& fp, int grid, double bytes_per_k
     return fpc;
 }
 
-// to: map over the output with boxes of 32 rows x 64 columns; read only when the output has the
+// to: map over the output with boxes of 32 rows (see encode_map_tile); read only when the output has the
 // operands' type (any valid map otherwise).
 // kF8: tq, tk, tv are maps over FP8 e4m3 bytes (boxes of 128 rows x 128 bytes) and T is the output type.
 // D: the head dimension, 128, or 64 with 16-bit operands (maps with boxes of 64 elements either way).

@@ -114,3 +114,24 @@ def test_other_forms_beside_a_kernel_that_holds_sms(fa, sms):  # noqa: F811
         sl = torch.tensor([smax - 77 * b for b in range(B)], dtype=torch.int32, device=DEV)
         ws = torch.empty(fa.fa_decode_workspace_bytes(B, 2 * Hkv, Hkv, smax, 128) + 16, dtype=torch.uint8, device=DEV)
         beside_neighbour(fa, lambda: fa.fa_decode(q, k, v, o, lse, sl, 0.1, ws), [o, lse], sms, overlaps=False)
+
+
+@pytest.mark.parametrize("B,H,S,d,causal", [(1, 2, 512, 128, True), (1, 1, 1, 128, False), (1, 4, 2048, 128, True), (1, 3, 3000, 128, False),
+                                            (3, 5, 700, 128, True), (8, 32, 512, 128, True), (4, 16, 600, 64, True)])
+def test_calls_that_read_what_the_call_before_wrote(fa, B, H, S, d, causal):
+    # every call starts while the one before it may still run, and decodes its first item then; each
+    # reads as its values what the last one wrote, into a buffer that the one before that reads.  Grids that leave SMs
+    # free, shared query tiles and full grids, against the same calls one by one.
+    q, k = (_rand((B, S, H, d), torch.float16, i) for i in (1, 2))
+    v0 = _rand((B, S, H, d), torch.float16, 3)
+    ends = []
+    for alone in (True, False):
+        bufs = [v0.clone(), torch.full_like(v0, float("nan"))]
+        for i in range(12):
+            fa.fa_forward(q, k, bufs[i & 1], bufs[1 - (i & 1)], None, causal, 0.1)
+            if alone:
+                torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        ends.append(bufs)
+    check_status(fa)
+    assert all(torch.equal(a, b) for a, b in zip(*ends)) and torch.isfinite(ends[0][0]).all()
