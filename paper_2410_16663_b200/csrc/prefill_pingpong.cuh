@@ -23,7 +23,9 @@
 // once O += P V of step g-1 has completed.  (Waiting for that hand-over costs nothing by itself: a form that
 // took the reference to be the one its own last step left, and looked only at the step's end, was 6 % slower.)  Each warpgroup keeps the row sum of its own steps;
 // the one that runs an item's last step adds the other's and writes O and LSE.
-// Synchronisation is by mbarriers, and every wait on one is bounded (see mbar_wait).  The form whose
+// Synchronisation is by mbarriers, and every wait on one is bounded (see mbar_wait); what the bound covers is this
+// kernel alone, as every role waits for the end of the kernel before it, without a bound, ahead of its first
+// wait for anything that follows from that (see PpTaker).  The form whose
 // CTAs share a query tile merges behind cluster barriers and a named barrier, which are not: every
 // thread reaches them, those of a CTA without work and of one that gave up a wait too, because a role
 // that stops only leaves its loop.
@@ -340,6 +342,14 @@ __device__ __forceinline__ uint32_t pp_bar(uint32_t bar0, int i) { return bar0 +
 
 // The other roles' end of the ring: the ord-th item, read by a single thread, which hands the slot
 // back at once.  False at the end of the list or after a wait that gave up.
+// The kernel before this one in the stream may still run when the first item is taken.  A dense call's is decoded
+// from the parameters alone, so the role first runs up to here, on cold instruction lines, and then waits for that
+// kernel; a packed batch's needs global memory.  The wait belongs to every role, not only to the loading
+// ones: what follows the item follows from the loads, and a bounded wait for that would count the time that
+// kernel takes, which has no bound (a collective of another library that releases its dependents and
+// waits for a peer).  (It costs next to nothing: with the loaders waiting alone 1 x 2 x 512 took 7.2 us, like this
+// 7.1; few query tiles over many keys 14.6 / 14.7; 8 x 32 x 512 41.8 / 42.0.)
+template <bool kVarlen>
 struct PpTaker {
     const PpItem* items;
     uint32_t bar0;
@@ -348,9 +358,11 @@ struct PpTaker {
     __device__ __forceinline__ bool next(PpItem& it, unsigned int where) {
         ++ord;
         const int slot = ord & (kPpSlots - 1);
+        if (kVarlen && ord == 0) grid_dep_wait();
         if (!mbar_wait(pp_bar(bar0, ppb::item_full + slot), (ord / kPpSlots) & 1, abort_flag, where)) return false;
         it = items[slot];
         mbar_arrive(pp_bar(bar0, ppb::item_empty + slot));
+        if (!kVarlen && ord == 0) grid_dep_wait();
         return it.n > 0;
     }
 };
@@ -428,7 +440,7 @@ struct PpRing {
 };
 
 // The thread that issues S = Q K^T of every step.
-template <typename T, bool kTmaOut, bool kF8, int D>
+template <typename T, bool kTmaOut, bool kVarlen, bool kF8, int D>
 __device__ __forceinline__ void pp_run_s(uint32_t bar0, uint32_t sQ, uint32_t sK, uint32_t tmem, const PpItem* slots,
                                          volatile uint32_t* abort_flag) {
     constexpr bool kBf16 = std::is_same<T, __nv_bfloat16>::value;
@@ -436,7 +448,7 @@ __device__ __forceinline__ void pp_run_s(uint32_t bar0, uint32_t sQ, uint32_t sK
     using Op = PpOperands<kF8, D>;
     uint32_t g = 0;
     PpRing<kPpNK> ring;
-    PpTaker items{slots, bar0, abort_flag};
+    PpTaker<kVarlen> items{slots, bar0, abort_flag};
     PpItem it;
     while (items.next(it, 133)) {
         const int ord = items.ord;
@@ -468,7 +480,7 @@ __device__ __forceinline__ void pp_run_s(uint32_t bar0, uint32_t sQ, uint32_t sK
 }
 
 // The thread that issues O += P V of every step.
-template <typename T, bool kF8, int D>
+template <typename T, bool kVarlen, bool kF8, int D>
 __device__ __forceinline__ void pp_run_pv(uint32_t bar0, uint32_t sV, uint32_t tmem, const PpItem* slots,
                                           volatile uint32_t* abort_flag) {
     constexpr bool kBf16 = std::is_same<T, __nv_bfloat16>::value;
@@ -476,7 +488,7 @@ __device__ __forceinline__ void pp_run_pv(uint32_t bar0, uint32_t sV, uint32_t t
     using Op = PpOperands<kF8, D>;
     uint32_t g = 0;
     PpRing<kPpNV> ring;
-    PpTaker items{slots, bar0, abort_flag};
+    PpTaker<kVarlen> items{slots, bar0, abort_flag};
     PpItem it;
     while (items.next(it, 143)) {
         const int ord = items.ord;
@@ -555,10 +567,10 @@ __device__ __forceinline__ void pp_run_load_qk(uint32_t bar0, uint32_t sQ, uint3
     PpSource<kVarlen> source{p, total_items, pp_bar(bar0, ppb::claim), smem_u32(&ss.claim_answer), abort_flag,
                              {p.deal_ctas, p.deal_rounds}};
     source.walk.take(blockIdx.x);
-    // The kernel before this one has ended: from here on global memory may be read, and what is written later is behind
-    // what the loads bring.  A dense call's first item needs no global memory: it is decoded, and the other
-    // roles get to their first waits, while that kernel may still run.  (1 x 2 x 512 8.1 -> 7.0 us, calls on
-    // few query tiles 17.2 -> 15.8, 14.8 -> 13.6; calls that fill the device level.)
+    // The kernel before this one has ended: from here on global memory may be read.  A dense call's first item
+    // needs none: it is decoded, and the other roles take it, while that kernel may still run (see PpTaker).
+    // (1 x 2 x 512 8.1 -> 7.0 us, calls on few query tiles 17.2 -> 15.8, 14.8 -> 13.6; calls that fill the device
+    // level.)
     auto after_last_kernel = [&]() {
         grid_dep_wait();
         if (p.early_next) grid_dep_launch();
@@ -571,7 +583,10 @@ __device__ __forceinline__ void pp_run_load_qk(uint32_t bar0, uint32_t sQ, uint3
         if (!mbar_wait(pp_bar(bar0, ppb::item_empty + slot), ((ord / kPpSlots) & 1) ^ 1, abort_flag, 154)) return;
         ss.items[slot] = it;
         mbar_arrive(pp_bar(bar0, ppb::item_full + slot));
-        if (!kVarlen && ord == 0) after_last_kernel();
+        if (!kVarlen && ord == 0) {
+            after_last_kernel();
+            if (*abort_flag) return;   // (a role did not get the item in time: nothing is loaded)
+        }
         if (it.n == 0) return;
         const uint32_t qb = ord & 1;
         // passes at once the first time each buffer is used
@@ -600,12 +615,10 @@ __device__ __forceinline__ void pp_run_load_v(uint32_t bar0, uint32_t sV, const 
     tma_prefetch_desc(tm_v);
     const uint64_t pol_kv = l2_policy_evict_last();
     PpRing<kPpNV> ring;
-    PpTaker items{slots, bar0, abort_flag};
+    PpTaker<kVarlen> items{slots, bar0, abort_flag};
     PpItem it;
-    bool waited = false;
     while (items.next(it, 155)) {
-        if (!waited) grid_dep_wait();
-        waited = true;
+        if (items.ord == 0 && *abort_flag) return;
         int page = (kVarlen && p.block_table != nullptr) ? it.page0 : 0;
         for (int j = 0; j < it.n; ++j, ring.next()) {
             const int page_next = pp_page_of<kVarlen>(p, it.b, j + 1, it.n, it.Skv);
@@ -961,11 +974,13 @@ __device__ __forceinline__ bool pp_attention(const CUtensorMap& tm_q, const CUte
         };
         for (int ord = 0; ok; ++ord) {
             const int slot = ord & (kPpSlots - 1);
+            if (kVarlen && ord == 0) grid_dep_wait();   // (see PpTaker)
             if (!pp_warp_wait(pp_bar(bar0, ppb::item_full + slot), (ord / kPpSlots) & 1, abort_flag, 122 + w)) break;
             // the epilogue reads the rest of the slot; it is handed back at the end of the item
             const PpItem& it = ss.items[slot];
             const int n = it.n, q0 = it.q0;
             if (n == 0) break;
+            if (!kVarlen && ord == 0) grid_dep_wait();
             const int row = q0 + r;   // within the sequence
             const int Sq_i = kVarlen ? it.Sq : p.Sq, Skv_i = kVarlen ? it.Skv : p.Skv;
             const int off_i = kVarlen ? it.Skv - it.Sq : off;
@@ -1143,8 +1158,8 @@ __device__ __forceinline__ bool pp_attention(const CUtensorMap& tm_q, const CUte
     } else {
         setmaxnreg_dec<kPipeOtherRegs>();
         if (lane == 0) {
-            if (warp == 8) pp_run_s<T, kTmaOut, kF8, D>(bar0, sQ, sK, tmem_base, ss.items, abort_flag);
-            else if (warp == 10) pp_run_pv<T, kF8, D>(bar0, sV, tmem_base, ss.items, abort_flag);
+            if (warp == 8) pp_run_s<T, kTmaOut, kVarlen, kF8, D>(bar0, sQ, sK, tmem_base, ss.items, abort_flag);
+            else if (warp == 10) pp_run_pv<T, kVarlen, kF8, D>(bar0, sV, tmem_base, ss.items, abort_flag);
             else if (warp == 9) pp_run_load_qk<kVarlen, kF8, D>(bar0, sQ, sK, &tm_q, &tm_k, p, total_items, ss, abort_flag);
             else pp_run_load_v<kVarlen, kF8, D>(bar0, sV, &tm_v, p, ss.items, abort_flag);
         }

@@ -121,8 +121,8 @@ __global__ void fa_selftest_wait_kernel(unsigned long long limit_ns, unsigned in
 // The attention kernels are launched as programmatic dependents of whatever precedes them in the
 // stream (launch_dependent in prefill_simple.cuh; not the simple kernels and not the fused projection):
 // the CTAs may start, and set up their barriers and tensor memory, while the kernel before still runs.  grid_dep_wait() blocks until that kernel
-// has completed and its writes are visible; nothing may read or write global memory before it (or before
-// something that follows it in another thread: in the ping-pong kernel only the loading threads wait), and
+// has completed and its writes are visible; nothing may read or write global memory before it, no
+// thread may enter a bounded wait before it for something that another thread does after it, and
 // nothing at all is read through the non-coherent path (__ldg, ld.global.nc), which wants data that
 // nobody writes while the kernel lives: its life begins while the kernel before it still writes.
 // grid_dep_launch() lets the next kernel of the stream start in the same way as soon as every CTA of

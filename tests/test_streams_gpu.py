@@ -3,6 +3,12 @@
 The persistent prefill kernel hands part of its work to whichever CTA is free, decode and small
 prefills run as clusters, and every kernel starts while the one before it in its stream still runs;
 all of this goes another way when a kernel of another stream keeps some of the SMs."""
+import ctypes
+import os
+import shutil
+import subprocess
+import time
+
 import pytest
 import torch
 
@@ -135,3 +141,71 @@ def test_calls_that_read_what_the_call_before_wrote(fa, B, H, S, d, causal):
         ends.append(bufs)
     check_status(fa)
     assert all(torch.equal(a, b) for a, b in zip(*ends)) and torch.isfinite(ends[0][0]).all()
+
+
+@pytest.fixture(scope="module")
+def early_release(tmp_path_factory):
+    """early_release(ns, src, dst): see gpu_helpers/early_release.cu; on the current stream."""
+    nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
+    nvcc = nvcc if os.path.exists(nvcc) else shutil.which("nvcc")
+    if nvcc is None:
+        pytest.skip("nvcc not found")
+    out = str(tmp_path_factory.mktemp("early_release") / "early_release.so")
+    src = os.path.join(os.path.dirname(os.path.abspath(__file__)), "gpu_helpers", "early_release.cu")
+    subprocess.run([nvcc, "-std=c++17", "-O2", "-gencode", "arch=compute_100a,code=sm_100a", "-shared", "-Xcompiler", "-fPIC", src,
+                    "-o", out], check=True, timeout=600)
+    fn = ctypes.CDLL(out).early_release
+    fn.argtypes = [ctypes.c_ulonglong, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_size_t, ctypes.c_void_p]
+
+    def call(ns, src, dst):
+        assert fn(ns, src.data_ptr(), dst.data_ptr(), src.numel() * src.element_size(), torch.cuda.current_stream().cuda_stream) == 0
+
+    return call
+
+
+WAIT_LIMIT_S = 4   # of every bounded wait in the kernels
+
+
+def test_a_kernel_before_that_outlasts_every_wait_limit(fa, early_release):  # noqa: F811
+    # The call starts while that kernel runs, which writes the call's values at its end, more than a wait limit later: no
+    # wait of the call may count that time.  The forms of the ping-pong kernel whose grids leave room for one
+    # another, each behind a kernel and on a stream of its own.
+    forms = []   # (values, output and log-sum-exp, call)
+    # (the second: a query tile shared by a cluster's CTAs)
+    for H, Sq, Skv, d, o_dtype in ((2, 512, 512, 128, None), (2, 100, 2048, 128, None), (2, 700, 700, 64, None), (2, 512, 512, 128, torch.float32)):
+        q, k, v, o, lse = _dense(1, H, H, Sq, Skv, d, torch.float16, o_dtype)
+        forms.append((v, [o, lse], lambda q=q, k=k, v=v, o=o, lse=lse: fa.fa_forward_ex(q, k, v, o, lse, True, 0.1)))
+    q, k, v, o, lse = _dense(1, 2, 2, 512, 512, 128, torch.float16)
+    q8, k8, v8 = synth.fp8_operands(q, k, v, 0.125, 0.25, 0.0625)
+    forms.append((v8, [o, lse], lambda q=q8, k=k8, v=v8, o=o, lse=lse: fa.fa_forward_fp8(q, k, v, o, lse, True, 0.1, 0.125, 0.25, 0.0625)))
+    lens = [300, 33, 128]
+    cu = torch.tensor([0] + lens).cumsum(0).to(torch.int32).to(DEV)
+    q, k, v = (_rand((sum(lens), 2, 128), torch.bfloat16, s) for s in (7, 8, 9))
+    o, lse = torch.empty_like(q), torch.empty(2, sum(lens), device=DEV)
+    forms.append((v, [o, lse], lambda q=q, k=k, v=v, o=o, lse=lse: fa.fa_forward_varlen(q, k, v, o, lse, cu, cu, max(lens), max(lens), True, 0.1)))
+    kp, vp, table = (t.to(DEV) for t in synth.paged_from_packed(k.cpu(), v.cpu(), lens, 128, seed=3))
+    sl = torch.tensor(lens, dtype=torch.int32, device=DEV)
+    o, lse = torch.empty_like(q), torch.empty(2, sum(lens), device=DEV)
+    forms.append((vp, [o, lse], lambda q=q, kp=kp, vp=vp, o=o, lse=lse: fa.fa_forward_varlen_paged(q, kp, vp, table, o, lse, cu, sl, max(lens), max(lens), True, 0.1)))
+    for _, _, call in forms:
+        call()
+    torch.cuda.synchronize()
+    check_status(fa)
+    alone = [[t.clone() for t in outs] for _, outs, _ in forms]
+    sources, streams = [v.clone() for v, _, _ in forms], [torch.cuda.Stream() for _ in forms]
+    for v, outs, _ in forms:
+        v.view(torch.uint8).zero_()
+        for t in outs:
+            t.fill_(float("nan"))
+    torch.cuda.synchronize()
+    t0 = time.monotonic()
+    for (v, _, call), src, stream in zip(forms, sources, streams):
+        with torch.cuda.stream(stream):
+            early_release(int((WAIT_LIMIT_S + 1) * 1e9), src, v)
+            call()
+    torch.cuda.synchronize()
+    assert WAIT_LIMIT_S + 0.5 < time.monotonic() - t0 < 4 * WAIT_LIMIT_S
+    check_status(fa)
+    for i, ((_, outs, _), want) in enumerate(zip(forms, alone)):
+        for a, b in zip(want, outs):
+            assert torch.equal(a, b), f"form {i}: {int((a != b).sum())} of {a.numel()} values differ"
