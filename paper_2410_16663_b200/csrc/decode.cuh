@@ -728,6 +728,7 @@ fa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
         }
         }
         asm volatile("bar.sync 1, 128;" ::: "memory");
+        settle_if(!ok);
         if (ok) {
             // a thread owns four output columns, so 512 / D rows go at a time
             const int col = 4 * (tid % (D / 4));

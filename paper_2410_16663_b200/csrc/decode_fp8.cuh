@@ -359,6 +359,7 @@ fa_decode_split_fp8_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
             }
         }
         asm volatile("bar.sync 1, %0;" ::"n"(kDec8Warps * 32) : "memory");
+        settle_if(!ok);
         if (ok) {
             const int col = 4 * (tid & 31);   // a thread owns four output columns, so four rows go at a time
             for (int r = tid >> 5; r < G; r += 4) {

@@ -343,6 +343,7 @@ fa_fwd_d256_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     tc_fence_before();
     __syncthreads();
     if (warp == 0) {
+        settle_if(abort_flag);
         __syncwarp();
         tmem_dealloc(tmem_base, 512);
     }

@@ -438,6 +438,7 @@ fa_fwd_d64_stream_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
     tc_fence_before();
     __syncthreads();
     if (warp == 16) {
+        settle_if(abort_word);
         __syncwarp();
         tmem_dealloc(tmem_base, 512);
     }

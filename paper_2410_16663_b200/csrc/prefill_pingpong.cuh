@@ -1188,6 +1188,7 @@ fa_fwd_pingpong_split_kernel(const __grid_constant__ CUtensorMap tm_q, const __g
     tc_fence_before();
     __syncthreads();
     if ((threadIdx.x >> 5) == 8) {
+        settle_if(ss.abort_flag);
         __syncwarp();
         tmem_dealloc(ss.tmem_holder, 512);
     }
@@ -1210,6 +1211,7 @@ fa_fwd_pingpong_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
     tc_fence_before();
     __syncthreads();
     if ((threadIdx.x >> 5) == 8) {
+        settle_if(ss.abort_flag);
         __syncwarp();
         tmem_dealloc(ss.tmem_holder, 512);
     }

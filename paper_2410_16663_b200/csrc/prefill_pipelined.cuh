@@ -605,6 +605,7 @@ fa_fwd_pipelined_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
     tc_fence_before();
     __syncthreads();
     if (warp == 8) {
+        settle_if(abort_flag);
         __syncwarp();
         tmem_dealloc(tmem_base, 512);
     }

@@ -209,6 +209,7 @@ fa_proj_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     tc_fence_before();
     __syncthreads();
     if (warp == 8) {
+        settle_if(abort_word);
         __syncwarp();
         tmem_dealloc(tmem_base, 512);
     }
@@ -248,6 +249,7 @@ fa_fwd_pingpong_proj_kernel(const __grid_constant__ CUtensorMap tm_q, const __gr
     tc_fence_before();
     __syncthreads();
     if ((threadIdx.x >> 5) == 8) {
+        settle_if(ss.abort_flag);
         __syncwarp();
         tmem_dealloc(ss.tmem_holder, 512);
     }

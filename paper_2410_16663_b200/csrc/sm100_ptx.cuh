@@ -74,7 +74,8 @@ __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
 }
 // Waits until the barrier's phase with the given parity has completed.  Gives up after
 // kWaitLimitNs or as soon as another thread of the CTA has given up (abort flag), records
-// the location, and returns false; the caller then leaves its loop and goes to teardown.
+// the location, and returns false; the caller then leaves its loop and goes to teardown, where
+// one thread sees to what is on its way (settle_if).
 __device__ __forceinline__ bool mbar_wait_for(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag,
                                               unsigned int where, unsigned long long limit_ns) {
     if (mbar_try_wait(bar, parity)) return true;
@@ -97,6 +98,22 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity,
     return mbar_wait_for(bar, parity, abort_flag, where, kWaitLimitNs);
 }
 
+// Where a CTA ends in which a wait may have given up: if one has, the thread stays for a millisecond longer.
+// The CTA's threads have left their roles by then and issue nothing more, and what is on its way into its shared or
+// tensor memory -- TMA loads, claims, matrix instructions, a few microseconds at the most -- arrives: the CTA must not
+// end before, as that memory is another's then.  (That every thread which issues such work counts it and waits
+// for exactly that was tried: 3 to 5 % slower on calls of 8 to 60 us, through the code alone.  Not
+// needed where the thread that issues everything also waits for it, in the simple kernel and the one for short d = 64
+// sequences: it probes 256 times before it leaves, which takes longer.)
+constexpr unsigned long long kSettleNs = 1000000ull;
+__device__ __noinline__ void settle() {
+    const unsigned long long t0 = globaltimer_ns();
+    while (globaltimer_ns() - t0 < kSettleNs) __nanosleep(1000);
+}
+__device__ __forceinline__ void settle_if(bool gave_up) {
+    if (__builtin_expect(gave_up, 0)) settle();
+}
+
 // Self-test of the give-up path above (fa_selftest_wait): one CTA waits, with a short limit, on a
 // barrier that is one arrival short of completing its phase and that nothing will ever complete.
 // The wait must run out, one thread records the location, the others see the abort flag, and
@@ -115,6 +132,7 @@ __global__ void fa_selftest_wait_kernel(unsigned long long limit_ns, unsigned in
     if (threadIdx.x == 0) mbar_arrive(bar);   // the second arrival never comes
     const bool ok = mbar_wait_for(bar, 0, &abort_flag, kSelftestWhere, limit_ns);
     if (!ok) atomicAdd(gave_up, 1u);
+    settle_if(!ok);
 }
 
 // ------------------------------------------------------------------ programmatic dependent launch

@@ -209,3 +209,17 @@ def test_a_kernel_before_that_outlasts_every_wait_limit(fa, early_release):  # n
     for i, ((_, outs, _), want) in enumerate(zip(forms, alone)):
         for a, b in zip(want, outs):
             assert torch.equal(a, b), f"form {i}: {int((a != b).sum())} of {a.numel()} values differ"
+
+
+def test_a_thread_that_gives_up_a_wait_lets_what_is_on_its_way_arrive(fa):  # noqa: F811
+    # copies that the CTA's threads have issued may be on their way into its shared memory; the thread
+    # whose time is up (0.05 ms here) stays for another millisecond before it and the CTA can leave
+    gave_up = torch.zeros(1, dtype=torch.int32, device=DEV)
+    t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    torch.cuda.synchronize()
+    t0.record()
+    fa.fa_selftest_wait(50, gave_up)
+    t1.record()
+    torch.cuda.synchronize()
+    assert int(gave_up.item()) == 64 and fa.fa_device_status()[:2] == (fa.FA_ERR_TIMEOUT, 990)
+    assert 1.0 <= t0.elapsed_time(t1) <= 500.0
