@@ -49,117 +49,78 @@ EncodeTiledFn get_encode_fn() {
     return fn;
 }
 
-// Tensor map over a [B, S, H, d] 16-bit tensor (d = 128 or 64) with element strides (sb, ss, sh);
-// a box is box_rows sequence positions x 64 elements of d for one (batch, head), 128-byte swizzled.
-int encode_map(CUtensorMap* tm, const void* base, int B, int S, int H, int64_t sb, int64_t ss, int64_t sh,
-               int box_rows, bool bf16, int d = 128) {
+// A tensor map with the 128-byte swizzle; rows out of range read as zeros.  strides: bytes, of the
+// dimensions from the second on.
+template <int N>
+int encode_tiled(CUtensorMap* tm, CUtensorMapDataType type, const void* base, const cuuint64_t (&dims)[N],
+                 const cuuint64_t (&strides)[N - 1], const cuuint32_t (&box)[N]) {
     EncodeTiledFn fn = get_encode_fn();
     if (!fn) return FA_ERR_DEVICE;
-    cuuint64_t dims[4] = {(cuuint64_t)d, (cuuint64_t)H, (cuuint64_t)S, (cuuint64_t)B};
-    cuuint64_t strides[3] = {(cuuint64_t)sh * 2, (cuuint64_t)ss * 2, (cuuint64_t)sb * 2};
-    // a dimension of extent 1 never advances; give it a harmless legal stride
-    if (H == 1) strides[0] = (cuuint64_t)d * 2;
-    if (S == 1) strides[1] = strides[0] * (cuuint64_t)H;
-    if (B == 1) strides[2] = strides[1] * (cuuint64_t)S;
-    cuuint32_t box[4] = {64, 1, (cuuint32_t)box_rows, 1};
-    cuuint32_t estr[4] = {1, 1, 1, 1};
-    CUresult r = fn(tm, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 4,
-                    const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                    CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) {
-        t_last_cuda_error = static_cast<int>(r);
-        return FA_ERR_CUDA;
-    }
-    return FA_OK;
-}
-
-// Tensor map of the ping-pong kernel over a [B, S, H, d] 16-bit tensor: for d = 128 a box is box_rows positions x
-// all of d for one (batch, head) -- the dimensions are (64 elements of d, S, 64-element blocks of d, H, B), so
-// it lands block by block, box_rows rows of 128 swizzled bytes each --, for d = 64 that of encode_map.
-int encode_map_tile(CUtensorMap* tm, const void* base, int B, int S, int H, int64_t sb, int64_t ss, int64_t sh,
-                    int box_rows, bool bf16, int d = 128) {
-    if (d == 64) return encode_map(tm, base, B, S, H, sb, ss, sh, box_rows, bf16, d);
-    EncodeTiledFn fn = get_encode_fn();
-    if (!fn) return FA_ERR_DEVICE;
-    cuuint64_t dims[5] = {64, (cuuint64_t)S, (cuuint64_t)(d / 64), (cuuint64_t)H, (cuuint64_t)B};
-    cuuint64_t strides[4] = {(cuuint64_t)ss * 2, 128, (cuuint64_t)sh * 2, (cuuint64_t)sb * 2};
-    // a dimension of extent 1 never advances; give it a harmless legal stride
-    if (H == 1) strides[2] = (cuuint64_t)d * 2;
-    if (S == 1) strides[0] = strides[2] * (cuuint64_t)H;
-    if (B == 1) strides[3] = strides[0] * (cuuint64_t)S;
-    cuuint32_t box[5] = {64, (cuuint32_t)box_rows, (cuuint32_t)(d / 64), 1, 1};
-    cuuint32_t estr[5] = {1, 1, 1, 1, 1};
-    CUresult r = fn(tm, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 5,
-                    const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                    CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) {
-        t_last_cuda_error = static_cast<int>(r);
-        return FA_ERR_CUDA;
-    }
-    return FA_OK;
-}
-
-// Tensor map over a contiguous 16-bit cache [slabs, S, H, d] (d = 128 or 64) whose box is box_rows keys
-// x all of d for one (slab, head): the dimensions are (64 elements of d, S, 64-element blocks of d, H,
-// slab), so a box lands block by block, box_rows rows of 128 swizzled bytes each.
-int encode_map_cache(CUtensorMap* tm, const void* base, int slabs, int S, int H, int box_rows, bool bf16, int d) {
-    EncodeTiledFn fn = get_encode_fn();
-    if (!fn) return FA_ERR_DEVICE;
-    const cuuint64_t row = (cuuint64_t)H * d * 2;
-    cuuint64_t dims[5] = {64, (cuuint64_t)S, (cuuint64_t)(d / 64), (cuuint64_t)H, (cuuint64_t)slabs};
-    cuuint64_t strides[4] = {row, 128, (cuuint64_t)d * 2, row * S};
-    cuuint32_t box[5] = {64, (cuuint32_t)box_rows, (cuuint32_t)(d / 64), 1, 1};
-    cuuint32_t estr[5] = {1, 1, 1, 1, 1};
-    CUresult r = fn(tm, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 5,
-                    const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                    CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) {
-        t_last_cuda_error = static_cast<int>(r);
-        return FA_ERR_CUDA;
-    }
-    return FA_OK;
-}
-
-// Tensor map over a [B, S, H, 128] one-byte tensor, contiguous: a box is box_rows sequence
-// positions x 128 bytes for one (batch, head), 128-byte swizzled.
-int encode_map_u8(CUtensorMap* tm, const void* base, int B, int S, int H, int box_rows) {
-    EncodeTiledFn fn = get_encode_fn();
-    if (!fn) return FA_ERR_DEVICE;
-    cuuint64_t dims[4] = {128, (cuuint64_t)H, (cuuint64_t)S, (cuuint64_t)B};
-    cuuint64_t strides[3] = {128, (cuuint64_t)H * 128, (cuuint64_t)S * H * 128};
-    cuuint32_t box[4] = {128, 1, (cuuint32_t)box_rows, 1};
-    cuuint32_t estr[4] = {1, 1, 1, 1};
-    CUresult r = fn(tm, CU_TENSOR_MAP_DATA_TYPE_UINT8, 4, const_cast<void*>(base), dims, strides, box, estr,
-                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) {
-        t_last_cuda_error = static_cast<int>(r);
-        return FA_ERR_CUDA;
-    }
-    return FA_OK;
-}
-
-// Tensor map over a row-major [rows, cols] 16-bit matrix: a box is 64 rows x 64 columns, 128-byte
-// swizzled (the projection weight, an N-major MMA operand).  Encoded with four dimensions so that
-// the kernels' one load wrapper serves it; the outer two have extent 1.
-int encode_map_matrix(CUtensorMap* tm, const void* base, int rows, int cols, bool bf16) {
-    EncodeTiledFn fn = get_encode_fn();
-    if (!fn) return FA_ERR_DEVICE;
-    cuuint64_t dims[4] = {(cuuint64_t)cols, (cuuint64_t)rows, 1, 1};
-    cuuint64_t strides[3] = {(cuuint64_t)cols * 2, (cuuint64_t)cols * 2 * rows, (cuuint64_t)cols * 2 * rows};
-    cuuint32_t box[4] = {64, 64, 1, 1};
-    cuuint32_t estr[4] = {1, 1, 1, 1};
-    CUresult r = fn(tm, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 4,
-                    const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+    cuuint32_t elem_strides[N];
+    for (int i = 0; i < N; ++i) elem_strides[i] = 1;
+    CUresult r = fn(tm, type, N, const_cast<void*>(base), dims, strides, box, elem_strides, CU_TENSOR_MAP_INTERLEAVE_NONE,
                     CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) {
         t_last_cuda_error = static_cast<int>(r);
         return FA_ERR_CUDA;
     }
     return FA_OK;
+}
+CUtensorMapDataType type16(bool bf16) { return bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16; }
+
+// Element strides of a [B, S, H, d] tensor.  A dimension of extent 1 never advances and may come with any
+// stride; it gets a harmless legal one.
+struct Strides { int64_t b, s, h; };
+Strides legal_strides(int B, int S, int H, int64_t sb, int64_t ss, int64_t sh, int d) {
+    if (H == 1) sh = d;
+    if (S == 1) ss = sh * H;
+    if (B == 1) sb = ss * S;
+    return {sb, ss, sh};
+}
+
+// Tensor map over a [B, S, H, d] 16-bit tensor with element strides (sb, ss, sh); a box is box_rows
+// sequence positions x 64 elements of d for one (batch, head).
+int encode_map(CUtensorMap* tm, const void* base, int B, int S, int H, int64_t sb, int64_t ss, int64_t sh,
+               int box_rows, bool bf16, int d = 128) {
+    const Strides st = legal_strides(B, S, H, sb, ss, sh, d);
+    return encode_tiled<4>(tm, type16(bf16), base, {(cuuint64_t)d, (cuuint64_t)H, (cuuint64_t)S, (cuuint64_t)B},
+                           {(cuuint64_t)st.h * 2, (cuuint64_t)st.s * 2, (cuuint64_t)st.b * 2}, {64, 1, (cuuint32_t)box_rows, 1});
+}
+
+// The same with boxes of box_rows positions x all of d: the dimensions are (64 elements of d, S, 64-element
+// blocks of d, H, B), so a box lands block by block, box_rows rows of 128 swizzled bytes each.
+int encode_map_blocks(CUtensorMap* tm, const void* base, int B, int S, int H, int64_t sb, int64_t ss, int64_t sh,
+                      int box_rows, bool bf16, int d) {
+    const Strides st = legal_strides(B, S, H, sb, ss, sh, d);
+    return encode_tiled<5>(tm, type16(bf16), base, {64, (cuuint64_t)S, (cuuint64_t)(d / 64), (cuuint64_t)H, (cuuint64_t)B},
+                           {(cuuint64_t)st.s * 2, 128, (cuuint64_t)st.h * 2, (cuuint64_t)st.b * 2},
+                           {64, (cuuint32_t)box_rows, (cuuint32_t)(d / 64), 1, 1});
+}
+
+// Tensor map of the ping-pong kernel: whole rows of d = 128, or d = 64, whose rows are one box wide anyway.
+int encode_map_tile(CUtensorMap* tm, const void* base, int B, int S, int H, int64_t sb, int64_t ss, int64_t sh,
+                    int box_rows, bool bf16, int d = 128) {
+    return (d == 64 ? encode_map : encode_map_blocks)(tm, base, B, S, H, sb, ss, sh, box_rows, bf16, d);
+}
+
+// Tensor map over a contiguous 16-bit cache [slabs, S, H, d] (d = 128 or 64) with boxes of box_rows keys x all of d.
+int encode_map_cache(CUtensorMap* tm, const void* base, int slabs, int S, int H, int box_rows, bool bf16, int d) {
+    return encode_map_blocks(tm, base, slabs, S, H, (int64_t)S * H * d, (int64_t)H * d, d, box_rows, bf16, d);
+}
+
+// Tensor map over a [B, S, H, 128] one-byte tensor, contiguous: a box is box_rows sequence
+// positions x 128 bytes for one (batch, head).
+int encode_map_u8(CUtensorMap* tm, const void* base, int B, int S, int H, int box_rows) {
+    return encode_tiled<4>(tm, CU_TENSOR_MAP_DATA_TYPE_UINT8, base, {128, (cuuint64_t)H, (cuuint64_t)S, (cuuint64_t)B},
+                           {128, (cuuint64_t)H * 128, (cuuint64_t)S * H * 128}, {128, 1, (cuuint32_t)box_rows, 1});
+}
+
+// Tensor map over a row-major [rows, cols] 16-bit matrix: a box is 64 rows x 64 columns (the projection
+// weight, an N-major MMA operand).  Encoded with four dimensions so that the kernels' one load
+// wrapper serves it; the outer two have extent 1.
+int encode_map_matrix(CUtensorMap* tm, const void* base, int rows, int cols, bool bf16) {
+    const cuuint64_t row = (cuuint64_t)cols * 2;
+    return encode_tiled<4>(tm, type16(bf16), base, {(cuuint64_t)cols, (cuuint64_t)rows, 1, 1}, {row, row * rows, row * rows}, {64, 64, 1, 1});
 }
 
 // a page holds a multiple of the 128-key tile, or 16, 32 or 64 keys (several pages per tile)
