@@ -96,7 +96,7 @@ typedef struct fa_params {
     int64_t v_stride[3];
     int64_t o_stride[3];
     int variant; /* 0 = default: the ping-pong kernel, or the paired-tile pipelined kernel for many short
-                    unmasked sequences.  Others force one kernel, for A/B timing and tests: 1, 2 = simple kernels
+                    unmasked sequences with fp32 output.  Others force one kernel, for A/B timing and tests: 1, 2 = simple kernels
                     (P through tensor / shared memory), 3 = ping-pong, 4 = paired-tile pipelined. */
 } fa_params;
 

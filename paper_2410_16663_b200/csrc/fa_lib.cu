@@ -226,8 +226,13 @@ fa::FwdParams dense_fwd_params(const fa_params& p) {
 }
 
 // Head dimension 64: keys from which the ping-pong kernel is used (128 < Skv <= 256 has the
-// short-sequence pipeline of its own; up to 128 keys the kernel with four small CTAs per SM, which
-// the ping-pong kernel ties there and beats by 3 to 37 % from 300 keys on).
+// short-sequence pipeline of its own, up to 128 keys the kernel with four small CTAs per SM).  Timed on both sides:
+// from 257 keys on the ping-pong kernel, 64 x 12 x 257 55.7 us, and 3 to 37 % ahead of the small one from 300 keys
+// on.  129 to 256 keys: the pipeline ahead nearly everywhere, 1024 x 12 x 197 392 against 532 us, 64 x 12 x 144
+// 22.0 / 32.9, 1024 x 12 x 256 498 / 535, 64 x 12 x 224 30.3 / 33.6, but 64 x 12 x 256 33.5 / 31.5.  Up to 128
+// keys neither everywhere: the small kernel ahead on calls of less than a round (9.0 / 9.2) and on up to 64 keys
+// (1024 x 12 x 64 173 / 179, x 32 158 / 174), the ping-pong kernel on many sequences of 128 (64 x 12 x 128 17.8 /
+// 13.7, 1024 x 12 x 128 210 / 192), which it only tied before its items of few steps got shorter.
 #ifndef FA_D64_PINGPONG_FROM
 #define FA_D64_PINGPONG_FROM 257
 #endif
@@ -278,16 +283,20 @@ int forward_impl(const fa_params& in, cudaStream_t st) {
 
     // Default choice, from timings of both kernels: the ping-pong kernel (one query tile per CTA,
     // Q K^T running ahead of the softmax), also on short sequences: paired tiles make half as many
-    // items of twice the length, which loses when there are few (1 x 2 heads x 512: 8.0 against 12.3
-    // us; 1 x 5 x 1000: 11.7 / 20.1; 1 x 32 x 512: 9.9 / 13.3), and an item boundary costs the
-    // ping-pong kernel less than it did (8 x 32 x 512: 42.0 / 48.9; 16 x 32 x 128: 18.5 / 25.3).  What
-    // is left to the paired kernel: without a mask, items of exactly two query and two kv tiles, at least three
-    // rounds of them (16 x 64/8 x 200: 56.1 against 61.8 us; 16 x 32 x 256: 38.1 / 39.8; causal level).
+    // items of twice the length, which loses when there are few (causal, 1 x 2 heads x 512: 9.1 against 13.3
+    // us, 1 x 5 x 1000 10.6 / 20.6, 1 x 32 x 512 9.0 / 14.1; by this entry point, whose calls take the host 9),
+    // and an item boundary costs the ping-pong kernel less (8 x 32 x 512 34.9 / 46.0; without a mask
+    // 16 x 32 x 128 12.5 / 22.0, 16 x 32 x 384 67.9 / 93.5).  What is left to the paired kernel: with fp32
+    // output, which every thread stores by itself, items without a mask of exactly two query and two kv tiles,
+    // at least three rounds of them (64 x 32 x 256 190.7 / 179.5, 16 x 64/8 x 200 78.9 / 75.0, though 16 x 32 x 256
+    // 48.3 / 55.1).  With 16-bit output, through shared memory and TMA stores, the ping-pong kernel is level or
+    // ahead there too: 16 x 64/8 x 200 49.9 / 56.2, 16 x 32 x 256 29.3 / 34.2, 64 x 32 x 256 126.1 / 126.2,
+    // 64 x 32 x 197 112.8 / 129.0, 128 x 32/8 x 256 213 / 225.
     int variant = p.variant;
     if (variant == 0 && p.d == 64) variant = p.Skv >= kD64PingPongFrom ? 3 : 0;
     else if (variant == 0 && p.d == 128) {
         const bool two_by_two = fp.n_qtiles == 2 && p.Skv > fa::kTile && p.Skv <= 2 * fa::kTile;
-        variant = (!p.causal && two_by_two && 2ll * p.B * p.Hq >= 3ll * sms) ? 4 : 3;
+        variant = (fp.o_fp32 && !p.causal && two_by_two && 2ll * p.B * p.Hq >= 3ll * sms) ? 4 : 3;
     }
     const auto encode = variant == 3 ? encode_map_tile : encode_map;
     CUtensorMap tq, tk, tv;

@@ -1,4 +1,5 @@
-// Prefill forward, paired-tile pipelined variant (the choice for short sequences of two tiles, see fa_lib.cu).
+// Prefill forward, paired-tile pipelined variant (the choice for short sequences of two tiles with
+// fp32 output, see fa_lib.cu).
 //
 // A persistent CTA (one per SM, 384 threads) walks a static list of work items, longest
 // first, in boustrophedon order over the CTAs.  An item is a pair of adjacent 128-row query

@@ -198,6 +198,22 @@ def test_scale_zero_and_large_scale(fa):
     full_case(fa, 1, 2, 2, 130, 260, False, "fp16", seed=6, scale=1.0, fp16_ulp=True)  # peaked softmax
 
 
+@pytest.mark.parametrize("dtype", ["fp16", "bf16"])
+@pytest.mark.parametrize("B,Hq,Hkv,Sq,Skv", [(7, 32, 8, 129, 256), (7, 32, 32, 256, 129), (14, 16, 16, 200, 200), (7, 32, 4, 256, 256)])
+def test_two_by_two_tiles_without_a_mask(fa, B, Hq, Hkv, Sq, Skv, dtype):
+    # where the two persistent kernels meet: 16-bit output is the ping-pong kernel's, fp32 output the paired one's
+    full_case(fa, B, Hq, Hkv, Sq, Skv, False, dtype, seed=Sq * 1000 + Skv)
+    cfg = synth.PrefillConfig("t", B, Hq, Hkv, Sq, Skv, dtype=dtype, causal=False, seed=6)
+    q, k, v = (t.to(DEV) for t in synth.prefill_inputs(cfg, "cpu"))
+    for o_dtype, kernel in ((None, 3), (torch.float32, 4)):
+        default, forced = (run_forward(fa, q, k, v, False, cfg.scale, o_dtype=o_dtype, variant=x) for x in (0, kernel))
+        assert all(torch.equal(a, b) for a, b in zip(default, forced))
+        # the same call head-major, as the default takes any strides
+        qh, kh, vh = (t.transpose(1, 2).contiguous().transpose(1, 2) for t in (q, k, v))
+        strided = run_forward(fa, qh, kh, vh, False, cfg.scale, o_dtype=o_dtype)
+        assert all(torch.equal(a, b) for a, b in zip(default, strided))
+
+
 @pytest.mark.parametrize("variant", [0, 3, 4])
 def test_bhsd_strided_layout(fa, variant):
     # (the ping-pong kernel writes its 16-bit output through a tensor map built from these strides)
