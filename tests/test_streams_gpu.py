@@ -122,25 +122,127 @@ def test_other_forms_beside_a_kernel_that_holds_sms(fa, sms):  # noqa: F811
         beside_neighbour(fa, lambda: fa.fa_decode(q, k, v, o, lse, sl, 0.1, ws), [o, lse], sms, overlaps=False)
 
 
-@pytest.mark.parametrize("B,H,S,d,causal", [(1, 2, 512, 128, True), (1, 1, 1, 128, False), (1, 4, 2048, 128, True), (1, 3, 3000, 128, False),
-                                            (3, 5, 700, 128, True), (8, 32, 512, 128, True), (4, 16, 600, 64, True)])
-def test_calls_that_read_what_the_call_before_wrote(fa, B, H, S, d, causal):
-    # every call starts while the one before it may still run, and decodes its first item then; each
-    # reads as its values what the last one wrote, into a buffer that the one before that reads.  Grids that leave SMs
-    # free, shared query tiles and full grids, against the same calls one by one.
-    q, k = (_rand((B, S, H, d), torch.float16, i) for i in (1, 2))
-    v0 = _rand((B, S, H, d), torch.float16, 3)
+# Calls that feed one another.  Every call starts while the one before it may still run; call i reads what call i - 1
+# wrote, as its queries, its keys or its values in turn (the other two are its own), and writes over what
+# that one read.  step(i, src, dst) is one call, src and dst [B, S, H, d] of 16 bits; the softmax scale grows from
+# call to call, so that no two of them write the same.
+def _scale(i):
+    return 0.2 + 0.03 * i
+
+
+def _dense_steps(fa, B, H, S, d, causal, dtype=torch.float16, o_dtype=None):
+    own = [_rand((B, S, H, d), dtype, 20 + i) for i in range(3)]
+    o32 = torch.empty(B, S, H, d, device=DEV) if o_dtype else None
+
+    def step(i, src, dst):
+        q, k, v = (src if i % 3 == n else own[n] for n in range(3))
+        fa.fa_forward_ex(q, k, v, dst if o32 is None else o32, None, causal, _scale(i))
+        if o32 is not None:
+            dst.copy_(o32)
+
+    return (B, S, H, d), dtype, step
+
+
+def _fp8_steps(fa, B, H, S, causal):
+    own = [_rand((B, S, H, 128), torch.float16, 30 + i).to(torch.float8_e4m3fn) for i in range(3)]
+    x8 = torch.empty_like(own[0])
+
+    def step(i, src, dst):
+        x8.copy_(src)
+        q, k, v = (x8 if i % 3 == n else own[n] for n in range(3))
+        fa.fa_forward_fp8(q, k, v, dst, None, causal, _scale(i), 1.0, 1.0, 1.0)
+
+    return (B, S, H, 128), torch.float16, step
+
+
+def _packed_steps(fa, lens, H, d, page):
+    """Prefix sums, lengths and block table are written on the device right before each call, which takes
+    the sequences in another order than the one before."""
+    n, total = len(lens), sum(lens)
+    own = [_rand((total, H, d), torch.bfloat16, 40 + i) for i in range(3)]
+    cu, sl = torch.zeros(n + 1, dtype=torch.int32, device=DEV), torch.zeros(n, dtype=torch.int32, device=DEV)
+    pages = -(-max(lens) // page) if page else 0
+    table = torch.zeros(n, max(1, pages), dtype=torch.int32, device=DEV)
+    orders = [torch.tensor(lens[i % n:] + lens[:i % n], dtype=torch.int32).to(DEV) for i in range(n)]
+    tables = [torch.randperm(n * pages).to(torch.int32).view(n, pages).to(DEV) for _ in range(n)] if page else None
+    pool = torch.zeros(2, n * pages, page, H, d, dtype=torch.bfloat16, device=DEV) if page else None
+    if page:
+        pool.copy_(_rand(pool.shape, torch.bfloat16, 44))
+
+    def step(i, src, dst):
+        src, dst = src.view(total, H, d), dst.view(total, H, d)
+        cu[1:].copy_(orders[i % n].cumsum(0))
+        if not page:
+            q, k, v = (src if i % 3 == m else own[m] for m in range(3))
+            fa.fa_forward_varlen(q, k, v, dst, None, cu, cu, max(lens), max(lens), True, _scale(i))
+        else:
+            sl.copy_(orders[i % n])
+            table.copy_(tables[i % n])
+            if i % 3:   # as keys or values: the first rows of the pool
+                pool[i % 3 - 1].view(-1, H, d)[:total].copy_(src)
+            fa.fa_forward_varlen_paged(own[0] if i % 3 else src, pool[0], pool[1], table, dst, None, cu, sl, max(lens), max(lens), True, _scale(i))
+
+    return (1, total, H, d), torch.bfloat16, step
+
+
+def _decode_and_prefill_steps(fa, B, H):
+    """A decode, a small prefill over its output, a decode with the prefill's output as its queries, ..."""
+    q0, k, v = _rand((1, B, H, 128), torch.float16, 50), _rand((B, 900, H, 128), torch.float16, 51), _rand((B, 900, H, 128), torch.float16, 52)
+    sl = torch.tensor([900 - 31 * b for b in range(B)], dtype=torch.int32, device=DEV)
+    ws = torch.empty(fa.fa_decode_workspace_bytes(B, H, H, 900, 128) + 16, dtype=torch.uint8, device=DEV)
+
+    def step(i, src, dst):
+        if i % 2 == 0:
+            fa.fa_decode(src.view(B, 1, H, 128), k, v, dst.view(B, 1, H, 128), None, sl, _scale(i), ws)
+        else:
+            fa.fa_forward(q0 if i % 4 == 1 else src, src, src, dst, None, True, _scale(i))
+
+    return (1, B, H, 128), torch.float16, step
+
+
+@pytest.mark.parametrize("form", [
+    lambda fa: _dense_steps(fa, 1, 2, 512, 128, True),
+    lambda fa: _dense_steps(fa, 1, 1, 5, 128, False),
+    lambda fa: _dense_steps(fa, 1, 4, 2048, 128, True),            # query tiles shared by a cluster's CTAs
+    lambda fa: _dense_steps(fa, 1, 3, 3000, 128, False, torch.bfloat16),
+    lambda fa: _dense_steps(fa, 3, 5, 700, 128, True),
+    lambda fa: _dense_steps(fa, 8, 32, 512, 128, True),            # a full grid
+    lambda fa: _dense_steps(fa, 4, 16, 600, 64, True),
+    lambda fa: _dense_steps(fa, 2, 6, 700, 128, True, o_dtype=torch.float32),
+    lambda fa: _fp8_steps(fa, 2, 8, 700, True),
+    lambda fa: _packed_steps(fa, [300, 33, 128, 517, 1], 4, 128, 0),
+    lambda fa: _packed_steps(fa, [300, 33, 128, 517, 1], 4, 64, 0),
+    lambda fa: _packed_steps(fa, [300, 33, 128, 517, 1], 4, 128, 128),
+    lambda fa: _decode_and_prefill_steps(fa, 16, 4),
+], ids=["small", "few rows", "shared tiles", "shared tiles bf16", "medium", "full grid", "d64", "fp32 output", "fp8", "packed", "packed d64",
+        "paged", "decode and prefill"])
+def test_calls_that_read_what_the_call_before_wrote(fa, form):  # noqa: F811
+    # The calls one by one, and queued up behind a call that outlasts their enqueueing: bit for bit the same.
+    near = Neighbour(fa, 4, 524288)
     ends = []
     for alone in (True, False):
-        bufs = [v0.clone(), torch.full_like(v0, float("nan"))]
-        for i in range(12):
-            fa.fa_forward(q, k, bufs[i & 1], bufs[1 - (i & 1)], None, causal, 0.1)
-            if alone:
-                torch.cuda.synchronize()
+        torch.manual_seed(3)
+        shape, dtype, step = form(fa)
+        x0 = _rand(shape, dtype, 3)
+        bufs, seen = [x0.clone(), torch.full_like(x0, float("nan"))], []
+        near.run()
         torch.cuda.synchronize()
+        gone = torch.cuda.Event()
+        if not alone:
+            near.run()
+            gone.record()
+        for i in range(12):
+            step(i, bufs[i & 1], bufs[1 - (i & 1)])
+            if alone:
+                seen.append(bufs[1 - (i & 1)].clone())
+                torch.cuda.synchronize()
+        assert alone or not gone.query()   # else the calls did not queue up and nothing has been tested
+        torch.cuda.synchronize()
+        check_status(fa)
+        for a, b in zip(seen, seen[2:]):   # a call that read a buffer as it was before would be found out
+            assert torch.isfinite(a).all() and torch.isfinite(b).all() and not torch.equal(a, b)
         ends.append(bufs)
-    check_status(fa)
-    assert all(torch.equal(a, b) for a, b in zip(*ends)) and torch.isfinite(ends[0][0]).all()
+    assert all(torch.equal(a, b) for a, b in zip(*ends))
 
 
 @pytest.fixture(scope="module")
