@@ -29,6 +29,10 @@
 // CTAs share a query tile merges behind cluster barriers and a named barrier, which are not: every
 // thread reaches them, those of a CTA without work and of one that gave up a wait too, because a role
 // that stops only leaves its loop.
+//
+// The times beside a step below are of the code before and after that step, in turn on one box, whose clock
+// and power state differ from box to box; steps measured apart do not multiply to the whole.  8 x 32 x 512
+// from the first step of "P stored in one piece" to here, in turn: 43.9 -> 41.4 us.
 #pragma once
 
 #include <type_traits>
@@ -787,7 +791,8 @@ struct PpSoftmax {
 
 // Merge of the parts that a cluster's CTAs computed of one query tile: CTA `rank` of `split` finishes
 // rows rank, rank + split, ..., one warp per row and four columns per lane, reading the parts through
-// distributed shared memory.
+// distributed shared memory.  (The spills of that kernel, 32 bytes stored and 76 loaded, are all this function's, which
+// runs once: without it there are none, with two rows at a time instead of four 16 and 48.)
 constexpr uint32_t kPpPartStats = 65536;   // bytes from a part's O to its (max, sum) pairs
 template <typename T>
 __device__ __forceinline__ void pp_split_merge(const FwdParams& p, uint32_t part, int tid) {
@@ -1086,8 +1091,11 @@ __device__ __forceinline__ bool pp_attention(const CUtensorMap& tm_q, const CUte
                     for (int c = 0; c < D / 8; ++c) {
                         // 16-byte chunk c & 7 of the row's half c >> 3, at its swizzled place
                         const uint32_t addr = row_base + (uint32_t)(c >> 3) * 4096u + (((uint32_t)(c & 7) ^ ((uint32_t)lane & 7u)) << 4);
-                        // (packed multiplications: 8 x 32 x 512 42.6 -> 42.0 us, 16 x 32 x 256 34.6 -> 34.3, others level; but
-                        // the packed batches' instantiation came out 1 to 2 % slower with them)
+                        // (packed multiplications: 8 x 32 x 512 42.6 -> 42.0 us, 16 x 32 x 256 34.6 -> 34.3, others level.  Not for
+                        // packed batches: 20 requests of 20 to 666 tokens 23.6 -> 24.0, 32 of 16 to 512 89.1 -> 89.9, 10 of 100
+                        // to 3000 442 -> 445, 32 of 256 to 8192 level.  The arithmetic is the same, and so are that
+                        // instantiation's registers and spills (88 bytes stored, none loaded) either way: presumably the order
+                        // that the compiler gives its epilogue.)
                         uint32_t wd[4];
 #pragma unroll
                         for (int q = 0; q < 4; ++q) {
@@ -1292,8 +1300,11 @@ int launch_pingpong(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensor
     // merge their parts through distributed shared memory, as many CTAs to a tile as the device runs
     // for all tiles at once.  A step takes 0.8 to 1 us, and the exchange of the parts (64 KiB a CTA,
     // two cluster barriers, the launch of clusters) about five more than an ordinary epilogue, so it
-    // pays from eight steps saved on the longest tile: 15 tiles over 157 kv tiles 128 -> 33 us, 32
-    // over 63 55 -> 25, 64 over 32 31.2 -> 23.3, 64 over 16 19.1 -> 17.9; 60 over 12 15.2 / 15.5.
+    // pays from about eight steps saved on the longest tile (not shared / shared): 15 tiles over 157 kv tiles
+    // 113.6 / 24.5 us (124 / 33 with 15 kv heads, whose keys come from HBM), 32 over 63 51.6 / 23.5, 64 over 32
+    // 28.0 / 21.7, 64 over 16 16.6 / 15.4, 24 over 16 16.1 / 13.4, 30 over 12 13.3 / 12.0.  At the line itself both
+    // sides occur: eight saved 74 over 16 21.0 / 22.0, 20 over 10 11.8 / 12.3; seven saved 30 over 10 level,
+    // 5 over 8 10.3 / 9.3; six saved 60 over 12 15.2 / 15.4.
     if constexpr (!kF8 && D == 128) {
         if (fp.split == 0 && !varlen) {
             const int kv_tiles = (fp.Skv + kTile - 1) / kTile;   // of the longest item
