@@ -113,7 +113,7 @@ fa_fwd_d256_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
 
     if (warp == 4) {
         // =========================== K loads and score MMAs: one thread
-        if (tid == 128 && n_tiles > 0) {
+        if (elect_one() && n_tiles > 0) {
             bool ok = mbar_wait(bar_q, 0, &abort_flag, 61);
             for (int t = 0; t < n_tiles && ok; ++t) {
                 const int buf = t & 1;
@@ -161,7 +161,7 @@ fa_fwd_d256_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
         __syncwarp();
     } else if (warp == 5) {
         // =========================== V loads and P V MMAs: one thread
-        if (tid == 160 && n_tiles > 0) {
+        if (elect_one() && n_tiles > 0) {
             bool ok = true;
             for (int j = 0; j < n_tiles && ok; ++j) {
                 const int buf = j & 1;

@@ -337,7 +337,7 @@ fa_fwd_d64_stream_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
                 }
             }
         }
-    } else if (lane == 0) {
+    } else if (elect_one()) {
         const uint32_t sStage0 = smem_base;
         if (warp == 16) {
             // ============================================================ S = Q K^T

@@ -1165,7 +1165,7 @@ __device__ __forceinline__ bool pp_attention(const CUtensorMap& tm_q, const CUte
         else if (kTmaOut && lane == 0) tma_store_wait_all();
     } else {
         setmaxnreg_dec<kPipeOtherRegs>();
-        if (lane == 0) {
+        if (elect_one()) {
             if (warp == 8) pp_run_s<T, kTmaOut, kVarlen, kF8, D>(bar0, sQ, sK, tmem_base, ss.items, abort_flag);
             else if (warp == 10) pp_run_pv<T, kVarlen, kF8, D>(bar0, sV, tmem_base, ss.items, abort_flag);
             else if (warp == 9) pp_run_load_qk<kVarlen, kF8, D>(bar0, sQ, sK, &tm_q, &tm_k, p, total_items, ss, abort_flag);

@@ -586,7 +586,7 @@ fa_fwd_pipelined_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
     }
     if (warp == 8 || warp == 10) {
         // ================================================================ MMA issue (role 0 / 1)
-        if (lane == 0) {
+        if (elect_one()) {
             MmaIssuer<T> mi;
             mi.bar0 = bar0;
             mi.sQ = sQ;
@@ -599,7 +599,7 @@ fa_fwd_pipelined_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
         __syncwarp();
     } else if (warp == 9) {
         // ================================================================ TMA loads
-        if (lane == 0) run_loader(bar0, sQ, sKV, &tm_q, &tm_k, &tm_v, p, total_items, n_qpairs, &abort_flag);
+        if (elect_one()) run_loader(bar0, sQ, sKV, &tm_q, &tm_k, &tm_v, p, total_items, n_qpairs, &abort_flag);
         __syncwarp();
     }
 

@@ -62,11 +62,11 @@ __device__ __forceinline__ void proj_item(const ProjParams& pp, int t, int& b, i
 template <typename T>
 __device__ __forceinline__ void proj_phase(const CUtensorMap* tm_a, const CUtensorMap* tm_w, const ProjParams& pp,
                                            uint32_t bar0, uint32_t smem, uint32_t tmem, volatile uint32_t* abort_flag) {
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = tid >> 5;
     const int total = pp.B * pp.n_qtiles * pp.n_cblocks;
     const int n_kb = pp.Hq * 2;   // k-blocks of 64
     if (warp == 9) {
-        if (lane == 0) {
+        if (elect_one()) {
             // ------------------------------------------------------------ loads
             tma_prefetch_desc(tm_a);
             tma_prefetch_desc(tm_w);
@@ -108,7 +108,7 @@ __device__ __forceinline__ void proj_phase(const CUtensorMap* tm_a, const CUtens
         }
         __syncwarp();
     } else if (warp == 8) {
-        if (lane == 0) {
+        if (elect_one()) {
             // ------------------------------------------------------------ MMA issue
             constexpr bool kBf16 = std::is_same<T, __nv_bfloat16>::value;
             constexpr uint32_t idesc = instr_desc_f16(kBf16, 128, 256, false, true);

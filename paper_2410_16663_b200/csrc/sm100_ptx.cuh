@@ -276,6 +276,23 @@ __device__ __forceinline__ void tma_store_wait_read() {
     asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
 }
 
+// ------------------------------------------------------------------ the issuing thread
+// True in one lane of the warp, always the same one (all lanes must be there).  Whoever issues tcgen05 or TMA instructions for
+// its warp is chosen by this and not by its lane number: the compiler takes a branch on the election for one that a
+// single lane enters, and keeps the descriptors that these instructions take from uniform registers there from the
+// start.  Behind a comparison of the lane number it moves them over for every instruction.  Eight 128 x 128 x 16
+// products back to back, clocks to issue: 389 by lane number, 90 to 158 elected; S and P V of a step from two threads, to the end:
+// 1134 to 1189, elected 1024 (which is what the tensor cores need).  1024 x 12 x 197, d = 64, 388.9 -> 366.5 us; d = 128: 8 x 32 x 512
+// 41.9 -> 40.8, 32 packed prompts 4113 -> 4084, 4 x 32 x 2048 with fp32 output 209 -> 202; d = 64 through the
+// ping-pong kernel, 16 x 16 x 512 26.6 -> 24.6; d = 256, 2 x 16 x 2048 103.4 -> 98.5; longer sequences of d = 128 level.
+// (Level, and left as they were: the decode kernels' loading threads, and the kernel for short d = 64 sequences, whose
+// issuing thread comes back to the others at every product.)
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
+
 // ------------------------------------------------------------------ tensor memory
 // Allocation is warp-wide; the base address (lane 0, first column) lands in shared memory.
 __device__ __forceinline__ void tmem_alloc(uint32_t dst_smem, uint32_t ncols) {
