@@ -50,7 +50,7 @@ fa_decode_split_fp8_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
     __shared__ volatile uint32_t abort_flag;
 
     const int tid = threadIdx.x;
-    const int warp = tid >> 5, lane = tid & 31;
+    const int warp = uniform(tid >> 5), lane = tid & 31;
     const int c = blockIdx.y;
     const int b = blockIdx.z;
     const int g_all = p.Hq / p.Hkv;

@@ -73,7 +73,7 @@ fa_fwd_d256_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     const uint32_t bar_sa = smem_u32(&bars[12]);   // the score MMAs over the first half of d completed
 
     const int tid = threadIdx.x;
-    const int warp = tid >> 5;
+    const int warp = uniform(tid >> 5);
     const int qt = p.n_qtiles - 1 - blockIdx.x;  // long (late) tiles first
     const int h = blockIdx.y;
     const int b = blockIdx.z;

@@ -45,7 +45,7 @@ fa_fwd_d64_slim_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
     const uint32_t bar_o = smem_u32(&bars[4]);
 
     const int tid = threadIdx.x;
-    const int warp = tid >> 5;
+    const int warp = uniform(tid >> 5);
     const int qt = p.n_qtiles - 1 - blockIdx.x;  // long (late) tiles first
     const int h = blockIdx.y;
     const int b = blockIdx.z;

@@ -104,7 +104,7 @@ fa_fwd_d64_stream_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
     const uint32_t bar0 = smem_u32(&bars[0]);
 
     const int tid = threadIdx.x;
-    const int warp = tid >> 5;
+    const int warp = uniform(tid >> 5);
     const int lane = tid & 31;
     if (tid == 0) {
         for (int i = 0; i < d64b::count; ++i) mbar_init(d64_bar(bar0, i), i >= d64b::row_max ? 2u : i >= d64b::s_free ? 8u : (i >= d64b::p_full ? 4u : 1u));

@@ -664,6 +664,7 @@ struct PpSoftmax {
     int r;                  // this thread's row of the tile
     // per item
     int row;                // query row of this thread
+    int lim0;               // packed batches: keys of the sequence that it sees
     float l_part;           // row sum over this warpgroup's steps, relative to m_loc
     float m_loc;            // reference max after this warpgroup's latest step
     float m_before;         // reference max that step received from the step before it
@@ -684,9 +685,16 @@ struct PpSoftmax {
         float m_prev = *m_other;
         if (masked) {
             // hidden scores become -inf (the scale is strictly positive, so they come out as exact zeros)
-            const int kv0 = kv_first + j * kTile;
-            int lim = Skv - kv0;
-            if (causal) lim = min(lim, row + off - kv0 + 1);
+            // (A packed item's lengths come from shared memory and live in registers, of which one is enough: 10 requests of 100
+            // to 3000 tokens 316 -> 313 us, 2 of 250 to 8000 233 -> 229.  A dense call's are parameters, and as fast as they are.)
+            int lim;
+            if (kVarlen) {
+                lim = lim0 - j * kTile;
+            } else {
+                const int kv0 = kv_first + j * kTile;
+                lim = Skv - kv0;
+                if (causal) lim = min(lim, row + off - kv0 + 1);
+            }
             // (bits of a word instead of a comparison per score: several predicates are set at a time; 4 x 32 x 2048
             // 173.9 -> 171.2 us, 32 packed prompts of 256 to 8192 tokens 4450 -> 4399, 8 x 32 x 512 43.1 -> 42.8)
 #pragma unroll
@@ -796,7 +804,7 @@ struct PpSoftmax {
 constexpr uint32_t kPpPartStats = 65536;   // bytes from a part's O to its (max, sum) pairs
 template <typename T>
 __device__ __forceinline__ void pp_split_merge(const FwdParams& p, uint32_t part, int tid) {
-    const int warp = tid >> 5, lane = tid & 31;
+    const int warp = uniform(tid >> 5), lane = tid & 31;
     const int split = p.split, idx = (int)blockIdx.x / split, rank = (int)blockIdx.x - idx * split;
     int bh, qt, b, h;
     pp_class_order(p, idx, bh, qt);
@@ -904,7 +912,7 @@ __device__ __forceinline__ bool pp_attention(const CUtensorMap& tm_q, const CUte
     volatile uint32_t* abort_flag = &ss.abort_flag;
 
     const int tid = threadIdx.x;
-    const int warp = tid >> 5;
+    const int warp = uniform(tid >> 5);
     const int lane = tid & 31;
     if (smem_base & 1023u) {  // uniform for the CTA: nothing has been set up yet
         if (tid == 0) record_timeout(900);
@@ -983,15 +991,15 @@ __device__ __forceinline__ bool pp_attention(const CUtensorMap& tm_q, const CUte
             if (!pp_warp_wait(pp_bar(bar0, ppb::item_full + slot), (ord / kPpSlots) & 1, abort_flag, 122 + w)) break;
             // the epilogue reads the rest of the slot; it is handed back at the end of the item
             const PpItem& it = ss.items[slot];
-            const int n = it.n, q0 = it.q0;
+            const int n = kVarlen ? uniform(it.n) : it.n, q0 = kVarlen ? uniform(it.q0) : it.q0;
             if (n == 0) break;
             if (!kVarlen && ord == 0) grid_dep_wait();
             const int row = q0 + r;   // within the sequence
-            const int Sq_i = kVarlen ? it.Sq : p.Sq, Skv_i = kVarlen ? it.Skv : p.Skv;
-            const int off_i = kVarlen ? it.Skv - it.Sq : off;
+            const int Sq_i = kVarlen ? it.Sq : p.Sq, Skv_i = kVarlen ? uniform(it.Skv) : p.Skv;
+            const int off_i = kVarlen ? Skv_i - Sq_i : off;
             if (kVarlen) {
                 sm.Skv = Skv_i;
-                sm.off = off_i;
+                sm.lim0 = p.causal ? min(Skv_i, row + off_i + 1) : Skv_i;
             }
             sm.row = row;
             sm.l_part = 0.f;
@@ -1091,21 +1099,13 @@ __device__ __forceinline__ bool pp_attention(const CUtensorMap& tm_q, const CUte
                     for (int c = 0; c < D / 8; ++c) {
                         // 16-byte chunk c & 7 of the row's half c >> 3, at its swizzled place
                         const uint32_t addr = row_base + (uint32_t)(c >> 3) * 4096u + (((uint32_t)(c & 7) ^ ((uint32_t)lane & 7u)) << 4);
-                        // (packed multiplications: 8 x 32 x 512 42.6 -> 42.0 us, 16 x 32 x 256 34.6 -> 34.3, others level.  Not for
-                        // packed batches: 20 requests of 20 to 666 tokens 23.6 -> 24.0, 32 of 16 to 512 89.1 -> 89.9, 10 of 100
-                        // to 3000 442 -> 445, 32 of 256 to 8192 level.  The arithmetic is the same, and so are that
-                        // instantiation's registers and spills (88 bytes stored, none loaded) either way: presumably the order
-                        // that the compiler gives its epilogue.)
+                        // (packed multiplications: 8 x 32 x 512 42.6 -> 42.0 us, 16 x 32 x 256 34.6 -> 34.3, 10 packed requests of 100 to 3000
+                        // tokens 325 -> 316, 32 of 256 to 8192 4158 -> 4072, others level)
                         uint32_t wd[4];
 #pragma unroll
                         for (int q = 0; q < 4; ++q) {
-                            float x0 = __uint_as_float(s[8 * c + 2 * q]), x1 = __uint_as_float(s[8 * c + 2 * q + 1]);
-                            if (kVarlen) {
-                                x0 *= inv_l;
-                                x1 *= inv_l;
-                            } else {
-                                f2_unpack(f2_mul(f2_pack(x0, x1), f2_pack(inv_l, inv_l)), x0, x1);
-                            }
+                            float x0, x1;
+                            f2_unpack(f2_mul(f2_pack(__uint_as_float(s[8 * c + 2 * q]), __uint_as_float(s[8 * c + 2 * q + 1])), f2_pack(inv_l, inv_l)), x0, x1);
                             wd[q] = pack2<T>(x0, x1);
                         }
                         asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(wd[0]), "r"(wd[1]), "r"(wd[2]), "r"(wd[3]) : "memory");

@@ -450,7 +450,7 @@ fa_fwd_pipelined_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
     auto o_final = [&](int t) { return bar0 + 8 * (8 + 2 * kStages + t); };
 
     const int tid = threadIdx.x;
-    const int warp = tid >> 5;
+    const int warp = uniform(tid >> 5);
     const int lane = tid & 31;
 
     if (tid == 0) {

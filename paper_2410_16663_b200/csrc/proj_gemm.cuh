@@ -62,7 +62,7 @@ __device__ __forceinline__ void proj_item(const ProjParams& pp, int t, int& b, i
 template <typename T>
 __device__ __forceinline__ void proj_phase(const CUtensorMap* tm_a, const CUtensorMap* tm_w, const ProjParams& pp,
                                            uint32_t bar0, uint32_t smem, uint32_t tmem, volatile uint32_t* abort_flag) {
-    const int tid = threadIdx.x, warp = tid >> 5;
+    const int tid = threadIdx.x, warp = uniform(tid >> 5);
     const int total = pp.B * pp.n_qtiles * pp.n_cblocks;
     const int n_kb = pp.Hq * 2;   // k-blocks of 64
     if (warp == 9) {
@@ -187,7 +187,7 @@ fa_proj_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     __shared__ uint32_t abort_word;
     const uint32_t smem_base = smem_u32(smem_raw);
     const uint32_t bar0 = smem_u32(&bars[0]);
-    const int tid = threadIdx.x, warp = tid >> 5;
+    const int tid = threadIdx.x, warp = uniform(tid >> 5);
     if (smem_base & 1023u) {
         if (tid == 0) record_timeout(901);
         return;
