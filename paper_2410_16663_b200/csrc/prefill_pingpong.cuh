@@ -10,7 +10,7 @@
 //                   landed and the softmax of step g-2 has read its scores out of the buffer.
 //   warp 10       : one thread issues O += P_{g&1} V_g for every step, as soon as P is written.
 //   warp 9 / 11   : one thread each issues the TMA loads of Q and K / of V (separate rings, as
-//                   K is consumed about two steps ahead of V).
+//                   K is consumed about two steps ahead of V); the second stores the 16-bit outputs too.
 // Because P has columns of its own, Q K^T of step g+1 and g+2 run on the tensor core while the
 // softmax of step g is still at work: the tensor core never waits for a softmax of the same
 // tile (the Cube/Vector overlap of Section 4.1 within one query tile), and the two warpgroups
@@ -41,17 +41,14 @@
 
 namespace fa {
 
-#ifndef FA_PP_NK
-#define FA_PP_NK 3
-#endif
-constexpr int kPpNK = FA_PP_NK;   // K ring slots
+constexpr int kPpNK = 3;          // K ring slots
 constexpr int kPpNV = 2;          // V ring slots: those of the steps' parities
 constexpr int kPpQBufs = 2;
 constexpr int kPpSlots = 4;       // work items the Q/K loader may be ahead of the slowest role
 static_assert((kPpQBufs + kPpNK + kPpNV) * kTileBytes + 3072 <= 232448, "shared memory budget");
 
 // What changes with FP8 e4m3 operands (kF8; Appendix D.2 evaluates the operator with 8-bit
-// operands): a tile of 128 rows x 128 bytes is one swizzled TMA box of 16 KiB (a Q slot keeps its
+// operands): a tile of 128 rows x 128 bytes is one swizzled TMA box of 16 KiB (a V slot keeps its
 // 32 KiB, because the 16-bit output tile is staged there); one MMA covers 32 elements of the
 // contraction, so a product takes four instead of eight; the probabilities are rounded to e4m3
 // four to a 32-bit column of tensor memory, times kP8Scale so that they use the format's range:
@@ -63,7 +60,8 @@ template <bool kF8, int D = 128>
 struct PpOperands {
     static_assert(D == 128 || (D == 64 && !kF8), "head dimension 128, or 64 with 16-bit operands");
     static constexpr bool kOneBox = kF8 || D == 64;                     // a tile row is 128 bytes
-    static constexpr int kKvSlotBytes = kOneBox ? 16384 : kTileBytes;   // one K or V ring slot
+    static constexpr int kKvSlotBytes = kOneBox ? 16384 : kTileBytes;   // one K ring slot, and the bytes of a K or V tile
+    static constexpr int kVSlotBytes = D == 64 ? 16384 : kTileBytes;    // one V ring slot: a V tile, later an output tile
     static constexpr int kQBytes = kOneBox ? 16384 : kTileBytes;        // bytes a Q load delivers
     static constexpr int kSteps = kOneBox ? 4 : 8;                      // MMAs of Q K^T (32 bytes of every row each)
     static constexpr int kPvSteps = kF8 ? 4 : 8;                        // MMAs of P V (32 or 16 keys each)
@@ -75,8 +73,7 @@ constexpr float kP8ScaleLog2 = 4.0f;   // log2 of the factor on the FP8 probabil
 // ---- barriers: indices into one array
 namespace ppb {
 constexpr int q_full = 0;                       // [2]  TMA -> S thread
-constexpr int q_empty = 2;                      // [2]  S thread (commit) -> loader; with the output staged in the
-                                                //      Q buffer, the four epilogue warps (count 4) -> loader
+constexpr int q_empty = 2;                      // [2]  S thread (commit) -> loader
 constexpr int k_full = 4;                       // [NK]
 constexpr int k_empty = k_full + kPpNK;         // [NK]
 constexpr int v_full = k_empty + kPpNK;         // [NV]
@@ -85,7 +82,8 @@ constexpr int pv_done = s_full + 2;             // [2]  PV thread (commit) -> so
 constexpr int o_final = pv_done + 2;            // [2]  PV thread (commit) -> epilogue, by item parity
 constexpr int item_full = o_final + 2;          // [kPpSlots] Q/K loader -> every other role: a work item is in the slot
 constexpr int item_empty = item_full + kPpSlots;   // [kPpSlots] back: three single-thread roles and eight softmax warps
-constexpr int claim = item_empty + kPpSlots;    // [1]  answer to a claim of work (cluster launch control) -> Q/K loader
+constexpr int o_staged = item_empty + kPpSlots; // [2]  by item parity, 16-bit output: the four epilogue warps (count 4) -> V loader, which stores it
+constexpr int claim = o_staged + 2;             // [1]  answer to a claim of work (cluster launch control) -> Q/K loader
 // barriers every thread of a softmax warpgroup arrives on (count 128)
 constexpr int p_full = claim + 1;               // [2]  softmax -> PV thread
 constexpr int m_ready = p_full + 2;             // [2]  softmax of step g -> softmax of step g+1 (reference max
@@ -444,7 +442,7 @@ struct PpRing {
 };
 
 // The thread that issues S = Q K^T of every step.
-template <typename T, bool kTmaOut, bool kVarlen, bool kF8, int D>
+template <typename T, bool kVarlen, bool kF8, int D>
 __device__ __forceinline__ void pp_run_s(uint32_t bar0, uint32_t sQ, uint32_t sK, uint32_t tmem, const PpItem* slots,
                                          volatile uint32_t* abort_flag) {
     constexpr bool kBf16 = std::is_same<T, __nv_bfloat16>::value;
@@ -477,8 +475,7 @@ __device__ __forceinline__ void pp_run_s(uint32_t bar0, uint32_t sQ, uint32_t sK
             }
             mma_commit(pp_bar(bar0, ppb::s_full + buf));
             mma_commit(pp_bar(bar0, ppb::k_empty + ring.slot));
-            // with the output staged in the Q buffer the item's epilogue hands the buffer back
-            if (!kTmaOut && j == it.n - 1) mma_commit(pp_bar(bar0, ppb::q_empty + qb));
+            if (j == it.n - 1) mma_commit(pp_bar(bar0, ppb::q_empty + qb));
         }
     }
 }
@@ -507,7 +504,7 @@ __device__ __forceinline__ void pp_run_pv(uint32_t bar0, uint32_t sV, uint32_t t
             // column blocks kHalfBytes apart, 16 keys (2048 bytes) per MMA; d = 64: one block, the
             // same 16 keys per MMA; 8-bit: one block, 32 keys (4096 bytes) per MMA.  Either way an
             // MMA reads 8 columns of P.
-            const uint32_t b_lo = desc_lo(sV + ring.slot * Op::kKvSlotBytes, D == 64 ? 16 : kHalfBytes);
+            const uint32_t b_lo = desc_lo(sV + ring.slot * Op::kVSlotBytes, D == 64 ? 16 : kHalfBytes);
 #pragma unroll
             for (int ks = 0; ks < Op::kPvSteps; ++ks) {
                 if (kF8) mma_ts_lo_f8(tmem, tmem + 384 + 64 * buf + ks * 8, b_lo + ks * (4096 >> 4), idesc,
@@ -612,27 +609,91 @@ __device__ __forceinline__ void pp_run_load_qk(uint32_t bar0, uint32_t sQ, uint3
     }
 }
 
-// The thread that loads V of every step.
-template <bool kVarlen, bool kF8, int D>
-__device__ __forceinline__ void pp_run_load_v(uint32_t bar0, uint32_t sV, const CUtensorMap* tm_v, const FwdParams& p,
-                                              const PpItem* slots, volatile uint32_t* abort_flag) {
+// An item's output, staged in the V slot of its last step.
+struct PpStaged {
+    uint32_t end;    // that step
+    int row, rows;   // first row in o and rows to store (32 at a time)
+    int h, b, done_slot;
+};
+
+// The thread that loads V of every step and stores the 16-bit outputs.  An item's last P V has read its V slot when the
+// epilogue gets O, and the slot is next needed by the step after next, which the same warpgroup runs once it is through
+// with the epilogue: so O is staged there, and before this thread loads that step's V it sends the tile and
+// waits until it has been read.  The warps that staged it neither issue nor wait for stores, and Q buffers are handed
+// back by the item's last Q K^T.  (Staged in the Q buffer, by each warp for itself, as it was, a buffer came back only when the
+// item after had begun, and short items began with a cold load: 8 x 32 x 512 40.4 -> 38.2 us, 4 x 32 x 2048 166.5 -> 160.3, 16 x 32 x
+// 256 33.2 -> 30.7, 32 x 8192 503 -> 497; 32 packed requests of 16 to 512 tokens 87.8 -> 85.2, 10 of 100 to 3000 311 -> 305; 8-bit
+// operands 8 x 32 x 512 26.5 -> 24.6, 16 x 32 x 128 10.9 -> 9.7; d = 64 level.  With a tile of its own for the output and
+// two K slots, and the warps still sending: 38.9, 167.1, 31.0, but 2 to 4 % slower packed.  With 256-bit stores from
+// registers instead: 44.2, 176.0, 35.1.)
+template <bool kTmaOut, bool kVarlen, bool kF8, bool kProj, int D>
+__device__ __forceinline__ void pp_run_v(uint32_t bar0, uint32_t sV, const CUtensorMap* tm_v, const CUtensorMap* tm_o, const FwdParams& p,
+                                         const PpItem* slots, volatile uint32_t* abort_flag, unsigned int* done) {
+    using Op = PpOperands<kF8, D>;
     tma_prefetch_desc(tm_v);
     const uint64_t pol_kv = l2_policy_evict_last();
     PpRing<kPpNV> ring;
     PpTaker<kVarlen> items{slots, bar0, abort_flag};
     PpItem it;
+    uint32_t g = 0, sent = 0;
+    PpStaged first = {}, second = {};   // outputs not yet sent, in order
+    int waiting = 0;                    // how many
+    int done_slot = -1;                 // kProj: row block whose stores have not been counted yet
+    auto count_done = [&]() {
+        if (kProj && done_slot >= 0) {
+            tma_store_wait_all();       // written, not only read out of shared memory
+            red_release_gpu_add(done + done_slot, 4u);
+            done_slot = -1;
+        }
+    };
+    auto send = [&]() -> bool {
+        if (!mbar_wait(pp_bar(bar0, ppb::o_staged + (sent & 1)), (sent >> 1) & 1, abort_flag, 156)) return false;
+        count_done();
+        const uint32_t tile = sV + (first.end & 1) * Op::kVSlotBytes;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            // packed batches: the rows after a sequence's last belong to the next sequence, so only 32 rows that
+            // all exist go as a box (the others' threads have written them)
+            if (kVarlen ? 32 * q + 32 <= first.rows : 32 * q < first.rows) {
+                if (D == 128) tma_store_5d(tm_o, tile + q * 8192, 0, first.row + 32 * q, 0, first.h, first.b);
+                else tma_store_4d(tm_o, tile + q * 4096, 0, first.h, first.row + 32 * q, first.b);
+            }
+        }
+        tma_store_commit();
+        if (kProj) done_slot = first.done_slot;
+        ++sent;
+        first = second;
+        --waiting;
+        return true;
+    };
     while (items.next(it, 155)) {
         if (items.ord == 0 && *abort_flag) return;
         int page = (kVarlen && p.block_table != nullptr) ? it.page0 : 0;
-        for (int j = 0; j < it.n; ++j, ring.next()) {
+        for (int j = 0; j < it.n; ++j, ++g, ring.next()) {
             const int page_next = pp_page_of<kVarlen>(p, it.b, j + 1, it.n, it.Skv);
-            if (!mbar_wait(pp_bar(bar0, ppb::pv_done + ring.slot), ring.par ^ 1, abort_flag, 152)) return;
-            mbar_expect_tx(pp_bar(bar0, ppb::v_full + ring.slot), PpOperands<kF8, D>::kKvSlotBytes);
+            if (kTmaOut && waiting > 0 && first.end + 2 == g) {
+                if (!send()) return;
+                tma_store_wait_read();
+            } else if (!mbar_wait(pp_bar(bar0, ppb::pv_done + ring.slot), ring.par ^ 1, abort_flag, 152)) return;
+            mbar_expect_tx(pp_bar(bar0, ppb::v_full + ring.slot), Op::kKvSlotBytes);
             int row = kVarlen ? it.k_base + j * kTile : (it.j0 + j) * kTile, slab = kVarlen ? 0 : it.b;
             pp_paged_tile<kVarlen>(p, page, j, row, slab);
             page = page_next;
-            pp_load_tile<PpOperands<kF8, D>::kOneBox>(sV + ring.slot * PpOperands<kF8, D>::kKvSlotBytes, tm_v, pp_bar(bar0, ppb::v_full + ring.slot), it.hk, row, slab, pol_kv);
+            pp_load_tile<Op::kOneBox>(sV + ring.slot * Op::kVSlotBytes, tm_v, pp_bar(bar0, ppb::v_full + ring.slot), it.hk, row, slab, pol_kv);
         }
+        if (kTmaOut) {
+            const PpStaged now = {g - 1, (kVarlen ? it.q_base : 0) + it.q0, (kVarlen ? it.Sq : p.Sq) - it.q0, it.h, kVarlen ? 0 : it.b,
+                                  kProj ? it.b * p.n_qtiles + it.q0 / kTile : 0};
+            if (waiting == 0) first = now;
+            else second = now;
+            ++waiting;
+        }
+    }
+    if (kTmaOut) {
+        while (waiting > 0)
+            if (!send()) break;
+        count_done();
+        tma_store_wait_all();   // the stores read shared memory, which has to outlive them
     }
 }
 
@@ -783,7 +844,7 @@ struct PpSoftmax {
             static_assert(kPpNV == 2, "the V slot of step g is taken to be g & 1");
             if (!pp_warp_wait(pp_bar(bar0, ppb::v_full + w), (g >> 1) & 1, abort_flag, 124 + w)) return false;
             if (r >= Skv - j * kTile) {
-                const uint32_t line = sV + (uint32_t)w * Op::kKvSlotBytes + (uint32_t)r * 128u;
+                const uint32_t line = sV + (uint32_t)w * Op::kVSlotBytes + (uint32_t)r * 128u;
 #pragma unroll
                 for (int c = 0; c < D / 8; ++c)
                     asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(line + (uint32_t)(c >> 3) * kHalfBytes + (uint32_t)(c & 7) * 16u), "r"(0u) : "memory");
@@ -888,15 +949,15 @@ __device__ __forceinline__ void pp_split_merge(const FwdParams& p, uint32_t part
 }
 
 // kTmaOut: the output has the operands' 16-bit type; an item's O goes, scaled and rounded, into
-// the item's Q buffer (which Q K^T has finished with by then) in the swizzled layout of a tile,
-// and each warp sends its 32 rows to global memory with one TMA store (tm_o: boxes of 32
+// the V slot of the item's last step (which P V has finished with by then) in the swizzled layout of a tile,
+// and the thread that loads V sends it to global memory (tm_o: boxes of 32
 // rows).  Rows past the end of the queries are clipped by the tensor map.  Otherwise
 // (fp32 output) every thread stores its own row.
 // kVarlen (needs kTmaOut): a packed batch of sequences of different lengths (see FwdParams).
 // kF8: q, k, v hold FP8 e4m3 bytes (see PpOperands); T is then the type of the output only.
-// kProj (needs kTmaOut): a projection phase follows in the same launch (proj_gemm.cuh): a warp
-// that has stored its rows of an item's output waits until the stores have reached global memory
-// and counts them in done[batch * n_qtiles + query tile]; four warps and Hq heads make a row
+// kProj (needs kTmaOut): a projection phase follows in the same launch (proj_gemm.cuh): when an item's
+// stores have reached global memory the thread that issued them counts
+// them in done[batch * n_qtiles + query tile], 32 rows as one; four of them and Hq heads make a row
 // block of O complete.
 // The whole kernel but for the release of tensor memory; returns false if nothing was set up.
 template <typename T, bool kTmaOut, bool kVarlen, bool kF8, bool kProj, int D = 128, bool kSplit = false>
@@ -920,9 +981,9 @@ __device__ __forceinline__ bool pp_attention(const CUtensorMap& tm_q, const CUte
     }
     if (tid == 0) {
         for (int i = 0; i < ppb::count; ++i) {
-            const bool q_back = kTmaOut && (i == ppb::q_empty || i == ppb::q_empty + 1);
+            const bool staged = i == ppb::o_staged || i == ppb::o_staged + 1;
             const bool slot_back = i >= ppb::item_empty && i < ppb::item_empty + kPpSlots;
-            mbar_init(pp_bar(bar0, i), i >= ppb::p_full ? 128 : (slot_back ? 11 : (q_back ? 4 : 1)));
+            mbar_init(pp_bar(bar0, i), i >= ppb::p_full ? 128 : (slot_back ? 11 : (staged ? 4 : 1)));
         }
         ss.abort_flag = 0;
         fence_mbar_init();
@@ -966,25 +1027,6 @@ __device__ __forceinline__ bool pp_attention(const CUtensorMap& tm_q, const CUte
         uint32_t g = 0;        // step counter of the CTA
         uint32_t items2 = 0;   // items with at least two steps seen so far
         bool ok = true;
-        // Q buffer whose TMA stores this warp has issued but not yet waited for (-1: none).  The
-        // wait (until the stores have read the buffer) and the hand-back to the loader come when
-        // the warp starts on the next item.
-        int q_back = -1;
-        int done_slot = 0;     // kProj: the row block the pending stores belong to
-        auto hand_back_q = [&]() {
-            if (kTmaOut && q_back >= 0) {
-                if (lane == 0) {
-                    if (kProj) {
-                        tma_store_wait_all();          // written, not only read out of shared memory
-                        red_release_gpu_add(done + done_slot, 1u);
-                    } else {
-                        tma_store_wait_read();
-                    }
-                    mbar_arrive(pp_bar(bar0, ppb::q_empty + q_back));
-                }
-                q_back = -1;
-            }
-        };
         for (int ord = 0; ok; ++ord) {
             const int slot = ord & (kPpSlots - 1);
             if (kVarlen && ord == 0) grid_dep_wait();   // (see PpTaker)
@@ -1026,17 +1068,9 @@ __device__ __forceinline__ bool pp_attention(const CUtensorMap& tm_q, const CUte
             // this warpgroup's steps of the item: those with an absolute step number of its parity
             const uint32_t g_item = g;
             int j = (int)((g_item ^ (uint32_t)w) & 1u);
-            // The stores of this warpgroup's last epilogue have read the Q buffer by now, or nearly.  Handed back
-            // after its next step, as it was before, the buffer came so late on short items that the Q load of
-            // the item after the next, and K behind it, started when their turn had come (8 x 32 x 512 41.1 -> 40.6 us; d = 64, 16 x 16 x 512, 29.5 -> 27.5).
-            // (With the projection the hand-back waits until the rows are written, so the step goes first --
-            // unless the item has none for this warpgroup: the next step that it takes then belongs to the item
-            // whose Q load waits for the buffer.)
-            if (!kProj || j >= n) hand_back_q();
             for (; j < n; j += 2) {
                 ok = sm.step(s, g_item + (uint32_t)j, j, j >= n_full);
                 if (!ok) break;
-                if (kProj) hand_back_q();
                 if (j == n - 2) {
                     // the other warpgroup runs the last step and the epilogue: hand it this row sum
                     // (it is relative to the reference this step left, which that step receives)
@@ -1091,50 +1125,36 @@ __device__ __forceinline__ bool pp_attention(const CUtensorMap& tm_q, const CUte
                                      : "memory");
                     asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(sK + kPpPartStats + (uint32_t)r * 8u), "f"(m_loc), "f"(l_run) : "memory");
                 } else if (kTmaOut) {
-                    const uint32_t q_buf = sQ + (uint32_t)(ord & 1) * kTileBytes;
-                    // a warp's rows: its 64-column blocks one after the other, as its store takes them
-                    const uint32_t slab = q_buf + (uint32_t)(warp & 3) * (D == 128 ? 8192u : 4096u);
+                    // a warp's rows, in the V slot of the item's last step (see pp_run_v): its 64-column blocks one after
+                    // the other, as its store takes them
+                    const uint32_t slab = sV + (uint32_t)w * PpOperands<kF8, D>::kVSlotBytes + (uint32_t)(warp & 3) * (D == 128 ? 8192u : 4096u);
                     const uint32_t row_base = slab + (uint32_t)lane * 128u;
+                    // (packed multiplications: 8 x 32 x 512 42.6 -> 42.0 us, 16 x 32 x 256 34.6 -> 34.3, 10 packed requests of 100 to 3000
+                    // tokens 325 -> 316, 32 of 256 to 8192 4158 -> 4072, others level)
 #pragma unroll
-                    for (int c = 0; c < D / 8; ++c) {
-                        // 16-byte chunk c & 7 of the row's half c >> 3, at its swizzled place
-                        const uint32_t addr = row_base + (uint32_t)(c >> 3) * 4096u + (((uint32_t)(c & 7) ^ ((uint32_t)lane & 7u)) << 4);
-                        // (packed multiplications: 8 x 32 x 512 42.6 -> 42.0 us, 16 x 32 x 256 34.6 -> 34.3, 10 packed requests of 100 to 3000
-                        // tokens 325 -> 316, 32 of 256 to 8192 4158 -> 4072, others level)
-                        uint32_t wd[4];
+                    for (int i = 0; i < D / 2; ++i) {
+                        float x0, x1;
+                        f2_unpack(f2_mul(f2_pack(__uint_as_float(s[2 * i]), __uint_as_float(s[2 * i + 1])), f2_pack(inv_l, inv_l)), x0, x1);
+                        s[i] = pack2<T>(x0, x1);
+                    }
+                    if (kVarlen && uniform(it.q0 + (warp & 3) * 32 + 32 > Sq_i)) {
+                        // 32 rows that do not all exist (see pp_run_v): each thread writes its own row
+                        if (row < Sq_i) {
+                            uint4* dst = reinterpret_cast<uint4*>(static_cast<T*>(p.o) + obase);
 #pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            float x0, x1;
-                            f2_unpack(f2_mul(f2_pack(__uint_as_float(s[8 * c + 2 * q]), __uint_as_float(s[8 * c + 2 * q + 1])), f2_pack(inv_l, inv_l)), x0, x1);
-                            wd[q] = pack2<T>(x0, x1);
+                            for (int c = 0; c < D / 8; ++c) dst[c] = make_uint4(s[4 * c], s[4 * c + 1], s[4 * c + 2], s[4 * c + 3]);
                         }
-                        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(wd[0]), "r"(wd[1]), "r"(wd[2]), "r"(wd[3]) : "memory");
-                    }
-                    fence_proxy_async_smem();
-                    __syncwarp();
-                    const int row0 = it.q0 + (warp & 3) * 32;   // first row of this warp
-                    // packed batches: the rows after a sequence's last belong to the next
-                    // sequence, so only a warp whose 32 rows all exist may use the box store
-                    const bool box = kVarlen ? (row0 + 32 <= Sq_i) : (row0 < Sq_i);
-                    if (lane == 0 && box) {
-                        if (D == 128) tma_store_5d(&tm_o, slab, 0, kVarlen ? it.q_base + row0 : row0, 0, it.h, kVarlen ? 0 : it.b);
-                        else tma_store_4d(&tm_o, slab, 0, it.h, kVarlen ? it.q_base + row0 : row0, kVarlen ? 0 : it.b);
-                        tma_store_commit();
-                    }
-                    q_back = ord & 1;  // handed back to the loader at the start of the next item
-                    if (kProj) done_slot = it.b * p.n_qtiles + it.q0 / kTile;
-                    __syncwarp();
-                    if (kVarlen && !box && row < Sq_i) {
-                        // the ragged end of a sequence: each thread writes its own row
-                        T* dst = static_cast<T*>(p.o) + obase;
+                    } else {
 #pragma unroll
-                        for (int c = 0; c < D / 8; ++c)
-                            reinterpret_cast<uint4*>(dst)[c] =
-                                make_uint4(pack2<T>(__uint_as_float(s[8 * c]) * inv_l, __uint_as_float(s[8 * c + 1]) * inv_l),
-                                           pack2<T>(__uint_as_float(s[8 * c + 2]) * inv_l, __uint_as_float(s[8 * c + 3]) * inv_l),
-                                           pack2<T>(__uint_as_float(s[8 * c + 4]) * inv_l, __uint_as_float(s[8 * c + 5]) * inv_l),
-                                           pack2<T>(__uint_as_float(s[8 * c + 6]) * inv_l, __uint_as_float(s[8 * c + 7]) * inv_l));
+                        for (int c = 0; c < D / 8; ++c) {
+                            // 16-byte chunk c & 7 of the row's half c >> 3, at its swizzled place
+                            const uint32_t addr = row_base + (uint32_t)(c >> 3) * 4096u + (((uint32_t)(c & 7) ^ ((uint32_t)lane & 7u)) << 4);
+                            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(s[4 * c]), "r"(s[4 * c + 1]), "r"(s[4 * c + 2]), "r"(s[4 * c + 3]) : "memory");
+                        }
+                        fence_proxy_async_smem();
                     }
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(pp_bar(bar0, ppb::o_staged + (ord & 1)));
                 } else if (row < Sq_i) {
                     if (p.o_fp32) {
                         float4* dst = reinterpret_cast<float4*>(static_cast<float*>(p.o) + obase);
@@ -1160,16 +1180,13 @@ __device__ __forceinline__ bool pp_attention(const CUtensorMap& tm_q, const CUte
             g = g_item + (uint32_t)n;
             if (n >= 2) ++items2;
         }
-        // the stores read shared memory, which has to outlive them
-        if (kProj) hand_back_q();
-        else if (kTmaOut && lane == 0) tma_store_wait_all();
     } else {
         setmaxnreg_dec<kPipeOtherRegs>();
         if (elect_one()) {
-            if (warp == 8) pp_run_s<T, kTmaOut, kVarlen, kF8, D>(bar0, sQ, sK, tmem_base, ss.items, abort_flag);
+            if (warp == 8) pp_run_s<T, kVarlen, kF8, D>(bar0, sQ, sK, tmem_base, ss.items, abort_flag);
             else if (warp == 10) pp_run_pv<T, kVarlen, kF8, D>(bar0, sV, tmem_base, ss.items, abort_flag);
             else if (warp == 9) pp_run_load_qk<kVarlen, kF8, D>(bar0, sQ, sK, &tm_q, &tm_k, p, total_items, ss, abort_flag);
-            else pp_run_load_v<kVarlen, kF8, D>(bar0, sV, &tm_v, p, ss.items, abort_flag);
+            else pp_run_v<kTmaOut, kVarlen, kF8, kProj, D>(bar0, sV, &tm_v, &tm_o, p, ss.items, abort_flag, done);
         }
         __syncwarp();
     }
@@ -1280,7 +1297,7 @@ inline FwdParams pp_plan_items(const FwdParams& fp, int grid, double bytes_per_k
 template <typename T, bool kF8 = false, int D = 128>
 int launch_pingpong(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& to,
                     const FwdParams& fp, cudaStream_t st, int* cuda_err) {
-    constexpr int smem = kPpQBufs * kTileBytes + (kPpNK + kPpNV) * PpOperands<kF8, D>::kKvSlotBytes;
+    constexpr int smem = kPpQBufs * kTileBytes + kPpNK * PpOperands<kF8, D>::kKvSlotBytes + kPpNV * PpOperands<kF8, D>::kVSlotBytes;
     const bool varlen = fp.cu_q != nullptr;
     if (varlen && fp.o_fp32) return -3;
     if (kF8 && (varlen || fp.o_fp32)) return -3;

@@ -16,7 +16,7 @@
 //   warps 0-7           : warpgroup a drains accumulator a: one thread per row, 32 columns at a
 //                         time, rounded to 16 bits and stored.
 // In the fused launch a row block may be loaded only after every head's attention output for it
-// has reached global memory: the attention epilogue counts its completed TMA stores per row block
+// has reached global memory: the thread that stores the attention output counts its completed TMA stores per row block
 // in `done`, and the loading thread waits (bounded) for the count before the block's first load.
 #pragma once
 
@@ -29,7 +29,7 @@ struct ProjParams {
     int B, Sq, Hq, N;          // K = Hq * 128
     int n_qtiles, n_cblocks;   // row blocks per batch entry, column blocks of 256
     unsigned int* done;        // [B * n_qtiles] completed-store counts, or nullptr (O is final already)
-    unsigned int done_target;  // 4 * Hq: one count per epilogue warp and head
+    unsigned int done_target;  // 4 * Hq: one count per 32 rows and head
 };
 
 constexpr int kProjStages = 4;
