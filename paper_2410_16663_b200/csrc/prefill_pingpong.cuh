@@ -722,7 +722,6 @@ struct PpSoftmax {
     int causal, Skv, off;
     int kv_first;           // first key of the item's first kv tile (0 unless CTAs share a query tile)
     uint32_t sV;            // V ring in shared memory (packed batches: see the end of step())
-    int r;                  // this thread's row of the tile
     // per item
     int row;                // query row of this thread
     int lim0;               // packed batches: keys of the sequence that it sees
@@ -839,15 +838,17 @@ struct PpSoftmax {
             // belong to the next sequence, or to the unused rest of a page, and may hold anything.
             // Their probabilities are exact zeros, but 0 * NaN would still poison O, so those
             // rows are cleared in shared memory before P V of this step may start (a contiguous
-            // tensor gets the same from the zero fill of its TMA loads).  Thread r owns key row r:
-            // its bytes are one 128-byte line in each 64-element half of the tile, whatever the swizzle.
+            // tensor gets the same from the zero fill of its TMA loads).  A row's bytes are one 128-byte line in each
+            // 64-element half of the tile, whatever the swizzle; eight threads clear a line.  (A thread per row hits the
+            // same banks with all lanes: 32 requests of 16 to 512 tokens, GQA, 85.2 -> 82.5 us, 20 chunks of up to 666 57.1 ->
+            // 55.1, 6 of up to 2000 21.9 -> 21.1, long requests level.)
             static_assert(kPpNV == 2, "the V slot of step g is taken to be g & 1");
             if (!pp_warp_wait(pp_bar(bar0, ppb::v_full + w), (g >> 1) & 1, abort_flag, 124 + w)) return false;
-            if (r >= Skv - j * kTile) {
-                const uint32_t line = sV + (uint32_t)w * Op::kVSlotBytes + (uint32_t)r * 128u;
+            const int dead = max(0, Skv - j * kTile);
+            for (int r0 = dead + (int)((threadIdx.x & 127) >> 3); r0 < kTile; r0 += 16) {
+                const uint32_t at = sV + (uint32_t)w * Op::kVSlotBytes + (uint32_t)r0 * 128u + (threadIdx.x & 7) * 16u;
 #pragma unroll
-                for (int c = 0; c < D / 8; ++c)
-                    asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(line + (uint32_t)(c >> 3) * kHalfBytes + (uint32_t)(c & 7) * 16u), "r"(0u) : "memory");
+                for (int h = 0; h < D / 64; ++h) asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(at + (uint32_t)h * kHalfBytes), "r"(0u) : "memory");
             }
             fence_proxy_async_smem();
         }
@@ -1010,7 +1011,6 @@ __device__ __forceinline__ bool pp_attention(const CUtensorMap& tm_q, const CUte
         const float scale_log2 = p.scale_log2;
         PpSoftmax<T, kVarlen, kF8, D> sm;
         sm.sV = sV;
-        sm.r = r;
         sm.bar0 = bar0;
         sm.abort_flag = abort_flag;
         sm.m_mine = &ss.m_xch[w][r];
