@@ -775,21 +775,44 @@ fa_decode_combine_kernel(const DecodeParams p, T* o, float* lse) {
     const int nc = (len + p.chunk - 1) / p.chunk;
     const float* lp = p.lse_part + (long long)bh * p.n_chunks;
     const float* op = p.o_part + (long long)bh * p.n_chunks * D;
-    float M = -INFINITY;
-    for (int c = 0; c < nc; ++c) M = fmaxf(M, lp[c]);
-    bool none = M == -INFINITY;   // no keys, or (several query rows) a token that sees none ...
-    if (none)                     // ... unless there is a NaN, which the max skips
-        for (int c = 0; c < nc; ++c) none = none && lp[c] == -INFINITY;
-    if (none) {
+    // One pass, some chunks at a time, whose loads are all on their way together; the weights are relative to the
+    // largest log-sum-exp so far.  (A pass for the maximum and one for the sums, a chunk at a time, waits for L2 twice
+    // per chunk: 4 sequences of up to 11139 keys, 2 tokens, 32/8 heads, 17.8 -> 17.3 us, 2 of up to 23723, 64/8 heads, 32.9 -> 32.2, 12 of up
+    // to 5861, 5 heads, 27.5 -> 27.0.  Two at a time where there are no more: with eight 64 of up to 3371, 4 tokens, 89.5 -> 90.7.)
+    float M = -INFINITY, wsum = 0.f, acc = 0.f;
+    auto merge = [&](auto chunks) {
+        constexpr int kN = decltype(chunks)::value;
+        for (int c0 = 0; c0 < nc; c0 += kN) {
+            float l[kN], v[kN], m = M;
+#pragma unroll
+            for (int i = 0; i < kN; ++i) {
+                const bool live = c0 + i < nc;
+                l[i] = live ? lp[c0 + i] : -INFINITY;
+                v[i] = live ? op[(long long)(c0 + i) * D + tid] : 0.f;
+            }
+#pragma unroll
+            for (int i = 0; i < kN; ++i) m = fmaxf(m, l[i]);
+            const float ref = m == -INFINITY ? 0.f : m;
+            const float keep = __expf(M - ref);
+            wsum *= keep;
+            acc *= keep;
+            M = m;
+#pragma unroll
+            for (int i = 0; i < kN; ++i) {
+                if (l[i] != -INFINITY) {   // (a chunk that the token sees nothing of; a NaN gets through)
+                    const float w = __expf(l[i] - ref);
+                    wsum += w;
+                    acc = fmaf(w, v[i], acc);
+                }
+            }
+        }
+    };
+    if (p.n_chunks <= 2) merge(std::integral_constant<int, 2>());
+    else merge(std::integral_constant<int, 8>());
+    if (wsum == 0.f) {   // no keys, or (several query rows) a token that sees none
         o[(long long)bh * D + tid] = T(0.f);
         if (lse && tid == 0) lse[lse_at] = -INFINITY;
         return;
-    }
-    float wsum = 0.f, acc = 0.f;
-    for (int c = 0; c < nc; ++c) {
-        const float w = __expf(lp[c] - M);
-        wsum += w;
-        acc = fmaf(w, op[(long long)c * D + tid], acc);
     }
     o[(long long)bh * D + tid] = T(acc / wsum);
     if (lse && tid == 0) lse[lse_at] = M + logf(wsum);
