@@ -66,6 +66,9 @@ struct DecodeParams {
     // long as without it, so it stays far inside fp32.
     int ref_tiles = 1 << 30;
     float ref_drop = 0.f;   // kDecRefDropLog2 / scale_log2
+    // Chunks cut by the sequences' own lengths (kDecBalanced, see DecBalance): CTAs per kv head over all
+    // sequences, and the tiles per chunk that are enough whatever the lengths are
+    int slots = 0, most_tiles = 0;
     int bf16_io = 0;      // 8-bit cache kernel only: q and o are bf16 (fp16 otherwise)
 };
 
@@ -126,6 +129,50 @@ struct DecTileLayout {
     __device__ __forceinline__ uint32_t key(int key) const {
         const uint32_t box = (uint32_t)key >> rows_log2;
         return (D / 64 - 1) * box * block + (uint32_t)key * 128u;
+    }
+};
+
+// How a call's sequences are cut: every DecodeParams::chunk keys (kDecPlain), the chunks of a sequence the CTAs of a cluster
+// (kDecCluster), or by the lengths that the device finds (kDecBalanced).
+constexpr int kDecPlain = 0, kDecCluster = 1, kDecBalanced = 2;
+constexpr int kDecBalancedSeqs = 32;
+
+// Chunks of equal length for sequences of different lengths, as short as p.slots CTAs per kv head allow, which the
+// device runs at once: worked out from the lengths by every warp for itself, a sequence per lane.  The sequences take the
+// CTAs one after the other, each at least one (it may have no keys).  (The loops are not unrolled: this runs once per CTA, and
+// fetching its instructions takes longer than executing them.)
+struct DecBalance {
+    int unit;                // tiles per chunk
+    int len, count, first;   // of sequence `lane`
+    // n / u, rounded up: exact for n below 2^15 at u up to 32 (the half keeps the quotient away from the whole numbers)
+    static __device__ __forceinline__ int parts(float n, int u) { return (int)((n - 0.5f) * __frcp_rn((float)u)) + 1; }
+    __device__ __forceinline__ DecBalance(const DecodeParams& p, int lane) {
+        const bool mine = lane < p.B;
+        len = mine ? max(0, min(p.seqlens[lane], p.Smax)) : 0;
+        const int t = max(1, (len + kDecTile - 1) / kDecTile);
+        int lo = max(1, (__reduce_add_sync(0xffffffffu, mine ? t : 0) + p.slots - 1) / p.slots), hi = max(lo, p.most_tiles);
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if (__reduce_add_sync(0xffffffffu, mine ? parts((float)t, mid) : 0) <= p.slots) hi = mid;
+            else lo = mid + 1;
+        }
+        unit = lo;
+        count = mine ? parts((float)t, unit) : 0;
+        int sum = count;
+#pragma unroll 1
+        for (int sh = 1; sh < p.B; sh <<= 1) {
+            const int low = __shfl_up_sync(0xffffffffu, sum, sh);
+            if (lane >= sh) sum += low;
+        }
+        first = sum - count;
+    }
+    // The sequence of CTA `at`, its chunk and length; false past the last chunk.
+    __device__ __forceinline__ bool find(int at, int& b, int& c, int& length) const {
+        b = __ffs(__ballot_sync(0xffffffffu, at >= first && at < first + count)) - 1;
+        if (b < 0) return false;
+        c = at - __shfl_sync(0xffffffffu, first, b);
+        length = __shfl_sync(0xffffffffu, len, b);
+        return true;
     }
 };
 
@@ -234,7 +281,7 @@ __device__ __forceinline__ void dec_store4(void* o, long long at, const float4& 
 // 2 t4, 2 t4 + 1 must not see (they came after the row's token).
 // Leaves each warp's (max, sum, O) in mo / ml in the layout the merge expects; returns false
 // after a wait that gave up.
-template <bool kMulti, typename T, int D, bool kCluster>
+template <bool kMulti, typename T, int D, bool kLower>
 __device__ __forceinline__ bool dec_consume_key_rows(const DecodeParams& p, uint64_t* bars, volatile uint32_t* abort_flag,
                                                      uint32_t sK, uint32_t sV, float* mo, float* ml, int warp, int lane,
                                                      const T* q_col, int hide0, int hide1, int len, int k_begin, int k_end,
@@ -266,7 +313,7 @@ __device__ __forceinline__ bool dec_consume_key_rows(const DecodeParams& p, uint
         const int st = t % kStages;
         const uint32_t parity = (t / kStages) & 1;
         const int valid = min(kDecTile, k_end - (k_begin + t * kDecTile)) - key_w;  // valid keys of this warp's 32
-        const float drop = kCluster && (t & (p.ref_tiles - 1)) == 0 ? p.ref_drop : 0.f;   // see DecodeParams
+        const float drop = kLower && (t & (p.ref_tiles - 1)) == 0 ? p.ref_drop : 0.f;   // see DecodeParams
         ok = mbar_wait(smem_u32(&bars[st]), parity, abort_flag, 20);
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
@@ -406,7 +453,7 @@ __device__ __forceinline__ bool dec_consume_key_rows(const DecodeParams& p, uint
 // several tokens were appended, Appendix C with more than one new token): the 16 MMA rows of a
 // CTA are then (token, head) pairs of one kv head, and query token t sees the keys up to
 // position len - Sq + t.  q is [B,Sq,Hq,d], the partials [B,Sq,Hq,NC,...].
-// grid: (Hkv * ceil(Sq * g / 16), n_chunks, B) with g = Hq / Hkv.  The kv head is the fastest
+// grid: (Hkv * ceil(Sq * g / 16), n_chunks, B), or (.., slots, 1) with kDecBalanced, with g = Hq / Hkv.  The kv head is the fastest
 // index: CTAs that run at the same time then read the same keys' rows of neighbouring heads,
 // which are contiguous in the cache (a key's Hkv * D elements), instead of key ranges whole
 // chunks apart (64 sequences of 1K to 32K keys, 32 kv heads: 2.39 against 2.48 ms).
@@ -414,14 +461,14 @@ __device__ __forceinline__ bool dec_consume_key_rows(const DecodeParams& p, uint
 // D: the head dimension, 128 or 64.
 // kKeyRows (at most 8 (token, head) rows per kv head): the consumers work in the keys-as-rows
 // form (dec_consume_key_rows).
-// kCluster: the chunks of a sequence are a cluster's CTAs (p.clustered).  (An instantiation of its own, as lowering
+// kMode: how the sequences are cut (kDecPlain and the others).  (The clustered form is an instantiation of its own, as lowering
 // the reference costs every tile two instructions and the merge below registers: 200 sequences of up to 600 keys,
 // not clustered, 10.14 us in one instantiation for both, 10.33 with the reference, 9.98 apart.)
 // (The kernels here do not release the next one early: its CTAs would take the places of this one's, or those
 // next to it, and wait there.  16 sequences of up to 4096 keys, d = 64, 22.3 us with an early release, 20.5
 // without; one of 32768 keys, 24.9 / 23.2; 8 of up to 8000, 30.5 / 29.6; 5 heads x 8192, 7.03 / 6.85; calls
 // of 6 us level.)
-template <bool kMulti, typename T, int D, bool kKeyRows, bool kCluster>
+template <bool kMulti, typename T, int D, bool kKeyRows, int kMode>
 __global__ void __launch_bounds__(kDecMmaThreads, DecShape<D>::kCtasPerSm)
 fa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                            const DecodeParams p) {
@@ -435,8 +482,7 @@ fa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
 
     const int tid = threadIdx.x;
     const int warp = uniform(tid >> 5), lane = tid & 31;
-    const int c = blockIdx.y;
-    const int b = blockIdx.z;
+    int c = blockIdx.y, b = blockIdx.z;   // (kDecBalanced: found below)
     const int g_all = p.Hq / p.Hkv;
     const int Sq = kMulti ? p.Sq : 1;
     const int rows_all = g_all * Sq;               // (token, head) rows that share a kv head
@@ -461,16 +507,28 @@ fa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
         tma_prefetch_desc(&tm_v);
     }
     grid_dep_wait();
-    int len = p.seqlens[b];
-    len = max(0, min(len, p.Smax));
-    const int k_begin = c * p.chunk;
-    const int k_end = min(len, k_begin + p.chunk);
+    int len, chunk = p.chunk;
+    if constexpr (kMode == kDecBalanced) {
+        const DecBalance bal(p, lane);
+        if (!bal.find(blockIdx.y, b, c, len)) return;   // (the same for all warps)
+        chunk = bal.unit * kDecTile;
+    } else {
+        len = max(0, min(p.seqlens[b], p.Smax));
+    }
+    const int k_begin = c * chunk;
+    const int k_end = min(len, k_begin + chunk);
+    // row r's place among the partial results
+    auto part_index = [&](int r) -> long long {
+        return kMode == kDecBalanced ? row_index(r) + ((long long)blockIdx.y - b) * Sq * p.Hq : row_index(r) * p.n_chunks + c;
+    };
     auto lse_index = [&](int r) -> long long {   // lse is [B,Hq,Sq]
         const int R = sub * 16 + r;
         return ((long long)b * p.Hq + hk * g_all + (kMulti ? R % g_all : R)) * Sq + row_token(r);
     };
     if (k_begin >= k_end) {  // uniform for the CTA
-        if (p.o_final != nullptr && c == 0 && tid < D) {   // a sequence without keys, and nobody else writes its rows
+        if (kMode == kDecBalanced) {
+            if (tid < G) p.lse_part[part_index(tid)] = -INFINITY;
+        } else if (p.o_final != nullptr && c == 0 && tid < D) {   // a sequence without keys, and nobody else writes its rows
             for (int r = 0; r < G; ++r) {
                 static_cast<T*>(p.o_final)[row_index(r) * D + tid] = T(0.f);
                 if (tid == 0 && p.lse_final) p.lse_final[lse_index(r)] = -INFINITY;
@@ -553,7 +611,7 @@ fa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
             const T* q_col = (g < G) ? static_cast<const T*>(p.q) + row_index(g) * D : nullptr;
             const int hide0 = kMulti ? Sq - 1 - row_token(min(2 * t4, G - 1)) : 0;
             const int hide1 = kMulti ? Sq - 1 - row_token(min(2 * t4 + 1, G - 1)) : 0;
-            ok = dec_consume_key_rows<kMulti, T, D, kCluster>(p, bars, &abort_flag, sK, sV, mo, ml, warp, lane, q_col, hide0, hide1,
+            ok = dec_consume_key_rows<kMulti, T, D, kMode != kDecPlain>(p, bars, &abort_flag, sK, sV, mo, ml, warp, lane, q_col, hide0, hide1,
                                                     len, k_begin, k_end, n_tiles);
         } else {
         // Q as A fragments for the D / 16 k-steps (rows >= G are zero)
@@ -584,7 +642,7 @@ fa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
             const int st = t % kStages;
             const uint32_t parity = (t / kStages) & 1;
             const int valid = min(kDecTile, k_end - (k_begin + t * kDecTile)) - key_w;  // valid keys of this warp's 32
-            const float drop = kCluster && (t & (p.ref_tiles - 1)) == 0 ? p.ref_drop : 0.f;   // see DecodeParams
+            const float drop = kMode != kDecPlain && (t & (p.ref_tiles - 1)) == 0 ? p.ref_drop : 0.f;   // see DecodeParams
             ok = mbar_wait(smem_u32(&bars[st]), parity, &abort_flag, 20);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
@@ -735,21 +793,21 @@ fa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
             for (int r = tid / (D / 4); r < G; r += 512 / D) {
                 float lse;
                 const float4 out = dec_warp_merge<D>(mo, ml, r, col, p.scale_log2, 1.f, lse);
-                if (kCluster) {
+                if (kMode == kDecCluster) {
                     *reinterpret_cast<float4*>(&part[r * D + col]) = out;
                     if (col == 0) part_lse[r] = lse;
                 } else if (p.o_final != nullptr) {   // the only chunk: this is the result
                     dec_store4<T>(p.o_final, row_index(r) * D + col, out);
                     if (col == 0 && p.lse_final) p.lse_final[lse_index(r)] = lse;
                 } else {
-                    const long long slot = row_index(r) * p.n_chunks + c;
+                    const long long slot = part_index(r);
                     *reinterpret_cast<float4*>(&p.o_part[slot * D + col]) = out;
                     if (col == 0) p.lse_part[slot] = lse;
                 }
             }
         }
     }
-    if constexpr (kCluster) {
+    if constexpr (kMode == kDecCluster) {
         const int n_live = (len + p.chunk - 1) / p.chunk;
         dec_cluster_merge<D>(part, part_lse, G, c, n_live, tid, [&](int r, int col, const float4& out, float lse) {
             dec_store4<T>(p.o_final, row_index(r) * D + col, out);
@@ -761,7 +819,7 @@ fa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
 // Merge of the per-chunk partials (rowmax/rowsum recurrence applied across chunks):
 //   M = max_c LSE_c, w_c = exp(LSE_c - M), O = sum_c w_c O_c / sum_c w_c, LSE = M + ln sum_c w_c.
 // grid: B * Sq * Hq blocks of D threads (row = (b, token, head)), thread t owns output dim t.
-template <typename T, int D = 128>
+template <typename T, int D = 128, bool kBalanced = false>
 __global__ void __launch_bounds__(128)
 fa_decode_combine_kernel(const DecodeParams p, T* o, float* lse) {
     const int bh = blockIdx.x;
@@ -769,12 +827,23 @@ fa_decode_combine_kernel(const DecodeParams p, T* o, float* lse) {
     // lse is [B,Hq,Sq]
     const long long lse_at = ((long long)b * p.Hq + bh % p.Hq) * p.Sq + (bh / p.Hq) % p.Sq;
     const int tid = threadIdx.x;
+    // The lengths may be read before the wait: this kernel starts when every CTA of the split kernel has ended, and those have
+    // waited for whoever wrote the lengths.  (Without a split kernel, as there are no keys, Smax is 0.)
+    int nc;
+    long long at = (long long)bh * p.n_chunks, step = 1;   // this row's first partial result, and how far the next one is
+    if constexpr (kBalanced) {
+        const DecBalance bal(p, tid & 31);
+        const int first = __shfl_sync(0xffffffffu, bal.first, b);
+        nc = __shfl_sync(0xffffffffu, bal.count, b);
+        step = (long long)p.Sq * p.Hq;
+        at = bh + (first - b) * step;
+    } else {
+        const int len = max(0, min(p.seqlens[b], p.Smax));
+        nc = (len + p.chunk - 1) / p.chunk;
+    }
     grid_dep_wait();   // the split kernel's partial results are complete and visible from here on
-    int len = p.seqlens[b];
-    len = max(0, min(len, p.Smax));
-    const int nc = (len + p.chunk - 1) / p.chunk;
-    const float* lp = p.lse_part + (long long)bh * p.n_chunks;
-    const float* op = p.o_part + (long long)bh * p.n_chunks * D;
+    const float* lp = p.lse_part + at;
+    const float* op = p.o_part + at * D;
     // One pass, some chunks at a time, whose loads are all on their way together; the weights are relative to the
     // largest log-sum-exp so far.  (A pass for the maximum and one for the sums, a chunk at a time, waits for L2 twice
     // per chunk: 4 sequences of up to 11139 keys, 2 tokens, 32/8 heads, 17.8 -> 17.3 us, 2 of up to 23723, 64/8 heads, 32.9 -> 32.2, 12 of up
@@ -787,8 +856,8 @@ fa_decode_combine_kernel(const DecodeParams p, T* o, float* lse) {
 #pragma unroll
             for (int i = 0; i < kN; ++i) {
                 const bool live = c0 + i < nc;
-                l[i] = live ? lp[c0 + i] : -INFINITY;
-                v[i] = live ? op[(long long)(c0 + i) * D + tid] : 0.f;
+                l[i] = live ? lp[(c0 + i) * step] : -INFINITY;
+                v[i] = live ? op[(c0 + i) * step * D + tid] : 0.f;
             }
 #pragma unroll
             for (int i = 0; i < kN; ++i) m = fmaxf(m, l[i]);

@@ -37,8 +37,9 @@ __device__ __forceinline__ uint32_t bf16x2_to_f16x2(uint32_t v) {
     return *reinterpret_cast<const uint32_t*>(&h);
 }
 
-// grid: (Hkv * ceil(g / 16), n_chunks, B) with g = Hq / Hkv (the kv head fastest, see decode.cuh)
-template <int NB, bool kCluster>
+// grid: (Hkv * ceil(g / 16), n_chunks, B), or (.., slots, 1) with kDecBalanced, with g = Hq / Hkv (the kv head fastest, see
+// decode.cuh)
+template <int NB, int kMode>
 __global__ void __launch_bounds__(kDec8Threads, 2)
 fa_decode_split_fp8_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                            const DecodeParams p) {
@@ -51,8 +52,7 @@ fa_decode_split_fp8_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
 
     const int tid = threadIdx.x;
     const int warp = uniform(tid >> 5), lane = tid & 31;
-    const int c = blockIdx.y;
-    const int b = blockIdx.z;
+    int c = blockIdx.y, b = blockIdx.z;   // (kDecBalanced: found below)
     const int g_all = p.Hq / p.Hkv;
     const int n_sub = (g_all + 15) / 16;           // CTAs per kv head when more than 16 heads share it
     const int hk = blockIdx.x / n_sub;
@@ -69,12 +69,24 @@ fa_decode_split_fp8_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
         tma_prefetch_desc(&tm_v);
     }
     grid_dep_wait();
-    int len = p.seqlens[b];
-    len = max(0, min(len, p.Smax));
-    const int k_begin = c * p.chunk;
-    const int k_end = min(len, k_begin + p.chunk);
+    int len, chunk = p.chunk;
+    if constexpr (kMode == kDecBalanced) {
+        const DecBalance bal(p, lane);
+        if (!bal.find(blockIdx.y, b, c, len)) return;   // (the same for all warps)
+        chunk = bal.unit * kDecTile;
+    } else {
+        len = max(0, min(p.seqlens[b], p.Smax));
+    }
+    const int k_begin = c * chunk;
+    const int k_end = min(len, k_begin + chunk);
+    // head h0 + r's place among the partial results
+    auto part_index = [&](int r) -> long long {
+        return kMode == kDecBalanced ? (long long)blockIdx.y * p.Hq + h0 + r : ((long long)b * p.Hq + h0 + r) * p.n_chunks + c;
+    };
     if (k_begin >= k_end) {  // uniform for the CTA
-        if (p.o_final != nullptr && c == 0 && tid < 128) {   // a sequence without keys, and nobody else writes its rows
+        if (kMode == kDecBalanced) {
+            if (tid < G) p.lse_part[part_index(tid)] = -INFINITY;
+        } else if (p.o_final != nullptr && c == 0 && tid < 128) {   // a sequence without keys, and nobody else writes its rows
             for (int r = 0; r < G; ++r) {
                 // (sixteen zero bits are 0.0 in fp16 and in bf16)
                 static_cast<__half*>(p.o_final)[((long long)b * p.Hq + h0 + r) * 128 + tid] = __half(0.f);
@@ -195,7 +207,7 @@ fa_decode_split_fp8_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
             const int st = t % kDec8Stages;
             const uint32_t parity = (t / kDec8Stages) & 1;
             const int valid = min(kDecTile, k_end - (k_begin + t * kDecTile)) - key_w;  // valid keys of this warp's 32
-            const float drop = kCluster && (t & (p.ref_tiles - 1)) == 0 ? p.ref_drop : 0.f;   // see DecodeParams
+            const float drop = kMode != kDecPlain && (t & (p.ref_tiles - 1)) == 0 ? p.ref_drop : 0.f;   // see DecodeParams
             ok = mbar_wait(smem_u32(&bars[st]), parity, &abort_flag, 20);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
@@ -366,7 +378,7 @@ fa_decode_split_fp8_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
                 float lse;
                 const float4 out = dec_warp_merge<128>(mo, ml, r, col, p.scale_log2, p.v_scale, lse);
                 const long long row = (long long)b * p.Hq + h0 + r;
-                if (kCluster) {
+                if (kMode == kDecCluster) {
                     *reinterpret_cast<float4*>(&part[r * 128 + col]) = out;
                     if (col == 0) part_lse[r] = lse;
                 } else if (p.o_final != nullptr) {   // the only chunk: this is the result
@@ -374,14 +386,14 @@ fa_decode_split_fp8_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
                     else dec_store4<__half>(p.o_final, row * 128 + col, out);
                     if (col == 0 && p.lse_final) p.lse_final[row] = lse;
                 } else {
-                    const long long slot = row * p.n_chunks + c;
+                    const long long slot = part_index(r);
                     *reinterpret_cast<float4*>(&p.o_part[slot * 128 + col]) = out;
                     if (col == 0) p.lse_part[slot] = lse;
                 }
             }
         }
     }
-    if constexpr (kCluster) {
+    if constexpr (kMode == kDecCluster) {
         const int n_live = (len + p.chunk - 1) / p.chunk;
         dec_cluster_merge<128>(part, part_lse, G, c, n_live, tid, [&](int r, int col, const float4& out, float lse) {
             const long long row = (long long)b * p.Hq + h0 + r;

@@ -440,9 +440,9 @@ int decode_chunk(int B, int Hkv, int Smax, bool long_ok = false) {
 
 // The clusters of a decode kernel that run at a time; kind: 0 = 16-bit, d = 128; 1 = 16-bit, d = 64; 2 = 8-bit.
 int decode_cluster_slots(int kind, fa::ClusterSlots* out) {
-    const void* kern = kind == 2   ? reinterpret_cast<const void*>(fa::fa_decode_split_fp8_kernel<1, true>)
-                       : kind == 1 ? reinterpret_cast<const void*>(fa::fa_decode_split_mma_kernel<false, __half, 64, true, true>)
-                                   : reinterpret_cast<const void*>(fa::fa_decode_split_mma_kernel<false, __half, 128, true, true>);
+    const void* kern = kind == 2   ? reinterpret_cast<const void*>(fa::fa_decode_split_fp8_kernel<1, fa::kDecCluster>)
+                       : kind == 1 ? reinterpret_cast<const void*>(fa::fa_decode_split_mma_kernel<false, __half, 64, true, fa::kDecCluster>)
+                                   : reinterpret_cast<const void*>(fa::fa_decode_split_mma_kernel<false, __half, 128, true, fa::kDecCluster>);
     const int smem = kind == 2 ? fa::kDec8Smem : kind == 1 ? fa::DecShape<64>::kSmem : fa::DecShape<128>::kSmem;
     const int ce = fa::cluster_slots(kern, smem, fa::kDecMmaThreads, out);
     return ce ? cuda_fail(static_cast<cudaError_t>(ce)) : FA_OK;
@@ -453,13 +453,16 @@ int decode_cluster_slots(int kind, fa::ClusterSlots* out) {
 struct DecodePlan {
     int chunk = 256, n_chunks = 1;
     bool clustered = false;
-    int plain_chunk = 256;   // keys per chunk without the cluster
+    int plain_chunk = 256;   // keys per chunk without the cluster, or the balancing
+    int slots = 0, most_tiles = 0;   // chunks cut on the device (see DecBalance); slots is 0 otherwise
     void fill(fa::DecodeParams* dp) const {   // (after scale_log2)
         dp->chunk = chunk;
         dp->n_chunks = n_chunks;
         dp->clustered = clustered;
+        dp->slots = slots;
+        dp->most_tiles = most_tiles;
         // (with next to no scale all scores count alike and no probability is rounded)
-        if (clustered && dp->scale_log2 > 1e-20f) {
+        if ((clustered || slots > 0) && dp->scale_log2 > 1e-20f) {
             dp->ref_tiles = plain_chunk / fa::kDecTile;
             dp->ref_drop = fa::kDecRefDropLog2 / dp->scale_log2;
         }
@@ -498,6 +501,25 @@ int decode_plan(int kind, int sms, long long ctas, int B, int Hkv, int Smax, boo
                 pl.n_chunks = (tiles + per - 1) / per;
                 pl.clustered = pl.n_chunks > 1;
             }
+        }
+    }
+    // Chunks cut by the device, out of the lengths that it finds.  The rule above makes 120 CTAs and more out of sequences as
+    // long as the longest: of sequences of different lengths, where chunks are long or two CTAs share an SM, those are
+    // too few.  One CTA for each place (us, by the longest / by the lengths): 12 x 5 heads of up to 5861 keys 27.0 / 21.8, all of
+    // 5861 32.7 / 31.1; 9 x 32/8, 4 tokens, up to 4266 31.3 / 18.5; 8-bit 28 x 5 up to 7562 34.8 / 27.6, all of 7562 47.0 / 47.0; 8-bit 7 x 8 up
+    // to 19641 35.7 / 30.2, 6 x 32/8 up to 31690 34.6 / 28.5.  Finding the lengths takes about a microsecond in both
+    // kernels: 16-bit chunks of 2048 keys and less stay (2 x 8 of up to 18909 12.8 / 10.8, but 7 x 32/8, 2 tokens, up to 4773 14.0 / 15.1,
+    // 8 x 8 of 4000 23.4 / 24.0); so do calls of four rounds of CTAs and more, whose CTAs balance as they end.
+    if (!pl.clustered && pl.n_chunks > 1 && (kind != 0 || pl.chunk >= 4096) && B <= fa::kDecBalancedSeqs &&
+        (long long)B * Hkv * ((Smax + 2047) / 2048) < 4ll * 148) {
+        const int ws_chunk = decode_chunk(B, Hkv, Smax);   // what the workspace is sized for
+        const long long room = (long long)B * ((Smax + ws_chunk - 1) / ws_chunk), run = (long long)sms * (kind == 0 ? 1 : 2) / (ctas / B);
+        const int slots = (int)(run < room ? run : room), per_seq = slots / B;
+        if (per_seq >= 2 && (tiles + per_seq - 1) / per_seq <= 32) {
+            pl.plain_chunk = pl.chunk;
+            pl.slots = slots;
+            pl.most_tiles = (tiles + per_seq - 1) / per_seq;
+            pl.n_chunks = (slots + B - 1) / B;   // (partial results of a sequence, on average)
         }
     }
     *plan = pl;
@@ -827,7 +849,8 @@ int decode_check_args(const void* q, const void* k_cache, const void* v_cache, c
 // writes are visible.
 template <typename T, int D>
 cudaError_t launch_combine(const fa::DecodeParams& dp, int blocks, void* o, float* lse, cudaStream_t st) {
-    return fa::launch_dependent(fa::fa_decode_combine_kernel<T, D>, dim3(blocks), D, 0, st, dp, static_cast<T*>(o), lse);
+    return fa::launch_dependent(dp.slots > 0 ? fa::fa_decode_combine_kernel<T, D, true> : fa::fa_decode_combine_kernel<T, D, false>, dim3(blocks), D, 0, st, dp,
+                                static_cast<T*>(o), lse);
 }
 
 // Launch of the split kernel and of the merge for one head dimension.
@@ -841,17 +864,18 @@ int decode_launch(const CUtensorMap& tk, const CUtensorMap& tv, const fa::Decode
         // at most 8 (token, head) rows per kv head: the keys-as-rows form of the consumers
         const bool key_rows = g * Sq <= 8;
         using Kernel = void (*)(CUtensorMap, CUtensorMap, fa::DecodeParams);
-        // by type, several query rows, consumer form, and whether the chunks of a sequence are one cluster
-        static const Kernel kernels[2][2][2][2] = {
-#define FA_DEC(T, M, R) {fa::fa_decode_split_mma_kernel<M, T, D, R, false>, fa::fa_decode_split_mma_kernel<M, T, D, R, true>}
+        // by type, several query rows, consumer form, and how the sequences are cut
+        static const Kernel kernels[2][2][2][3] = {
+#define FA_DEC(T, M, R) {fa::fa_decode_split_mma_kernel<M, T, D, R, fa::kDecPlain>, fa::fa_decode_split_mma_kernel<M, T, D, R, fa::kDecCluster>, fa::fa_decode_split_mma_kernel<M, T, D, R, fa::kDecBalanced>}
             {{FA_DEC(__half, false, false), FA_DEC(__half, false, true)}, {FA_DEC(__half, true, false), FA_DEC(__half, true, true)}},
             {{FA_DEC(__nv_bfloat16, false, false), FA_DEC(__nv_bfloat16, false, true)},
              {FA_DEC(__nv_bfloat16, true, false), FA_DEC(__nv_bfloat16, true, true)}}};
 #undef FA_DEC
-        const Kernel kern = kernels[bf16][Sq > 1][key_rows][dp.clustered != 0];
+        const Kernel kern = kernels[bf16][Sq > 1][key_rows][dp.slots > 0 ? fa::kDecBalanced : dp.clustered ? fa::kDecCluster : fa::kDecPlain];
         if (int ce = fa::prepare_big_smem_kernel(reinterpret_cast<const void*>(kern), smem, &sm_count))
             return cuda_fail(static_cast<cudaError_t>(ce));
         dim3 grid(Hkv * ((g * Sq + 15) / 16), dp.n_chunks, B);   // 16 (token, head) rows per CTA
+        if (dp.slots > 0) grid.y = dp.slots, grid.z = 1;
         const cudaError_t e = fa::launch_dependent_clusters(kern, grid, 1, dp.clustered ? dp.n_chunks : 1, fa::kDecMmaThreads, smem, st, tk, tv, dp);
         if (e != cudaSuccess) return cuda_fail(e);
     }
@@ -892,7 +916,7 @@ int decode_impl(const void* q, const void* k_cache, const void* v_cache, void* o
     plan.fill(&dp);
     if (dp.n_chunks > 65535) return FA_ERR_UNSUPPORTED;   // the chunks are the grid's second dimension
     dp.o_part = static_cast<float*>(workspace);
-    dp.lse_part = dp.o_part + (size_t)B * Sq * Hq * dp.n_chunks * d;
+    dp.lse_part = dp.o_part + (size_t)Sq * Hq * (dp.slots > 0 ? (size_t)dp.slots : (size_t)B * dp.n_chunks) * d;
     dp.block_table = block_table;
     dp.page_size = block_table ? page_size : 1;
     dp.table_stride = table_stride;
@@ -962,7 +986,7 @@ static int decode_fp8_impl(const void* q, const void* k_cache, const void* v_cac
     plan.fill(&dp);
     if (dp.n_chunks > 65535) return FA_ERR_UNSUPPORTED;   // the chunks are the grid's second dimension
     dp.o_part = static_cast<float*>(workspace);
-    dp.lse_part = dp.o_part + (size_t)B * Hq * dp.n_chunks * 128;
+    dp.lse_part = dp.o_part + (size_t)Hq * (dp.slots > 0 ? (size_t)dp.slots : (size_t)B * dp.n_chunks) * 128;
     dp.block_table = block_table;
     dp.page_size = block_table ? page_size : 1;
     dp.table_stride = table_stride;
@@ -985,11 +1009,15 @@ static int decode_fp8_impl(const void* q, const void* k_cache, const void* v_cac
         constexpr int smem = fa::kDec8Smem;
         int sm_count = 0;
         // keys as the MMA's rows and up to 8 query heads as its columns (two column blocks for 9..16 heads)
-        auto kern = dp.clustered ? ((g > 8) ? fa::fa_decode_split_fp8_kernel<2, true> : fa::fa_decode_split_fp8_kernel<1, true>)
-                                 : ((g > 8) ? fa::fa_decode_split_fp8_kernel<2, false> : fa::fa_decode_split_fp8_kernel<1, false>);
+        using Kernel = void (*)(CUtensorMap, CUtensorMap, fa::DecodeParams);
+        static const Kernel kernels[2][3] = {
+            {fa::fa_decode_split_fp8_kernel<1, fa::kDecPlain>, fa::fa_decode_split_fp8_kernel<1, fa::kDecCluster>, fa::fa_decode_split_fp8_kernel<1, fa::kDecBalanced>},
+            {fa::fa_decode_split_fp8_kernel<2, fa::kDecPlain>, fa::fa_decode_split_fp8_kernel<2, fa::kDecCluster>, fa::fa_decode_split_fp8_kernel<2, fa::kDecBalanced>}};
+        const Kernel kern = kernels[g > 8][dp.slots > 0 ? fa::kDecBalanced : dp.clustered ? fa::kDecCluster : fa::kDecPlain];
         if (int ce = fa::prepare_big_smem_kernel(reinterpret_cast<const void*>(kern), smem, &sm_count))
             return cuda_fail(static_cast<cudaError_t>(ce));
         dim3 grid(Hkv * ((g + 15) / 16), dp.n_chunks, B);
+        if (dp.slots > 0) grid.y = dp.slots, grid.z = 1;
         const cudaError_t e = fa::launch_dependent_clusters(kern, grid, 1, dp.clustered ? dp.n_chunks : 1, fa::kDec8Threads, smem, st, tk, tv, dp);
         rc = e == cudaSuccess ? FA_OK : cuda_fail(e);
         if (rc) return rc;

@@ -1533,6 +1533,37 @@ def test_decode_chunks_in_one_cluster(fa, B, hq, hkv, smax, d):
         assert_close_to_oracle(o[:, 0], lse, o_ref, l_ref, what=f"cluster fp8 B{B} {hkv} {smax}")
 
 
+@pytest.mark.parametrize("B,hq,hkv,smax,d", [(12, 5, 5, 4500, 128), (9, 8, 8, 4300, 128), (28, 5, 5, 4300, 64), (32, 4, 4, 4200, 128), (33, 4, 4, 4200, 128),
+                                             (2, 16, 8, 9000, 128), (4, 68, 4, 14500, 128)])
+def test_decode_chunks_cut_by_the_lengths(fa, B, hq, hkv, smax, d):
+    # long chunks, or two CTAs to an SM: the device cuts chunks of one length out of the lengths it finds; sequences
+    # without keys, of one key, on and off whole tiles, of the full length; lanes of the last sequences (32, and 33, which
+    # is cut by the longest).  One and three query rows, fp16 and (d = 128) the FP8 cache; exact workspaces, guarded.
+    cfg = synth.DecodeConfig("t", B, hq, hkv, smax, 1, smax, d=d, seed=2100 + B + smax)
+    q, k, v, sl = synth.decode_inputs(cfg, "cpu", poison=False)
+    for b, n in enumerate([smax, 0, 1, 128, 129]):
+        if b < B:
+            sl[b] = n
+    kn, vn = k.clone(), v.clone()
+    for b in range(B):
+        kn[b, int(sl[b]):] = float("nan")
+        vn[b, int(sl[b]):] = float("nan")
+    o_ref, l_ref = oracle.decode(q, k, v, sl, cfg.scale)
+    o, lse = run_decode(fa, q.to(DEV), kn.to(DEV), vn.to(DEV), sl.to(DEV), cfg.scale)
+    assert_close_to_oracle(o[:, 0], lse, o_ref, l_ref, what=f"balanced decode B{B} {hkv} {smax}")
+    if smax < 10000:
+        q3 = torch.cat([q, q.flip(2), -q], dim=1)
+        o_ref, l_ref = oracle.decode_append(q3, k, v, sl, cfg.scale)
+        o, lse = run_decode_append(fa, q3.to(DEV), kn.to(DEV), vn.to(DEV), sl.to(DEV), cfg.scale)
+        assert_close_to_oracle(o, lse, o_ref, l_ref, what=f"balanced append B{B} {hkv} {smax}")
+    if d == 128:
+        k8, v8 = synth.fp8_cache(k, v, sl, 0.25, 0.125)
+        kc, vc = synth.fp8_cache(k, v, sl, 0.25, 0.125, poison=False)
+        o_ref, l_ref = oracle.decode_fp8(q, kc, vc, sl, cfg.scale, 0.25, 0.125)
+        o, lse = run_decode_fp8(fa, q.to(DEV), k8.to(DEV), v8.to(DEV), sl.to(DEV), cfg.scale, 0.25, 0.125)
+        assert_close_to_oracle(o[:, 0], lse, o_ref, l_ref, what=f"balanced fp8 B{B} {hkv} {smax}")
+
+
 @pytest.mark.parametrize("causal", [False, True])
 @pytest.mark.parametrize("B,hq,hkv,sq,skv,dtype", [(1, 2, 2, 1500, 1500, "fp16"), (1, 3, 3, 1279, 1281, "fp16"), (1, 8, 1, 128, 4000, "bf16"),
                                                    (1, 1, 1, 1, 2100, "fp16"), (1, 1, 1, 100, 1300, "bf16"), (2, 4, 2, 300, 1500, "fp16"),
