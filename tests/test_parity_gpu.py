@@ -232,6 +232,30 @@ def test_bhsd_strided_layout(fa, variant):
     assert_close_to_oracle(o, lse, o_ref, l_ref, what="BHSD views")
 
 
+
+@pytest.mark.parametrize("causal", [False, True])
+@pytest.mark.parametrize("B,hq,hkv,sq,skv,dtype", [(40, 16, 4, 128, 128, "fp16"), (24, 16, 16, 250, 250, "bf16"), (20, 16, 8, 384, 384, "fp16"),
+                                                   (14, 16, 16, 129, 300, "fp16"), (10, 16, 2, 513, 513, "bf16")])
+def test_outputs_of_short_items_one_after_the_other(fa, B, hq, hkv, sq, skv, dtype, causal):
+    # several items of one to five steps on every CTA: an item's output is staged in the V slot of its last step while
+    # the next items' loads, products and epilogues go on; ragged last tiles.  Every element against the simple
+    # kernel, as closely as two kernels that round P and O to 16 bits agree (each is within TOL_O, of bf16 2^-8 of the
+    # output and of sum P |V| more: |O| <= 5 here), the sums to fp32; the packed form, same items, bit for bit.
+    cfg = synth.PrefillConfig("t", B, hq, hkv, sq, skv, dtype=dtype, causal=causal, seed=2300 + sq + skv)
+    q, k, v = synth.prefill_inputs(cfg, DEV)
+    o1, l1 = run_forward(fa, q, k, v, causal, cfg.scale)
+    o2, l2 = run_forward(fa, q, k, v, causal, cfg.scale, variant=2)
+    tol = 2 * TOL_O + (2 * 5 * 2.0 ** -8 if dtype == "bf16" else 0.0)
+    assert float((o1.float() - o2.float()).abs().max()) <= tol
+    assert float((l1 - l2).abs().max()) <= 2 * TOL_LSE
+    o3, l3 = torch.empty_like(q).flatten(0, 1), torch.empty(hq, B * sq, device=DEV)
+    cu_q, cu_k = (torch.arange(B + 1, dtype=torch.int32, device=DEV) * n for n in (sq, skv))
+    fa.fa_forward_varlen(q.flatten(0, 1), k.flatten(0, 1), v.flatten(0, 1), o3, l3, cu_q, cu_k, sq, skv, causal, cfg.scale)
+    torch.cuda.synchronize()
+    check_status(fa)
+    assert torch.equal(o3, o1.flatten(0, 1)) and torch.equal(l3.view(hq, B, sq).transpose(0, 1), l1)
+
+
 @pytest.mark.parametrize("variant", [0, 3, 4])
 def test_output_aligned_to_16_but_not_32_bytes(fa, variant):
     # rows that start on a 16-byte but not a 32-byte boundary take the 128-bit store path of the
