@@ -225,18 +225,15 @@ fa::FwdParams dense_fwd_params(const fa_params& p) {
     return fp;
 }
 
-// Head dimension 64: keys from which the ping-pong kernel is used (128 < Skv <= 256 has the
-// short-sequence pipeline of its own, up to 128 keys the kernel with four small CTAs per SM).  Timed on both sides:
-// from 257 keys on the ping-pong kernel, 64 x 12 x 257 55.7 us, and 3 to 37 % ahead of the small one from 300 keys
-// on.  129 to 256 keys: the pipeline ahead nearly everywhere, 1024 x 12 x 197 392 against 532 us, 64 x 12 x 144
-// 22.0 / 32.9, 1024 x 12 x 256 498 / 535, 64 x 12 x 224 30.3 / 33.6, but 64 x 12 x 256 33.5 / 31.5.  Up to 128
-// keys neither everywhere: the small kernel ahead on calls of less than a round (9.0 / 9.2) and on up to 64 keys
-// (1024 x 12 x 64 173 / 179, x 32 158 / 174), the ping-pong kernel on many sequences of 128 (64 x 12 x 128 17.8 /
-// 13.7, 1024 x 12 x 128 210 / 192), which it only tied before its items of few steps got shorter.
-#ifndef FA_D64_PINGPONG_FROM
-#define FA_D64_PINGPONG_FROM 257
-#endif
-constexpr int kD64PingPongFrom = FA_D64_PINGPONG_FROM;
+// Head dimension 64, which kernel: timed on both sides (us, the other kernel / the ping-pong kernel, inputs of the small calls in L2).
+// More than 256 keys: the ping-pong kernel, 3 to 37 % ahead of the small one (four CTAs per SM).  129 to 256 keys: the short-sequence
+// pipeline, 64 x 12 x 144 21.2 / 30.1, x 197 26.4 / 30.6, x 240 29.9 / 31.0, 512 x 12 x 197 189 / 252, x 256 237 / 253 (but 64 x 12 x 256
+// 32.7 / 29.0).  Up to 128 keys: the ping-pong kernel where the query tiles are more than the SMs, 16 x 12 x 128 9.1 / 9.0, 25 x 12 x 128 11.7 /
+// 9.0, 64 x 12 x 128 17.3 / 11.3, 64 x 12 x 50 15.2 / 11.5, 1024 x 12 x 100 223 / 139, 256 x 12 x 30 42.2 / 32.0, 64 x 12 of 256 over 128 29.1 / 18.1, fp32
+// output 64 x 12 x 128 24.2 / 20.8; the small one below that, 12 x 12 x 128 8.9 / 9.1, 4 x 12 x 100 8.8 / 9.0.
+bool d64_takes_pingpong(const fa::FwdParams& fp, int sms) {
+    return fp.Skv > 256 || (fp.Skv <= fa::kTile && (long long)fp.n_qtiles * fp.B * fp.Hq > sms);
+}
 
 int forward_impl(const fa_params& in, cudaStream_t st) {
     fa_params p = in;
@@ -293,7 +290,7 @@ int forward_impl(const fa_params& in, cudaStream_t st) {
     // ahead there too: 16 x 64/8 x 200 49.9 / 56.2, 16 x 32 x 256 29.3 / 34.2, 64 x 32 x 256 126.1 / 126.2,
     // 64 x 32 x 197 112.8 / 129.0, 128 x 32/8 x 256 213 / 225.
     int variant = p.variant;
-    if (variant == 0 && p.d == 64) variant = p.Skv >= kD64PingPongFrom ? 3 : 0;
+    if (variant == 0 && p.d == 64) variant = d64_takes_pingpong(fp, sms) ? 3 : 0;
     else if (variant == 0 && p.d == 128) {
         const bool two_by_two = fp.n_qtiles == 2 && p.Skv > fa::kTile && p.Skv <= 2 * fa::kTile;
         variant = (fp.o_fp32 && !p.causal && two_by_two && 2ll * p.B * p.Hq >= 3ll * sms) ? 4 : 3;
@@ -322,7 +319,7 @@ int forward_impl(const fa_params& in, cudaStream_t st) {
         return bf16 ? fa::launch_d64_stream<__nv_bfloat16>(tq, tk, tv, fp, st, &t_last_cuda_error)
                     : fa::launch_d64_stream<__half>(tq, tk, tv, fp, st, &t_last_cuda_error);
     }
-    if (p.d == 64) {  // one CTA per (batch, head, query tile), four CTAs per SM
+    if (p.d == 64) {  // few tiles: one CTA per (batch, head, query tile), four CTAs per SM
         auto kern = bf16 ? fa::fa_fwd_d64_slim_kernel<__nv_bfloat16> : fa::fa_fwd_d64_slim_kernel<__half>;
         int sm_count = 0;
         if (int ce = fa::prepare_big_smem_kernel(reinterpret_cast<const void*>(kern), fa::kD64SlimSmem, &sm_count))

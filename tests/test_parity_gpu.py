@@ -424,6 +424,31 @@ def test_d64_shape_grid(fa, sq, skv, causal):
     full_case_d64(fa, 2, 3, 3, sq, skv, causal, "fp16", seed=sq * 1000 + skv + 11)
 
 
+@pytest.mark.parametrize("causal", [False, True])
+@pytest.mark.parametrize("sq,skv", [(1, 1), (1, 128), (16, 100), (64, 64), (65, 65), (127, 127), (128, 128), (129, 128), (300, 70)])
+def test_d64_up_to_128_keys_of_many_sequences(fa, sq, skv, causal):
+    # more query tiles than SMs: the ping-pong kernel, with one kv tile per item (both types, fp32 output with bf16, grouped
+    # heads); then the same out of one [B, S, 3, H, 64] tensor into every second row, against the kernel for few tiles a sequence at a time
+    if causal and sq > skv:
+        sq = skv
+    full_case_d64(fa, 40, 8, 8, sq, skv, causal, "fp16", seed=2500 + sq + skv)
+    full_case_d64(fa, 60, 6, 3, sq, skv, causal, "bf16", seed=2600 + sq + skv)
+    if sq != skv:
+        return
+    qkv = torch.randn(40, sq, 3, 8, 64, generator=torch.Generator().manual_seed(sq)).half().to(DEV)
+    q, k, v = qkv.unbind(2)
+    o = torch.full((40, 2 * sq, 8, 64), float("nan"), dtype=torch.float16, device=DEV)
+    lse = torch.empty(40, 8, sq, device=DEV)
+    fa.fa_forward_ex(q, k, v, o[:, ::2], lse, causal, 0.125)
+    torch.cuda.synchronize()
+    check_status(fa)
+    assert torch.isnan(o[:, 1::2]).all()
+    for b in range(0, 40, 13):
+        o1, l1 = run_forward(fa, q[b:b + 1].contiguous(), k[b:b + 1].contiguous(), v[b:b + 1].contiguous(), causal, 0.125)
+        assert float((o[b:b + 1, ::2].float() - o1.float()).abs().max()) <= 2 * TOL_O
+        assert float((lse[b:b + 1] - l1).abs().max()) <= 2 * TOL_LSE
+
+
 def test_d64_short_sequence_kernel(fa):
     # 128 < Skv <= 256: all keys as one tile, a persistent pipeline over (batch, head, two query
     # tiles).  More items than CTAs, with one or two query tiles each, many query tiles over few
