@@ -5,9 +5,10 @@
 // N-major operand.  Three kernels:
 //   fa_fwd_d64_stream_kernel (prefill_d64_stream.cuh)  128 < Skv <= 256: all keys as one tile,
 //                            single-pass softmax, a persistent pipeline over (batch, head, two query tiles)
-//   fa_fwd_pingpong_kernel   (prefill_pingpong.cuh, D = 64)  longer sequences and packed batches
-//   fa_fwd_d64_slim_kernel   (here) any Skv, used up to 128 keys: online softmax over 128-key
-//                            tiles, one thread per query row, O kept in registers
+//   fa_fwd_pingpong_kernel   (prefill_pingpong.cuh, D = 64)  longer sequences, packed batches, and up
+//                            to 128 keys where the query tiles are more than the SMs
+//   fa_fwd_d64_slim_kernel   (here) any Skv, used up to 128 keys by the calls of fewer tiles: online
+//                            softmax over 128-key tiles, one thread per query row, O kept in registers
 #pragma once
 
 #include "prefill_simple.cuh"
