@@ -827,8 +827,9 @@ fa_decode_combine_kernel(const DecodeParams p, T* o, float* lse) {
     // lse is [B,Hq,Sq]
     const long long lse_at = ((long long)b * p.Hq + bh % p.Hq) * p.Sq + (bh / p.Hq) % p.Sq;
     const int tid = threadIdx.x;
-    // The lengths may be read before the wait: this kernel starts when every CTA of the split kernel has ended, and those have
-    // waited for whoever wrote the lengths.  (Without a split kernel, as there are no keys, Smax is 0.)
+    // The split kernel's partial results are complete and visible from here on, and so is what came before it.  (The
+    // lengths too: that every CTA of the split kernel has waited for whoever wrote them orders those CTAs, not this kernel.)
+    grid_dep_wait();
     int nc;
     long long at = (long long)bh * p.n_chunks, step = 1;   // this row's first partial result, and how far the next one is
     if constexpr (kBalanced) {
@@ -841,7 +842,6 @@ fa_decode_combine_kernel(const DecodeParams p, T* o, float* lse) {
         const int len = max(0, min(p.seqlens[b], p.Smax));
         nc = (len + p.chunk - 1) / p.chunk;
     }
-    grid_dep_wait();   // the split kernel's partial results are complete and visible from here on
     const float* lp = p.lse_part + at;
     const float* op = p.o_part + at * D;
     // One pass, some chunks at a time, whose loads are all on their way together; the weights are relative to the

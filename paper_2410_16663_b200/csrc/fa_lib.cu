@@ -841,9 +841,9 @@ int decode_check_args(const void* q, const void* k_cache, const void* v_cache, c
 }
 
 // Launch of the merge kernel as a programmatic dependent of the split kernel before it in the
-// stream: its launch is processed while the split kernel still runs, and its blocks start (they
-// wait in griddepcontrol.wait) when the last block of the split kernel has finished and its
-// writes are visible.
+// stream: its launch is processed while the split kernel still runs, its blocks start when the last
+// block of the split kernel has ended, and read nothing before they have waited for its writes
+// (griddepcontrol.wait).
 template <typename T, int D>
 cudaError_t launch_combine(const fa::DecodeParams& dp, int blocks, void* o, float* lse, cudaStream_t st) {
     return fa::launch_dependent(dp.slots > 0 ? fa::fa_decode_combine_kernel<T, D, true> : fa::fa_decode_combine_kernel<T, D, false>, dim3(blocks), D, 0, st, dp,

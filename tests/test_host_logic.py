@@ -1,6 +1,7 @@
 """Host-side logic of the CUDA sources that can run without a GPU: compiled as host code with
 nvcc (the image has it; no device is touched) and executed."""
 import os
+import re
 import shutil
 import subprocess
 import sys
@@ -44,6 +45,22 @@ def test_kernels_read_nothing_through_the_non_coherent_path():
         for n, line in enumerate(open(os.path.join(csrc, name)), 1):
             code = line.split("//")[0]
             assert "__ldg" not in code and "global.nc" not in code, f"{name}:{n}: {line.strip()}"
+
+
+def test_kernels_read_no_lengths_tables_or_partials_before_they_wait():
+    """What a kernel before wrote is visible to a programmatic dependent behind its own wait only."""
+    csrc = os.path.join(ROOT, "paper_2410_16663_b200", "csrc")
+    kernels = 0
+    for name in sorted(os.listdir(csrc)):
+        text = re.sub(r"//[^\n]*", "", open(os.path.join(csrc, name)).read())
+        for body in text.split("__global__")[1:]:
+            if "grid_dep_wait();" not in body:   # (waits in a function of its own, or is launched in order)
+                continue
+            kernels += 1
+            early = body[:body.index("grid_dep_wait();")]
+            read = re.search(r"(seqlens|block_table|table|cu_[qk]|\w+_part|\blp|\bop)\s*\[|\bDecBalance\s+\w+\s*\(", early)
+            assert read is None, f"{name}: {read.group(0)} ahead of the wait"
+    assert kernels >= 6
 
 
 def test_paged_from_packed_keeps_every_row_where_the_table_says():

@@ -245,6 +245,52 @@ def test_calls_that_read_what_the_call_before_wrote(fa, form):  # noqa: F811
     assert all(torch.equal(a, b) for a, b in zip(*ends))
 
 
+# 120 CTAs each, fewer than the SMs, and a merge kernel: chunks of one length out of the longest sequence's, and out of the lengths
+# that the device finds (one and three tokens, 8-bit keys)
+@pytest.mark.parametrize("B,Hkv,smax,sq,fp8", [(3, 1, 40000, 1, False), (12, 5, 5861, 1, False), (12, 5, 5861, 3, False), (7, 8, 19641, 1, True)],
+                         ids=["by the longest", "by the lengths", "by the lengths, 3 tokens", "by the lengths, 8-bit"])
+def test_decodes_whose_lengths_are_written_right_before(fa, B, Hkv, smax, sq, fp8):  # noqa: F811
+    # Each call's lengths are written on the device right before it, in another order than the call before had them, and its
+    # queries are the output of that call: one by one, and queued up behind a call that outlasts their enqueueing, bit for bit.
+    near = Neighbour(fa, 4, 524288)
+    k, v = (_rand((B, smax, Hkv, 128), torch.float16, s) for s in (61, 62))
+    if fp8:
+        k, v = (t.to(torch.float8_e4m3fn).view(torch.uint8) for t in (k, v))
+    lens = [smax, sq, 128, 129] + [max(sq, smax * (2 * b + 1) // (2 * B + 3)) for b in range(B)]
+    orders = [torch.tensor((lens * 2)[i:i + B], dtype=torch.int32).to(DEV) for i in range(len(lens))]
+    sl = torch.zeros(B, dtype=torch.int32, device=DEV)
+    ws = torch.empty(fa.fa_decode_append_workspace_bytes(B, sq, Hkv, Hkv, smax, 128) + 16, dtype=torch.uint8, device=DEV)
+    x0 = _rand((B, sq, Hkv, 128), torch.float16, 63)
+    ends = []
+    for alone in (True, False):
+        bufs, seen = [x0.clone(), torch.full_like(x0, float("nan"))], []
+        sl.zero_()
+        ws.fill_(0xff)   # NaNs
+        near.run()
+        torch.cuda.synchronize()
+        gone = torch.cuda.Event()
+        if not alone:
+            near.run()
+            gone.record()
+        for i in range(20):
+            src, dst = bufs[i & 1], bufs[1 - (i & 1)]
+            sl.copy_(orders[i % len(lens)])
+            if fp8:
+                fa.fa_decode_fp8(src, k, v, dst, None, sl, 0.3, 1.0, 1.0, ws)
+            else:
+                fa.fa_decode_ex(src, k, v, dst, None, sl, 0.3, ws)
+            if alone:
+                seen.append(dst.clone())
+                torch.cuda.synchronize()
+        assert alone or not gone.query()   # else the calls did not queue up and nothing has been tested
+        torch.cuda.synchronize()
+        check_status(fa)
+        for a, b in zip(seen, seen[1:]):
+            assert torch.isfinite(a).all() and torch.isfinite(b).all() and not torch.equal(a, b)
+        ends.append(bufs)
+    assert all(torch.equal(a, b) for a, b in zip(*ends))
+
+
 @pytest.fixture(scope="module")
 def early_release(tmp_path_factory):
     """early_release(ns, src, dst): see gpu_helpers/early_release.cu; on the current stream."""
