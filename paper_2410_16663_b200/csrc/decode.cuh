@@ -59,11 +59,14 @@ struct DecodeParams {
     // Tiles (a power of two) after which the reference of the probabilities, the running max, is lowered
     // by ref_drop.  The probabilities are rounded to 16 bits for the second product, all but that of the
     // key that sets the reference, which is exactly 1: the fewer keys share a reference, the smaller is
-    // the rounding error.  Chunks that are longer only because a sequence is one cluster's (see
-    // decode_plan) lower it where they would end without the cluster, so that the next keys set their
+    // the rounding error.  Chunks that are longer only because a sequence is one cluster's, or because the
+    // device cuts them (see decode_plan), lower it where they would end otherwise, so that the next keys set their
     // own (1 sequence, 5 heads, 8192 keys: 2.54e-4 from the result in 64 bits, 2.61e-4 without this).
-    // What has been summed grows by up to 2^6 each time; a cluster's chunks are at most eight times as
-    // long as without it, so it stays far inside fp32.
+    // What has been summed grows by up to 2^6 each time.  With 16-bit caches by no more than 2^42 in all, however long the
+    // chunk is (see dec_lowered): the sums of probabilities stay far inside fp32, and those of the values times them do
+    // for values up to 2^74.  8-bit values are below 2^9, and their chunks lower it 15 times at most, by 2^90 (see
+    // DecodePlan::fill; the limit in the kernel cost two column blocks 3 %: 8 x 64/2 over 27389 keys 38.9 -> 40.3 us.  The
+    // 16-bit kernels are level with it: 1 x 5 over 8192 8.4 / 8.4, 12 x 5 over up to 5861 23.9 / 23.9).
     int ref_tiles = 1 << 30;
     float ref_drop = 0.f;   // kDecRefDropLog2 / scale_log2
     // Chunks cut by the sequences' own lengths (kDecBalanced, see DecBalance): CTAs per kv head over all
@@ -131,6 +134,14 @@ struct DecTileLayout {
         return (D / 64 - 1) * box * block + (uint32_t)key * 128u;
     }
 };
+
+// The reference of a row (its running max, m) lowered by `drop` (see DecodeParams::ref_tiles), but no further than seven
+// times that below the highest one that the chunk has had, `top`: keys whose scores do not reach up to there weigh
+// less than 2^-42 of that one.
+__device__ __forceinline__ float dec_lowered(float m, float& top, float drop) {
+    top = fmaxf(top, m);
+    return fmaxf(m - drop, fmaf(-7.f, drop, top));
+}
 
 // How a call's sequences are cut: every DecodeParams::chunk keys (kDecPlain), the chunks of a sequence the CTAs of a cluster
 // (kDecCluster), or by the lengths that the device finds (kDecBalanced).
@@ -302,6 +313,7 @@ __device__ __forceinline__ bool dec_consume_key_rows(const DecodeParams& p, uint
 #pragma unroll
     for (int i = 0; i < D / 16; ++i) o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f;
     float m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f};  // heads 2 t4 and 2 t4 + 1
+    float top[2] = {-INFINITY, -INFINITY};   // (kLower: see dec_lowered)
     const int key_w = warp * 32;  // this warp's keys inside a tile
     bool ok = true;
     // this lane's key of each block of 16, for the K and for the V matrices
@@ -313,7 +325,7 @@ __device__ __forceinline__ bool dec_consume_key_rows(const DecodeParams& p, uint
         const int st = t % kStages;
         const uint32_t parity = (t / kStages) & 1;
         const int valid = min(kDecTile, k_end - (k_begin + t * kDecTile)) - key_w;  // valid keys of this warp's 32
-        const float drop = kLower && (t & (p.ref_tiles - 1)) == 0 ? p.ref_drop : 0.f;   // see DecodeParams
+        const bool lower = kLower && (t & (p.ref_tiles - 1)) == 0;   // see DecodeParams
         ok = mbar_wait(smem_u32(&bars[st]), parity, abort_flag, 20);
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
@@ -359,7 +371,8 @@ __device__ __forceinline__ bool dec_consume_key_rows(const DecodeParams& p, uint
             }
             // finite when key 0 of the warp is visible (always with one query token; an earlier
             // token of several may see none of the warp's keys: its state then stays empty)
-            const float mn0 = fmaxf(m_run[0] - drop, mx0), mn1 = fmaxf(m_run[1] - drop, mx1);
+            const float mn0 = fmaxf(lower ? dec_lowered(m_run[0], top[0], p.ref_drop) : m_run[0], mx0);
+            const float mn1 = fmaxf(lower ? dec_lowered(m_run[1], top[1], p.ref_drop) : m_run[1], mx1);
             const float a0 = (m_run[0] == -INFINITY) ? 0.f : fast_exp2((m_run[0] - mn0) * p.scale_log2);
             const float a1 = (m_run[1] == -INFINITY) ? 0.f : fast_exp2((m_run[1] - mn1) * p.scale_log2);
             m_run[0] = mn0;
@@ -635,6 +648,7 @@ fa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
 #pragma unroll
         for (int i = 0; i < D / 8; ++i) o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f;
         float m_lo = -INFINITY, m_hi = -INFINITY, l_lo = 0.f, l_hi = 0.f;  // rows g and g + 8
+        float top_lo = -INFINITY, top_hi = -INFINITY;   // (not kDecPlain: see dec_lowered)
         const int key_w = warp * 32;  // this warp's keys inside a tile
         const DecTileLayout<D> lay(p);
 
@@ -642,7 +656,7 @@ fa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
             const int st = t % kStages;
             const uint32_t parity = (t / kStages) & 1;
             const int valid = min(kDecTile, k_end - (k_begin + t * kDecTile)) - key_w;  // valid keys of this warp's 32
-            const float drop = kMode != kDecPlain && (t & (p.ref_tiles - 1)) == 0 ? p.ref_drop : 0.f;   // see DecodeParams
+            const bool lower = kMode != kDecPlain && (t & (p.ref_tiles - 1)) == 0;   // see DecodeParams
             ok = mbar_wait(smem_u32(&bars[st]), parity, &abort_flag, 20);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
@@ -691,7 +705,8 @@ fa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
                 mx_hi = fmaxf(mx_hi, __shfl_xor_sync(0xffffffffu, mx_hi, 2));
                 // finite when key 0 of the warp is visible (always with one query row; an earlier
                 // token of several may see none of the warp's keys: its state then stays empty)
-                const float mn_lo = fmaxf(m_lo - drop, mx_lo), mn_hi = fmaxf(m_hi - drop, mx_hi);
+                const float mn_lo = fmaxf(lower ? dec_lowered(m_lo, top_lo, p.ref_drop) : m_lo, mx_lo);
+                const float mn_hi = fmaxf(lower ? dec_lowered(m_hi, top_hi, p.ref_drop) : m_hi, mx_hi);
                 const float a_lo = (m_lo == -INFINITY) ? 0.f : fast_exp2((m_lo - mn_lo) * p.scale_log2);
                 const float a_hi = (m_hi == -INFINITY) ? 0.f : fast_exp2((m_hi - mn_hi) * p.scale_log2);
                 m_lo = mn_lo;

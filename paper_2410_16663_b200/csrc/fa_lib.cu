@@ -452,7 +452,7 @@ struct DecodePlan {
     bool clustered = false;
     int plain_chunk = 256;   // keys per chunk without the cluster, or the balancing
     int slots = 0, most_tiles = 0;   // chunks cut on the device (see DecBalance); slots is 0 otherwise
-    void fill(fa::DecodeParams* dp) const {   // (after scale_log2)
+    void fill(fa::DecodeParams* dp, bool kv8) const {   // (after scale_log2)
         dp->chunk = chunk;
         dp->n_chunks = n_chunks;
         dp->clustered = clustered;
@@ -461,6 +461,8 @@ struct DecodePlan {
         // (with next to no scale all scores count alike and no probability is rounded)
         if ((clustered || slots > 0) && dp->scale_log2 > 1e-20f) {
             dp->ref_tiles = plain_chunk / fa::kDecTile;
+            const int most = slots > 0 ? most_tiles : chunk / fa::kDecTile;   // tiles of a chunk
+            while (kv8 && (long long)dp->ref_tiles * 16 < most) dp->ref_tiles *= 2;
             dp->ref_drop = fa::kDecRefDropLog2 / dp->scale_log2;
         }
     }
@@ -910,7 +912,7 @@ int decode_impl(const void* q, const void* k_cache, const void* v_cache, void* o
     rc = decode_plan(d == 64 ? 1 : 0, sms, (long long)B * Hkv * ((g * Sq + 15) / 16), B, Hkv, Skv_max, true, &plan);
     if (rc) return rc;
     dp.scale_log2 = scale * 1.4426950408889634f;
-    plan.fill(&dp);
+    plan.fill(&dp, false);
     if (dp.n_chunks > 65535) return FA_ERR_UNSUPPORTED;   // the chunks are the grid's second dimension
     dp.o_part = static_cast<float*>(workspace);
     dp.lse_part = dp.o_part + (size_t)Sq * Hq * (dp.slots > 0 ? (size_t)dp.slots : (size_t)B * dp.n_chunks) * d;
@@ -980,7 +982,7 @@ static int decode_fp8_impl(const void* q, const void* k_cache, const void* v_cac
     rc = decode_plan(2, sms, (long long)B * Hkv * ((g + 15) / 16), B, Hkv, Skv_max, false, &plan);
     if (rc) return rc;
     dp.scale_log2 = scale * k_scale * 1.4426950408889634f;   // the scores are q . (k_scale * k8)
-    plan.fill(&dp);
+    plan.fill(&dp, true);
     if (dp.n_chunks > 65535) return FA_ERR_UNSUPPORTED;   // the chunks are the grid's second dimension
     dp.o_part = static_cast<float*>(workspace);
     dp.lse_part = dp.o_part + (size_t)Hq * (dp.slots > 0 ? (size_t)dp.slots : (size_t)B * dp.n_chunks) * 128;

@@ -1613,6 +1613,37 @@ def test_decode_chunks_cut_by_the_lengths(fa, B, hq, hkv, smax, d):
         assert_close_to_oracle(o[:, 0], lse, o_ref, l_ref, what=f"balanced fp8 B{B} {hkv} {smax}")
 
 
+# (chunks of 14 and of 32 tiles by the lengths instead of 2 by the longest; clusters with chunks of 64 tiles instead of 2, of one
+# row block and, 16 tiles, keys as rows; 8-bit, up to 128 tiles)
+@pytest.mark.parametrize("B,tokens,hq,smax,d,fp8", [(2, 32, 8, 16128, 64, False), (2, 64, 8, 16128, 64, False), (1, 64, 8, 32768, 128, False),
+                                                    (1, 1, 1, 32768, 128, False), (1, 1, 512, 32768, 128, True), (1, 1, 2048, 32768, 128, True)])
+def test_decode_first_key_outweighs_all_others_with_large_values(fa, B, tokens, hq, smax, d, fp8):
+    # One key's score is 120 nats above all others': the output is its value and the log-sum-exp its score, to fp32.  Chunks
+    # that lower the probabilities' reference behind that key scale what they have summed up by 2^6 each
+    # time, values of 2^50 among it, and have to stay finite.
+    gen = torch.Generator(device=DEV).manual_seed(2700 + tokens)
+    q = (1 + torch.randn(B, tokens, hq, d, generator=gen, device=DEV) / 16).to(torch.float16 if fp8 else torch.bfloat16)
+    k, v = (torch.randn(B, smax, 1, d, generator=gen, device=DEV).bfloat16() for _ in range(2))
+    k[:, 0] = 128.0 / d * 8
+    v[:, 0] = v[:, 0].clamp(-0.75, 0.75)
+    k8, v8 = (t.to(torch.float8_e4m3fn) for t in (k, v))
+    sl = torch.tensor([smax, smax - 77][:B], dtype=torch.int32, device=DEV)
+    o, lse = torch.empty_like(q), torch.empty(B, hq, tokens, device=DEV)
+    ws = torch.empty(fa.fa_decode_append_workspace_bytes(B, tokens, hq, 1, smax, d), dtype=torch.uint8, device=DEV)
+    if fp8:
+        fa.fa_decode_fp8(q, k8.view(torch.uint8), v8.view(torch.uint8), o, lse, sl, 0.125, 1.0, 1.0, ws)
+        want = v8.float()[:, :1].expand(o.shape)
+    else:
+        big = v * 2.0 ** 50   # exact
+        fa.fa_decode_ex(q, k, big, o, lse, sl, 0.125, ws)
+        want = big.float()[:, :1].expand(o.shape)
+    torch.cuda.synchronize()
+    check_status(fa)
+    assert torch.equal(o.float(), want)   # (within 2^-20 before it is rounded, and a number of the format)
+    score = (q.double() * k[:, :1].double()).sum(3).transpose(1, 2) * 0.125
+    assert float((lse.double() - score).abs().max()) <= TOL_LSE
+
+
 @pytest.mark.parametrize("causal", [False, True])
 @pytest.mark.parametrize("B,hq,hkv,sq,skv,dtype", [(1, 2, 2, 1500, 1500, "fp16"), (1, 3, 3, 1279, 1281, "fp16"), (1, 8, 1, 128, 4000, "bf16"),
                                                    (1, 1, 1, 1, 2100, "fp16"), (1, 1, 1, 100, 1300, "bf16"), (2, 4, 2, 300, 1500, "fp16"),
