@@ -389,6 +389,14 @@ int fa_device_status(unsigned int detail[2]);
  */
 int fa_selftest_wait(unsigned int limit_us, unsigned int* gave_up, void* stream);
 
+/*
+ * How a decode of these sizes is cut on the current device (kv8: an FP8 cache; nothing is launched, and no call depends on
+ * it): so that a test can tell which form of the kernels it reaches.  cut[0] = 0 chunks of one length, 1 a sequence's
+ * chunks are one cluster, 2 cut by the lengths that the device finds; cut[1] = chunks of a sequence (2: of all sequences
+ * together), cut[2] = tiles of 128 keys in the longest chunk, cut[3] = in a chunk of form 0.
+ */
+int fa_selftest_decode_cut(int B, int Sq, int Hq, int Hkv, int Skv_max, int d, int kv8, int cut[4]);
+
 const char* fa_strerror(int code);
 int fa_version(void);         /* major * 10000 + minor * 100 + patch */
 int fa_last_cuda_error(void); /* cudaError_t of the last failed CUDA call on this thread */

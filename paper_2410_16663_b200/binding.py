@@ -89,6 +89,8 @@ lib.fa_device_status.restype = _i
 lib.fa_device_status.argtypes = [ctypes.POINTER(ctypes.c_uint * 2)]
 lib.fa_selftest_wait.restype = _i
 lib.fa_selftest_wait.argtypes = [ctypes.c_uint, _p, _p]
+lib.fa_selftest_decode_cut.restype = _i
+lib.fa_selftest_decode_cut.argtypes = [_i, _i, _i, _i, _i, _i, _i, ctypes.POINTER(_i * 4)]
 lib.fa_strerror.restype = ctypes.c_char_p
 lib.fa_strerror.argtypes = [_i]
 lib.fa_version.restype = _i
@@ -98,7 +100,7 @@ FA_DECODE_NOALLOC_BYTES = 4 << 20
 
 EXPORTS = ["fa_forward", "fa_forward_bf16", "fa_forward_ex", "fa_forward_fp8", "fa_forward_proj", "fa_forward_proj_workspace_bytes", "fa_decode", "fa_decode_workspace_bytes",
            "fa_decode_noalloc", "fa_decode_paged", "fa_forward_varlen", "fa_decode_fp8", "fa_decode_fp8_paged", "fa_decode_fp8_bf16", "fa_decode_fp8_paged_bf16", "fa_decode_append", "fa_decode_append_workspace_bytes", "fa_decode_ex", "fa_forward_varlen_paged",
-           "fa_forward_host", "fa_forward_host_staging_bytes", "fa_device_status", "fa_selftest_wait", "fa_strerror",
+           "fa_forward_host", "fa_forward_host_staging_bytes", "fa_device_status", "fa_selftest_wait", "fa_selftest_decode_cut", "fa_strerror",
            "fa_version", "fa_last_cuda_error"]
 
 
@@ -396,3 +398,11 @@ def fa_device_status():
     detail = (ctypes.c_uint * 2)(0, 0)
     rc = int(lib.fa_device_status(ctypes.byref(detail)))
     return rc, int(detail[0]), int(detail[1])
+
+
+def fa_selftest_decode_cut(B: int, Sq: int, Hq: int, Hkv: int, Skv_max: int, d: int, kv8: bool = False):
+    """``fa_selftest_decode_cut``: (form, chunks, tiles of the longest chunk, tiles of a chunk of form 0) of a decode of these
+    sizes; form 0: chunks of one length, 1: a sequence's chunks are one cluster, 2: cut by the lengths the device finds."""
+    cut = (_i * 4)()
+    _check(lib.fa_selftest_decode_cut(B, Sq, Hq, Hkv, Skv_max, d, int(kv8), ctypes.byref(cut)), "fa_selftest_decode_cut", True)
+    return tuple(cut)

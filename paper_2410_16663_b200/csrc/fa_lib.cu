@@ -524,6 +524,10 @@ int decode_plan(int kind, int sms, long long ctas, int B, int Hkv, int Smax, boo
     *plan = pl;
     return FA_OK;
 }
+int decode_plan_of(bool kv8, int sms, int B, int Sq, int Hq, int Hkv, int Smax, int d, DecodePlan* plan) {
+    const int rows = Hq / Hkv * Sq;   // (token, head) rows that share a kv head
+    return decode_plan(kv8 ? 2 : d == 64 ? 1 : 0, sms, (long long)B * Hkv * ((rows + 15) / 16), B, Hkv, Smax, !kv8, plan);
+}
 
 }  // namespace
 
@@ -909,7 +913,7 @@ int decode_impl(const void* q, const void* k_cache, const void* v_cache, void* o
     dp.Sq = Sq;
     const int g = Hq / Hkv;
     DecodePlan plan;
-    rc = decode_plan(d == 64 ? 1 : 0, sms, (long long)B * Hkv * ((g * Sq + 15) / 16), B, Hkv, Skv_max, true, &plan);
+    rc = decode_plan_of(false, sms, B, Sq, Hq, Hkv, Skv_max, d, &plan);
     if (rc) return rc;
     dp.scale_log2 = scale * 1.4426950408889634f;
     plan.fill(&dp, false);
@@ -979,7 +983,7 @@ static int decode_fp8_impl(const void* q, const void* k_cache, const void* v_cac
     dp.B = B; dp.Hq = Hq; dp.Hkv = Hkv; dp.Smax = Skv_max;
     const int g = Hq / Hkv;
     DecodePlan plan;
-    rc = decode_plan(2, sms, (long long)B * Hkv * ((g + 15) / 16), B, Hkv, Skv_max, false, &plan);
+    rc = decode_plan_of(true, sms, B, 1, Hq, Hkv, Skv_max, d, &plan);
     if (rc) return rc;
     dp.scale_log2 = scale * k_scale * 1.4426950408889634f;   // the scores are q . (k_scale * k8)
     plan.fill(&dp, true);
@@ -1250,6 +1254,23 @@ int fa_selftest_wait(unsigned int limit_us, unsigned int* gave_up, void* stream)
     fa::fa_selftest_wait_kernel<<<1, 64, 0, static_cast<cudaStream_t>(stream)>>>(1000ull * limit_us, gave_up);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? FA_OK : cuda_fail(e);
+}
+
+int fa_selftest_decode_cut(int B, int Sq, int Hq, int Hkv, int Skv_max, int d, int kv8, int cut[4]) {
+    if (!cut) return FA_ERR_NULL;
+    if (B <= 0 || Sq < 1 || Hq <= 0 || Hkv <= 0 || Skv_max <= 0 || Hq % Hkv) return FA_ERR_SHAPE;
+    if ((d != 128 && d != 64) || (kv8 && (d != 128 || Sq != 1)) || Sq > 64) return FA_ERR_UNSUPPORTED;
+    int sms = 0;
+    int rc = check_device(&sms);
+    if (rc) return rc;
+    DecodePlan plan;
+    rc = decode_plan_of(kv8 != 0, sms, B, Sq, Hq, Hkv, Skv_max, d, &plan);
+    if (rc) return rc;
+    cut[0] = plan.slots > 0 ? fa::kDecBalanced : plan.clustered ? fa::kDecCluster : fa::kDecPlain;
+    cut[1] = plan.slots > 0 ? plan.slots : plan.n_chunks;
+    cut[2] = plan.slots > 0 ? plan.most_tiles : plan.chunk / fa::kDecTile;
+    cut[3] = (plan.slots > 0 || plan.clustered ? plan.plain_chunk : plan.chunk) / fa::kDecTile;
+    return FA_OK;
 }
 
 const char* fa_strerror(int code) {

@@ -293,6 +293,16 @@ def test_selftest_wait_validates_before_any_cuda_call(fa):
     assert fa.lib.fa_selftest_wait(100001, c.data_ptr(), None) == fa.FA_ERR_UNSUPPORTED
 
 
+def test_selftest_decode_cut_validates_before_any_cuda_call(fa):
+    cut = (ctypes.c_int * 4)()
+    L = fa.lib.fa_selftest_decode_cut
+    assert L(1, 1, 8, 8, 1000, 128, 0, None) == fa.FA_ERR_NULL
+    for bad in ((0, 1, 8, 8, 1000, 128, 0), (1, 0, 8, 8, 1000, 128, 0), (1, 1, 8, 3, 1000, 128, 0), (1, 1, 8, 8, 0, 128, 0)):
+        assert L(*bad, cut) == fa.FA_ERR_SHAPE
+    for bad in ((1, 1, 8, 8, 1000, 256, 0), (1, 65, 8, 8, 1000, 128, 0), (1, 2, 8, 8, 1000, 128, 1), (1, 1, 8, 8, 1000, 64, 1)):
+        assert L(*bad, cut) == fa.FA_ERR_UNSUPPORTED
+
+
 def test_forward_fp8_validation(fa):
     q = torch.zeros(1, 4, 4, 128, dtype=torch.uint8)
     o = torch.zeros(1, 4, 4, 128, dtype=torch.float16)

@@ -1613,6 +1613,64 @@ def test_decode_chunks_cut_by_the_lengths(fa, B, hq, hkv, smax, d):
         assert_close_to_oracle(o[:, 0], lse, o_ref, l_ref, what=f"balanced fp8 B{B} {hkv} {smax}")
 
 
+# (d, kv8, B, hq, hkv, smax, tokens, dtype, page): keys as rows and heads as rows, one token and several, more than one row block
+# per kv head, both types, contiguous and in pages of 16 and of one tile; the last three of d = 64 make longer chunks than
+# without the device's cut
+@pytest.mark.parametrize("d,kv8,B,hq,hkv,smax,sq,dtype,page", [
+    (128, False, 9, 32, 8, 4300, 1, "bf16", 0), (128, False, 9, 32, 8, 4300, 2, "fp16", 16), (128, False, 9, 32, 8, 4300, 2, "bf16", 128),
+    (128, False, 9, 32, 8, 4300, 4, "fp16", 0), (128, False, 9, 32, 8, 4300, 4, "bf16", 16), (128, False, 9, 32, 8, 4300, 4, "fp16", 128),
+    (128, False, 9, 72, 8, 4500, 1, "fp16", 128), (128, False, 9, 72, 8, 4500, 1, "bf16", 0),
+    (64, False, 28, 5, 5, 4300, 1, "bf16", 0), (64, False, 28, 5, 5, 4300, 1, "fp16", 16), (64, False, 16, 32, 8, 4500, 2, "bf16", 128),
+    (64, False, 16, 32, 8, 4500, 4, "fp16", 0), (64, False, 16, 32, 8, 4500, 4, "bf16", 16), (64, False, 16, 72, 8, 4500, 1, "fp16", 0),
+    (64, False, 15, 32, 1, 6564, 4, "bf16", 0), (64, False, 2, 32, 8, 18875, 8, "fp16", 128), (64, False, 2, 8, 1, 29144, 8, "bf16", 16),
+    (128, True, 28, 5, 5, 4300, 1, "bf16", 0), (128, True, 28, 5, 5, 4300, 1, "fp16", 16), (128, True, 16, 32, 8, 4500, 1, "bf16", 128),
+    (128, True, 16, 72, 8, 4500, 1, "fp16", 0), (128, True, 16, 72, 8, 4500, 1, "bf16", 16), (128, True, 5, 128, 4, 12769, 1, "fp16", 128),
+])
+def test_decode_every_form_cut_by_the_lengths(fa, d, kv8, B, hq, hkv, smax, sq, dtype, page):
+    if torch.cuda.get_device_properties(0).multi_processor_count == 148:   # (how many chunks run at once decides)
+        assert fa.fa_selftest_decode_cut(B, sq, hq, hkv, smax, d, kv8)[0] == 2
+    dt = torch.bfloat16 if dtype == "bf16" else torch.float16
+    gen = torch.Generator().manual_seed(2800 + B + hq + smax + sq)
+    q = torch.randn(B, sq, hq, d, generator=gen).to(dt)
+    k, v = (torch.randn(B, smax, hkv, d, generator=gen).to(dt) for _ in range(2))
+    sl = torch.randint(1, smax + 1, (B,), generator=gen, dtype=torch.int32)
+    for b, n in enumerate([smax, 0, 1, 128, 129]):
+        if b < B and B > 2:
+            sl[b] = n
+    scale = 1 / math.sqrt(d)
+    if kv8:
+        k, v = synth.fp8_cache(k, v, sl, 0.25, 0.125, poison=False)
+        o_ref, l_ref = oracle.decode_fp8(q, k, v, sl, scale, 0.25, 0.125)
+        o_ref, l_ref, absv, none = o_ref[:, None], l_ref[:, :, None], None, 0x7f
+    else:
+        o_ref, l_ref = oracle.decode_append(q, k, v, sl, scale)
+        absv, none = oracle.decode_append(q, k, v.abs(), sl, scale)[0] if dtype == "bf16" else None, float("nan")
+    if page:
+        there = synth.paged_cache(torch.ones_like(k), v, sl, page, seed=9, poison=False)[0] != 0
+        k, v, table = synth.paged_cache(k, v, sl, page, seed=9, poison=False)
+        table, most = table.to(DEV), table.shape[1] * page
+    else:
+        there = (torch.arange(smax)[None] < sl[:, None])[:, :, None, None].expand(k.shape)
+        table, most = None, smax
+    k, v = (t.masked_fill(~there, none).to(DEV) for t in (k, v))
+    o, chk_o = guard_alloc((B, sq, hq, d), dt, DEV)
+    lse, chk_l = guard_alloc((B, hq, sq), torch.float32, DEV)
+    ws, chk_w = guard_alloc((fa.fa_decode_append_workspace_bytes(B, sq, hq, hkv, most, d) // 4,), torch.float32, DEV)
+    q, sl = q.to(DEV), sl.to(DEV)
+    if kv8:
+        args = (o, lse, sl, scale, 0.25, 0.125, ws)
+        if page:
+            (fa.fa_decode_fp8_paged_bf16 if dtype == "bf16" else fa.fa_decode_fp8_paged)(q, k, v, table, *args)
+        else:
+            (fa.fa_decode_fp8_bf16 if dtype == "bf16" else fa.fa_decode_fp8)(q, k, v, *args)
+    else:
+        fa.fa_decode_ex(q, k, v, o, lse, sl, scale, ws, block_table=table)
+    torch.cuda.synchronize()
+    check_status(fa)
+    chk_o(); chk_l(); chk_w()
+    assert_close_to_oracle(o, lse, o_ref, l_ref, stored_bf16=dtype == "bf16", p_absv=absv, what="every form")
+
+
 # (chunks of 14 and of 32 tiles by the lengths instead of 2 by the longest; clusters with chunks of 64 tiles instead of 2, of one
 # row block and, 16 tiles, keys as rows; 8-bit, up to 128 tiles)
 @pytest.mark.parametrize("B,tokens,hq,smax,d,fp8", [(2, 32, 8, 16128, 64, False), (2, 64, 8, 16128, 64, False), (1, 64, 8, 32768, 128, False),
