@@ -502,22 +502,35 @@ int decode_plan(int kind, int sms, long long ctas, int B, int Hkv, int Smax, boo
             }
         }
     }
-    // Chunks cut by the device, out of the lengths that it finds.  The rule above makes 120 CTAs and more out of sequences as
-    // long as the longest: of sequences of different lengths, where chunks are long or two CTAs share an SM, those are
-    // too few.  One CTA for each place (us, by the longest / by the lengths): 12 x 5 heads of up to 5861 keys 27.0 / 21.8, all of
-    // 5861 32.7 / 31.1; 9 x 32/8, 4 tokens, up to 4266 31.3 / 18.5; 8-bit 28 x 5 up to 7562 34.8 / 27.6, all of 7562 47.0 / 47.0; 8-bit 7 x 8 up
-    // to 19641 35.7 / 30.2, 6 x 32/8 up to 31690 34.6 / 28.5.  Finding the lengths takes about a microsecond in both
-    // kernels: 16-bit chunks of 2048 keys and less stay (2 x 8 of up to 18909 12.8 / 10.8, but 7 x 32/8, 2 tokens, up to 4773 14.0 / 15.1,
-    // 8 x 8 of 4000 23.4 / 24.0); so do calls of four rounds of CTAs and more, whose CTAs balance as they end.
+    // Chunks cut by the device, of equal length out of the lengths that it finds.  The rule above makes 120 chunks and more out
+    // of sequences as long as the longest, some of them empty where the lengths differ.  The device spreads what there
+    // is over as many CTAs as run at once, or as the workspace has room for (what decode_chunk makes) if that is fewer.
+    // Finding the lengths takes about a microsecond in both kernels, which sequences of equal length pay for nothing (us,
+    // by the longest / by the lengths, different lengths and equal ones): 12 x 5 heads of up to 5861 keys 26.8 / 24.1, 32.6 / 31.9;
+    // 9 x 32/8, 4 tokens, 4266 31.4 / 21.6, 33.3 / 32.6; 8-bit 28 x 5 of 7562 35.3 / 32.9, 47.2 / 47.9, 4 x 32/8 of 20000 26.4 / 20.6, 34.3 / 35.1, 7
+    // x 8 of 19641 40.8 / 42.5, 47.9 / 48.4; d = 64 4 x 8 of 20000 21.8 / 19.8, 29.9 / 30.7, 7 x 8 of 9000 23.7 / 18.0, 26.6 / 25.6.
+    // So not where chunks are short, and there are many to merge: 16-bit, d = 128, chunks of 2048 keys and less (7 x 32/8, 2 tokens,
+    // 4773 14.0 / 15.1, 8 x 8 of 4000 23.4 / 24.0, but 2 x 8 of 18909 12.8 / 10.8), the others of 1024 and less (8-bit 4 x 8/1
+    // of 43306 14.1 / 16.5, 2 x 8/2 of 44647 14.1 / 15.1, d = 64 3 x 4/1 of 37440 13.1 / 16.4, but 8-bit 3 x 16/1 of 53058 20.4 / 19.4); and
+    // not in calls of four rounds of CTAs and more, which balance as they end.  Several row blocks per kv head make
+    // several rounds of CTAs out of chunks that are short already: then one round of longer chunks (d = 64, 2 x 8/1, 32
+    // tokens, 16128 29.4 / 15.1, 36.2 / 17.2, 6 x 64/2, 2 tokens, 19137 19.1 / 19.1, 32.2 / 25.4; 8-bit 8 x 64/2 of 27389 45.5 / 32.6, 45.5 / 39.0), unless equal
+    // lengths would leave many places without one, as whole chunks per sequence do not add up to a round: by the tiles of
+    // the longest chunk over those per place, 8-bit 1.32 14 x 128/4 of 7589 29.0 / 32.0, 48.0 / 49.5, 1.20 2 x 512/16 of 9255 27.0 / 24.5, 30.8
+    // / 33.4, 1.16 17 x 32/1 of 13413 18.4 / 18.3, 30.4 / 26.5, but 1.40 27 x 64/2 of 5160 28.1 / 25.5, 37.3 / 37.7; d = 64 1.51 5 x 40/5, 8 tokens, 5409
+    // 13.6 / 15.3, 21.3 / 24.0, 1.53 25 x 32/2, 2 tokens, 3860 13.1 / 14.0, 20.8 / 20.9, 1.35 7 x 256/8 of 6170 18.7 / 18.9, 31.2 / 27.0.
     if (!pl.clustered && pl.n_chunks > 1 && (kind != 0 || pl.chunk >= 4096) && B <= fa::kDecBalancedSeqs &&
-        (long long)B * Hkv * ((Smax + 2047) / 2048) < 4ll * 148) {
+        (long long)B * Hkv * ((Smax + 2047) / 2048) < 4ll * sms) {
+        const long long places = (long long)sms * (kind == 0 ? 1 : 2), run = places / (ctas / B);
         const int ws_chunk = decode_chunk(B, Hkv, Smax);   // what the workspace is sized for
-        const long long room = (long long)B * ((Smax + ws_chunk - 1) / ws_chunk), run = (long long)sms * (kind == 0 ? 1 : 2) / (ctas / B);
+        const long long room = (long long)B * ((Smax + ws_chunk - 1) / ws_chunk);
         const int slots = (int)(run < room ? run : room), per_seq = slots / B;
-        if (per_seq >= 2 && (tiles + per_seq - 1) / per_seq <= 32) {
+        const int most = per_seq >= 2 ? (tiles + per_seq - 1) / per_seq : 0;
+        const bool pays = most * fa::kDecTile <= pl.chunk ? pl.chunk >= 2048 : 100 * most * places <= (kind == 2 ? 130 : 145) * ctas * tiles;
+        if (per_seq >= 2 && most <= 32 && pays) {
             pl.plain_chunk = pl.chunk;
             pl.slots = slots;
-            pl.most_tiles = (tiles + per_seq - 1) / per_seq;
+            pl.most_tiles = most;
             pl.n_chunks = (slots + B - 1) / B;   // (partial results of a sequence, on average)
         }
     }

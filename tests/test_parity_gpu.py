@@ -1671,6 +1671,17 @@ def test_decode_every_form_cut_by_the_lengths(fa, d, kv8, B, hq, hkv, smax, sq, 
     assert_close_to_oracle(o, lse, o_ref, l_ref, stored_bf16=dtype == "bf16", p_absv=absv, what="every form")
 
 
+@pytest.mark.parametrize("B,sq,hq,hkv,smax,d,kv8,form", [
+    (28, 1, 5, 5, 7562, 128, True, 2), (2, 8, 8, 1, 29144, 64, False, 2), (8, 1, 64, 2, 27389, 128, True, 2),
+    # longer chunks that leave a third of the places idle; chunks of 1024 keys, all of which run at once
+    (5, 8, 40, 5, 5409, 64, False, 0), (14, 1, 128, 4, 7589, 128, True, 0), (4, 1, 8, 1, 43306, 128, True, 0), (3, 1, 4, 1, 37440, 64, False, 0),
+])
+def test_decode_is_cut_by_the_lengths_where_that_is_faster(fa, B, sq, hq, hkv, smax, d, kv8, form):
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("the forms are those of 148 SMs")
+    assert fa.fa_selftest_decode_cut(B, sq, hq, hkv, smax, d, kv8)[0] == form
+
+
 # (chunks of 14 and of 32 tiles by the lengths instead of 2 by the longest; clusters with chunks of 64 tiles instead of 2, of one
 # row block and, 16 tiles, keys as rows; 8-bit, up to 128 tiles)
 @pytest.mark.parametrize("B,tokens,hq,smax,d,fp8", [(2, 32, 8, 16128, 64, False), (2, 64, 8, 16128, 64, False), (1, 64, 8, 32768, 128, False),
