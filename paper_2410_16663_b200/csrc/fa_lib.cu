@@ -319,13 +319,12 @@ int forward_impl(const fa_params& in, cudaStream_t st) {
         return bf16 ? fa::launch_d64_stream<__nv_bfloat16>(tq, tk, tv, fp, st, &t_last_cuda_error)
                     : fa::launch_d64_stream<__half>(tq, tk, tv, fp, st, &t_last_cuda_error);
     }
-    if (p.d == 64) {  // few tiles: one CTA per (batch, head, query tile), four CTAs per SM
+    if (p.d == 64) {  // up to 128 keys, few tiles: one CTA per (batch, head, query tile), four of which fit on an SM
         auto kern = bf16 ? fa::fa_fwd_d64_slim_kernel<__nv_bfloat16> : fa::fa_fwd_d64_slim_kernel<__half>;
         int sm_count = 0;
         if (int ce = fa::prepare_big_smem_kernel(reinterpret_cast<const void*>(kern), fa::kD64SlimSmem, &sm_count))
             return cuda_fail(static_cast<cudaError_t>(ce));
         dim3 grid(fp.n_qtiles, fp.Hq, fp.B);
-        fp.early_next = (long long)fp.n_qtiles * fp.Hq * fp.B < 4ll * sm_count;
         const cudaError_t e = fa::launch_dependent(kern, grid, 128, fa::kD64SlimSmem, st, tq, tk, tv, fp);
         return e == cudaSuccess ? FA_OK : cuda_fail(e);
     }
