@@ -226,13 +226,16 @@ fa::FwdParams dense_fwd_params(const fa_params& p) {
 }
 
 // Head dimension 64, which kernel: timed on both sides (us, the other kernel / the ping-pong kernel, inputs of the small calls in L2).
-// More than 256 keys: the ping-pong kernel, 3 to 37 % ahead of the small one (four CTAs per SM).  129 to 256 keys: the short-sequence
+// More than 256 keys: the ping-pong kernel.  129 to 256 keys: the short-sequence
 // pipeline, 64 x 12 x 144 21.2 / 30.1, x 197 26.4 / 30.6, x 240 29.9 / 31.0, 512 x 12 x 197 189 / 252, x 256 237 / 253 (but 64 x 12 x 256
-// 32.7 / 29.0).  Up to 128 keys: the ping-pong kernel where the query tiles are more than the SMs, 16 x 12 x 128 9.1 / 9.0, 25 x 12 x 128 11.7 /
-// 9.0, 64 x 12 x 128 17.3 / 11.3, 64 x 12 x 50 15.2 / 11.5, 1024 x 12 x 100 223 / 139, 256 x 12 x 30 42.2 / 32.0, 64 x 12 of 256 over 128 29.1 / 18.1, fp32
-// output 64 x 12 x 128 24.2 / 20.8; the small one below that, 12 x 12 x 128 8.9 / 9.1, 4 x 12 x 100 8.8 / 9.0.
+// 32.7 / 29.0).  Up to 128 keys: the small kernel, four CTAs to an SM, where there are more query tiles than SMs and the keys are
+// no more than 64: 49 x 12 x 16 7.0 / 9.5, x 48 7.4 / 9.6, x 64 7.6 / 9.7, 25 x 12 x 48 7.2 / 7.7, 100 x 12 x 48 14.5 / 16.1, 400 x 12 x 16 43.3 / 47.7, x 64 49.9 /
+// 49.5, fp32 output 100 x 12 x 48 15.6 / 18.5, 25 x 12 x 64 9.7 / 9.4; the ping-pong kernel on fewer tiles (4 x 12 x 48 4.9 / 4.7, 12 x 12 x 48 5.3 / 5.4, 4 x
+// 12 x 128 5.2 / 4.7, 12 x 12 x 128 5.5 / 5.4) and on more keys (25 x 12 x 72 7.5 / 7.9, x 96 8.4 / 7.9, 49 x 12 x 96 8.7 / 10.0, 100 x 12 x 72 15.3 / 16.2, x 96
+// 17.4 / 16.4, x 128 21.5 / 15.5, 400 x 12 x 72 52.6 / 49.8, x 128 70.8 / 52.5).
 bool d64_takes_pingpong(const fa::FwdParams& fp, int sms) {
-    return fp.Skv > 256 || (fp.Skv <= fa::kTile && (long long)fp.n_qtiles * fp.B * fp.Hq > sms);
+    const bool small = fp.Skv <= 64 && (long long)fp.n_qtiles * fp.B * fp.Hq > sms;
+    return fp.Skv > 256 || (fp.Skv <= fa::kTile && !small);
 }
 
 int forward_impl(const fa_params& in, cudaStream_t st) {
@@ -319,12 +322,13 @@ int forward_impl(const fa_params& in, cudaStream_t st) {
         return bf16 ? fa::launch_d64_stream<__nv_bfloat16>(tq, tk, tv, fp, st, &t_last_cuda_error)
                     : fa::launch_d64_stream<__half>(tq, tk, tv, fp, st, &t_last_cuda_error);
     }
-    if (p.d == 64) {  // up to 128 keys, few tiles: one CTA per (batch, head, query tile), four of which fit on an SM
+    if (p.d == 64) {  // few keys, many tiles: one CTA per (batch, head, query tile), four of which fit on an SM
         auto kern = bf16 ? fa::fa_fwd_d64_slim_kernel<__nv_bfloat16> : fa::fa_fwd_d64_slim_kernel<__half>;
         int sm_count = 0;
         if (int ce = fa::prepare_big_smem_kernel(reinterpret_cast<const void*>(kern), fa::kD64SlimSmem, &sm_count))
             return cuda_fail(static_cast<cudaError_t>(ce));
         dim3 grid(fp.n_qtiles, fp.Hq, fp.B);
+        fp.early_next = (long long)fp.n_qtiles * fp.Hq * fp.B < 4ll * sm_count;
         const cudaError_t e = fa::launch_dependent(kern, grid, 128, fa::kD64SlimSmem, st, tq, tk, tv, fp);
         return e == cudaSuccess ? FA_OK : cuda_fail(e);
     }

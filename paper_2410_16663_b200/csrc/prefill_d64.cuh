@@ -5,10 +5,10 @@
 // N-major operand.  Three kernels:
 //   fa_fwd_d64_stream_kernel (prefill_d64_stream.cuh)  128 < Skv <= 256: all keys as one tile,
 //                            single-pass softmax, a persistent pipeline over (batch, head, two query tiles)
-//   fa_fwd_pingpong_kernel   (prefill_pingpong.cuh, D = 64)  longer sequences, packed batches, and up
-//                            to 128 keys where the query tiles are more than the SMs
-//   fa_fwd_d64_slim_kernel   (here) up to 128 keys, calls of fewer tiles: all keys as one tile, one
-//                            thread per query row
+//   fa_fwd_pingpong_kernel   (prefill_pingpong.cuh, D = 64)  longer sequences, packed batches, and most
+//                            calls of up to 128 keys
+//   fa_fwd_d64_slim_kernel   (here) few keys where the query tiles are more than the SMs: all keys as
+//                            one tile, one thread per query row
 #pragma once
 
 #include "prefill_simple.cuh"
@@ -21,7 +21,7 @@ constexpr int kD64TileBytes = 16384;   // 128 rows x 64 16-bit elements: one TMA
 // At most 128 keys, small enough for four CTAs per SM.  One CTA per (batch, head, query tile), 128
 // threads, 49 KiB of shared memory (a tile each of Q, K and V) and 128 columns of tensor memory: S
 // in [0,128), P packed over [0,64), and P V in [64,128) (columns of S the thread has read by
-// then).  The calls that come here have no more CTAs than SMs, so the next kernel may start at once.
+// then).
 constexpr int kD64SlimSmem = 1024 + 3 * kD64TileBytes;
 
 template <typename T>
@@ -67,7 +67,7 @@ fa_fwd_d64_slim_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    grid_dep_launch();
+    if (p.early_next) grid_dep_launch();
     const uint32_t tmem_base = tmem_holder;
     const uint32_t tS = tmem_base + (static_cast<uint32_t>(warp * 32) << 16);
 

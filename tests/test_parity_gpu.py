@@ -449,6 +449,17 @@ def test_d64_up_to_128_keys_of_many_sequences(fa, sq, skv, causal):
         assert float((lse[b:b + 1] - l1).abs().max()) <= 2 * TOL_LSE
 
 
+@pytest.mark.parametrize("causal", [False, True])
+@pytest.mark.parametrize("sq,skv", [(1, 1), (1, 64), (3, 5), (64, 50), (63, 63), (65, 64), (129, 64), (300, 33), (64, 65), (100, 128)])
+def test_d64_up_to_64_keys_of_many_and_of_few_sequences(fa, sq, skv, causal):
+    # more query tiles than SMs and up to 64 keys: the kernel with four CTAs to an SM; otherwise the ping-pong kernel
+    if causal and sq > skv:
+        sq = skv
+    for B in (50, 2):
+        full_case_d64(fa, B, 8, 8, sq, skv, causal, "fp16", seed=2900 + sq + skv)
+        full_case_d64(fa, B, 6, 3, sq, skv, causal, "bf16", seed=3000 + sq + skv)
+
+
 def test_d64_short_sequence_kernel(fa):
     # 128 < Skv <= 256: all keys as one tile, a persistent pipeline over (batch, head, two query
     # tiles).  More items than CTAs, with one or two query tiles each, many query tiles over few
