@@ -256,6 +256,14 @@ def test_outputs_of_short_items_one_after_the_other(fa, B, hq, hkv, sq, skv, dty
     assert torch.equal(o3, o1.flatten(0, 1)) and torch.equal(l3.view(hq, B, sq).transpose(0, 1), l1)
 
 
+@pytest.mark.parametrize("causal", [False, True])
+@pytest.mark.parametrize("B,hq,hkv,sq,skv,dtype", [(40, 16, 4, 128, 128, "fp16"), (24, 16, 16, 250, 250, "bf16"), (20, 16, 8, 384, 384, "fp16"),
+                                                   (14, 16, 16, 129, 300, "fp16"), (10, 16, 2, 513, 513, "bf16")])
+def test_outputs_of_short_items_against_the_oracle(fa, B, hq, hkv, sq, skv, dtype, causal):
+    # every element of the calls of test_outputs_of_short_items_one_after_the_other
+    full_case(fa, B, hq, hkv, sq, skv, causal, dtype, seed=2300 + sq + skv)
+
+
 @pytest.mark.parametrize("variant", [0, 3, 4])
 def test_output_aligned_to_16_but_not_32_bytes(fa, variant):
     # rows that start on a 16-byte but not a 32-byte boundary take the 128-bit store path of the
