@@ -62,8 +62,9 @@ struct PpOperands {
     static constexpr bool kOneBox = kF8 || D == 64;                     // a tile row is 128 bytes
     static constexpr int kKvSlotBytes = kOneBox ? 16384 : kTileBytes;   // one K ring slot, and the bytes of a K or V tile
     static constexpr int kVSlotBytes = D == 64 ? 16384 : kTileBytes;    // one V ring slot: a V tile, later an output tile
-    static constexpr int kQBytes = kOneBox ? 16384 : kTileBytes;        // one Q buffer, and the bytes of a Q tile
-    static constexpr int kSmem = kPpQBufs * kQBytes + kPpNK * kKvSlotBytes + kPpNV * kVSlotBytes;   // 224 KiB; 8-bit 144, d = 64 112
+    static constexpr int kQBytes = kOneBox ? 16384 : kTileBytes;        // bytes a Q load delivers
+    static constexpr int kQBufBytes = kF8 ? 16384 : kTileBytes;         // one Q buffer (d = 64 with 16 KiB: 512 x 12 x 128 66.4 -> 66.8 us)
+    static constexpr int kSmem = kPpQBufs * kQBufBytes + kPpNK * kKvSlotBytes + kPpNV * kVSlotBytes;   // 224 KiB; 8-bit and d = 64 144
     static constexpr int kSteps = kOneBox ? 4 : 8;                      // MMAs of Q K^T (32 bytes of every row each)
     static constexpr int kPvSteps = kF8 ? 4 : 8;                        // MMAs of P V (32 or 16 keys each)
     static constexpr int kPCols = kF8 ? 8 : 16;                         // tensor-memory columns of 32 probabilities
@@ -457,7 +458,7 @@ __device__ __forceinline__ void pp_run_s(uint32_t bar0, uint32_t sQ, uint32_t sK
         const int ord = items.ord;
         const uint32_t qb = ord & 1;
         if (!mbar_wait(pp_bar(bar0, ppb::q_full + qb), (ord >> 1) & 1, abort_flag, 130)) return;
-        const uint32_t a_lo = desc_lo(sQ + qb * Op::kQBytes, 16);
+        const uint32_t a_lo = desc_lo(sQ + qb * Op::kQBufBytes, 16);
         for (int j = 0; j < it.n; ++j, ++g, ring.next()) {
             const uint32_t buf = g & 1;
             if (!mbar_wait(pp_bar(bar0, ppb::k_full + ring.slot), ring.par, abort_flag, 131)) return;
@@ -594,7 +595,7 @@ __device__ __forceinline__ void pp_run_load_qk(uint32_t bar0, uint32_t sQ, uint3
         // passes at once the first time each buffer is used
         if (!mbar_wait(pp_bar(bar0, ppb::q_empty + qb), ((ord >> 1) & 1) ^ 1, abort_flag, 150)) return;
         mbar_expect_tx(pp_bar(bar0, ppb::q_full + qb), PpOperands<kF8, D>::kQBytes);
-        pp_load_tile<PpOperands<kF8, D>::kOneBox>(sQ + qb * PpOperands<kF8, D>::kQBytes, tm_q, pp_bar(bar0, ppb::q_full + qb), it.h,
+        pp_load_tile<PpOperands<kF8, D>::kOneBox>(sQ + qb * PpOperands<kF8, D>::kQBufBytes, tm_q, pp_bar(bar0, ppb::q_full + qb), it.h,
                        kVarlen ? it.q_base + it.q0 : it.q0, kVarlen ? 0 : it.b, pol_q);
         int page = (kVarlen && p.block_table != nullptr) ? it.page0 : 0;
         for (int j = 0; j < it.n; ++j, ring.next()) {
@@ -969,7 +970,7 @@ __device__ __forceinline__ bool pp_attention(const CUtensorMap& tm_q, const CUte
     static_assert(!kSplit || (!kTmaOut && !kVarlen && !kF8 && !kProj && D == 128), "one form shares query tiles");
     static_assert(!kProj || (kTmaOut && !kVarlen && D == 128), "the projection phase reads a contiguous 16-bit O of d = 128");
     const uint32_t sQ = smem_base;
-    const uint32_t sK = sQ + kPpQBufs * PpOperands<kF8, D>::kQBytes;
+    const uint32_t sK = sQ + kPpQBufs * PpOperands<kF8, D>::kQBufBytes;
     const uint32_t sV = sK + kPpNK * PpOperands<kF8, D>::kKvSlotBytes;
     const uint32_t bar0 = smem_u32(&ss.bars[0]);
     volatile uint32_t* abort_flag = &ss.abort_flag;
