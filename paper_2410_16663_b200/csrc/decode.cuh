@@ -33,13 +33,13 @@ struct DecShape {
 };
 
 struct DecodeParams {
-    const void* q;        // [B,1,Hq,d] 16-bit
+    const void* q;        // [B,Sq,Hq,d] 16-bit
     const int* seqlens;   // [B] device
-    float* o_part;        // [B,Hq,NC,d]
-    float* lse_part;      // [B,Hq,NC]
+    float* o_part;        // [B,Sq,Hq,n_chunks,d]; cut by the device (slots > 0): [slots,Sq,Hq,d], a chunk of any sequence in each
+    float* lse_part;      // the same without d
     int B, Hq, Hkv, Smax;
-    int chunk;            // keys per chunk (multiple of kDecTile)
-    int n_chunks;         // ceil(Smax / chunk)
+    int chunk;            // keys per chunk (multiple of kDecTile); cut by the device: what it would be otherwise
+    int n_chunks;         // ceil(Smax / chunk); cut by the device: the mean number per sequence, rounded up
     float scale_log2;
     // paged cache (block_table != nullptr): key j of sequence b is row j % page_size of page
     // block_table[b * table_stride + j / page_size]; the tensor maps then run over
@@ -148,8 +148,8 @@ __device__ __forceinline__ float dec_lowered(float m, float& top, float drop) {
 constexpr int kDecPlain = 0, kDecCluster = 1, kDecBalanced = 2;
 constexpr int kDecBalancedSeqs = 32;
 
-// Chunks of equal length for sequences of different lengths, as short as p.slots CTAs per kv head allow, which the
-// device runs at once: worked out from the lengths by every warp for itself, a sequence per lane.  The sequences take the
+// Chunks of equal length for sequences of different lengths, as short as p.slots CTAs per kv head allow (no more than the
+// device runs at once, and than the workspace has room for): worked out from the lengths by every warp for itself, a sequence per lane.  The sequences take the
 // CTAs one after the other, each at least one (it may have no keys).  (The loops are not unrolled: this runs once per CTA, and
 // fetching its instructions takes longer than executing them.)
 struct DecBalance {
@@ -465,7 +465,7 @@ __device__ __forceinline__ bool dec_consume_key_rows(const DecodeParams& p, uint
 // kMulti: Sq > 1 query rows per sequence, the last Sq positions of its cache (decoding after
 // several tokens were appended, Appendix C with more than one new token): the 16 MMA rows of a
 // CTA are then (token, head) pairs of one kv head, and query token t sees the keys up to
-// position len - Sq + t.  q is [B,Sq,Hq,d], the partials [B,Sq,Hq,NC,...].
+// position len - Sq + t.  q is [B,Sq,Hq,d], the partials see DecodeParams.
 // grid: (Hkv * ceil(Sq * g / 16), n_chunks, B), or (.., slots, 1) with kDecBalanced, with g = Hq / Hkv.  The kv head is the fastest
 // index: CTAs that run at the same time then read the same keys' rows of neighbouring heads,
 // which are contiguous in the cache (a key's Hkv * D elements), instead of key ranges whole

@@ -863,8 +863,7 @@ struct PpSoftmax {
 
 // Merge of the parts that a cluster's CTAs computed of one query tile: CTA `rank` of `split` finishes
 // rows rank, rank + split, ..., one warp per row and four columns per lane, reading the parts through
-// distributed shared memory.  (The spills of that kernel, 32 bytes stored and 76 loaded, are all this function's, which
-// runs once: without it there are none, with two rows at a time instead of four 16 and 48.)
+// distributed shared memory.
 constexpr uint32_t kPpPartStats = 65536;   // bytes from a part's O to its (max, sum) pairs
 template <typename T>
 __device__ __forceinline__ void pp_split_merge(const FwdParams& p, uint32_t part, int tid) {
@@ -1228,7 +1227,7 @@ fa_fwd_pingpong_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
                        const FwdParams p, const int total_items) {
     // Shared memory is used to the last byte: 3 KiB of static state (sized so that the dynamic
     // part that follows it starts on a 1024-byte boundary, which the 128-byte swizzle needs)
-    // plus seven 32 KiB tiles.  The alignment is checked rather than assumed.
+    // plus seven 32 KiB tiles (d = 128, 16 bits).  The alignment is checked rather than assumed.
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     __shared__ __align__(1024) uint8_t static_raw[kPpStaticBytes];
     PpStatic& ss = *reinterpret_cast<PpStatic*>(static_raw);

@@ -276,24 +276,23 @@ __device__ __forceinline__ void tma_store_wait_read() {
     asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
 }
 
-// ------------------------------------------------------------------ the issuing thread
-// A value that is the same in all lanes (all of them must be there), such as the warp's number, in a form that
-// the compiler knows to be: it then lives in uniform registers, and so do the addresses of barriers and
-// tensor memory that follow from it, which the instructions that take those want there.
-// (The warp's number: 4 x 32 x 2048 170.9 -> 168.3 us, 5 heads x 4096 30.2 -> 29.8, 32 x 32768 7429 -> 7320, 8-bit operands 8 x 32 x 512
+// ------------------------------------------------------------------ values that are the same in all lanes
+// A value that all lanes share (all of them must be there), such as the warp's number, taken from lane 0, so that the
+// compiler can tell that they do.
+// (The warp's number: 4 x 32 x 2048 170.9 -> 168.3 us, 8-bit operands 8 x 32 x 512
 // 27.7 -> 26.5, 4 x 32 x 2048 126 -> 121; d = 64 16 x 16 x 512 26.5 -> 25.4; decode of 8 x 32/8 over up to 4000 keys in pages of 16
-// 20.9 -> 20.1, with 4 tokens of 64/8 heads 29.7 -> 28.1, of 64 x 32/8 over up to 32768 8-bit keys 372 -> 366.)
+// 20.9 -> 20.1, with 4 tokens of 64/8 heads 29.7 -> 28.1, of 64 x 32/8 over up to 32768 8-bit keys 372 -> 366; 5 heads x 4096 and 32 x
+// 32768 level.)
 __device__ __forceinline__ int uniform(int x) { return __shfl_sync(0xffffffffu, x, 0); }
 
+// ------------------------------------------------------------------ the issuing thread
 // True in one lane of the warp, always the same one (all lanes must be there).  Whoever issues tcgen05 or TMA instructions for
-// its warp is chosen by this and not by its lane number: the compiler takes a branch on the election for one that a
-// single lane enters, and keeps the descriptors that these instructions take from uniform registers there from the
-// start.  Behind a comparison of the lane number it moves them over for every instruction.  Eight 128 x 128 x 16
-// products back to back, clocks to issue: 389 by lane number, 90 to 158 elected; S and P V of a step from two threads, to the end:
+// its warp is chosen by this and not by its lane number, as that is how fast they issue: eight 128 x 128 x 16
+// products back to back, clocks to issue, 389 by lane number, 90 to 158 elected; S and P V of a step from two threads, to the end:
 // 1134 to 1189, elected 1024 (which is what the tensor cores need).  1024 x 12 x 197, d = 64, 388.9 -> 366.5 us; d = 128: 8 x 32 x 512
 // 41.9 -> 40.8, 32 packed prompts 4113 -> 4084, 4 x 32 x 2048 with fp32 output 209 -> 202; d = 64 through the
 // ping-pong kernel, 16 x 16 x 512 26.6 -> 24.6; d = 256, 2 x 16 x 2048 103.4 -> 98.5; longer sequences of d = 128 level.
-// (Level, and left as they were: the decode kernels' loading threads, and the kernel for short d = 64 sequences, whose
+// (Level, and left as they were: the decode kernels' loading threads, and the kernel for few d = 64 keys, whose
 // issuing thread comes back to the others at every product.)
 __device__ __forceinline__ bool elect_one() {
     uint32_t p;
