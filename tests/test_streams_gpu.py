@@ -291,6 +291,42 @@ def test_decodes_whose_lengths_are_written_right_before(fa, B, Hkv, smax, sq, fp
     assert all(torch.equal(a, b) for a, b in zip(*ends))
 
 
+@pytest.mark.parametrize("B,Hkv,smax,sq", [(3, 1, 40000, 1), (12, 5, 5861, 2), (1, 5, 8192, 1)], ids=["by the longest", "by the lengths", "cluster"])
+def test_captured_decodes_take_the_lengths_of_the_replay(fa, B, Hkv, smax, sq):  # noqa: F811
+    # two decodes in one graph, the second with the first one's output as its queries; each replay bit for bit what the
+    # calls give with its lengths
+    k, v = (_rand((B, smax, Hkv, 128), torch.float16, s) for s in (71, 72))
+    q = _rand((B, sq, Hkv, 128), torch.float16, 73)
+    sl = torch.full((B,), smax, dtype=torch.int32, device=DEV)
+    ws = torch.empty(fa.fa_decode_append_workspace_bytes(B, sq, Hkv, Hkv, smax, 128) + 16, dtype=torch.uint8, device=DEV)
+    outs = [torch.empty_like(q), torch.empty_like(q), torch.empty(B, Hkv, sq, device=DEV)]
+
+    def calls():
+        fa.fa_decode_ex(q, k, v, outs[0], None, sl, 0.1, ws)
+        fa.fa_decode_ex(outs[0], k, v, outs[1], outs[2], sl, 0.3, ws)
+
+    calls()   # (set-up before the capture)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        calls()
+    seen = []
+    for lens in ([smax] * B, [smax // (b + 2) for b in range(B)], [1 + 128 * b for b in range(B)], [0] + [smax - 5] * (B - 1)):
+        sl.copy_(torch.tensor(lens, dtype=torch.int32))
+        ws.fill_(0xff)
+        calls()
+        want = [t.clone() for t in outs]
+        for t in outs:
+            t.fill_(float("nan"))
+        ws.fill_(0xff)
+        graph.replay()
+        torch.cuda.synchronize()
+        check_status(fa)
+        assert all(torch.equal(a, b) for a, b in zip(want, outs)) and not torch.isnan(outs[1]).any()
+        seen.append(want[1])
+    assert not any(torch.equal(a, b) for a, b in zip(seen, seen[1:]))
+
+
 @pytest.fixture(scope="module")
 def early_release(tmp_path_factory):
     """early_release(ns, src, dst): see gpu_helpers/early_release.cu; on the current stream."""
